@@ -1,0 +1,50 @@
+"""Canonical order of hashed results at the sizes and key ranges where the radix sort takes another path: one tile,
+one more, the most pieces, every number of digit passes, equal keys, lists in order already."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_07632_b200 as sjq
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(keys, capacity):
+    n = len(keys)
+    rng = np.random.default_rng(n)
+    allk = np.full(capacity, 5, dtype=np.int64)
+    allk[:n] = keys
+    sums, counts = rng.integers(-2**62, 2**62, capacity), rng.integers(0, 2**40, capacity)
+    res = sjq.Result("HASHED", torch.from_numpy(sums).cuda(), torch.from_numpy(counts).cuda(),
+                     torch.from_numpy(allk.copy()).cuda(), torch.tensor([n], dtype=torch.int64, device="cuda"),
+                     torch.zeros(1, dtype=torch.int32, device="cuda"), None)
+    res.sort()
+    order = np.concatenate([np.argsort(keys, kind="stable"), np.arange(n, capacity)])
+    for got, want in ((res.keys, allk), (res.sums, sums), (res.counts, counts)):
+        assert np.array_equal(got.cpu().numpy(), want[order])
+
+
+@pytest.mark.parametrize("n", [2, 31, 2047, 2048, 2049, 4095, 4096, 4097, 148 * 2048 - 1, 148 * 2048 + 1,
+                               148 * 4096 + 33, 2_000_003])
+def test_list_lengths_around_pieces_and_tiles(n):
+    keys = np.random.default_rng(n).permutation(n).astype(np.int64) * 0x9E3779B97F4A7 - 2**40
+    _check(keys, n + 7)
+
+
+@pytest.mark.parametrize("bits", [1, 8, 9, 16, 24, 33, 40, 48, 56, 63])
+def test_every_number_of_passes_with_equal_keys(bits):
+    n = 20_011
+    rng = np.random.default_rng(bits)
+    lo = -(2**(bits - 1)) + 12_345
+    keys = rng.integers(0, 2**bits - 1, n, endpoint=True, dtype=np.int64) + np.int64(lo)
+    keys[:2] = lo, lo + 2**bits - 1  # the whole range, so that the pass count is the intended one
+    keys[100:5_000] = keys[7]
+    _check(keys, 32_768)
+
+
+def test_list_in_order_and_list_of_equal_keys_stay_as_they_are():
+    _check(np.arange(100_000, dtype=np.int64) * 3 - 150_000, 131_072)
+    _check(np.full(10_000, -9, dtype=np.int64), 10_000)
+    swapped = np.arange(60_000, dtype=np.int64)
+    swapped[[2047, 2048]] = swapped[[2048, 2047]]  # out of order only across a piece's edge
+    _check(swapped, 60_000)
