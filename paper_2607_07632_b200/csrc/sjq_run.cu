@@ -54,7 +54,8 @@ struct StageSpec {
     int index;    // predicate or join index (-1 for loads)
     int col;      // fact column
     double sel;   // estimated fraction of rows passing
-    double cost;  // relative cost per row evaluated
+    int width;    // bytes of a value of the column
+    double cost;  // picoseconds per row evaluated, the column's bytes apart
     int prefilter; // 1: only the presence bitmap of a hashed join; 2: the exact probe that follows one
 };
 
@@ -91,9 +92,88 @@ bool valid_term(const sjq_term &t, int nfact, const sjq_join *joins, int njoins)
     return false;
 }
 
+// What a filter stage costs, in picoseconds per fact row on the whole chip (148 SMs, 1.9 GHz, 6.5 TB/s).
+constexpr double kPsByte = 0.154;  // a byte of DRAM traffic
+constexpr double kPsIssue = 0.3;   // evaluating a row (about ten instructions)
+constexpr double kPsShared = 0.4;  // a probe of a table staged in shared memory (random banks)
+constexpr double kPsGlobal = 3.4;  // a probe of a global table: 32 random lines take the L1 32 cycles, whatever hits
+constexpr double kPsFar = 10.0;    // ... of a table that the L2 cannot hold
+constexpr size_t kStageBytes = (size_t)32 << 10; // tables up to this size are copied into shared memory
+constexpr size_t kNearL2 = (size_t)64 << 20;
+
+// DRAM delivers 64-byte pieces: one of a column is read iff one of its rows is still alive.
+double column_ps(int width, double reach)
+{
+    double dead = 1.0 - std::min(1.0, reach);
+    for (int rows = 64 / width; rows > 1; rows >>= 1) dead *= dead;
+    return kPsByte * width * (1.0 - dead);
+}
+
+// The order of the filter stages with the least estimated time: the sum over the stages of the column's bytes
+// (once per column, at the share of rows that reach it) and of the probes.  The share depends only on which stages
+// came before, so the best order is found over subsets (up to 8 stages; one at a time, cheapest per row dropped
+// first, beyond).  Exact probes behind a presence bitmap go last: they run at the final level.
+// (Ranking by (1 - selectivity) / cost with one cost for every table below 200 KB left city x brand to chance: two
+// joins that keep one row in 25, one probing 25 KB in shared memory, the other 175 KB through the L1, which is
+// 0.67 or 3.3 ms for 600 M rows with the one or the other first.)
+std::vector<int> cheapest_order(const std::vector<StageSpec> &specs)
+{
+    constexpr int kExhaustive = 8;
+    const int n = (int)specs.size();
+    int early[64], m = 0;
+    std::vector<int> order;
+    order.reserve(n);
+    for (int i = 0; i < n; ++i)
+        if (specs[i].prefilter != 2) early[m++] = i;
+    auto cost = [&](int i, double reach, bool column_read) {
+        return (column_read ? 0.0 : column_ps(specs[i].width, reach)) + reach * specs[i].cost;
+    };
+    if (m <= kExhaustive) {
+        struct Best { double ps, reach; int last; } best[1 << kExhaustive];
+        unsigned same_col[kExhaustive]; // the stages that read the column of stage i
+        for (int i = 0; i < m; ++i) {
+            same_col[i] = 0;
+            for (int j = 0; j < m; ++j) same_col[i] |= (unsigned)(specs[early[j]].col == specs[early[i]].col) << j;
+        }
+        const unsigned all = (1u << m) - 1u;
+        for (unsigned set = 0; set <= all; ++set) best[set] = Best{set ? 1e300 : 0.0, 1.0, -1};
+        for (unsigned set = 0; set < all; ++set) {
+            for (int i = 0; i < m; ++i) {
+                if (set >> i & 1u) continue;
+                const double ps = best[set].ps + cost(early[i], best[set].reach, (same_col[i] & set) != 0);
+                Best &to = best[set | 1u << i];
+                if (ps < to.ps) to = Best{ps, best[set].reach * specs[early[i]].sel, i};
+            }
+        }
+        for (unsigned set = all; set; set ^= 1u << best[set].last) order.push_back(early[best[set].last]);
+        std::reverse(order.begin(), order.end());
+    } else {
+        double reach = 1.0;
+        std::vector<char> used(n, 0);
+        for (int k = 0; k < m; ++k) {
+            int pick = -1;
+            double least = 0.0;
+            for (int e = 0; e < m; ++e) {
+                const int i = early[e];
+                if (used[i]) continue;
+                bool column_read = false;
+                for (int j : order) column_read |= specs[j].col == specs[i].col;
+                const double per_drop = cost(i, reach, column_read) / std::max(1e-9, 1.0 - specs[i].sel);
+                if (pick < 0 || per_drop < least) pick = i, least = per_drop;
+            }
+            used[pick] = 1;
+            order.push_back(pick);
+            reach *= specs[pick].sel;
+        }
+    }
+    for (int i = 0; i < n; ++i)
+        if (specs[i].prefilter == 2) order.push_back(i);
+    return order;
+}
+
 // The filter stages of a query (its predicates and joins; a hashed join with a presence bitmap is two
-// stages) with estimated selectivities and relative costs, and the order they are evaluated in: the
-// caller's, or by rank (1 - selectivity) / cost.
+// stages) with estimated selectivities and costs, and the order they are evaluated in: the caller's, or
+// the cheapest.
 sjq_status order_stages(const sjq_col *fact, const sjq_pred *preds, int npreds, const sjq_join *joins, int njoins,
                         const sjq_run_opts &opts, std::vector<StageSpec> *specs_out, std::vector<int> *order_out)
 {
@@ -104,35 +184,38 @@ sjq_status order_stages(const sjq_col *fact, const sjq_pred *preds, int npreds, 
         const int32_t ppm = opts.pass_ppm[i];
         return ppm > 0 ? std::min(1.0, ppm / 1e6) : estimate;
     };
-    for (int p = 0; p < npreds; ++p) {
-        const double bytes = fact[preds[p].col].dtype == SJQ_I64 ? 2.0 : 1.0;
-        specs.push_back({ST_PRED, p, preds[p].col, hinted(p, pred_selectivity(preds[p])), bytes, 0});
-    }
+    for (int p = 0; p < npreds; ++p)
+        specs.push_back({ST_PRED, p, preds[p].col, hinted(p, pred_selectivity(preds[p])),
+                         fact[preds[p].col].dtype == SJQ_I64 ? 8 : 4, kPsIssue, 0});
     for (int j = 0; j < njoins; ++j) {
         const sjq_table *T = joins[j].table;
         const sjq_dim_layout &L = T->layout;
-        const double bytes = L.key_dtype == SJQ_I64 ? 2.0 : 1.0;
+        const int width = L.key_dtype == SJQ_I64 ? 8 : 4;
         const double sel = hinted(npreds + j, L.dim_rows > 0 ? (double)L.entries / (double)L.dim_rows : 0.0);
         // bytes a filter stage on this table touches: the presence bitmap when a direct table has one
-        const size_t tb = (is_direct_kind(L.kind) && L.filter_bits > 0 && T->filter && !opts.no_filter_bitmap)
-                              ? (size_t)(L.filter_bits / 8)
-                              : L.table_bytes;
-        // relative cost of one probe: a table the L1 mostly holds, one the L2 holds (measured on the four-join
-        // workload: the 3 MB map before the 175 KB bitmap when it drops twice as many rows), one in HBM
-        double probe = tb <= (size_t)200 << 10 ? 0.3 : tb <= (size_t)32 << 20 ? 0.6 : 4.0;
+        const bool direct = is_direct_kind(L.kind);
+        const size_t tb = !direct ? L.table_bytes
+                          : (L.filter_bits > 0 && T->filter && !opts.no_filter_bitmap) ? (size_t)(L.filter_bits / 8)
+                                                                                      : T->slots_bytes;
+        const size_t staged_up_to = opts.smem_tables == 0 ? kStageBytes
+                                    : opts.smem_tables == 1 ? 0
+                                    : opts.smem_tables >= 1024 ? (size_t)opts.smem_tables
+                                                               : (size_t)128 << 10;
+        const double probe = direct && tb <= staged_up_to ? kPsShared : tb <= kNearL2 ? kPsGlobal : kPsFar;
         if (is_hash_kind(L.kind) && T->filter && L.filter_bits > 0) {
             // a hashed join is two stages: its presence bitmap (cheap, passes the hits and ~1/16 of the
             // misses) early, the exact probe (expensive) on what is left
             const double fp = std::min(1.0, (double)L.entries / (double)L.filter_bits);
             const double pass = std::min(1.0, sel + (1.0 - sel) * fp);
-            specs.push_back({ST_PROBE, j, joins[j].fk_col, pass, bytes + 0.7, 1});
-            specs.push_back({ST_PROBE, j, joins[j].fk_col, pass > 0 ? std::min(1.0, sel / pass) : 1.0,
-                             bytes + probe + 4.0, 2});
+            specs.push_back({ST_PROBE, j, joins[j].fk_col, pass, width, kPsGlobal + kPsIssue, 1});
+            specs.push_back({ST_PROBE, j, joins[j].fk_col, pass > 0 ? std::min(1.0, sel / pass) : 1.0, width,
+                             probe + kPsIssue, 2});
             continue;
         }
-        specs.push_back({ST_PROBE, j, joins[j].fk_col, std::min(1.0, sel), bytes + probe, 0});
+        specs.push_back({ST_PROBE, j, joins[j].fk_col, std::min(1.0, sel), width, probe + kPsIssue, 0});
     }
     const int nfilter = (int)specs.size();
+    static_assert(SJQ_MAX_PREDS + 2 * SJQ_MAX_JOINS <= 64, "cheapest_order lists the stages in 64 places");
     if (opts.norder) {
         // the caller orders predicates and joins; a hashed join's bitmap and exact probe stay adjacent
         std::vector<char> seen(npreds + njoins, 0);
@@ -147,13 +230,7 @@ sjq_status order_stages(const sjq_col *fact, const sjq_pred *preds, int npreds, 
             }
         }
     } else {
-        order.resize(nfilter);
-        for (int i = 0; i < nfilter; ++i) order[i] = i;
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-            // exact probes of prefiltered hashed joins go last: they run at the final level
-            if ((specs[a].prefilter == 2) != (specs[b].prefilter == 2)) return specs[b].prefilter == 2;
-            return (1.0 - specs[a].sel) / specs[a].cost > (1.0 - specs[b].sel) / specs[b].cost;
-        });
+        order = cheapest_order(specs);
     }
 
     return SJQ_OK;
@@ -476,7 +553,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
         if (c.src == SJQ_SRC_FACT) {
             if (stage_of_col[c.a] < 0) { // a column nobody filters on: plain load stage at the end
                 if (ns >= kMaxStages) return SJQ_ERR_UNSUPPORTED;
-                StageSpec sp{ST_LOAD, -1, c.a, 1.0, 1.0, 0};
+                StageSpec sp{ST_LOAD, -1, c.a, 1.0, 4, 0.0, 0};
                 fill_stage(P.st[ns], sp);
                 stage_of_col[c.a] = ns;
                 stage_label.push_back(-1);
@@ -721,7 +798,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
                 const size_t tb = align_up(S.tab_bytes, 16);
                 if (tables + tb > table_budget) continue;
                 // larger tables are left to L1/L2: shared memory taken here is L1 capacity lost to every other table
-                if (opts.smem_tables == 0 && tb > (size_t)32 << 10) continue;
+                if (opts.smem_tables == 0 && tb > kStageBytes) continue;
                 if (opts.smem_tables >= 1024 && tb > (size_t)opts.smem_tables) continue; // experiment: size limit in bytes
                 // worth it only if a block probes the table more often than it costs to copy
                 const double probes_per_cta = (double)n * reach[s] / approx_grid;
