@@ -34,7 +34,8 @@ __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
 }
 
 struct CompactParams {
-    const int64_t *gkeys, *gsums, *gcounts;
+    const int64_t *gkeys;
+    const longlong2 *cells; // {sum, count}
     int64_t dense_base; // indexed: cell number = key + dense_base
     int32_t indexed;    // the table is indexed by the key itself and has no key array
     int64_t gslots; // regular slots; the side slot follows (direct-indexed: cells - 1)
@@ -52,13 +53,14 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactParams C)
         const bool direct = C.indexed != 0;
         const bool side = !direct && i == C.gslots;
         const int64_t k = direct ? i - C.dense_base : side ? kEmptyKey64 : C.gkeys[i];
-        const bool used = (direct || side) ? (C.gcounts[i] != 0) : (k != kEmptyKey64);
-        if (!used) continue;
+        if (!direct && !side && k == kEmptyKey64) continue;
+        const longlong2 cell = C.cells[i];
+        if ((direct || side) && cell.y == 0) continue;
         const int64_t pos = (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(C.n_groups), 1ull);
         if (pos < C.capacity) {
             C.keys[pos] = k;
-            C.sums[pos] = C.gsums[i];
-            C.counts[pos] = C.gcounts[i];
+            C.sums[pos] = cell.x;
+            C.counts[pos] = cell.y;
         } else {
             set_status(C.status, SJQ_ERR_GROUP_OVERFLOW);
         }
@@ -68,7 +70,7 @@ __global__ void __launch_bounds__(256) compact_kernel(const CompactParams C)
 struct MergeParams {
     const int64_t *keys, *sums, *counts; // the lists to merge, n entries
     int64_t n;
-    int64_t *gkeys, *gsums, *gcounts; // group table
+    int64_t *gkeys, *cells; // group table
     uint64_t gmask;
     int32_t *status;
 };
@@ -77,8 +79,23 @@ struct MergeParams {
 __global__ void __launch_bounds__(256) merge_kernel(const MergeParams M)
 {
     const int64_t stride = (int64_t)blockDim.x * gridDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M.n; i += stride)
-        group_table_add(M.gkeys, M.gsums, M.gcounts, M.gmask, M.status, M.keys[i], M.sums[i], M.counts[i]);
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = first; i - (threadIdx.x & 31) < M.n; i += stride) { // whole warps stay together
+        uint64_t cell = ~0ull;
+        int64_t sum = 0, count = 0;
+        if (i < M.n) {
+            cell = group_cell(M.gkeys, M.gmask, M.status, M.keys[i]);
+            sum = M.sums[i];
+            count = M.counts[i];
+        }
+        unsigned long long *cells = reinterpret_cast<unsigned long long *>(M.cells);
+        if (M.gmask < 0xFFFFFFFEull) {
+            add_pairs<false>(cells, (uint32_t)cell, (uint64_t)sum, (uint64_t)count, cell != ~0ull);
+        } else if (cell != ~0ull) {
+            atomicAdd(cells + 2 * cell, (unsigned long long)sum);
+            atomicAdd(cells + 2 * cell + 1, (unsigned long long)count);
+        }
+    }
 }
 
 struct SampleParams {
@@ -225,22 +242,21 @@ sjq_status sample_launch(const sjq_col *fact, const DPred *preds, int npreds, in
 }
 
 sjq_status merge_launch(const int64_t *keys, const int64_t *sums, const int64_t *counts, int64_t n, int64_t *gkeys,
-                        int64_t *gsums, int64_t *gcounts, uint64_t gmask, int32_t *status, int sm_count,
-                        cudaStream_t stream)
+                        int64_t *cells, uint64_t gmask, int32_t *status, int sm_count, cudaStream_t stream)
 {
     if (n <= 0) return SJQ_OK;
-    MergeParams M{keys, sums, counts, n, gkeys, gsums, gcounts, gmask, status};
+    MergeParams M{keys, sums, counts, n, gkeys, cells, gmask, status};
     int64_t blocks = (n + 255) / 256;
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     merge_kernel<<<(int)blocks, 256, 0, stream>>>(M);
     return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 
-sjq_status compact_launch(const int64_t *gkeys, const int64_t *gsums, const int64_t *gcounts, int64_t gslots,
-                          bool indexed, int64_t dense_base, int64_t *keys, int64_t *sums, int64_t *counts,
-                          int64_t capacity, int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream)
+sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gslots, bool indexed,
+                          int64_t dense_base, int64_t *keys, int64_t *sums, int64_t *counts, int64_t capacity,
+                          int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream)
 {
-    CompactParams C{gkeys, gsums, gcounts, dense_base, indexed ? 1 : 0, gslots, keys, sums, counts, capacity, n_groups,
+    CompactParams C{gkeys, reinterpret_cast<const longlong2 *>(cells), dense_base, indexed ? 1 : 0, gslots, keys, sums, counts, capacity, n_groups,
                     status};
     int64_t blocks = (gslots + 256) / 256;
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;

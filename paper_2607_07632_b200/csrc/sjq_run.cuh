@@ -109,8 +109,8 @@ struct RunParams {
     uint64_t modmask; // modulo - 1 when modulo is a power of two, else 0
     int64_t num_groups;
     uint64_t gmask; // hashed: group-table slots - 1
-    int64_t *sums;  // scalar/dense: result; hashed: table sums
-    int64_t *counts; // may be NULL
+    int64_t *sums;  // scalar/dense: result; hashed: the table's {sum, count} cells
+    int64_t *counts; // may be NULL; hashed: sums + 1
     int64_t *gkeys;  // hashed: table keys
     int32_t *status;
     int32_t nstages;
@@ -132,6 +132,8 @@ struct RunParams {
     uint32_t smem_l0;     // byte offset of the per-warp staging buffers of the first column (then their mbarriers)
     int32_t sparse_push;  // few rows survive level 0: the push into the first queue walks the set bits of the mask
     int32_t count32;      // fewer than 2^32 fact rows: a block's count of a group fits 32 bits (no carry into the high word)
+    int32_t cell_shift;   // log2 of the distance between two groups' sums: 1 when sums and counts alternate, else 0
+    int32_t pairs;        // ... and two lanes share a row's two adds
     int32_t l0_bulk;      // compiled kernels: the first column arrives by bulk-asynchronous copies into shared memory
 };
 

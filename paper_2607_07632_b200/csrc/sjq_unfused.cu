@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(256) unfused_aggregate_kernel(const __grid_con
                 accumulate<MUL, int32_t, 4>(S, v, code, m, key, X, Y);
             }
         }
-        terminal<AGG, MUL, 4>(P, nullptr, key, X, Y, m, lsum, lcnt);
+        terminal<AGG, MUL, 4, false>(P, nullptr, key, X, Y, m, lsum, lcnt);
     }
     if (AGG == AGG_SCALAR) scalar_block_reduce(P, lsum, lcnt);
 }

@@ -1,0 +1,42 @@
+"""The evaluation order the planner chooses, and parity where its search changes form."""
+import numpy as np
+import pytest
+import torch
+
+from datagen.workloads import AggExpr, Pred, Term
+
+pytestmark = pytest.mark.gpu
+
+sjq = pytest.importorskip("paper_2607_07632_b200") if torch.cuda.is_available() else None
+
+from gpuhelpers import compare, run_both  # noqa: E402
+from qhelpers import adhoc  # noqa: E402
+
+
+@pytest.mark.parametrize("small_first", [True, False])
+def test_of_two_equally_selective_joins_the_one_in_shared_memory_goes_first(small_first):
+    n, rng = 50_003, np.random.default_rng(3)
+    sizes = {"small": 100_000, "large": 1_000_000}  # bitmaps of 12 KB and 125 KB
+    dims = [(nm, {"k": np.arange(rows, dtype=np.int32), "a": (np.arange(rows) % 25).astype(np.int32)}, "k",
+             [Pred("a", "EQ", 7)], []) for nm, rows in sizes.items()]
+    fact = {nm: rng.integers(0, rows, n).astype(np.int32) for nm, rows in sizes.items()}
+    fact["m"] = rng.integers(0, 1000, n).astype(np.int32)
+    names = list(sizes) if small_first else list(sizes)[::-1]
+    w = adhoc("order", fact, dims, [(nm, nm) for nm in names], [], None, AggExpr("COL", Term("FACT", "m")), "SCALAR")
+    res, exp, _ = run_both(w, fact, {d[0]: d[1] for d in dims})
+    compare(w, res, exp)
+    assert res.info.order[0] == names.index("small")
+
+
+@pytest.mark.parametrize("npreds", [1, 8, 9, 16])
+def test_any_number_of_filters(npreds):
+    n, rng = 20_011, np.random.default_rng(npreds)
+    fact = {f"c{i}": rng.integers(0, 100, n).astype(np.int32) for i in range(npreds)}
+    dim = {"k": np.arange(100, dtype=np.int32), "a": (np.arange(100) % 2).astype(np.int32)}
+    w = adhoc("many", fact, [("d", dim, "k", [Pred("a", "EQ", 1)], [])], [("c0", "d")],
+              [Pred(f"c{i}", "LT", 80 + i) for i in range(npreds)], None, AggExpr("COL", Term("FACT", "c0")), "SCALAR")
+    for opts in (sjq.RunOpts(), sjq.RunOpts(specialise=True)):
+        res, exp, _ = run_both(w, fact, {"d": dim}, opts=opts)
+        assert res.status() == 0
+        compare(w, res, exp)
+        assert sorted(res.info.order[: npreds + 1]) == list(range(npreds + 1))
