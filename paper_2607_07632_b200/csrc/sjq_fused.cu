@@ -18,16 +18,23 @@ struct ClearParams {
     int32_t *status;
 };
 
+// (every array starts on a 16-byte boundary; the odd last word is thread 0's)
 __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
 {
     const int64_t stride = (int64_t)blockDim.x * gridDim.x;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t i = t; i < C.cells; i += stride) {
-        C.sums[i] = 0;
-        if (C.counts) C.counts[i] = 0;
+    const longlong2 zero = make_longlong2(0, 0), empty = make_longlong2(kEmptyKey64, kEmptyKey64);
+    for (int64_t i = t; i < C.cells / 2; i += stride) {
+        reinterpret_cast<longlong2 *>(C.sums)[i] = zero;
+        if (C.counts) reinterpret_cast<longlong2 *>(C.counts)[i] = zero;
     }
-    for (int64_t i = t; i < C.gslots; i += stride) C.gkeys[i] = kEmptyKey64;
+    for (int64_t i = t; i < C.gslots / 2; i += stride) reinterpret_cast<longlong2 *>(C.gkeys)[i] = empty;
     if (t == 0) {
+        if (C.cells & 1) {
+            C.sums[C.cells - 1] = 0;
+            if (C.counts) C.counts[C.cells - 1] = 0;
+        }
+        if (C.gslots & 1) C.gkeys[C.gslots - 1] = kEmptyKey64;
         if (C.status) *C.status = 0;
         if (C.n_groups) *C.n_groups = 0;
     }
@@ -38,33 +45,113 @@ struct CompactParams {
     const longlong2 *cells; // {sum, count}
     int64_t dense_base; // indexed: cell number = key + dense_base
     int32_t indexed;    // the table is indexed by the key itself and has no key array
-    int64_t gslots; // regular slots; the side slot follows (direct-indexed: cells - 1)
+    int64_t ncells;     // indexed: all; otherwise the regular slots and the side slot after them
+    int64_t tiles_per_block;
+    unsigned int *block_counts; // indexed: used cells per block, so that the list comes out in key order; else NULL
     int64_t *keys, *sums, *counts;
     int64_t capacity;
     int64_t *n_groups;
     int32_t *status;
 };
 
-// Group table -> list of (key, sum, count).
-__global__ void __launch_bounds__(256) compact_kernel(const CompactParams C)
+constexpr int kCompactThreads = 256;
+constexpr int kCompactRounds = 8; // cells per thread and tile, all loaded before the first is used
+constexpr int kCompactTile = kCompactThreads * kCompactRounds;
+
+__global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const CompactParams C)
 {
-    const int64_t stride = (int64_t)blockDim.x * gridDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= C.gslots; i += stride) {
-        const bool direct = C.indexed != 0;
-        const bool side = !direct && i == C.gslots;
-        const int64_t k = direct ? i - C.dense_base : side ? kEmptyKey64 : C.gkeys[i];
-        if (!direct && !side && k == kEmptyKey64) continue;
-        const longlong2 cell = C.cells[i];
-        if ((direct || side) && cell.y == 0) continue;
-        const int64_t pos = (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(C.n_groups), 1ull);
-        if (pos < C.capacity) {
-            C.keys[pos] = k;
-            C.sums[pos] = cell.x;
-            C.counts[pos] = cell.y;
-        } else {
-            set_status(C.status, SJQ_ERR_GROUP_OVERFLOW);
-        }
+    const int64_t lo = (int64_t)blockIdx.x * C.tiles_per_block * kCompactTile;
+    int64_t hi = lo + C.tiles_per_block * kCompactTile;
+    hi = hi < C.ncells ? hi : C.ncells;
+    unsigned int used = 0;
+#pragma unroll 8
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kCompactThreads) used += C.cells[i].y != 0;
+    used = __reduce_add_sync(0xffffffffu, used);
+    __shared__ unsigned int part[kCompactThreads / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = used;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kCompactThreads / 32; ++w) used += part[w];
+        C.block_counts[blockIdx.x] = used;
     }
+}
+
+// Group table -> list of (key, sum, count).  A block owns consecutive tiles of cells; a warp takes 256 consecutive
+// cells of a tile.  The place of a block's groups is the number of groups before it (an indexed table: the list comes
+// out in ascending key order), or is drawn from the common counter, once per tile.
+__global__ void __launch_bounds__(kCompactThreads) compact_kernel(const CompactParams C)
+{
+    __shared__ unsigned int part[kCompactThreads / 32];
+    __shared__ long long draw;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long place = 0;
+    if (C.block_counts) {
+        unsigned int before = 0;
+        for (int b = threadIdx.x; b < (int)blockIdx.x; b += kCompactThreads) before += C.block_counts[b];
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0) part[warp] = before;
+        __syncthreads();
+        for (int w = 0; w < kCompactThreads / 32; ++w) place += part[w];
+        __syncthreads();
+    }
+    const int64_t lo = (int64_t)blockIdx.x * C.tiles_per_block * kCompactTile;
+    int64_t hi = lo + C.tiles_per_block * kCompactTile;
+    hi = hi < C.ncells ? hi : C.ncells;
+    for (int64_t tile = lo; tile < hi; tile += kCompactTile) {
+        const int64_t first = tile + warp * (32 * kCompactRounds) + lane;
+        longlong2 cell[kCompactRounds];
+        long long key[kCompactRounds];
+        unsigned int lanes[kCompactRounds], mine = 0;
+#pragma unroll
+        for (int r = 0; r < kCompactRounds; ++r) {
+            const int64_t i = first + 32 * r;
+            cell[r] = make_longlong2(0, 0);
+            key[r] = kEmptyKey64;
+            if (i < hi) {
+                cell[r] = C.cells[i];
+                key[r] = C.indexed ? i - C.dense_base : i == C.ncells - 1 ? kEmptyKey64 : C.gkeys[i];
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kCompactRounds; ++r) {
+            const int64_t i = first + 32 * r;
+            // a claimed slot holds a group whatever its count (merged lists may carry zeros); the side slot and the
+            // cells of an indexed table do when a row was counted there
+            const bool used = i < hi && (C.indexed || i == C.ncells - 1 ? cell[r].y != 0 : key[r] != kEmptyKey64);
+            lanes[r] = __ballot_sync(0xffffffffu, used);
+            mine += __popc(lanes[r]);
+        }
+        if (lane == 0) part[warp] = mine;
+        __syncthreads();
+        unsigned int before = 0, total = 0;
+        for (int w = 0; w < kCompactThreads / 32; ++w) {
+            before += w < warp ? part[w] : 0u;
+            total += part[w];
+        }
+        if (!C.block_counts) {
+            if (threadIdx.x == 0) draw = (long long)atomicAdd(reinterpret_cast<unsigned long long *>(C.n_groups), (unsigned long long)total);
+            __syncthreads();
+            place = draw;
+        }
+        long long at = place + before;
+#pragma unroll
+        for (int r = 0; r < kCompactRounds; ++r) {
+            if ((lanes[r] >> lane) & 1u) {
+                const long long pos = at + __popc(lanes[r] & ((1u << lane) - 1u));
+                if (pos < C.capacity) {
+                    C.keys[pos] = key[r];
+                    C.sums[pos] = cell[r].x;
+                    C.counts[pos] = cell[r].y;
+                } else {
+                    set_status(C.status, SJQ_ERR_GROUP_OVERFLOW);
+                }
+            }
+            at += __popc(lanes[r]);
+        }
+        place += total;
+        __syncthreads(); // the shared words are written again for the next tile
+    }
+    if (C.block_counts && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *C.n_groups = place;
 }
 
 struct MergeParams {
@@ -210,7 +297,7 @@ sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *
                         int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream)
 {
     ClearParams C{sums, counts, cells, gkeys, gslots, n_groups, status};
-    int64_t work = cells > gslots ? cells : gslots;
+    const int64_t work = (cells > gslots ? cells : gslots) / 2;
     int64_t blocks = (work + 255) / 256;
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     if (blocks < 1) blocks = 1;
@@ -252,15 +339,25 @@ sjq_status merge_launch(const int64_t *keys, const int64_t *sums, const int64_t 
     return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 
+// gslots: regular slots of the hash table (a side slot follows), or the cells of an indexed table.  `block_counts`
+// (device, one word per 2048 cells): an indexed table is listed in key order, by two kernels; NULL: in no order, by one.
 sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gslots, bool indexed,
-                          int64_t dense_base, int64_t *keys, int64_t *sums, int64_t *counts, int64_t capacity,
-                          int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream)
+                          int64_t dense_base, unsigned int *block_counts, int64_t *keys, int64_t *sums,
+                          int64_t *counts, int64_t capacity, int64_t *n_groups, int32_t *status, int sm_count,
+                          cudaStream_t stream, int *launches)
 {
-    CompactParams C{gkeys, reinterpret_cast<const longlong2 *>(cells), dense_base, indexed ? 1 : 0, gslots, keys, sums, counts, capacity, n_groups,
-                    status};
-    int64_t blocks = (gslots + 256) / 256;
-    if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
-    compact_kernel<<<(int)blocks, 256, 0, stream>>>(C);
+    const int64_t ncells = indexed ? gslots : gslots + 1;
+    const int64_t tiles = (ncells + kCompactTile - 1) / kCompactTile;
+    const int64_t per = (tiles + (int64_t)sm_count * 8 - 1) / ((int64_t)sm_count * 8);
+    const int blocks = (int)((tiles + per - 1) / per);
+    CompactParams C{gkeys, reinterpret_cast<const longlong2 *>(cells), dense_base, indexed ? 1 : 0, ncells, per,
+                    block_counts, keys, sums, counts, capacity, n_groups, status};
+    if (block_counts) {
+        compact_count_kernel<<<blocks, kCompactThreads, 0, stream>>>(C);
+        ++*launches;
+    }
+    compact_kernel<<<blocks, kCompactThreads, 0, stream>>>(C);
+    ++*launches;
     return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 

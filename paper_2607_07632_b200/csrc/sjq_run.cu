@@ -33,8 +33,9 @@ sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
                         int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream);
 sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gslots, bool indexed,
-                          int64_t dense_base, int64_t *keys, int64_t *sums, int64_t *counts, int64_t capacity,
-                          int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream);
+                          int64_t dense_base, unsigned int *block_counts, int64_t *keys, int64_t *sums,
+                          int64_t *counts, int64_t capacity, int64_t *n_groups, int32_t *status, int sm_count,
+                          cudaStream_t stream, int *launches);
 
 size_t unfused_scratch_bytes(int64_t n, int gathering_joins);
 sjq_status unfused_launch(const RunParams &P, int nfilter, int agg, bool mul, bool has_hash, void *scratch,
@@ -963,11 +964,12 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     if (opts.event_after && cudaEventRecord((cudaEvent_t)opts.event_after, stream) != cudaSuccess)
         return SJQ_ERR_CUDA;
     if (spec->mode == SJQ_HASHED) {
-        st = compact_launch(gkeys, cells, direct_groups ? table_groups - 1 : (int64_t)gslots,
-                            direct_groups, P.post_offset, out->keys, out->sums, out->counts, spec->capacity,
-                            out->n_groups, out->status, dev.sm_count, stream);
+        // (an indexed table has no use for the key array: it holds the block counts of the ordered list)
+        st = compact_launch(gkeys, cells, direct_groups ? table_groups : (int64_t)gslots, direct_groups, P.post_offset,
+                            direct_groups && !opts.unfused ? reinterpret_cast<unsigned int *>(gkeys) : nullptr,
+                            out->keys, out->sums, out->counts, spec->capacity, out->n_groups, out->status,
+                            dev.sm_count, stream, &launches);
         if (st != SJQ_OK) return st;
-        ++launches;
     }
     if (info) {
         std::memset(info, 0, sizeof(*info));
@@ -1021,8 +1023,9 @@ extern "C" sjq_status sjq_merge_groups(const int64_t *keys, const int64_t *sums,
     if ((st = merge_launch(keys, sums, counts, n, gkeys, cells, gslots - 1, out->status, dev.sm_count,
                            stream)) != SJQ_OK)
         return st;
-    return compact_launch(gkeys, cells, (int64_t)gslots, false, 0, out->keys, out->sums, out->counts, capacity,
-                          out->n_groups, out->status, dev.sm_count, stream);
+    int launches = 0;
+    return compact_launch(gkeys, cells, (int64_t)gslots, false, 0, nullptr, out->keys, out->sums, out->counts, capacity,
+                          out->n_groups, out->status, dev.sm_count, stream, &launches);
 }
 
 // ---------------------------------------------------------------------------
