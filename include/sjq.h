@@ -215,9 +215,9 @@ sjq_status sjq_dim_plan_end(const sjq_col *cols, int ncols, int key_col, int npa
  * is consistent but too small for the data is caught on the device
  * (LAYOUT_MISMATCH: key or payload outside the planned ranges; TABLE_FULL:
  * the open-addressing table has no free slot left).  Enqueues
- * a fill, the build kernel and a verification kernel; does not synchronise.
+ * a fill and the build kernel; does not synchronise.
  * Direct tables are written by race-free direct stores indexed by key
- * (Section 3.3); hash tables by atomicCAS on the key word with a bounded
+ * (Section 3.3), and the presence bits beside them tell a repeated key; hash tables by atomicCAS on the key word with a bounded
  * linear probe.  Keys must be unique among the passing rows: a repeated key
  * sets SJQ_ERR_DUP_KEY in *status_dev.  Zero passing rows is valid (every
  * probe then misses).  *status_dev is NOT cleared by this call.
@@ -225,6 +225,32 @@ sjq_status sjq_dim_plan_end(const sjq_col *cols, int ncols, int key_col, int npa
 sjq_status sjq_build_dim(const sjq_col *cols, int ncols, const sjq_pred *preds, int npreds, int key_col,
                          const int *payload_cols, int npayload, const sjq_dim_layout *layout, void *table_mem,
                          size_t table_bytes, int32_t *status_dev, void *stream, sjq_table **table);
+
+/*
+ * The tables of several dimensions at once: the same scans, layouts and builds as sjq_dim_plan and sjq_build_dim give
+ * one by one, with one scan kernel and one wait, then one kernel that prepares the memory and one build kernel, for
+ * up to eight dimensions (a query asked once plans and builds all of its tables before it can run, and its small
+ * dimensions cost little but the launches and the waits).
+ *   dims              `ndims` descriptions, as the arguments of sjq_dim_plan
+ *   scratch_dev       device scratch of ndims * SJQ_PLAN_SCRATCH_BYTES bytes
+ *   layouts           receives (plan) or gives (build) `ndims` layouts
+ *   table_mem etc.    one entry per dimension, as the arguments of sjq_build_dim; the status words ARE cleared
+ * sjq_dims_plan SYNCHRONISES the stream; sjq_dims_build does not.  After an error no table has been created.
+ */
+typedef struct sjq_dim_desc {
+    const sjq_col *cols;
+    int32_t ncols;
+    const sjq_pred *preds;
+    int32_t npreds;
+    int32_t key_col;
+    const int *payload_cols;
+    int32_t npayload;
+    const sjq_build_opts *opts; /* NULL = defaults */
+} sjq_dim_desc;
+sjq_status sjq_dims_plan(const sjq_dim_desc *dims, int ndims, void *scratch_dev, size_t scratch_bytes, void *stream,
+                         sjq_dim_layout *layouts);
+sjq_status sjq_dims_build(const sjq_dim_desc *dims, int ndims, const sjq_dim_layout *layouts, void *const *table_mem,
+                          const size_t *table_bytes, int32_t *const *status_dev, void *stream, sjq_table **tables);
 
 /*
  * Device bytes a table of the given shape occupies, recomputed from `kind`,
@@ -242,8 +268,8 @@ sjq_status sjq_dim_layout_bytes(const sjq_dim_layout *layout, size_t *bytes);
  * whether the probed structure stays in L1 / L2 (Section 3.3: the packed map is sized to stay cache-resident). */
 sjq_status sjq_table_info(const sjq_table *table, sjq_dim_layout *layout);
 
-/* Kernels sjq_build_dim enqueued for this table: one that prepares the memory, the build unless the dimension
- * is empty, and for a direct table the occupancy count that ends with the duplicate check. */
+/* Kernels sjq_build_dim enqueued for this table: one that prepares the memory and the build unless the dimension is
+ * empty.  (sjq_dims_build counts those of a batch with its first table.) */
 int32_t sjq_table_kernel_launches(const sjq_table *table);
 
 /* Frees the host handle only (the device memory belongs to the caller). */

@@ -8,6 +8,8 @@
 // key range is verified at run time and the packed or unpacked form chosen.
 #include <algorithm>
 #include <new>
+#include <type_traits>
+#include <utility>
 
 #include "sjq_internal.h"
 
@@ -17,133 +19,279 @@ namespace {
 
 constexpr int kMaxDimCols = 32;
 
-struct DimParams {
-    const void *col[kMaxDimCols];
-    uint8_t is64[kMaxDimCols];
-    DPred preds[SJQ_MAX_PREDS];
-    int32_t npreds;
-    int32_t key_col;
-    int32_t pay_col[SJQ_MAX_PAYLOADS];
-    int32_t npayload;
+// A launch works on up to kBatchDims dimensions (and their filters, together at most kBatchPreds): the scans, the
+// fills and the builds of a query's tables are one launch each.  A block belongs to one dimension; its threads take
+// four consecutive rows at two places at a time (one where 64-bit values fill the registers), so that every column is
+// read with 128-bit loads and six of them are in flight per thread before the first is used.  What bounds these kernels: latency for the small dimensions (2,556
+// to 200,000 rows), instructions as much as the columns' bytes for those of millions; so the code for 32-bit keys and
+// payloads keeps to 32-bit arithmetic.
+constexpr int kBatchDims = 8;
+constexpr int kBatchPreds = 16;
+constexpr int kFillThreads = 256;
+constexpr int kBuildThreads = 256;
+constexpr int kScanThreads = 512;
+
+struct DimRows {
     int64_t n;
+    const void *key;
+    const void *pay[SJQ_MAX_PAYLOADS];
+    int32_t npayload;
+    int32_t pred0, npreds; // its conjunction in the launch's list
+    uint32_t block0, blocks;
+    uint8_t key64, pay64[SJQ_MAX_PAYLOADS];
 };
 
-__device__ inline bool dim_row_passes(const DimParams &P, int64_t r)
+struct DimFilters {
+    DPred d[kBatchPreds];
+    const void *col[kBatchPreds];
+};
+
+// Four consecutive values of a column as T (a 32-bit column may be read as 64-bit values, not the other way round).
+template <typename T>
+__device__ __forceinline__ void load4(const void *col, bool is64, int64_t r, int rows, T *v)
 {
-    bool ok = true;
-    for (int k = 0; k < P.npreds && ok; ++k) {
-        const DPred &d = P.preds[k];
-        if (d.is64) ok = pred_eval<int64_t>(d, static_cast<const int64_t *>(P.col[d.col])[r]);
-        else ok = pred_eval<int32_t>(d, static_cast<const int32_t *>(P.col[d.col])[r]);
+    if (rows == 4) {
+        if (sizeof(T) == 8 && is64) {
+            const longlong2 a = __ldg(static_cast<const longlong2 *>(col) + r / 2);
+            const longlong2 b = __ldg(static_cast<const longlong2 *>(col) + r / 2 + 1);
+            v[0] = (T)a.x, v[1] = (T)a.y, v[2] = (T)b.x, v[3] = (T)b.y;
+        } else {
+            const int4 a = __ldg(static_cast<const int4 *>(col) + r / 4);
+            v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+        }
+        return;
     }
-    return ok;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = k < rows ? (T)load_cell(col, sizeof(T) == 8 && is64, r + k) : (T)0;
 }
 
-__device__ inline int64_t warp_min(int64_t v)
+// The rows a thread has in hand, Q groups of four: keys of type K and up to N payloads of type V, and which pass the
+// filter.  Usual keeps to the tables of most dimensions: at most one payload, of 32 bits.
+template <typename K, typename V, int N, int Q>
+struct RowSet {
+    static constexpr int kPayloads = N, kQuads = Q, kRows = 4 * Q;
+    typedef K Key;
+    typedef V Payload;
+    K key[kRows];
+    V pay[N][kRows];
+    uint32_t m;
+};
+template <typename K>
+using Usual = RowSet<K, int32_t, 1, 2>;
+template <typename K>
+using Wide = RowSet<K, int64_t, SJQ_MAX_PAYLOADS, 1>;
+__host__ __device__ inline bool usual_payloads(const DimRows &D) { return D.npayload == 0 || (D.npayload == 1 && !D.pay64[0]); }
+
+template <typename T>
+__device__ __forceinline__ uint32_t filter4(const DPred &d, const T *v)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        int64_t t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = t < v ? t : v;
+    uint32_t pass = 0;
+    if (d.nset) {
+        for (int i = 0; i < d.nset; ++i) {
+            const int64_t lit = d.set[i];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) pass |= (uint32_t)((int64_t)v[k] == lit) << k;
+        }
+        return pass;
     }
-    return v;
-}
-__device__ inline int64_t warp_max(int64_t v)
-{
-    for (int o = 16; o > 0; o >>= 1) {
-        int64_t t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = t > v ? t : v;
+    if (sizeof(T) == 4) {
+        const uint32_t lo = (uint32_t)d.lo32, width = (uint32_t)d.hi32 - lo;
+        if (!d.never) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) pass |= (uint32_t)((uint32_t)v[k] - lo <= width) << k;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) pass |= (uint32_t)(((int64_t)v[k] >= d.lo) & ((int64_t)v[k] <= d.hi)) << k;
     }
-    return v;
-}
-__device__ inline int64_t warp_sum(int64_t v)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    return d.neg ? ~pass : pass;
 }
 
-// Sum over a block of at most 256 threads; the total is valid in thread 0.
-__device__ inline unsigned long long block_sum(unsigned long long v)
+// Rows r .. r + 3 and r + apart .. r + apart + 3 (those below D.n).  The first filter's column is requested with the
+// others; further filters are read one after the other.
+template <typename Set>
+__device__ __forceinline__ void read_rows(const DimRows &D, const DimFilters &F, int64_t r, int64_t apart, Set &R)
 {
-    __shared__ unsigned long long part[8];
-    v = (unsigned long long)warp_sum((int64_t)v);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
-    __syncthreads();
-    unsigned long long t = 0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += part[w];
+    typedef typename Set::Key K;
+    typedef typename Set::Payload V;
+    constexpr int kDimQuads = Set::kQuads;
+    R.m = 0;
+    int first[Set::kRows];
+    const bool ahead = D.npreds > 0 && !F.d[D.pred0].is64;
+#pragma unroll
+    for (int q = 0; q < kDimQuads; ++q) {
+        const int64_t at = r + q * apart, left = D.n - at;
+        const int rows = left >= 4 ? 4 : left > 0 ? (int)left : 0;
+        R.m |= ((1u << rows) - 1u) << (4 * q);
+        if (!rows) continue;
+        load4<K>(D.key, D.key64, at, rows, &R.key[4 * q]);
+        if (ahead) load4<int>(F.col[D.pred0], false, at, rows, &first[4 * q]);
+#pragma unroll
+        for (int i = 0; i < Set::kPayloads; ++i)
+            if (i < D.npayload) load4<V>(D.pay[i], D.pay64[i], at, rows, &R.pay[i][4 * q]);
+    }
+    if (ahead) {
+#pragma unroll
+        for (int q = 0; q < kDimQuads; ++q)
+            if ((R.m >> (4 * q)) & 0xFu) R.m &= ~(0xFu << (4 * q)) | (filter4<int>(F.d[D.pred0], &first[4 * q]) & 0xFu) << (4 * q);
+    }
+    for (int p = D.pred0 + (ahead ? 1 : 0); p < D.pred0 + D.npreds; ++p) {
+        const DPred &d = F.d[p];
+#pragma unroll
+        for (int q = 0; q < kDimQuads; ++q) {
+            const int64_t at = r + q * apart, left = D.n - at;
+            if (left <= 0) continue;
+            int64_t v[4];
+            load4<int64_t>(F.col[p], d.is64, at, left >= 4 ? 4 : (int)left, v);
+            int v32[4] = {(int)v[0], (int)v[1], (int)v[2], (int)v[3]};
+            const uint32_t pass = d.is64 ? filter4<int64_t>(d, v) : filter4<int>(d, v32);
+            R.m &= ~(0xFu << (4 * q)) | (pass & 0xFu) << (4 * q);
+        }
+    }
+}
+
+// (a launch's tasks in the order of their blocks)
+struct BuildTask;
+struct FillTask;
+__device__ __forceinline__ uint32_t first_block(const DimRows &t) { return t.block0; }
+__device__ __forceinline__ uint32_t first_block(const BuildTask &t);
+__device__ __forceinline__ uint32_t first_block(const FillTask &t);
+
+template <typename Task>
+__device__ __forceinline__ int task_of_block(const Task *tasks, int n)
+{
+    int t = 0;
+    while (t + 1 < n && blockIdx.x >= first_block(tasks[t + 1])) ++t;
     return t;
 }
 
-// scratch: [0] kmin [1] kmax [2] count [3] p0min [4] p0max [5] p1min [6] p1max
-__global__ void plan_init_kernel(int64_t *s)
+__device__ __forceinline__ unsigned long long ordered(int64_t v) { return (unsigned long long)v ^ 0x8000000000000000ull; }
+__device__ __forceinline__ int64_t unordered(unsigned long long v) { return (int64_t)(v ^ 0x8000000000000000ull); }
+
+// Statistics of a dimension, kScratchWords words of scratch that start as zeros: while the blocks add to them, words
+// 4 i, each in a sector of its own, hold i = 0 the largest of ~ordered(key) (so the smallest key), 1 of ordered(key),
+// 2 the passing rows, 3..6 the payloads' like 0 and 1, 7 the blocks done; the block that comes last leaves kmin, kmax,
+// count, p0min, p0max, p1min, p1max, 0 in words 0..7.
+constexpr int kScratchWords = 32;
+static_assert(kScratchWords * 8 == SJQ_PLAN_SCRATCH_BYTES, "one dimension's statistics fill the scratch of a plan");
+
+struct ScanParams {
+    DimRows dim[kBatchDims];
+    DimFilters filters;
+    int32_t ndims;
+    unsigned long long *scratch;
+    int64_t *host; // page-locked, eight words per dimension, or NULL: the statistics stay in the scratch
+};
+
+constexpr int kExtremes = 2 + 2 * SJQ_MAX_PAYLOADS; // [min, max] of the key and of each payload
+
+// Extremes (as ~ordered(min), ordered(max)) and count of the passing rows that this thread owns.
+template <typename Set>
+__device__ __forceinline__ void scan_rows(const DimRows &D, const DimFilters &F, unsigned long long (&ext)[kExtremes], unsigned int &cnt)
 {
-    if (threadIdx.x < 8) {
-        int64_t v = 0;
-        if (threadIdx.x == 0 || threadIdx.x == 3 || threadIdx.x == 5) v = INT64_MAX;
-        if (threadIdx.x == 1 || threadIdx.x == 4 || threadIdx.x == 6) v = INT64_MIN;
-        s[threadIdx.x] = v;
+    typedef typename Set::Key K;
+    typedef typename Set::Payload V;
+    constexpr int kPayloads = Set::kPayloads;
+    constexpr K kmost = sizeof(K) == 8 ? (K)INT64_MAX : (K)INT32_MAX;
+    constexpr V vmost = sizeof(V) == 8 ? (V)INT64_MAX : (V)INT32_MAX;
+    K kmin = kmost, kmax = -kmost - 1;
+    V pmin[kPayloads], pmax[kPayloads];
+#pragma unroll
+    for (int i = 0; i < kPayloads; ++i) pmin[i] = vmost, pmax[i] = -vmost - 1;
+    const int64_t apart = 4 * (int64_t)D.blocks * kScanThreads;
+    for (int64_t r = 4 * ((int64_t)(blockIdx.x - D.block0) * kScanThreads + threadIdx.x); r < D.n; r += Set::kQuads * apart) {
+        Set R;
+        read_rows(D, F, r, apart, R);
+        cnt += __popc(R.m);
+#pragma unroll
+        for (int k = 0; k < Set::kRows; ++k) {
+            const bool on = (R.m >> k) & 1u;
+            const K lo = on ? R.key[k] : kmost, hi = on ? R.key[k] : (K)(-kmost - 1);
+            kmin = lo < kmin ? lo : kmin;
+            kmax = hi > kmax ? hi : kmax;
+#pragma unroll
+            for (int i = 0; i < kPayloads; ++i) {
+                if (i >= D.npayload) continue;
+                const V plo = on ? R.pay[i][k] : vmost, phi = on ? R.pay[i][k] : (V)(-vmost - 1);
+                pmin[i] = plo < pmin[i] ? plo : pmin[i];
+                pmax[i] = phi > pmax[i] ? phi : pmax[i];
+            }
+        }
+    }
+    if (cnt == 0) return;
+    ext[0] = ~ordered(kmin);
+    ext[1] = ordered(kmax);
+#pragma unroll
+    for (int i = 0; i < kPayloads; ++i) {
+        if (i >= D.npayload) continue;
+        ext[2 + 2 * i] = ~ordered(pmin[i]);
+        ext[3 + 2 * i] = ordered(pmax[i]);
     }
 }
 
-__global__ void __launch_bounds__(256) plan_scan_kernel(const __grid_constant__ DimParams P, int64_t *scratch)
+__global__ void __launch_bounds__(kScanThreads, 2) plan_scan_kernel(const __grid_constant__ ScanParams P)
 {
-    int64_t kmin = INT64_MAX, kmax = INT64_MIN, cnt = 0;
-    int64_t pmin[SJQ_MAX_PAYLOADS] = {INT64_MAX, INT64_MAX}, pmax[SJQ_MAX_PAYLOADS] = {INT64_MIN, INT64_MIN};
-    const int64_t stride = (int64_t)blockDim.x * gridDim.x;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < P.n; r += stride) {
-        if (!dim_row_passes(P, r)) continue;
-        int64_t k = load_cell(P.col[P.key_col], P.is64[P.key_col], r);
-        kmin = k < kmin ? k : kmin;
-        kmax = k > kmax ? k : kmax;
-        ++cnt;
-        for (int i = 0; i < P.npayload; ++i) {
-            int64_t v = load_cell(P.col[P.pay_col[i]], P.is64[P.pay_col[i]], r);
-            pmin[i] = v < pmin[i] ? v : pmin[i];
-            pmax[i] = v > pmax[i] ? v : pmax[i];
-        }
-    }
-    kmin = warp_min(kmin);
-    kmax = warp_max(kmax);
-    cnt = warp_sum(cnt);
-    for (int i = 0; i < SJQ_MAX_PAYLOADS; ++i) {
-        pmin[i] = warp_min(pmin[i]);
-        pmax[i] = warp_max(pmax[i]);
-    }
-    // one set of atomics per block, not per warp: they all land on the same seven words
-    __shared__ int64_t part[8][3 + 2 * SJQ_MAX_PAYLOADS];
+    const int which = task_of_block(P.dim, P.ndims);
+    const DimRows &D = P.dim[which];
+    unsigned long long *const scratch = P.scratch + which * kScratchWords;
+    unsigned long long ext[kExtremes];
+#pragma unroll
+    for (int i = 0; i < kExtremes; ++i) ext[i] = 0;
+    unsigned int cnt = 0;
+    if (!usual_payloads(D)) scan_rows<Wide<int64_t>>(D, P.filters, ext, cnt);
+    else if (D.key64) scan_rows<Usual<int64_t>>(D, P.filters, ext, cnt);
+    else scan_rows<Usual<int32_t>>(D, P.filters, ext, cnt);
+    // one set of atomics per block: they all land on the same seven words
+    __shared__ unsigned long long part[kScanThreads / 32][kExtremes + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        part[warp][0] = kmin;
-        part[warp][1] = kmax;
-        part[warp][2] = cnt;
-        for (int i = 0; i < SJQ_MAX_PAYLOADS; ++i) {
-            part[warp][3 + 2 * i] = pmin[i];
-            part[warp][4 + 2 * i] = pmax[i];
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+#pragma unroll
+    for (int i = 0; i < kExtremes; ++i) {
+        if (i >= 2 + 2 * D.npayload) continue;
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, ext[i], o);
+            ext[i] = v > ext[i] ? v : ext[i];
         }
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < kExtremes; ++i) part[warp][i] = ext[i];
+        part[warp][kExtremes] = cnt;
     }
     __syncthreads();
-    if (threadIdx.x < 3 + 2 * SJQ_MAX_PAYLOADS) {
-        const int f = threadIdx.x; // 0 kmin, 1 kmax, 2 count, then (min, max) per payload
-        const bool is_min = f == 0 || (f >= 3 && ((f - 3) & 1) == 0), is_sum = f == 2;
-        int64_t v = part[0][f];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-            const int64_t t = part[w][f];
-            v = is_sum ? v + t : is_min ? (t < v ? t : v) : (t > v ? t : v);
+    if (warp <= kExtremes) { // one warp per word
+        unsigned long long v = lane < kScanThreads / 32 ? part[lane][warp] : 0ull;
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o);
+            v = warp == kExtremes ? v + t : t > v ? t : v;
         }
-        int64_t block_cnt = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) block_cnt += part[w][2];
-        if (block_cnt > 0 && f < 3 + 2 * P.npayload) {
-            if (is_sum) atomicAdd((unsigned long long *)&scratch[f], (unsigned long long)v);
-            else if (is_min) atomicMin((long long *)&scratch[f], (long long)v);
-            else atomicMax((long long *)&scratch[f], (long long)v);
+        if (lane == 0) {
+            if (warp == kExtremes) atomicAdd(&scratch[4 * 2], v);
+            else if (warp < 2 + 2 * D.npayload) atomicMax(&scratch[4 * (warp < 2 ? warp : warp + 1)], v);
+            __threadfence();
+        }
+    }
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&scratch[4 * 7], 1ull) == D.blocks - 1;
+    __syncthreads();
+    if (last && warp == 0) {
+        const int i = lane & 7;
+        const unsigned long long v = i < 7 ? atomicAdd(&scratch[4 * i], 0ull) : 0ull;
+        const int64_t stat = i == 2 || i == 7 ? (int64_t)v : (i == 0 || i == 3 || i == 5) ? unordered(~v) : unordered(v);
+        __syncwarp();
+        if (lane < 8) {
+            scratch[i] = (unsigned long long)stat;
+            if (P.host) P.host[8 * which + i] = stat;
         }
     }
 }
 
-struct BuildParams {
-    DimParams dim;
+struct BuildTask {
+    DimRows rows;
     int32_t kind;
     int32_t code_bits;
+    int32_t usual; // no payload or a 32-bit one, slot indexes of a direct table below 2^32
     int64_t kmin;
     uint64_t span;  // direct
     uint32_t buckets; // hash: number of buckets
@@ -154,37 +302,62 @@ struct BuildParams {
     void *slots;
     unsigned int *filter; // presence bitmap words (hash: indexed by a hash of the key; direct with payloads: by slot)
     uint32_t fmask;       // hash: filter bits - 1
-    unsigned long long *header; // [0] rows inserted, [1] slots occupied
+    long long expect_full; // >= 0: the layout promises that every key of the range is present: so many rows are stored
+    unsigned long long *header; // [0] rows inserted, [1] blocks done (only with such a promise)
     int32_t *status;
 };
 
-// One launch prepares a table's memory: the header counters and the presence bitmap to zero, the slot array to
-// its empty pattern (bitmap: zeros; packed codes: all ones; open addressing: the empty key in every word).
-// All three regions start on 16-byte boundaries and are padded to a multiple of 16 bytes by the layout.
-struct InitParams {
-    uint4 *header, *slots, *filter;
-    size_t header16, slots16, filter16; // sizes in 16-byte units
-    uint4 pattern;
+__device__ __forceinline__ uint32_t first_block(const BuildTask &t) { return t.rows.block0; }
+
+struct BuildParams {
+    BuildTask task[kBatchDims];
+    DimFilters filters;
+    int32_t ntasks;
 };
 
-__global__ void __launch_bounds__(256) table_init_kernel(const __grid_constant__ InitParams I)
+// One launch prepares the memory of the tables: the header counters and the presence bitmap to zero, the slot array
+// to its empty pattern (bitmap: zeros; packed codes: all ones; open addressing: the empty key in every word).
+// All regions start on 16-byte boundaries and are padded to a multiple of 16 bytes by the layout.
+constexpr int kFillTile = 4 * kFillThreads; // 16-byte units per block and step
+
+struct FillTask {
+    uint4 *at;
+    uint64_t units; // of 16 bytes
+    uint4 pattern;
+    uint32_t block0, blocks;
+};
+
+__device__ __forceinline__ uint32_t first_block(const FillTask &t) { return t.block0; }
+
+struct FillParams {
+    FillTask task[3 * kBatchDims];
+    int32_t *clear_status[kBatchDims]; // NULL: left as it is
+    int32_t ntasks;
+};
+
+__global__ void __launch_bounds__(kFillThreads) table_init_kernel(const __grid_constant__ FillParams P)
 {
-    const size_t stride = (size_t)blockDim.x * gridDim.x;
-    const size_t total = I.header16 + I.slots16 + I.filter16;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        if (i < I.header16) I.header[i] = zero;
-        else if (i < I.header16 + I.slots16) I.slots[i - I.header16] = I.pattern;
-        else I.filter[i - I.header16 - I.slots16] = zero;
+    cudaTriggerProgrammaticLaunchCompletion(); // the build is launched behind and waits for this kernel on the device
+    if (blockIdx.x == 0 && threadIdx.x < kBatchDims && P.clear_status[threadIdx.x]) *P.clear_status[threadIdx.x] = 0;
+    const FillTask &T = P.task[task_of_block(P.task, P.ntasks)];
+    for (uint64_t base = (uint64_t)(blockIdx.x - T.block0) * kFillTile; base < T.units; base += (uint64_t)T.blocks * kFillTile) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint64_t i = base + k * kFillThreads + threadIdx.x;
+            if (i < T.units) T.at[i] = T.pattern;
+        }
     }
 }
 
-__device__ inline bool pack_code(const BuildParams &B, int64_t r, uint64_t *code)
+template <typename Set>
+__device__ __forceinline__ bool pack_code(const BuildTask &B, const Set &R, int k, uint64_t *code)
 {
     uint64_t c = 0;
     int shift = 0;
-    for (int i = 0; i < B.dim.npayload; ++i) {
-        int64_t v = load_cell(B.dim.col[B.dim.pay_col[i]], B.dim.is64[B.dim.pay_col[i]], r);
+#pragma unroll
+    for (int i = 0; i < Set::kPayloads; ++i) {
+        if (i >= B.rows.npayload) continue;
+        const int64_t v = R.pay[i][k];
         if (v < B.pay_min[i] || v > B.pay_max[i]) return false;
         c |= ((uint64_t)v - (uint64_t)B.pay_min[i]) << shift;
         shift += B.pay_bits[i];
@@ -192,146 +365,288 @@ __device__ inline bool pack_code(const BuildParams &B, int64_t r, uint64_t *code
     *code = c;
     return true;
 }
-
-__device__ inline void store_code(void *codes, int bits, uint64_t idx, uint64_t c)
+// (one 32-bit payload whose layout's bounds are 32-bit values)
+template <typename Set>
+__device__ __forceinline__ bool pack_code(const BuildTask &B, const Set &R, int k, uint32_t *code)
 {
+    *code = B.rows.npayload ? (uint32_t)R.pay[0][k] - (uint32_t)B.pay_min[0] : 0u;
+    return *code <= (uint32_t)B.pay_max[0] - (uint32_t)B.pay_min[0];
+}
+
+// Set one bit per row of the warp in a bitmap and report a bit that two rows set.  All lanes call it.  A dimension
+// that lists its keys in ascending order, as most do, gives a warp 128 neighbouring bits: the rows of a thread that
+// share a word are joined first, then the words that several threads share (up to eight of them), so that five adds
+// leave the warp instead of a hundred.
+template <typename I>
+__device__ __forceinline__ void set_bits(unsigned int *bits, const I *idx, uint32_t m, int32_t *status)
+{
+    const int lane = threadIdx.x & 31;
+    I word = 0;
+    unsigned int mine = 0, rows = 0, seen[4] = {0, 0, 0, 0};
+    bool dup = false;
+    // (nothing waits for an atomic's answer before the last of them is on its way)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!((m >> k) & 1u)) continue;
+        const unsigned int bit = 1u << (idx[k] & 31);
+        if (!rows) word = idx[k] >> 5;
+        if (idx[k] >> 5 == word) {
+            mine |= bit;
+            ++rows;
+        } else {
+            seen[k] = atomicOr(bits + (idx[k] >> 5), bit);
+        }
+    }
+    unsigned int joined = 0; // leader of a word that several threads share: their bits
+    unsigned int pending = __ballot_sync(0xffffffffu, rows != 0);
+    for (int it = 0; it < 8 && pending; ++it) {
+        const int leader = __ffs((int)pending) - 1;
+        const I w = __shfl_sync(0xffffffffu, word, leader);
+        const bool in = rows && word == w;
+        const unsigned int same = __ballot_sync(0xffffffffu, in);
+        if (it == 0 && __popc(same) == 1 && __popc(pending) > 1) break; // scattered keys: every lane for itself
+        const unsigned int all = __reduce_or_sync(0xffffffffu, in ? mine : 0u);
+        const unsigned int n = __reduce_add_sync(0xffffffffu, in ? rows : 0u);
+        if (lane == leader) {
+            joined = all;
+            dup = (int)n != __popc(all);
+        }
+        pending &= ~same;
+    }
+    if ((pending >> lane) & 1u) {
+        joined = mine;
+        dup = (int)rows != __popc(mine);
+    }
+    if (joined) dup |= (atomicOr(bits + word, joined) & joined) != 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dup |= (seen[k] >> (idx[k] & 31)) & 1u;
+    if (dup) set_status(status, SJQ_ERR_DUP_KEY);
+}
+
+// The packed codes of a thread's rows into a direct table.  A table with a presence bitmap finds repeated keys there;
+// without one (wide codes only) the store itself tells, since a code is never all ones, which is what a slot starts as.
+template <typename I, typename C>
+__device__ __forceinline__ void store_codes(const BuildTask &B, const I *idx, const C *code, uint32_t m)
+{
+    const int bits = B.code_bits;
     if (bits < 8) {
-        // several codes share a word that starts as all ones: clear this code's zero bits (the keys are
-        // unique, so no two rows touch the same bits)
-        const int per = 32 / bits;
-        const unsigned int sh = (unsigned int)(idx % (uint64_t)per) * (unsigned int)bits;
-        const unsigned int mask = ((1u << bits) - 1u) << sh;
-        atomicAnd(static_cast<unsigned int *>(codes) + idx / (uint64_t)per, ~mask | ((unsigned int)c << sh));
+        // several codes share a word that starts as all ones: clear this code's zero bits, the rows of a thread that
+        // share a word at once (the keys are unique, so no two rows touch the same bits)
+        const unsigned int per = 32u / (unsigned int)bits, low = (1u << bits) - 1u;
+        unsigned int *const words = static_cast<unsigned int *>(B.slots);
+        const int log_per = bits == 2 ? 4 : 3;
+        I word = ~(I)0; // no slot's word
+        unsigned int keep = ~0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (!((m >> k) & 1u)) continue;
+            const I w = idx[k] >> log_per;
+            const unsigned int sh = ((unsigned int)idx[k] & (per - 1u)) * (unsigned int)bits;
+            if (w != word) {
+                if (word != ~(I)0) atomicAnd(words + word, keep);
+                word = w;
+                keep = ~0u;
+            }
+            keep &= ~(low << sh) | ((unsigned int)code[k] << sh);
+        }
+        if (word != ~(I)0) atomicAnd(words + word, keep);
         return;
     }
-    switch (bits) {
-    case 8: static_cast<uint8_t *>(codes)[idx] = (uint8_t)c; break;
-    case 16: static_cast<uint16_t *>(codes)[idx] = (uint16_t)c; break;
-    case 32: static_cast<uint32_t *>(codes)[idx] = (uint32_t)c; break;
-    case 64: static_cast<uint64_t *>(codes)[idx] = c; break;
-    default: break;
+    bool dup = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!((m >> k) & 1u)) continue;
+        const uint64_t i = idx[k], c = code[k];
+        if (B.filter) {
+            if (bits == 8) static_cast<uint8_t *>(B.slots)[i] = (uint8_t)c;
+            else if (bits == 16) static_cast<uint16_t *>(B.slots)[i] = (uint16_t)c;
+            else if (bits == 32) static_cast<uint32_t *>(B.slots)[i] = (uint32_t)c;
+            else static_cast<uint64_t *>(B.slots)[i] = c;
+        } else if (bits == 64) {
+            dup |= atomicExch(static_cast<unsigned long long *>(B.slots) + i, (unsigned long long)c) != ~0ull;
+        } else if (bits == 32) {
+            dup |= atomicExch(static_cast<unsigned int *>(B.slots) + i, (unsigned int)c) != ~0u;
+        } else {
+            const unsigned int per = 32u / (unsigned int)bits, sh = (unsigned int)(i % per) * (unsigned int)bits;
+            const unsigned int low = ((1u << bits) - 1u) << sh;
+            const unsigned int old = atomicAnd(static_cast<unsigned int *>(B.slots) + i / per, ~low | ((unsigned int)c << sh));
+            dup |= (old & low) != low;
+        }
     }
+    if (dup) set_status(B.status, SJQ_ERR_DUP_KEY);
 }
 
-// Claim the first free slot on the key's probe path (bucket after bucket from its home bucket, the slots of
-// a bucket in order) with atomicCAS on the key word, then store the code beside it.  Bounded by the number
-// of buckets; a key met on the way is a duplicate.
-template <typename W>
-__device__ inline void hash_insert(const BuildParams &B, W key, W empty, uint64_t hashed, uint64_t code)
+// Build a direct table from the rows that this thread owns; returns how many it stored.  I: type of a slot index of
+// a direct table; C: of a code.
+template <typename Set, typename I, typename C>
+__device__ __forceinline__ unsigned int build_rows(const BuildTask &B, const DimFilters &F)
 {
-    char *base = static_cast<char *>(B.slots);
-    uint32_t b = home_bucket(hashed, B.buckets);
-    for (uint32_t it = 0; it < B.buckets; ++it) {
-        char *bucket = base + (size_t)b * kBucketBytes;
-        W *keys = reinterpret_cast<W *>(bucket);
-        for (int j = 0; j < B.bucket_k; ++j) {
-            W old = *reinterpret_cast<volatile W *>(&keys[j]);
-            if (old == empty) old = atomicCAS(&keys[j], empty, key);
-            if (old == empty) {
-                if (B.code_bits == 32) reinterpret_cast<uint32_t *>(bucket + B.code_off)[j] = (uint32_t)code;
-                else if (B.code_bits == 64) reinterpret_cast<uint64_t *>(bucket + B.code_off)[j] = code;
-                return;
-            }
-            if (old == key) {
-                set_status(B.status, SJQ_ERR_DUP_KEY);
-                return;
+    constexpr int kRows = Set::kRows;
+    const int64_t apart = 4 * (int64_t)B.rows.blocks * kBuildThreads;
+    unsigned int inserted = 0;
+    for (int64_t r = 4 * ((int64_t)(blockIdx.x - B.rows.block0) * kBuildThreads + threadIdx.x);
+         r - 4 * (int64_t)(threadIdx.x & 31) < B.rows.n; r += Set::kQuads * apart) { // whole warps stay together
+        Set R;
+        read_rows(B.rows, F, r, apart, R);
+        C code[kRows];
+        uint32_t mismatch = 0;
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+            code[k] = 0;
+            if (((R.m >> k) & 1u) && !pack_code(B, R, k, &code[k])) mismatch |= 1u << k;
+        }
+        I idx[kRows];
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+            const uint64_t i = (uint64_t)(int64_t)R.key[k] - (uint64_t)B.kmin;
+            idx[k] = (I)i;
+            if (((R.m >> k) & 1u) && i >= B.span) mismatch |= 1u << k;
+        }
+        if (mismatch) set_status(B.status, SJQ_ERR_LAYOUT_MISMATCH);
+        R.m &= ~mismatch;
+#pragma unroll
+        for (int q = 0; q < Set::kQuads; ++q) {
+            const uint32_t m = (R.m >> (4 * q)) & 0xFu;
+            if (B.kind == SJQ_TABLE_DIRECT_BITMAP) {
+                set_bits<I>(static_cast<unsigned int *>(B.slots), &idx[4 * q], m, B.status);
+            } else {
+                store_codes(B, &idx[4 * q], &code[4 * q], m);
+                if (B.filter) set_bits<I>(B.filter, &idx[4 * q], m, B.status);
             }
         }
-        b = b + 1 == B.buckets ? 0 : b + 1;
+        inserted += __popc(R.m);
     }
-    set_status(B.status, SJQ_ERR_TABLE_FULL);
+    return inserted;
 }
 
-__global__ void __launch_bounds__(256) build_kernel(const __grid_constant__ BuildParams B)
+__global__ void __launch_bounds__(kBuildThreads, 4) direct_build_kernel(const __grid_constant__ BuildParams P)
 {
-    const DimParams &P = B.dim;
-    const int64_t stride = (int64_t)blockDim.x * gridDim.x;
-    unsigned long long inserted = 0;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < P.n; r += stride) {
-        if (!dim_row_passes(P, r)) continue;
-        const int64_t k = load_cell(P.col[P.key_col], P.is64[P.key_col], r);
-        uint64_t code = 0;
-        if (!pack_code(B, r, &code)) {
-            set_status(B.status, SJQ_ERR_LAYOUT_MISMATCH);
-            continue;
-        }
-        ++inserted;
-        if (B.kind != SJQ_TABLE_HASH_I32 && B.kind != SJQ_TABLE_HASH_I64) {
-            const uint64_t idx = (uint64_t)k - (uint64_t)B.kmin;
-            if (idx >= B.span) {
-                set_status(B.status, SJQ_ERR_LAYOUT_MISMATCH);
-                continue;
-            }
-            if (B.kind == SJQ_TABLE_DIRECT_BITMAP)
-                atomicOr(static_cast<unsigned int *>(B.slots) + (idx >> 5), 1u << (idx & 31));
-            else {
-                store_code(B.slots, B.code_bits, idx, code); // race-free: keys are unique
-                if (B.filter) atomicOr(B.filter + (idx >> 5), 1u << (idx & 31));
-            }
-        } else if (B.kind == SJQ_TABLE_HASH_I64) {
-            if (k == kEmptyKey64) {
-                set_status(B.status, SJQ_ERR_RESERVED_KEY);
-                continue;
-            }
-            if (B.filter) {
-                const uint32_t fb = filter_hash((uint64_t)k) & B.fmask;
-                atomicOr(B.filter + (fb >> 5), 1u << (fb & 31));
-            }
-            hash_insert<unsigned long long>(B, (unsigned long long)k, (unsigned long long)kEmptyKey64, (uint64_t)k, code);
-        } else { // HASH_I32
-            const int32_t k32 = (int32_t)k;
-            if (k32 == kEmptyKey32) {
-                set_status(B.status, SJQ_ERR_RESERVED_KEY);
-                continue;
-            }
-            if (B.filter) {
-                const uint32_t fb = filter_hash((uint64_t)(int64_t)k32) & B.fmask;
-                atomicOr(B.filter + (fb >> 5), 1u << (fb & 31));
-            }
-            hash_insert<unsigned int>(B, (unsigned int)k32, (unsigned int)kEmptyKey32, (uint64_t)(int64_t)k32, code);
-        }
-    }
-    inserted = block_sum(inserted);
-    if (threadIdx.x == 0 && inserted) atomicAdd(&B.header[0], inserted);
-}
-
-// Count occupied slots of a direct table; a repeated key leaves fewer occupied slots than inserted rows.  The
-// block that finishes last (a ticket in header[2]) compares the two counters.  `expect_full` >= 0: the layout
-// promises that every key of the range is present (a probe then trusts the range test alone), so exactly that
-// many rows must have been stored.
-__global__ void __launch_bounds__(256) direct_count_kernel(const __grid_constant__ BuildParams B, long long expect_full)
-{
-    const uint64_t stride = (uint64_t)blockDim.x * gridDim.x;
-    unsigned long long occ = 0;
-    if (B.kind == SJQ_TABLE_DIRECT_BITMAP || B.filter) {
-        // one bit per occupied slot: the table itself, or the presence bitmap beside the codes
-        const uint64_t words = (B.span + 31) >> 5;
-        const unsigned int *w = B.kind == SJQ_TABLE_DIRECT_BITMAP ? static_cast<const unsigned int *>(B.slots) : B.filter;
-        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += stride) occ += __popc(w[i]);
-    } else {
-        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < B.span; i += stride) {
-            bool set;
-            switch (B.code_bits) {
-            case 8: set = static_cast<const uint8_t *>(B.slots)[i] != 0xFFu; break;
-            case 16: set = static_cast<const uint16_t *>(B.slots)[i] != 0xFFFFu; break;
-            case 32: set = static_cast<const uint32_t *>(B.slots)[i] != 0xFFFFFFFFu; break;
-            default: set = static_cast<const uint64_t *>(B.slots)[i] != ~0ULL; break;
-            }
-            occ += set;
-        }
-    }
-    occ = block_sum(occ);
+    const BuildTask &B = P.task[task_of_block(P.task, P.ntasks)];
+    const DimRows &D = B.rows;
+    cudaGridDependencySynchronize(); // the tables' memory is prepared by the kernel before this one
+    unsigned int inserted;
+    if (B.usual && !D.key64) inserted = build_rows<Usual<int32_t>, uint32_t, uint32_t>(B, P.filters);
+    else if (B.usual) inserted = build_rows<Usual<int64_t>, uint32_t, uint32_t>(B, P.filters);
+    else if (!D.key64) inserted = build_rows<Wide<int32_t>, uint64_t, uint64_t>(B, P.filters);
+    else inserted = build_rows<Wide<int64_t>, uint64_t, uint64_t>(B, P.filters);
+    if (B.expect_full < 0) return;
+    // A probe of this table trusts the range test alone, so exactly so many rows must have been stored: the block
+    // that comes last compares (repeated keys have been reported by then).
+    __shared__ unsigned int part[kBuildThreads / 32];
+    inserted = __reduce_add_sync(0xffffffffu, inserted);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = inserted;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (occ) atomicAdd(&B.header[1], occ);
+        for (int w = 1; w < kBuildThreads / 32; ++w) inserted += part[w];
+        if (inserted) atomicAdd(&B.header[0], (unsigned long long)inserted);
         __threadfence();
-        if (atomicAdd(&B.header[2], 1ULL) == (unsigned long long)gridDim.x - 1) {
+        if (atomicAdd(&B.header[1], 1ull) == B.rows.blocks - 1ull) {
             __threadfence();
-            const unsigned long long inserted = atomicAdd(&B.header[0], 0ULL), occupied = atomicAdd(&B.header[1], 0ULL);
-            if (inserted != occupied) set_status(B.status, SJQ_ERR_DUP_KEY);
-            else if (expect_full >= 0 && occupied != (unsigned long long)expect_full)
-                set_status(B.status, SJQ_ERR_LAYOUT_MISMATCH);
+            if (atomicAdd(&B.header[0], 0ull) != (unsigned long long)B.expect_full) set_status(B.status, SJQ_ERR_LAYOUT_MISMATCH);
         }
     }
+}
+
+// Open addressing.  A key claims the first free slot on its probe path (bucket after bucket from its home bucket, the
+// slots of a bucket in order) with atomicCAS on the key word, one CAS a step and no look before it (at the default load
+// 1.3 steps place a key), then its code goes beside it.  Bounded by the number of buckets; a key met on the way is a
+// duplicate.  The passing rows of a warp are gathered in shared memory and placed 32 at a time, so that every lane of
+// the chain of CASes, whose latency bounds the kernel, has a key.  2 M keys of 8 M rows of 16 bytes into 80 MB: 100 us,
+// 135 with each lane placing its own rows, 125 one row per thread; the CASes alone, random, take 45, the rows 20.
+constexpr int kHashThreads = 256;
+constexpr int kHashQueue = 31 + 128; // what is left of a batch and a warp's next rows
+
+template <typename W, typename C>
+__device__ __forceinline__ void hash_place(const BuildTask &B, W key, C code)
+{
+    const W empty = sizeof(W) == 8 ? (W)kEmptyKey64 : (W)(uint32_t)kEmptyKey32;
+    const uint64_t hashed = sizeof(W) == 8 ? (uint64_t)key : (uint64_t)(int64_t)(int32_t)key;
+    if (B.filter) {
+        const uint32_t fb = filter_hash(hashed) & B.fmask;
+        atomicOr(B.filter + (fb >> 5), 1u << (fb & 31));
+    }
+    uint32_t b = home_bucket(hashed, B.buckets), it = 0;
+    int j = 0;
+    for (;;) {
+        char *const bucket = static_cast<char *>(B.slots) + (size_t)b * kBucketBytes;
+        const W old = atomicCAS(reinterpret_cast<W *>(bucket) + j, empty, key);
+        if (old == empty) {
+            if (B.code_bits == 32) reinterpret_cast<uint32_t *>(bucket + B.code_off)[j] = (uint32_t)code;
+            else if (B.code_bits == 64) reinterpret_cast<uint64_t *>(bucket + B.code_off)[j] = code;
+            return;
+        }
+        if (old == key) {
+            set_status(B.status, SJQ_ERR_DUP_KEY);
+            return;
+        }
+        if (++j == B.bucket_k) {
+            j = 0;
+            b = b + 1 == B.buckets ? 0 : b + 1;
+            if (++it == B.buckets) {
+                set_status(B.status, SJQ_ERR_TABLE_FULL);
+                return;
+            }
+        }
+    }
+}
+
+template <typename Set, typename C>
+__device__ __forceinline__ void hash_rows(const BuildTask &B, const DimFilters &F, void *queue)
+{
+    typedef typename std::conditional<sizeof(typename Set::Key) == 8, unsigned long long, unsigned int>::type W;
+    static_assert(Set::kQuads == 1, "the queue takes 128 rows at a time");
+    const W empty = sizeof(W) == 8 ? (W)kEmptyKey64 : (W)(uint32_t)kEmptyKey32;
+    const int lane = threadIdx.x & 31;
+    W *const qkey = static_cast<W *>(queue);
+    C *const qcode = reinterpret_cast<C *>(qkey + kHashQueue + 1);
+    int waiting = 0;
+    for (int64_t r = 4 * ((int64_t)(blockIdx.x - B.rows.block0) * kHashThreads + threadIdx.x);
+         r - 4 * lane < B.rows.n; r += 4 * (int64_t)B.rows.blocks * kHashThreads) { // whole warps stay together
+        Set R;
+        read_rows(B.rows, F, r, 0, R);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            bool on = (R.m >> k) & 1u;
+            C code = 0;
+            if (on && !pack_code(B, R, k, &code)) {
+                set_status(B.status, SJQ_ERR_LAYOUT_MISMATCH);
+                on = false;
+            }
+            if (on && (W)R.key[k] == empty) {
+                set_status(B.status, SJQ_ERR_RESERVED_KEY);
+                on = false;
+            }
+            const unsigned int lanes = __ballot_sync(0xffffffffu, on);
+            if (on) {
+                const int at = waiting + __popc(lanes & ((1u << lane) - 1u));
+                qkey[at] = (W)R.key[k];
+                qcode[at] = code;
+            }
+            waiting += __popc(lanes);
+        }
+        __syncwarp();
+        while (waiting >= 32) {
+            waiting -= 32;
+            hash_place<W>(B, qkey[waiting + lane], qcode[waiting + lane]);
+            __syncwarp();
+        }
+    }
+    if (lane < waiting) hash_place<W>(B, qkey[lane], qcode[lane]);
+}
+
+template <typename K>
+using UsualQuad = RowSet<K, int32_t, 1, 1>;
+
+__global__ void __launch_bounds__(kHashThreads, 5) hash_build_kernel(const __grid_constant__ BuildParams P)
+{
+    __shared__ __align__(16) unsigned char queues[kHashThreads / 32][(kHashQueue + 1) * 16];
+    const BuildTask &B = P.task[task_of_block(P.task, P.ntasks)];
+    void *const queue = queues[threadIdx.x >> 5];
+    cudaGridDependencySynchronize(); // the tables' memory is prepared by the kernel before this one
+    if (B.usual && !B.rows.key64) hash_rows<UsualQuad<int32_t>, uint32_t>(B, P.filters, queue);
+    else if (B.usual) hash_rows<UsualQuad<int64_t>, uint32_t>(B, P.filters, queue);
+    else if (!B.rows.key64) hash_rows<Wide<int32_t>, uint64_t>(B, P.filters, queue);
+    else hash_rows<Wide<int64_t>, uint64_t>(B, P.filters, queue);
 }
 
 int bits_for(uint64_t range)
@@ -383,43 +698,102 @@ bool layout_table_bytes(const sjq_dim_layout &L, size_t *bytes)
     return false;
 }
 
-sjq_status fill_dim_params(const sjq_col *cols, int ncols, const sjq_pred *preds, int npreds, int key_col,
-                           const int *payload_cols, int npayload, DimParams *P)
+// What the kernels read of one dimension, checked; its filters are appended to the launch's list.
+sjq_status fill_rows(const sjq_dim_desc &d, DimRows *D, DimFilters *F, int *nfilters)
 {
-    if (!cols || ncols <= 0 || ncols > kMaxDimCols || npreds < 0 || npreds > SJQ_MAX_PREDS || (npreds && !preds) ||
-        key_col < 0 || key_col >= ncols || npayload < 0 || npayload > SJQ_MAX_PAYLOADS || (npayload && !payload_cols))
+    if (!d.cols || d.ncols <= 0 || d.ncols > kMaxDimCols || d.npreds < 0 || d.npreds > SJQ_MAX_PREDS ||
+        (d.npreds && !d.preds) || d.key_col < 0 || d.key_col >= d.ncols || d.npayload < 0 ||
+        d.npayload > SJQ_MAX_PAYLOADS || (d.npayload && !d.payload_cols))
         return SJQ_ERR_INVALID_ARG;
-    const int64_t n = cols[key_col].n;
+    const int64_t n = d.cols[d.key_col].n;
     if (n < 0) return SJQ_ERR_INVALID_ARG;
-    for (int c = 0; c < ncols; ++c) {
-        if (cols[c].n != n || (cols[c].dtype != SJQ_I32 && cols[c].dtype != SJQ_I64)) return SJQ_ERR_INVALID_ARG;
-        if (n > 0 && !cols[c].data) return SJQ_ERR_INVALID_ARG;
-        if (!aligned16(cols[c].data)) return SJQ_ERR_ALIGN;
-        P->col[c] = cols[c].data;
-        P->is64[c] = (uint8_t)cols[c].dtype;
+    for (int c = 0; c < d.ncols; ++c) {
+        const sjq_col &col = d.cols[c];
+        if (col.n != n || (col.dtype != SJQ_I32 && col.dtype != SJQ_I64)) return SJQ_ERR_INVALID_ARG;
+        if (n > 0 && !col.data) return SJQ_ERR_INVALID_ARG;
+        if (!aligned16(col.data)) return SJQ_ERR_ALIGN;
     }
-    for (int k = 0; k < npreds; ++k) {
-        if (preds[k].col < 0 || preds[k].col >= ncols) return SJQ_ERR_INVALID_ARG;
-        if (!canon_pred(preds[k], cols[preds[k].col].dtype, &P->preds[k])) return SJQ_ERR_INVALID_ARG;
+    *D = DimRows{};
+    D->n = n;
+    D->key = d.cols[d.key_col].data;
+    D->key64 = (uint8_t)d.cols[d.key_col].dtype;
+    D->npayload = d.npayload;
+    for (int i = 0; i < d.npayload; ++i) {
+        if (d.payload_cols[i] < 0 || d.payload_cols[i] >= d.ncols) return SJQ_ERR_INVALID_ARG;
+        D->pay[i] = d.cols[d.payload_cols[i]].data;
+        D->pay64[i] = (uint8_t)d.cols[d.payload_cols[i]].dtype;
     }
-    for (int i = 0; i < npayload; ++i) {
-        if (payload_cols[i] < 0 || payload_cols[i] >= ncols) return SJQ_ERR_INVALID_ARG;
-        P->pay_col[i] = payload_cols[i];
+    D->pred0 = *nfilters;
+    D->npreds = d.npreds;
+    for (int k = 0; k < d.npreds; ++k) {
+        const int c = d.preds[k].col;
+        if (c < 0 || c >= d.ncols) return SJQ_ERR_INVALID_ARG;
+        if (!canon_pred(d.preds[k], d.cols[c].dtype, &F->d[*nfilters])) return SJQ_ERR_INVALID_ARG;
+        F->col[*nfilters] = d.cols[c].data;
+        ++*nfilters;
     }
-    P->npreds = npreds;
-    P->key_col = key_col;
-    P->npayload = npayload;
-    P->n = n;
     return SJQ_OK;
 }
 
-int grid_for(int64_t n, int sm_count)
+// How many of the dimensions from `first` on one launch can take.
+int batch_of(const sjq_dim_desc *dims, int ndims, int first)
 {
-    int64_t blocks = (n + 255) / 256;
-    int64_t cap = (int64_t)sm_count * 8;
-    if (blocks > cap) blocks = cap;
-    return blocks < 1 ? 1 : (int)blocks;
+    int n = 0, preds = 0;
+    while (first + n < ndims && n < kBatchDims) {
+        preds += std::max(0, dims[first + n].npreds);
+        if (n > 0 && preds > kBatchPreds) break;
+        ++n;
+    }
+    return n;
 }
+
+// Blocks for tasks of `second` steps each: about `room` of them in all, at least one per task.  Returns the grid.
+template <typename Get>
+uint32_t share_blocks(int ntasks, int64_t room, Get task)
+{
+    int64_t total = 0;
+    for (int i = 0; i < ntasks; ++i) total += task(i).second;
+    const int64_t per = std::max<int64_t>(1, (total + room - 1) / room);
+    uint32_t at = 0;
+    for (int i = 0; i < ntasks; ++i) {
+        auto t = task(i);
+        t.first->block0 = at;
+        t.first->blocks = (uint32_t)std::max<int64_t>(1, (t.second + per - 1) / per);
+        at += t.first->blocks;
+    }
+    return at;
+}
+
+// Enqueue the scans of a batch; the statistics of dimension i go to scratch + i * kScratchWords (and host + 8 i).
+sjq_status scan_launch(const sjq_dim_desc *dims, int ndims, unsigned long long *scratch, int64_t *host, int sm_count,
+                       cudaStream_t stream)
+{
+    ScanParams P;
+    int nfilters = 0;
+    bool rows = false;
+    for (int i = 0; i < ndims; ++i) {
+        const sjq_status st = fill_rows(dims[i], &P.dim[i], &P.filters, &nfilters);
+        if (st != SJQ_OK) return st;
+        rows = rows || P.dim[i].n > 0;
+    }
+    P.ndims = ndims;
+    P.scratch = scratch;
+    P.host = host;
+    if (cudaMemsetAsync(scratch, 0, (size_t)ndims * kScratchWords * 8, stream) != cudaSuccess) return SJQ_ERR_CUDA;
+    if (rows || host) { // (a dimension without rows still has its statistics written)
+        const uint32_t grid = share_blocks(ndims, 2 * sm_count, [&](int i) {
+            return std::make_pair(&P.dim[i], (P.dim[i].n + 8 * kScanThreads - 1) / (8 * kScanThreads));
+        });
+        plan_scan_kernel<<<grid, kScanThreads, 0, stream>>>(P);
+    }
+    return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
+}
+
+// Page-locked memory of this thread for the statistics that a waiting plan reads back.
+struct HostStats {
+    int64_t *words = nullptr;
+};
+thread_local HostStats g_host_stats;
 
 } // namespace
 
@@ -506,36 +880,84 @@ extern "C" sjq_status sjq_dim_plan_begin(const sjq_col *cols, int ncols, const s
 {
     if (!scratch_dev || !host_stats) return SJQ_ERR_INVALID_ARG;
     if (!aligned16(scratch_dev)) return SJQ_ERR_ALIGN;
-    DimParams P{};
-    sjq_status st = fill_dim_params(cols, ncols, preds, npreds, key_col, payload_cols, npayload, &P);
-    if (st != SJQ_OK) return st;
+    const sjq_dim_desc d{cols, ncols, preds, npreds, key_col, payload_cols, npayload, nullptr};
     DeviceInfo dev;
-    if ((st = device_info(&dev)) != SJQ_OK) return st;
+    sjq_status st = device_info(&dev);
+    DimRows check_rows; // (argument errors come before a missing device)
+    DimFilters check_filters;
+    int nfilters = 0;
+    const sjq_status bad = fill_rows(d, &check_rows, &check_filters, &nfilters);
+    if (bad != SJQ_OK) return bad;
+    if (st != SJQ_OK) return st;
     cudaStream_t stream = (cudaStream_t)stream_;
-    int64_t *scratch = static_cast<int64_t *>(scratch_dev);
-    plan_init_kernel<<<1, 32, 0, stream>>>(scratch);
-    if (P.n > 0) plan_scan_kernel<<<grid_for(P.n, dev.sm_count), 256, 0, stream>>>(P, scratch);
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(host_stats, scratch, 8 * sizeof(int64_t), cudaMemcpyDeviceToHost, stream) != cudaSuccess) {
+    st = scan_launch(&d, 1, static_cast<unsigned long long *>(scratch_dev), nullptr, dev.sm_count, stream);
+    if (st == SJQ_OK &&
+        cudaMemcpyAsync(host_stats, scratch_dev, 8 * sizeof(int64_t), cudaMemcpyDeviceToHost, stream) != cudaSuccess)
+        st = SJQ_ERR_CUDA;
+    if (st == SJQ_ERR_CUDA) (void)cudaGetLastError();
+    return st;
+}
+
+namespace sjq {
+int host_stats_release()
+{
+    if (!g_host_stats.words) return 0;
+    if (cudaFreeHost(g_host_stats.words) != cudaSuccess) (void)cudaGetLastError();
+    g_host_stats.words = nullptr;
+    return 1;
+}
+} // namespace sjq
+
+extern "C" sjq_status sjq_dims_plan(const sjq_dim_desc *dims, int ndims, void *scratch_dev, size_t scratch_bytes,
+                                    void *stream_, sjq_dim_layout *layouts)
+{
+    if (!dims || ndims <= 0 || !scratch_dev || !layouts) return SJQ_ERR_INVALID_ARG;
+    if (!aligned16(scratch_dev)) return SJQ_ERR_ALIGN;
+    const int most = std::min(ndims, kBatchDims);
+    if (scratch_bytes < (size_t)most * SJQ_PLAN_SCRATCH_BYTES) return SJQ_ERR_BUFFER_SMALL;
+    for (int i = 0; i < ndims; ++i) {
+        DimRows rows;
+        DimFilters filters;
+        int nfilters = 0;
+        const sjq_status st = fill_rows(dims[i], &rows, &filters, &nfilters);
+        if (st != SJQ_OK) return st;
+    }
+    DeviceInfo dev;
+    sjq_status st = device_info(&dev);
+    if (st != SJQ_OK) return st;
+    cudaStream_t stream = (cudaStream_t)stream_;
+    int64_t *&host = g_host_stats.words;
+    if (!host && cudaHostAlloc(reinterpret_cast<void **>(&host), kBatchDims * 8 * sizeof(int64_t),
+                               cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
         (void)cudaGetLastError();
+        host = nullptr;
         return SJQ_ERR_CUDA;
+    }
+    for (int first = 0; first < ndims;) {
+        const int n = batch_of(dims, ndims, first);
+        st = scan_launch(dims + first, n, static_cast<unsigned long long *>(scratch_dev), host, dev.sm_count, stream);
+        // the kernel writes the statistics into the page-locked words itself
+        if (st == SJQ_OK && cudaStreamSynchronize(stream) != cudaSuccess) st = SJQ_ERR_CUDA;
+        if (st != SJQ_OK) {
+            (void)cudaGetLastError();
+            return st;
+        }
+        for (int i = 0; i < n; ++i) {
+            const sjq_dim_desc &d = dims[first + i];
+            st = sjq_dim_plan_end(d.cols, d.ncols, d.key_col, d.npayload, d.opts, host + 8 * i, &layouts[first + i]);
+            if (st != SJQ_OK) return st;
+        }
+        first += n;
     }
     return SJQ_OK;
 }
 
 extern "C" sjq_status sjq_dim_plan(const sjq_col *cols, int ncols, const sjq_pred *preds, int npreds, int key_col,
                                    const int *payload_cols, int npayload, const sjq_build_opts *opts,
-                                   void *scratch_dev, void *stream_, sjq_dim_layout *layout)
+                                   void *scratch_dev, void *stream, sjq_dim_layout *layout)
 {
-    int64_t h[8];
-    sjq_status st = sjq_dim_plan_begin(cols, ncols, preds, npreds, key_col, payload_cols, npayload, scratch_dev, h,
-                                       stream_);
-    if (st != SJQ_OK) return st;
-    if (cudaStreamSynchronize((cudaStream_t)stream_) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return SJQ_ERR_CUDA;
-    }
-    return sjq_dim_plan_end(cols, ncols, key_col, npayload, opts, h, layout);
+    const sjq_dim_desc d{cols, ncols, preds, npreds, key_col, payload_cols, npayload, opts};
+    return sjq_dims_plan(&d, 1, scratch_dev, SJQ_PLAN_SCRATCH_BYTES, stream, layout);
 }
 
 extern "C" sjq_status sjq_dim_plan_end(const sjq_col *cols, int ncols, int key_col, int npayload,
@@ -636,108 +1058,192 @@ extern "C" sjq_status sjq_dim_plan_end(const sjq_col *cols, int ncols, int key_c
     return SJQ_OK;
 }
 
-extern "C" sjq_status sjq_build_dim(const sjq_col *cols, int ncols, const sjq_pred *preds, int npreds, int key_col,
-                                    const int *payload_cols, int npayload, const sjq_dim_layout *layout,
-                                    void *table_mem, size_t table_bytes, int32_t *status_dev, void *stream_,
-                                    sjq_table **table)
+namespace sjq {
+namespace {
+
+// Check one table of a batch and describe its build and the fills before it.
+sjq_status describe_build(const sjq_dim_desc &d, const sjq_dim_layout &L, void *table_mem, size_t table_bytes,
+                          int32_t *status_dev, BuildTask *B, DimFilters *F, int *nfilters, FillParams *I, sjq_table *T)
 {
-    if (!layout || !table_mem || !status_dev || !table) return SJQ_ERR_INVALID_ARG;
+    if (!table_mem || !status_dev) return SJQ_ERR_INVALID_ARG;
     if (!aligned16(table_mem)) return SJQ_ERR_ALIGN;
-    BuildParams B{};
-    sjq_status st = fill_dim_params(cols, ncols, preds, npreds, key_col, payload_cols, npayload, &B.dim);
+    *B = BuildTask{};
+    sjq_status st = fill_rows(d, &B->rows, F, nfilters);
     if (st != SJQ_OK) return st;
-    const sjq_dim_layout &L = *layout;
     // The layout is the caller's: every size used below is recomputed from its shape fields, never taken
     // from its table_bytes, and a layout whose fields contradict one another is rejected here.
     size_t need_bytes = 0;
-    if (L.npayload != npayload || L.key_dtype != cols[key_col].dtype || L.dim_rows != B.dim.n ||
+    if (L.npayload != d.npayload || L.key_dtype != d.cols[d.key_col].dtype || L.dim_rows != B->rows.n ||
         !layout_table_bytes(L, &need_bytes) || need_bytes != L.table_bytes)
         return SJQ_ERR_INVALID_ARG;
-    for (int i = 0; i < npayload; ++i)
+    for (int i = 0; i < d.npayload; ++i)
         if (L.pay_bits[i] < 0 || L.pay_bits[i] > 63) return SJQ_ERR_INVALID_ARG;
     if (table_bytes < need_bytes) return SJQ_ERR_BUFFER_SMALL;
-    DeviceInfo dev;
-    if ((st = device_info(&dev)) != SJQ_OK) return st;
-    cudaStream_t stream = (cudaStream_t)stream_;
 
-    sjq_table *T = new (std::nothrow) sjq_table();
-    if (!T) return SJQ_ERR_INVALID_ARG;
     T->layout = L;
     T->base = static_cast<char *>(table_mem);
     T->slots = T->base + kTableHeaderBytes;
     T->filter = nullptr;
+    T->launches = 0;
     T->magic = kTableMagic;
 
-    B.kind = L.kind;
-    B.code_bits = L.code_bits;
-    B.kmin = L.kmin;
-    B.span = (uint64_t)L.slots;
+    B->kind = L.kind;
+    B->code_bits = L.code_bits;
+    B->kmin = L.kmin;
+    B->span = (uint64_t)L.slots;
     for (int i = 0; i < SJQ_MAX_PAYLOADS; ++i) {
-        B.pay_min[i] = L.pay_min[i];
-        B.pay_max[i] = L.pay_max[i];
-        B.pay_bits[i] = L.pay_bits[i];
+        B->pay_min[i] = L.pay_min[i];
+        B->pay_max[i] = L.pay_max[i];
+        B->pay_bits[i] = L.pay_bits[i];
     }
-    B.header = reinterpret_cast<unsigned long long *>(T->base);
-    B.status = status_dev;
-    B.slots = T->slots;
-
-    InitParams I{};
-    I.header = reinterpret_cast<uint4 *>(T->base);
-    I.header16 = kTableHeaderBytes / 16;
-    I.slots = reinterpret_cast<uint4 *>(T->slots);
+    B->header = reinterpret_cast<unsigned long long *>(T->base);
+    B->status = status_dev;
+    B->slots = T->slots;
     const bool direct = is_direct_kind(L.kind);
-    size_t filter_bytes = 0;
+    B->usual = usual_payloads(B->rows) && (!direct || L.slots <= INT32_MAX) && L.pay_min[0] >= INT32_MIN &&
+               L.pay_max[0] <= INT32_MAX && L.pay_min[0] <= L.pay_max[0];
+    B->expect_full = direct && L.code_bits > 0 && L.code_bits < 8 && L.entries == L.slots ? (long long)L.entries : -1;
+
+    uint4 pattern;
     if (direct) {
-        const size_t bytes = direct_array_bytes(L);
-        T->slots_bytes = bytes;
+        T->slots_bytes = direct_array_bytes(L);
         const unsigned int fill = L.kind == SJQ_TABLE_DIRECT_BITMAP ? 0u : 0xFFFFFFFFu;
-        I.pattern = make_uint4(fill, fill, fill, fill);
-        if (L.filter_bits) {
-            T->filter = T->slots + align_up(bytes, 256);
-            B.filter = reinterpret_cast<unsigned int *>(T->filter);
-            filter_bytes = (size_t)(L.filter_bits / 8);
-        }
+        pattern = make_uint4(fill, fill, fill, fill);
     } else {
         const int kb = L.key_dtype == SJQ_I64 ? 8 : 4, cb = L.code_bits / 8;
-        B.bucket_k = bucket_keys(kb, cb);
-        B.code_off = bucket_code_offset(kb, cb, B.bucket_k);
-        B.buckets = (uint32_t)(L.slots / B.bucket_k);
-        const size_t bytes = (size_t)B.buckets * kBucketBytes;
-        T->slots_bytes = bytes;
-        if (L.filter_bits) {
-            T->filter = T->slots + align_up(bytes, 256);
-            B.filter = reinterpret_cast<unsigned int *>(T->filter);
-            B.fmask = (uint32_t)(L.filter_bits - 1);
-            filter_bytes = (size_t)(L.filter_bits / 8);
-        }
+        B->bucket_k = bucket_keys(kb, cb);
+        B->code_off = bucket_code_offset(kb, cb, B->bucket_k);
+        B->buckets = (uint32_t)(L.slots / B->bucket_k);
+        B->fmask = (uint32_t)(L.filter_bits - 1);
+        T->slots_bytes = (size_t)B->buckets * kBucketBytes;
         // Every word of a bucket starts as the empty marker's pattern: both markers (the minimum of the key
         // type) are a repeated 0x80 00 .. 00 word, so the codes start as that pattern too and are overwritten
         // when their slot is claimed.
-        I.pattern = L.key_dtype == SJQ_I64 ? make_uint4(0u, 0x80000000u, 0u, 0x80000000u)
-                                           : make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
+        pattern = L.key_dtype == SJQ_I64 ? make_uint4(0u, 0x80000000u, 0u, 0x80000000u)
+                                         : make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
     }
-    I.slots16 = (T->slots_bytes + 15) / 16;
-    I.filter = reinterpret_cast<uint4 *>(T->filter);
-    I.filter16 = (filter_bytes + 15) / 16; // the layout pads the bitmap's region to 256 bytes
-    table_init_kernel<<<grid_for((int64_t)(I.header16 + I.slots16 + I.filter16), dev.sm_count), 256, 0, stream>>>(I);
-    ++T->launches;
-    if (B.dim.n > 0) {
-        build_kernel<<<grid_for(B.dim.n, dev.sm_count), 256, 0, stream>>>(B);
-        ++T->launches;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    if (B->expect_full >= 0) I->task[I->ntasks++] = {reinterpret_cast<uint4 *>(T->base), kTableHeaderBytes / 16, zero, 0, 0};
+    I->task[I->ntasks++] = {reinterpret_cast<uint4 *>(T->slots), (T->slots_bytes + 15) / 16, pattern, 0, 0};
+    if (L.filter_bits) {
+        T->filter = T->slots + align_up(T->slots_bytes, 256);
+        B->filter = reinterpret_cast<unsigned int *>(T->filter);
+        // (the layout pads the bitmap's region to 256 bytes)
+        I->task[I->ntasks++] = {reinterpret_cast<uint4 *>(T->filter), ((size_t)(L.filter_bits / 8) + 15) / 16, zero, 0, 0};
     }
-    if (direct) {
-        const bool promises_every_key = L.code_bits > 0 && L.code_bits < 8 && L.entries == L.slots;
-        direct_count_kernel<<<grid_for(L.slots, dev.sm_count), 256, 0, stream>>>(
-            B, promises_every_key ? (long long)L.entries : -1);
-        ++T->launches;
-    }
-    if (cudaGetLastError() != cudaSuccess) {
-        (void)cudaGetLastError();
-        delete T;
-        return SJQ_ERR_CUDA;
-    }
-    *table = T;
     return SJQ_OK;
+}
+
+// Launch a build kernel behind the fills: it waits for them on the device.
+bool launch_behind(void (*kernel)(BuildParams), BuildParams &B, int threads, int blocks_per_sm, int sm_count, cudaStream_t stream)
+{
+    const uint32_t grid = share_blocks(B.ntasks, (int64_t)blocks_per_sm * sm_count, [&](int i) {
+        return std::make_pair(&B.task[i].rows, (B.task[i].rows.n + 4 * threads - 1) / (4 * threads));
+    });
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, B) == cudaSuccess;
+}
+
+// Enqueue the fills and the builds of a batch: one launch for the direct tables, one for those with open addressing.
+sjq_status build_launch(const sjq_dim_desc *dims, int ndims, const sjq_dim_layout *layouts, void *const *table_mem,
+                        const size_t *table_bytes, int32_t *const *status_dev, bool clear_status, void *stream_,
+                        sjq_table **tables)
+{
+    cudaStream_t stream = (cudaStream_t)stream_;
+    BuildParams B, H;
+    FillParams I{};
+    int nfilters = 0;
+    B.ntasks = H.ntasks = 0;
+    sjq_status st = SJQ_OK;
+    for (int i = 0; i < ndims && st == SJQ_OK; ++i) { // (the entries of `tables` are NULL before)
+        tables[i] = new (std::nothrow) sjq_table();
+        if (!tables[i]) {
+            st = SJQ_ERR_INVALID_ARG;
+            break;
+        }
+        BuildParams &to = is_hash_kind(layouts[i].kind) ? H : B;
+        BuildTask &task = to.task[to.ntasks];
+        st = describe_build(dims[i], layouts[i], table_mem[i], table_bytes[i], status_dev[i], &task, &B.filters,
+                            &nfilters, &I, tables[i]);
+        if (clear_status) I.clear_status[i] = status_dev[i];
+        if (task.rows.n > 0) ++to.ntasks;
+    }
+    DeviceInfo dev;
+    if (st == SJQ_OK) st = device_info(&dev);
+    if (st == SJQ_OK) {
+        const uint32_t fill_grid = share_blocks(I.ntasks, 8 * dev.sm_count, [&](int i) {
+            return std::make_pair(&I.task[i], (int64_t)((I.task[i].units + kFillTile - 1) / kFillTile));
+        });
+        table_init_kernel<<<fill_grid, kFillThreads, 0, stream>>>(I);
+        bool ok = cudaGetLastError() == cudaSuccess;
+        int launches = 1;
+        if (ok && B.ntasks) {
+            ok = launch_behind(direct_build_kernel, B, kBuildThreads, 4, dev.sm_count, stream);
+            ++launches;
+        }
+        if (ok && H.ntasks) {
+            H.filters = B.filters;
+            ok = launch_behind(hash_build_kernel, H, kHashThreads, 5, dev.sm_count, stream);
+            ++launches;
+        }
+        tables[0]->launches = launches;
+        if (!ok) {
+            (void)cudaGetLastError();
+            st = SJQ_ERR_CUDA;
+        }
+    }
+    if (st != SJQ_OK)
+        for (int i = 0; i < ndims; ++i) {
+            delete tables[i];
+            tables[i] = nullptr;
+        }
+    return st;
+}
+
+} // namespace
+} // namespace sjq
+
+extern "C" sjq_status sjq_dims_build(const sjq_dim_desc *dims, int ndims, const sjq_dim_layout *layouts,
+                                     void *const *table_mem, const size_t *table_bytes, int32_t *const *status_dev,
+                                     void *stream, sjq_table **tables)
+{
+    if (!dims || ndims <= 0 || !layouts || !table_mem || !table_bytes || !status_dev || !tables) return SJQ_ERR_INVALID_ARG;
+    for (int i = 0; i < ndims; ++i) tables[i] = nullptr;
+    for (int first = 0; first < ndims;) {
+        const int n = batch_of(dims, ndims, first);
+        const sjq_status st = build_launch(dims + first, n, layouts + first, table_mem + first, table_bytes + first,
+                                           status_dev + first, true, stream, tables + first);
+        if (st != SJQ_OK) {
+            for (int i = 0; i < ndims; ++i) {
+                delete tables[i];
+                tables[i] = nullptr;
+            }
+            return st;
+        }
+        first += n;
+    }
+    return SJQ_OK;
+}
+
+extern "C" sjq_status sjq_build_dim(const sjq_col *cols, int ncols, const sjq_pred *preds, int npreds, int key_col,
+                                    const int *payload_cols, int npayload, const sjq_dim_layout *layout,
+                                    void *table_mem, size_t table_bytes, int32_t *status_dev, void *stream,
+                                    sjq_table **table)
+{
+    if (!layout || !table_mem || !status_dev || !table) return SJQ_ERR_INVALID_ARG;
+    const sjq_dim_desc d{cols, ncols, preds, npreds, key_col, payload_cols, npayload, nullptr};
+    sjq_table *made = nullptr;
+    const sjq_status st = build_launch(&d, 1, layout, &table_mem, &table_bytes, &status_dev, false, stream, &made);
+    if (st == SJQ_OK) *table = made;
+    return st;
 }
 
 extern "C" sjq_status sjq_dim_layout_bytes(const sjq_dim_layout *layout, size_t *bytes)

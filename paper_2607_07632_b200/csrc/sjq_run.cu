@@ -37,6 +37,7 @@ sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gs
                           int64_t *counts, int64_t capacity, int64_t *n_groups, int32_t *status, int sm_count,
                           cudaStream_t stream, int *launches);
 
+int host_stats_release();
 size_t unfused_scratch_bytes(int64_t n, int gathering_joins);
 sjq_status unfused_launch(const RunParams &P, int nfilter, int agg, bool mul, bool has_hash, void *scratch,
                           size_t scratch_bytes, int sm_count, cudaStream_t stream, int *launches);
@@ -1291,6 +1292,7 @@ extern "C" int32_t sjq_release(void)
     }
     if (have_device) (void)cudaSetDevice(current);
     (void)cudaGetLastError();
+    released += sjq::host_stats_release();
     released += sjq_jit_cache_clear();
     released += sjq::fused_cache_clear();
     return released;

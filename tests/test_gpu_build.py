@@ -1,0 +1,112 @@
+"""Table builds at the sizes and key orders where their kernels take another path: parts of a thread's four rows, a
+warp's 128, a block's 1024; neighbouring, descending, scattered and widely spaced keys; repeated keys inside a thread,
+a warp, a block and across blocks; tables without a presence bitmap; batches of more dimensions and filters than one
+launch takes."""
+import numpy as np
+import pytest
+import torch
+
+from datagen.workloads import AggExpr, KeyExpr, Pred, Term
+
+pytestmark = pytest.mark.gpu
+
+sjq = pytest.importorskip("paper_2607_07632_b200") if torch.cuda.is_available() else None
+
+from gpuhelpers import compare, run_both, to_dev  # noqa: E402
+from qhelpers import adhoc  # noqa: E402
+
+SIZES = [1, 3, 4, 5, 127, 128, 129, 1023, 1024, 1025, 40_961]
+
+
+def _keys(n, order, wide, rng):
+    k = np.arange(n, dtype=np.int64)
+    if order == "descending":
+        k = k[::-1].copy()
+    elif order == "scattered":
+        k = rng.permutation(n)
+    elif order == "spaced":
+        k = k * 37
+    k = k - n // 2
+    return k if wide else k.astype(np.int32)
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("order", ["ascending", "descending", "scattered", "spaced"])
+def test_tables_of_every_form(n, order):
+    rng = np.random.default_rng(n)
+    for wide in (False, True):
+        keys = _keys(n, order, wide, rng)
+        for span, forced in ((0, False), (3, False), (13, False), (200, False), (40_000, False), (2**31 - 1, False),
+                             (2**40, False), (0, True), (1000, True), (2**40, True)):
+            dim = {"k": keys, "f": rng.integers(0, 3, n).astype(np.int32)}
+            pay = []
+            if span:
+                dim["p"] = rng.integers(0, span, n, endpoint=True).astype(np.int64 if span > 2**31 else np.int32)
+                pay = ["p"]
+            fk = rng.integers(int(keys.min()) - 5, int(keys.max()) + 6, 3 * n + 7)
+            fact = {"fk": fk.astype(keys.dtype), "m": rng.integers(0, 1000, len(fk)).astype(np.int32)}
+            agg = AggExpr("ADD", Term("FACT", "m"), Term("PAYLOAD", 0, 0)) if pay else AggExpr("COL", Term("FACT", "m"))
+            w = adhoc("forms", fact, [("d", dim, "k", [Pred("f", "NE", 1)], pay, forced)], [("fk", "d")], [], None, agg,
+                      "SCALAR")
+            res, exp, _ = run_both(w, fact, {"d": dim})
+            assert res.status() == 0
+            compare(w, res, exp)
+
+
+@pytest.mark.parametrize("apart", [1, 3, 40, 500, 30_000])
+@pytest.mark.parametrize("order", ["ascending", "scattered"])
+def test_a_repeated_key_is_found_wherever_its_rows_are(apart, order):
+    n, rng = 40_000, np.random.default_rng(apart)
+    keys = _keys(n, order, False, rng)
+    at = 5_001
+    keys[at + apart] = keys[at]
+    for pay_max, forced in ((0, False), (13, False), (200, False), (40_000, False), (2**31 - 1, False), (1000, True)):
+        cols = {"k": keys, "p": np.full(n, pay_max, np.int32)}
+        cols["p"][0] = 0
+        dev = to_dev(cols)
+        pay = ("p",) if pay_max else ()
+        assert sjq.build_dim(dev, "k", (), pay, force_kind=sjq.sjq.FORCE_HASH if forced else 0).status() == 16
+        if pay_max >= 200 and not forced:  # codes of a byte and more may do without the bitmap
+            def bare(L):
+                L.filter_bits = 0
+                L.table_bytes = sjq.layout_bytes(L)
+
+            assert sjq.build_dim(dev, "k", (), pay, edit_layout=bare).status() == 16
+            keep = np.delete(np.arange(n), at + apart)
+            t = sjq.build_dim(to_dev({c: v[keep] for c, v in cols.items()}), "k", (), pay, edit_layout=bare)
+            assert t.status() == 0
+
+
+def test_more_dimensions_and_filters_than_one_launch_takes():
+    rng = np.random.default_rng(5)
+    n, fact, dims, joins, host = 30_011, {}, [], [], {}
+    for j in range(8):
+        rows = [2_500, 1, 1024, 70_000, 33, 5_000, 128, 10][j]
+        dim = {"k": rng.permutation(rows).astype(np.int32)}
+        preds = []
+        for f in range(j + 1):
+            dim[f"f{f}"] = rng.integers(0, 100, rows).astype(np.int32)
+            preds.append(Pred(f"f{f}", "GE", 1))
+        dim["p"] = rng.integers(0, 50, rows).astype(np.int32)
+        fact[f"fk{j}"] = rng.integers(0, rows, n).astype(np.int32)
+        dims.append((f"d{j}", dim, "k", preds, ["p"]))
+        joins.append((f"fk{j}", f"d{j}"))
+        host[f"d{j}"] = dim
+    w = adhoc("eight", fact, dims, joins, [], KeyExpr((Term("PAYLOAD", 0, 0),)),
+              AggExpr("ADD", Term("PAYLOAD", 3, 0), Term("PAYLOAD", 7, 0)), "DENSE", num_groups=50)
+    res, exp, tables = run_both(w, fact, host)
+    assert res.status() == 0
+    compare(w, res, exp)
+    one = {d[0]: sjq.build_dim(to_dev(d[1]), d[2], d[3], d[4]) for d in dims}  # one by one: the same tables
+    for name, t in tables.items():
+        assert t.status() == one[name].status() == 0
+        for f, _ in sjq.DimLayout._fields_:
+            a, b = getattr(t.layout, f), getattr(one[name].layout, f)
+            assert (list(a) == list(b)) if hasattr(a, "__len__") else a == b
+
+
+def test_empty_dimension_in_a_batch():
+    empty = {"k": np.zeros(0, np.int32), "p": np.zeros(0, np.int32)}
+    full = {"k": np.arange(9, dtype=np.int32), "p": np.arange(9, dtype=np.int32)}
+    tables = sjq.sjq._build_tables([(to_dev(d), "k", (), ("p",), sjq.sjq._BuildOpts()) for d in (empty, full, empty)])
+    assert [t.layout.entries for t in tables] == [0, 9, 0] and all(t.status() == 0 for t in tables)
