@@ -4,12 +4,14 @@ from __future__ import annotations
 import glob
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libsjq.so")
 OBJ = os.path.join(HERE, "csrc", "obj")  # one object per translation unit, so that an edit recompiles only its own
+MARSHAL = os.path.join(HERE, "_marshal.so")  # CPython extension: the binding's argument marshalling, linked to LIB
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 
@@ -36,6 +38,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     headers = _headers()
     todo = [s for s in sources() if force or extra or _stale(_object(s), [s] + headers)]
     if not todo and not _stale(LIB, [_object(s) for s in sources()]):
+        _build_marshal(force)
         return LIB
     os.makedirs(OBJ, exist_ok=True)
 
@@ -47,8 +50,17 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
     with ThreadPoolExecutor(max_workers=max(1, min(len(todo), os.cpu_count() or 1))) as pool:
         list(pool.map(compile_one, todo))
-    subprocess.check_call(["nvcc", "-shared", *NVCC_FLAGS[:2], "-o", LIB, *[_object(s) for s in sources()]], cwd=HERE)
+    subprocess.check_call(["nvcc", "-shared", *NVCC_FLAGS[:2], "-Xlinker", "-soname=libsjq.so", "-o", LIB, *[_object(s) for s in sources()]], cwd=HERE)
+    _build_marshal(force)
     return LIB
+
+
+def _build_marshal(force: bool) -> None:
+    src = os.path.join(HERE, "csrc", "sjq_py.cpp")
+    if force or _stale(MARSHAL, [src, os.path.join(ROOT, "include", "sjq.h")]):
+        subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-fPIC", "-shared", "-fvisibility=hidden",
+                               "-I" + os.path.join(ROOT, "include"), "-I" + sysconfig.get_paths()["include"], src, LIB,
+                               "-Wl,-rpath,$ORIGIN", "-o", MARSHAL], cwd=HERE)
 
 
 if __name__ == "__main__":

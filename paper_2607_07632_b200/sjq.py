@@ -73,6 +73,12 @@ class DimLayout(ctypes.Structure):
         return TABLE_KINDS.get(self.kind, str(self.kind))
 
 
+class _DimDesc(ctypes.Structure):
+    _fields_ = [("cols", ctypes.POINTER(_Col)), ("ncols", ctypes.c_int32), ("preds", ctypes.POINTER(_Pred)),
+                ("npreds", ctypes.c_int32), ("key_col", ctypes.c_int32), ("payload_cols", ctypes.POINTER(ctypes.c_int)),
+                ("npayload", ctypes.c_int32), ("opts", ctypes.POINTER(_BuildOpts))]
+
+
 class _Join(ctypes.Structure):
     _fields_ = [("fk_col", ctypes.c_int32), ("table", ctypes.c_void_p)]
 
@@ -194,6 +200,11 @@ def lib():
         L.sjq_build_dim.restype = ctypes.c_int32
         L.sjq_build_dim.argtypes = [ctypes.POINTER(_Col), ip, ctypes.POINTER(_Pred), ip, ip, ctypes.POINTER(ip), ip,
                                     ctypes.POINTER(DimLayout), vp, ctypes.c_size_t, vp, vp, ctypes.POINTER(vp)]
+        L.sjq_dims_plan.restype = ctypes.c_int32
+        L.sjq_dims_plan.argtypes = [ctypes.POINTER(_DimDesc), ip, vp, ctypes.c_size_t, vp, ctypes.POINTER(DimLayout)]
+        L.sjq_dims_build.restype = ctypes.c_int32
+        L.sjq_dims_build.argtypes = [ctypes.POINTER(_DimDesc), ip, ctypes.POINTER(DimLayout), ctypes.POINTER(vp),
+                                     ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(vp), vp, ctypes.POINTER(vp)]
         L.sjq_dim_layout_bytes.restype = ctypes.c_int32
         L.sjq_dim_layout_bytes.argtypes = [ctypes.POINTER(DimLayout), ctypes.POINTER(ctypes.c_size_t)]
         L.sjq_table_info.restype = ctypes.c_int32
@@ -232,12 +243,31 @@ def lib():
     return _lib
 
 
+_marshal = None
+
+
+def marshal():
+    """The extension module that fills the argument structures of sjq_run; raises if it has not been built."""
+    global _marshal
+    if _marshal is None:
+        lib()  # the module is linked to the library: both must be there
+        from . import _marshal as m
+        m.init(torch.int32, torch.int64, OPS, AGGS)
+        _marshal = m
+    return _marshal
+
+
 def strerror(status: int) -> str:
     return lib().sjq_strerror(int(status)).decode()
 
 
 def version() -> str:
     return lib().sjq_version().decode()
+
+
+def _raw_stream(index: int) -> int:
+    """The current stream of a device, without building a Stream object for it."""
+    return torch._C._cuda_getCurrentRawStream(index)
 
 
 def _stream_ptr(device) -> int:
@@ -300,33 +330,47 @@ def build_dim(cols: dict, key: str, preds=(), payloads=(), force_kind: int = 0, 
     the layout from its caller: tests use this to hand it an undersized or inconsistent one).  `mem_offset`
     (a multiple of 16) places the table that many bytes into its allocation: table memory only has to be
     16-byte aligned, and tests use this to get exactly that."""
-    names = list(cols.keys())
-    tensors = [cols[n] for n in names]
-    device = tensors[0].device
+    return _build_tables([(cols, key, preds, payloads, _BuildOpts(force_kind, hash_load_pct, max_direct_bytes,
+                                                                  min_code_bits, 0))], edit_layout, mem_offset)[0]
+
+
+def _build_tables(dims, edit_layout=None, mem_offset: int = 0) -> list:
+    """sjq_dims_plan + sjq_dims_build: the tables of several dimensions of one device with one wait.  dims: sequence
+    of (columns, key, predicates, payloads, _BuildOpts)."""
+    n = len(dims)
+    descs, keep = (_DimDesc * n)(), []
+    device = next(iter(dims[0][0].values())).device
     with torch.cuda.device(device):
-        carr = _cols(tensors)
-        parr, keep = _preds(preds, names)
-        pay = (ctypes.c_int * max(1, len(payloads)))(*[names.index(p) for p in payloads])
-        opts = _BuildOpts(force_kind, hash_load_pct, max_direct_bytes, min_code_bits, 0)
-        scratch = torch.empty(PLAN_SCRATCH_BYTES, dtype=torch.uint8, device=device)
-        layout = DimLayout()
-        stream = _stream_ptr(device)
-        rc = lib().sjq_dim_plan(carr, len(names), parr, len(preds), names.index(key), pay, len(payloads),
-                                ctypes.byref(opts), scratch.data_ptr(), stream, ctypes.byref(layout))
+        for i, (cols, key, preds, payloads, opts) in enumerate(dims):
+            names = list(cols.keys())
+            carr = _cols([cols[c] for c in names])
+            parr, values = _preds(preds, names)
+            pay = (ctypes.c_int * max(1, len(payloads)))(*[names.index(p) for p in payloads])
+            keep.append((carr, parr, values, pay, opts))
+            descs[i] = _DimDesc(carr, len(names), parr, len(preds), names.index(key), pay, len(payloads),
+                                ctypes.pointer(opts))
+        L, stream = lib(), _stream_ptr(device)
+        scratch = torch.empty(n * PLAN_SCRATCH_BYTES, dtype=torch.uint8, device=device)
+        layouts = (DimLayout * n)()
+        rc = L.sjq_dims_plan(descs, n, scratch.data_ptr(), scratch.numel(), stream, layouts)
         if rc != 0:
             raise SjqError(rc, "sjq_dim_plan")
-        planned_bytes = layout.table_bytes
+        planned = [x.table_bytes for x in layouts]
         if edit_layout is not None:
-            edit_layout(layout)
-        mem = torch.empty(max(planned_bytes, layout.table_bytes) + mem_offset, dtype=torch.uint8, device=device)[mem_offset:]
-        status = torch.zeros(1, dtype=torch.int32, device=device)
-        handle = ctypes.c_void_p()
-        rc = lib().sjq_build_dim(carr, len(names), parr, len(preds), names.index(key), pay, len(payloads),
-                                 ctypes.byref(layout), mem.data_ptr(), mem.numel(), status.data_ptr(), stream,
-                                 ctypes.byref(handle))
+            for x in layouts:
+                edit_layout(x)
+        mems = [torch.empty(max(p, x.table_bytes) + mem_offset, dtype=torch.uint8, device=device)[mem_offset:]
+                for p, x in zip(planned, layouts)]
+        status = torch.empty(n, dtype=torch.int32, device=device)  # cleared by the build
+        statuses = [status[i:i + 1] for i in range(n)]
+        vp = ctypes.c_void_p
+        handles = (vp * n)()
+        rc = L.sjq_dims_build(descs, n, layouts, (vp * n)(*[m.data_ptr() for m in mems]),
+                              (ctypes.c_size_t * n)(*[m.numel() for m in mems]),
+                              (vp * n)(*[s.data_ptr() for s in statuses]), stream, handles)
         if rc != 0:
             raise SjqError(rc, "sjq_build_dim")
-    return Table(handle.value, layout, mem, status)
+    return [Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], statuses[i]) for i in range(n)]
 
 
 class TableBuilder:
@@ -659,25 +703,19 @@ def _result_struct(res: "Result") -> _Result:
 def run(fact: dict, preds=(), joins=(), key=None, agg=None, mode: str = "SCALAR", num_groups: int = 1,
         capacity: int = 0, opts: Optional[RunOpts] = None, result: Optional[Result] = None) -> Result:
     """sjq_run over a dict of CUDA tensors.  joins: sequence of (fk column name, Table)."""
-    names = list(fact.keys())
-    tensors = [fact[n] for n in names]
-    device = tensors[0].device
-    with torch.cuda.device(device):
-        carr = _cols(tensors)
-        parr, jarr, kexpr, aexpr, keep = _query(names, preds, joins, key, agg)
-        spec = _ResultSpec(MODES[mode], num_groups, capacity)
-        res = result if result is not None else alloc_result(mode, num_groups, capacity, agg.want_count, device)
-        cres = _result_struct(res)
-        copts = (opts or RunOpts()).to_c()
-        if not copts.hot_scratch and copts.hot_keys != 2 and any(t.layout.kind_name.startswith("HASH") for _, t in joins):
-            scratch = _hot_scratch(device)  # one per device, reused by every run (runs on one stream are ordered)
-            copts.hot_scratch, copts.hot_scratch_bytes = scratch.data_ptr(), scratch.numel()
-        rc = lib().sjq_run(carr, len(names), parr, len(preds), jarr, len(joins),
-                           ctypes.byref(kexpr) if kexpr is not None else None, ctypes.byref(aexpr),
-                           ctypes.byref(spec), ctypes.byref(cres), ctypes.byref(copts), _stream_ptr(device),
-                           ctypes.byref(res.info))
-        if rc != 0:
-            raise SjqError(rc, "sjq_run")
+    device = next(iter(fact.values())).device
+    if device.type != "cuda":
+        raise ValueError("columns must be contiguous 1-D int32/int64 CUDA tensors")
+    index = device.index
+    if index != torch.cuda.current_device():
+        with torch.cuda.device(device):
+            return run(fact, preds, joins, key, agg, mode, num_groups, capacity, opts, result)
+    res = result if result is not None else alloc_result(mode, num_groups, capacity, agg.want_count, device)
+    # (one hot-key scratch per device, reused by every run: runs on one stream are ordered)
+    rc = marshal().run(fact, preds, joins, key, agg, MODES[mode], num_groups, capacity, opts, res,
+                       _raw_stream(index), lambda: _hot_scratch(device))
+    if rc != 0:
+        raise SjqError(rc, "sjq_run")
     return res
 
 
@@ -842,11 +880,11 @@ def release() -> int:
 
 def build_workload_tables(w, dims: dict) -> dict:
     """dims: dimension name -> dict of CUDA column tensors (a workload description's dims)."""
-    out = {}
-    for d in w.dims:
-        out[d.name] = build_dim(dims[d.name], d.key, d.preds, d.payloads,
-                                force_kind=FORCE_HASH if d.force_hash else 0)
-    return out
+    if not w.dims:
+        return {}
+    tables = _build_tables([(dims[d.name], d.key, d.preds, d.payloads, _BuildOpts(FORCE_HASH if d.force_hash else 0))
+                            for d in w.dims])
+    return {d.name: t for d, t in zip(w.dims, tables)}
 
 
 def run_workload(w, fact: dict, tables: dict, opts: Optional[RunOpts] = None,
