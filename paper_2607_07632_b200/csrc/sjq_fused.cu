@@ -21,6 +21,7 @@ struct ClearParams {
 // (every array starts on a 16-byte boundary; the odd last word is thread 0's)
 __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
 {
+    asm volatile("griddepcontrol.launch_dependents;"); // the fused kernel may start and wait for this one on the device
     const int64_t stride = (int64_t)blockDim.x * gridDim.x;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const longlong2 zero = make_longlong2(0, 0), empty = make_longlong2(kEmptyKey64, kEmptyKey64);
@@ -284,12 +285,23 @@ sjq_status fused_occupancy(int agg, bool mul, bool hash, int block, size_t smem,
     return SJQ_OK;
 }
 
-sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, const RunParams &P,
-                        cudaStream_t stream)
+sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, bool behind,
+                        const RunParams &P, cudaStream_t stream)
 {
-    fused_fn fn = pick_kernel(agg, mul, hash);
-    fn<<<grid, block, smem, stream>>>(P);
-    if (cudaGetLastError() != cudaSuccess) return SJQ_ERR_CUDA;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = behind ? 1 : 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, pick_kernel(agg, mul, hash), P) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return SJQ_ERR_CUDA;
+    }
     return SJQ_OK;
 }
 

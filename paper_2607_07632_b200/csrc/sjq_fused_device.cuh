@@ -1100,6 +1100,8 @@ __device__ __forceinline__ void fused_body(const RunParams &P, unsigned char *sm
         for (int64_t i = tid; i < cells; i += blockDim.x) ss[i] = 0ull;
     }
     __syncthreads();
+    // launched behind the kernel that clears the results: nothing above touches them, everything below may
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     int64_t lsum = 0, lcnt = 0;
 

@@ -359,7 +359,7 @@ sjq_status jit_occupancy(const RunParams &P, int agg, bool mul, bool hash, int b
 }
 
 sjq_status jit_launch(const RunParams &P, int agg, bool mul, bool hash, int grid, int block, int lb_blocks,
-                      size_t smem, cudaStream_t stream)
+                      size_t smem, bool behind, cudaStream_t stream)
 {
     cudaKernel_t kernel;
     {
@@ -379,8 +379,17 @@ sjq_status jit_launch(const RunParams &P, int agg, bool mul, bool hash, int grid
     std::memcpy(packed, P.st, nst * sizeof(DStage));
     std::memcpy(packed + nst * sizeof(DStage), reinterpret_cast<const unsigned char *>(&P) + tail_from, tail_bytes);
     void *args[] = {packed};
-    if (cudaLaunchKernel(reinterpret_cast<const void *>(kernel), dim3(grid), dim3(block), args, smem, stream) !=
-        cudaSuccess) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = behind ? 1 : 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), args) != cudaSuccess) {
         (void)cudaGetLastError();
         return SJQ_ERR_CUDA;
     }

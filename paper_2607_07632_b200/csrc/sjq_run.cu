@@ -27,9 +27,9 @@ sjq_status fused_occupancy(int agg, bool mul, bool hash, int block, size_t smem,
 sjq_status jit_occupancy(const RunParams &P, int agg, bool mul, bool hash, int block, int lb_blocks, size_t smem,
                          int *ctas_per_sm);
 sjq_status jit_launch(const RunParams &P, int agg, bool mul, bool hash, int grid, int block, int lb_blocks,
-                      size_t smem, cudaStream_t stream);
-sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, const RunParams &P,
-                        cudaStream_t stream);
+                      size_t smem, bool behind, cudaStream_t stream);
+sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, bool behind,
+                        const RunParams &P, cudaStream_t stream);
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
                         int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream);
 sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gslots, bool indexed,
@@ -963,8 +963,12 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
                             dev.sm_count, stream, &launches);
         if (st != SJQ_OK) return st;
     } else if (n > 0) {
-        st = jit ? jit_launch(P, aggp, mul, has_hash, grid, block, lb_blocks, smem, stream)
-                 : fused_launch(aggp, mul, has_hash, grid, block, smem, P, stream);
+        // Directly behind the clear the kernel is launched while that one still runs (programmatic dependent launch): it
+        // stages its tables, which were complete before the clear began, and waits for the clear before it touches a
+        // result (two-join query, 60 M rows: 94 -> 92 us; filter and sum, 6 M rows: 20.5 -> 18.5 us back to back).
+        const bool behind = !opts.accumulate && hot_stage < 0 && !opts.event_before;
+        st = jit ? jit_launch(P, aggp, mul, has_hash, grid, block, lb_blocks, smem, behind, stream)
+                 : fused_launch(aggp, mul, has_hash, grid, block, smem, behind, P, stream);
         if (st != SJQ_OK) return st;
         ++launches;
     }
