@@ -520,7 +520,12 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     const bool register_terminal = spec->mode == SJQ_SCALAR || (spec->mode == SJQ_DENSE && spec->num_groups == 1);
     const bool mostly_survive = opts.specialise && opts.compaction == 0 &&
                                 reach[nfilter] >= (register_terminal ? kDirectSurvival : kDirectSurvivalGrouped);
-    const bool direct = opts.eager_loads || opts.compaction == 1 || nfilter == 0 || opts.unfused || mostly_survive;
+    // Few rows: the kernel's time is a chain of memory latencies, one per queue level, and without queues it is one in
+    // all (compiled, 400 thousand rows: city x city 12.5 -> 8.7 us, city x brand 14.6 -> 12.6, the others alike;
+    // interpreted: four joins 16.6 -> 12.5, two joins 14.5 -> 10.5, filter and sum 12.5 -> 10.4; at 800 thousand rows
+    // some gain and some lose).
+    const bool few_rows = n <= (int64_t)1 << 19 && opts.compaction == 0;
+    const bool direct = few_rows || opts.eager_loads || opts.compaction == 1 || nfilter == 0 || opts.unfused || mostly_survive;
     if (!direct) {
         nd0 = 1;
         if (opts.compaction != 2) {
@@ -528,8 +533,15 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
             while (nd0 < nfilter && specs[order[nd0]].sel < 0.9 && reach[nd0] > dense_reach &&
                    specs[order[nd0]].prefilter != 2)
                 ++nd0;
+            // A queue of its own pays for a filter that still sees more than about one row in eight; a later one is
+            // better taken at the final level, whose columns a compiled kernel requests together (600 M rows: four
+            // joins, the third filter reached by 6 % of the rows, 1286 us with a queue for it and 1223 without, but
+            // 1295 without one for the second, reached by 20 %; filter and sum, 4 %: 1280 and 1109; two joins, 4 %:
+            // 783 and 735).  The interpreting kernel loads its columns one after the other and is better off with
+            // queues (four joins, 60 M rows: 175 us against 290 without any).
+            const double queue_reach = opts.specialise ? 0.12 : 0.002;
             while (nd0 + nfq < nfilter && nfq < kMaxQueues - 1 && specs[order[nd0 + nfq]].sel < 0.9 &&
-                   reach[nd0 + nfq] > 0.002 && specs[order[nd0 + nfq]].prefilter != 2)
+                   reach[nd0 + nfq] > queue_reach && specs[order[nd0 + nfq]].prefilter != 2)
                 ++nfq;
         }
     }
@@ -537,13 +549,20 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     P.nd0 = nd0;
     P.nq = direct ? 0 : nfq + 1;
     P.rows = opts.rows_per_lane ? opts.rows_per_lane : 4;
-    P.slots = (opts.specialise && opts.dense_slots == 4) ? 4 : 2;
+    // Few survivors of level 0 leave a compiled kernel room for sixteen rows per thread: twice the loads in flight for
+    // the column that every row reads (200 M rows: two joins, 4 % left, 282 -> 250 us; city x brand, 4 %, 261 -> 220;
+    // the sweep into a thousand groups at 1, 3, 6, 10 %, 210 -> 201, 297 -> 290, 354 -> 348, 412 -> 406).  With more
+    // left the first queue, twice as large, costs more than it gives (14 % 447 -> 447, 20 % 477 -> 485; four joins,
+    // 20 %, 409 -> 438), with next to none the lane's longer test of its rows does (0.1 % 127 -> 131).
+    const bool few_left = opts.specialise && P.nq && reach[nd0] < 0.15;
+    const bool sixteen = opts.dense_slots == 4 || (opts.dense_slots == 0 && few_left && reach[nd0] >= 0.005 && reach[nd0] < 0.12);
+    P.slots = opts.specialise && sixteen ? 4 : 2;
     // a third or more of the rows reaching the first queue: pushes are dense enough for bank conflicts to matter
     P.qfold = (opts.specialise && P.nq && reach[nd0] >= 0.3) ? 7u : 0u;
     // fewer than about one row in seven surviving level 0: pushing by walking the set bits of a thread's mask beats
     // testing its eight rows one by one (city x brand 0.72 -> 0.68 ms, city x city 0.72 -> 0.71; at one in five,
     // the four-join workload, it loses: 1.19 -> 1.21 ms)
-    P.sparse_push = (opts.specialise && P.nq && reach[nd0] < 0.15) ? 1 : 0;
+    P.sparse_push = few_left ? 1 : 0;
 
     // Sources of the accumulators.  A dense stage cannot feed an accumulator
     // (it only keeps a bit per row), so a value it would supply is gathered
@@ -783,7 +802,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     // drop (the sweep at 50 %, one group: 1.48 -> 1.41 ms) and cost a little when none does (100 %: 2.18 -> 2.22).
     const bool two_wide_blocks = opts.specialise && !opts.unfused && !opts.block_threads && !opts.ctas_per_sm &&
                                  P.nq == 0 && (aggp == AGG_SMEM || (aggp == AGG_SCALAR && reach[nfilter] < 0.8));
-    if (two_wide_blocks) block = aggp == AGG_SMEM ? 640 : 768;
+    if (two_wide_blocks) block = few_rows && aggp != AGG_SMEM ? 256 : aggp == AGG_SMEM ? 640 : 768;
     const size_t smem_cap = (size_t)dev.max_smem_optin - 1024; // static reduce scratch + slack
     const size_t stage_bytes = align_up((size_t)ns * sizeof(DStage), 16);
     if (hot_bytes && stage_bytes + hot_bytes + group_bytes +
@@ -835,34 +854,27 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     // queues.  A kernel compiled for the query can run as one block of 1024 threads per SM instead: one
     // copy, 32 warps instead of 24.  Measured better whenever the copies are sizeable or shared memory
     // would crowd out the L1 (config 3: 1.43 -> 1.32 ms, config 5: 2.8 -> 1.8 ms), given enough tiles per
-    // block to even out the tail.
-    bool single_block = false;
-    // Between the two: a kernel with queues whose shared memory is moderate (more than three 384-thread blocks
-    // could share, at most 100 KB as a 640-thread block) runs as two 640-thread blocks: 40 warps instead of 24 or
-    // 32 and the L1 keeps half of the SM's memory (two-join workload 0.101 -> 0.094 ms, city x brand 0.681 ->
-    // 0.667, city x city 0.700 -> 0.691).
-    bool two_wide_queue_blocks = false;
-    if (opts.specialise && !opts.block_threads && !opts.ctas_per_sm && P.nq && !opts.unfused &&
-        stage_bytes + tables + hot_bytes + group_bytes + queue_bytes(block) > ((size_t)48 << 10)) {
-        size_t tables640 = 0;
-        if (stage_tables(640, &tables640) &&
-            stage_bytes + tables640 + hot_bytes + group_bytes + queue_bytes(640) <= ((size_t)100 << 10)) {
-            block = 640;
-            tables = tables640;
-            two_wide_queue_blocks = true;
-        } else if (!stage_tables(block, &tables)) {
-            return SJQ_ERR_UNSUPPORTED;
-        }
-    }
-    if (opts.specialise && !opts.block_threads && !opts.ctas_per_sm && P.nq && !two_wide_queue_blocks) {
-        const size_t copies = tables + hot_bytes + group_bytes;
+    // block to even out the tail (four joins: 140 -> 135 us at 60 M rows, 49 tiles a block; 23.3 -> 23.0 at 6 M; two
+    // joins with sixteen rows per thread: 84.8 -> 84.9 at 60 M, 25 tiles, 14.5 -> 15.8 at 6 M, 2 tiles).
+    // Failing that, a kernel whose shared memory is moderate (more than three 384-thread blocks
+    // could share, at most 100 KB as a 640-thread block) runs as two 640-thread blocks: 40 warps instead of 24 and the
+    // L1 keeps half of the SM's memory (two-join workload 0.101 -> 0.094 ms with eight rows per thread).  With sixteen
+    // rows per thread its queues leave the L1 too little once survivors gather at random (the sweep, 200 M rows, as two
+    // blocks of 640 or of 384: 1 % 201 and 210 us, 3 % 294 and 290, 10 % 462 and 406).
+    bool single_block = false, two_wide_queue_blocks = false;
+    if (opts.specialise && !opts.block_threads && !opts.ctas_per_sm && P.nq && !opts.unfused) {
+        const size_t copies = tables + hot_bytes + group_bytes, as384 = stage_bytes + copies + queue_bytes(block);
         const int64_t tiles_per_block = n / ((int64_t)1024 * 4 * P.slots) / dev.sm_count;
-        size_t tables1024 = 0;
-        if ((copies >= ((size_t)16 << 10) || stage_bytes + copies + queue_bytes(block) > ((size_t)80 << 10)) &&
-            tiles_per_block >= 128 && stage_tables(1024, &tables1024)) {
+        size_t other = 0;
+        if ((copies >= ((size_t)16 << 10) || as384 > ((size_t)80 << 10)) && tiles_per_block >= 16 && stage_tables(1024, &other)) {
             block = 1024;
             single_block = true;
-            tables = tables1024;
+            tables = other;
+        } else if (as384 > ((size_t)48 << 10) && (P.slots == 2 || reach[nd0] < 0.03) && stage_tables(640, &other) &&
+                   stage_bytes + other + hot_bytes + group_bytes + queue_bytes(640) <= ((size_t)100 << 10)) {
+            block = 640;
+            two_wide_queue_blocks = true;
+            tables = other;
         } else if (!stage_tables(block, &tables)) {
             return SJQ_ERR_UNSUPPORTED;
         }

@@ -40,3 +40,23 @@ def test_any_number_of_filters(npreds):
         assert res.status() == 0
         compare(w, res, exp)
         assert sorted(res.info.order[: npreds + 1]) == list(range(npreds + 1))
+
+
+@pytest.mark.parametrize("n", [2**19 - 1, 2**19, 2**19 + 1, 700_001])
+@pytest.mark.parametrize("below", [2, 10, 60, 130, 400])
+def test_launch_shapes_by_rows_and_survivors(n, below):
+    """Queue-free plans up to 2^19 rows, queues beyond; eight or sixteen rows per thread at level 0; a queue for the
+    second filter or not."""
+    rng = np.random.default_rng(below)
+    fact = {"p": rng.integers(0, 1000, n).astype(np.int32), "q": rng.integers(0, 1000, n).astype(np.int32),
+            "fk": rng.integers(0, 50_000, n).astype(np.int32), "m": rng.integers(-2**31, 2**31 - 1, n).astype(np.int32)}
+    dim = {"k": np.arange(50_000, dtype=np.int32), "a": (np.arange(50_000) % 3).astype(np.int32)}
+    preds = [Pred("p", "LT", below), Pred("q", "LT", 300)]
+    w = adhoc("shapes", fact, [("d", dim, "k", [Pred("a", "EQ", 1)], [])], [("fk", "d")], preds, None,
+              AggExpr("COL", Term("FACT", "m")), "SCALAR")
+    ppm = [below * 1000, 300_000]
+    for opts in (sjq.RunOpts(pass_ppm=ppm), sjq.RunOpts(specialise=True, pass_ppm=ppm)):
+        res, exp, _ = run_both(w, fact, {"d": dim}, opts=opts)
+        assert res.status() == 0
+        compare(w, res, exp)
+        assert (res.info.reserved_levels == 0) == (n <= 2**19)
