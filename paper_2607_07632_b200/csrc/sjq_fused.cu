@@ -1,5 +1,6 @@
 // Ahead-of-time instantiations of the fused probe kernel (the query is a descriptor interpreted at
 // run time), result housekeeping kernels and the launch helpers used by the planner.
+#include <cstring>
 #include <mutex>
 #include <unordered_map>
 
@@ -222,13 +223,13 @@ __global__ void __launch_bounds__(256) sample_kernel(const __grid_constant__ Sam
         atomicAdd(&S.counts[threadIdx.x], (unsigned long long)block_counts[threadIdx.x]);
 }
 
-fused_fn pick_kernel(int agg, bool mul, bool hash)
+const void *pick_kernel(int agg, bool mul, bool hash, bool few)
 {
     switch (agg) {
-    case AGG_SCALAR: return fused_variant_scalar(mul, hash);
-    case AGG_SMEM: return fused_variant_smem(mul, hash);
-    case AGG_GLOBAL: return fused_variant_global(mul, hash);
-    default: return fused_variant_hash(mul, hash);
+    case AGG_SCALAR: return few ? reinterpret_cast<const void *>(fused_few_scalar(mul, hash)) : reinterpret_cast<const void *>(fused_variant_scalar(mul, hash));
+    case AGG_SMEM: return few ? reinterpret_cast<const void *>(fused_few_smem(mul, hash)) : reinterpret_cast<const void *>(fused_variant_smem(mul, hash));
+    case AGG_GLOBAL: return few ? reinterpret_cast<const void *>(fused_few_global(mul, hash)) : reinterpret_cast<const void *>(fused_variant_global(mul, hash));
+    default: return few ? reinterpret_cast<const void *>(fused_few_hash(mul, hash)) : reinterpret_cast<const void *>(fused_variant_hash(mul, hash));
     }
 }
 
@@ -252,18 +253,19 @@ int fused_cache_clear()
     return n;
 }
 
-sjq_status fused_occupancy(int agg, bool mul, bool hash, int block, size_t smem, int *ctas_per_sm)
+sjq_status fused_occupancy(int agg, bool mul, bool hash, int nstages, int block, size_t smem, int *ctas_per_sm)
 {
+    const bool few = nstages <= kFewStages;
     std::mutex &mutex = g_occ_mutex;
     std::unordered_map<uint64_t, int> &occupancy = g_occupancy;
     std::unordered_map<uint32_t, int> &opted = g_opted;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SJQ_ERR_CUDA;
-    const uint32_t variant = (uint32_t)(agg * 4 + (mul ? 2 : 0) + (hash ? 1 : 0));
+    const uint32_t variant = (uint32_t)(agg * 8 + (mul ? 4 : 0) + (hash ? 2 : 0) + (few ? 1 : 0));
     const uint32_t fkey = (uint32_t)dev * 64u + variant;
     const uint64_t okey = ((uint64_t)fkey << 40) | ((uint64_t)block << 24) | (uint64_t)(smem & 0xFFFFFF);
     std::lock_guard<std::mutex> lock(mutex);
-    fused_fn fn = pick_kernel(agg, mul, hash);
+    const void *fn = pick_kernel(agg, mul, hash, few);
     auto o = opted.find(fkey);
     if (o == opted.end() || o->second < (int)smem) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
@@ -298,7 +300,16 @@ sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, pick_kernel(agg, mul, hash), P) != cudaSuccess) {
+    void *args[1];
+    RunParamsFew little;
+    if (P.nstages <= kFewStages) {
+        std::memcpy(little.st, P.st, (size_t)P.nstages * sizeof(DStage));
+        static_cast<RunCore &>(little) = P;
+        args[0] = &little;
+    } else {
+        args[0] = const_cast<RunParams *>(&P);
+    }
+    if (cudaLaunchKernelExC(&cfg, pick_kernel(agg, mul, hash, P.nstages <= kFewStages), args) != cudaSuccess) {
         (void)cudaGetLastError();
         return SJQ_ERR_CUDA;
     }

@@ -57,6 +57,14 @@ namespace sjq {
 
 namespace {
 
+// The parameter block as the functions below see it: a compiled kernel's stages are parameters like the rest, the
+// interpreting kernels pass theirs along as a copy in shared memory.
+#if defined(SJQ_JIT)
+typedef RunParams RunArg;
+#else
+typedef RunCore RunArg;
+#endif
+
 template <typename T>
 struct Vec4;
 template <>
@@ -131,7 +139,7 @@ __device__ __forceinline__ uint32_t body_pred_range(const DStage &S, const T (&v
 }
 
 template <typename T, int NR>
-__device__ __forceinline__ uint32_t body_pred_set(const RunParams &P, const DStage &S, const T (&v)[NR], uint32_t m)
+__device__ __forceinline__ uint32_t body_pred_set(const RunArg &P, const DStage &S, const T (&v)[NR], uint32_t m)
 {
     uint32_t pass = 0;
     for (int k = 0; k < S.nset; ++k) {
@@ -391,7 +399,7 @@ __device__ __forceinline__ uint32_t body_hashbits(const DStage &S, const unsigne
 }
 
 template <typename T, int NR, bool WANT, bool HASH>
-__device__ __forceinline__ uint32_t run_stage(const RunParams &P, const DStage &S, const unsigned char *smem,
+__device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, const unsigned char *smem,
                                               const T (&v)[NR], uint32_t m, uint64_t (&code)[NR])
 {
     switch (S.op * 2 + S.in_smem) {
@@ -575,7 +583,7 @@ __device__ __forceinline__ uint64_t smem_cell(const unsigned int *words, uint64_
 // aggregation; every test on the query shape is uniform and outside the row loops.
 // PAIRS: every lane of the warp arrives here (with or without rows), so lanes may work on each other's rows.
 template <int AGG, bool MUL, int NR, bool PAIRS = true>
-__device__ __forceinline__ void terminal(const RunParams &P, unsigned char *smem, const int64_t (&key)[NR],
+__device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, const int64_t (&key)[NR],
                                          const int64_t (&X)[NR], const int64_t (&Y)[NR], uint32_t m, int64_t &lsum,
                                          int64_t &lcnt)
 {
@@ -743,7 +751,7 @@ __device__ __forceinline__ void load_rows(const DStage &S, int64_t base, const u
 
 // One pure filter stage on a batch: returns the mask of rows that pass.
 template <bool HASH, int NR>
-__device__ __forceinline__ uint32_t filter_rows(const RunParams &P, const DStage &S, const unsigned char *smem,
+__device__ __forceinline__ uint32_t filter_rows(const RunArg &P, const DStage &S, const unsigned char *smem,
                                                 int64_t base, const uint32_t (&off)[NR], uint32_t valid)
 {
     uint64_t unused[NR];
@@ -761,7 +769,7 @@ __device__ __forceinline__ uint32_t filter_rows(const RunParams &P, const DStage
 // the next stage is requested before the current stage's probe is resolved, so
 // a stage costs one memory latency, not two.
 template <int AGG, bool MUL, bool CONTIG, bool HASH, int NR>
-__device__ __forceinline__ void final_rows(const RunParams &P, const DStage *st, unsigned char *smem, int first,
+__device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, unsigned char *smem, int first,
                                            int64_t base, const uint32_t (&off)[NR], uint32_t valid, int64_t &lsum,
                                            int64_t &lcnt)
 {
@@ -832,7 +840,7 @@ __device__ __forceinline__ void final_rows(const RunParams &P, const DStage *st,
 // whose rows survive, where every column is read whole anyway): one 128-bit load per column, issued up
 // front, four columns deep.
 template <int AGG, bool MUL, bool HASH, bool CONTIG, int NR>
-__device__ __forceinline__ void final_rows_scheduled(const RunParams &P, unsigned char *smem, int first, int64_t base,
+__device__ __forceinline__ void final_rows_scheduled(const RunArg &P, unsigned char *smem, int first, int64_t base,
                                                      const uint32_t (&off)[NR], uint32_t valid, int64_t &lsum,
                                                      int64_t &lcnt)
 {
@@ -897,7 +905,7 @@ __device__ __forceinline__ void final_rows_scheduled(const RunParams &P, unsigne
 // `staged` != nullptr: the tile's values of this column were copied into shared memory by a bulk-asynchronous
 // copy (in table order); the thread reads its four values of each slice from there.
 template <typename T, bool FULL, bool HASH>
-__device__ __forceinline__ uint32_t dense_stage(const RunParams &P, const DStage &S, const unsigned char *smem,
+__device__ __forceinline__ uint32_t dense_stage(const RunArg &P, const DStage &S, const unsigned char *smem,
                                                 int64_t row0, int32_t slot_stride, uint32_t valid, uint32_t alive,
                                                 const unsigned char *staged = nullptr)
 {
@@ -933,7 +941,7 @@ __device__ __forceinline__ uint32_t dense_stage(const RunParams &P, const DStage
 }
 
 template <bool FULL, bool HASH>
-__device__ __forceinline__ uint32_t level0(const RunParams &P, const DStage *st, const unsigned char *smem,
+__device__ __forceinline__ uint32_t level0(const RunArg &P, const DStage *st, const unsigned char *smem,
                                            int64_t row0, int32_t slot_stride, uint32_t valid,
                                            const unsigned char *staged = nullptr)
 {
@@ -1030,7 +1038,7 @@ __device__ __forceinline__ uint32_t queue_base(int l)
 
 // The scalar terminal's tail (Section 3.2: one atomic per block instead of one per matching row): warp
 // shuffle reduce, block reduce through shared memory, one global atomic per block.
-__device__ __forceinline__ void scalar_block_reduce(const RunParams &P, int64_t lsum, int64_t lcnt)
+__device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsum, int64_t lcnt)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
@@ -1058,8 +1066,9 @@ __device__ __forceinline__ void scalar_block_reduce(const RunParams &P, int64_t 
     }
 }
 
+// `given`: the stage descriptors of the parameter block.
 template <int AGG, bool MUL, bool HASH>
-__device__ __forceinline__ void fused_body(const RunParams &P, unsigned char *smem)
+__device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given, unsigned char *smem)
 {
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -1070,7 +1079,7 @@ __device__ __forceinline__ void fused_body(const RunParams &P, unsigned char *sm
 #if !defined(SJQ_JIT)
     {
         const uint32_t words = (uint32_t)(P.nstages * sizeof(DStage) / 8);
-        const uint64_t *src = reinterpret_cast<const uint64_t *>(&P.st[0]);
+        const uint64_t *src = reinterpret_cast<const uint64_t *>(given);
         uint64_t *dst = reinterpret_cast<uint64_t *>(st);
         for (uint32_t i = tid; i < words; i += blockDim.x) dst[i] = src[i];
     }
@@ -1080,7 +1089,7 @@ __device__ __forceinline__ void fused_body(const RunParams &P, unsigned char *sm
 #if defined(SJQ_JIT)
         const DStage &S = SJQ_STAGE(s);
 #else
-        const DStage &S = P.st[s];
+        const DStage &S = given[s];
 #endif
         if (S.in_smem) {
             const uint4 *src = static_cast<const uint4 *>(S.tab);
@@ -1373,11 +1382,19 @@ __device__ __forceinline__ void fused_body(const RunParams &P, unsigned char *sm
 
 
 #if !defined(SJQ_JIT)
-template <int AGG, bool MUL, bool HASH>
-__global__ void __launch_bounds__(SJQ_LB_THREADS, SJQ_LB_BLOCKS) fused_kernel(const __grid_constant__ RunParams P)
+template <typename Params, int AGG, bool MUL, bool HASH>
+__global__ void __launch_bounds__(SJQ_LB_THREADS, SJQ_LB_BLOCKS) fused_kernel(const __grid_constant__ Params P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    fused_body<AGG, MUL, HASH>(P, smem);
+    fused_body<AGG, MUL, HASH>(P, P.st, smem);
+}
+
+// The kernel of one aggregation path for a parameter block.
+template <typename Params, int AGG>
+auto fused_variant(bool mul, bool hash) -> void (*)(const Params)
+{
+    if (mul) return hash ? fused_kernel<Params, AGG, true, true> : fused_kernel<Params, AGG, true, false>;
+    return hash ? fused_kernel<Params, AGG, false, true> : fused_kernel<Params, AGG, false, false>;
 }
 #endif
 
@@ -1390,7 +1407,7 @@ extern "C" __global__ void __launch_bounds__(SJQ_LB_THREADS, SJQ_LB_BLOCKS)
     sjq_jit_kernel(const __grid_constant__ sjq::RunParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    sjq::fused_body<SJQ_JIT_AGG, (SJQ_JIT_MUL != 0), (SJQ_JIT_HASH != 0)>(P, smem);
+    sjq::fused_body<SJQ_JIT_AGG, (SJQ_JIT_MUL != 0), (SJQ_JIT_HASH != 0)>(P, P.st, smem);
 }
 #endif
 #endif

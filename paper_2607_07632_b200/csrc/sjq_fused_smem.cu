@@ -1,13 +1,9 @@
 // Ahead-of-time instantiations of the fused kernel for one aggregation path (AGG_SMEM); one translation unit per
-// path so that the four compile in parallel.
+// path and size of the parameter block so that they compile in parallel.
 #include "sjq_fused_device.cuh"
 
 namespace sjq {
 
-fused_fn fused_variant_smem(bool mul, bool hash)
-{
-    if (mul) return hash ? fused_kernel<AGG_SMEM, true, true> : fused_kernel<AGG_SMEM, true, false>;
-    return hash ? fused_kernel<AGG_SMEM, false, true> : fused_kernel<AGG_SMEM, false, false>;
-}
+fused_fn fused_variant_smem(bool mul, bool hash) { return fused_variant<RunParams, AGG_SMEM>(mul, hash); }
 
 } // namespace sjq

@@ -203,29 +203,37 @@ namespace {
 
 // Everything jit_shape_header prints, as bytes: cheap to build on every run; the text itself is only
 // generated when the key is new.
-std::string shape_key(const RunParams &P, int agg, bool mul, bool hash, int lb_threads, int lb_blocks)
+struct ShapeKey {
+    size_t size = 0;
+    unsigned char bytes[128 + 160 * kMaxStages];
+
+    void put(const void *p, size_t n)
+    {
+        std::memcpy(bytes + size, p, n);
+        size += n;
+    }
+};
+
+void shape_key(const RunParams &P, int agg, bool mul, bool hash, int lb_threads, int lb_blocks, ShapeKey *k)
 {
-    std::string k;
-    k.reserve(64 + (size_t)P.nstages * 128);
-    auto put_raw = [&](const void *p, size_t n) { k.append(static_cast<const char *>(p), n); };
     const int32_t head[] = {agg, mul ? 1 : 0, hash ? 1 : 0, lb_threads, lb_blocks, P.nstages, P.nd0, P.nq,
                             P.rows, P.want_count, P.eager, P.has_key, P.mod32, (int32_t)P.qfold, P.slots, P.warp_agg,
                             P.l0_bulk, P.count32, P.sparse_push, P.cell_shift, P.pairs};
-    put_raw(head, sizeof(head));
-    put_raw(&P.modulo, sizeof(P.modulo));
-    put_raw(&P.modmask, sizeof(P.modmask));
+    static_assert(sizeof(head) + 16 <= 128, "room for the head");
+    k->put(head, sizeof(head));
+    k->put(&P.modulo, sizeof(P.modulo));
+    k->put(&P.modmask, sizeof(P.modmask));
     for (int s = 0; s < P.nstages; ++s) {
         const DStage &S = P.st[s];
         const uint8_t b[] = {S.op, S.is64, S.neg, S.never, S.nset, S.set_idx, S.in_smem, S.kind, S.simple, S.code_bits,
                              (uint8_t)S.issue_after, S.full, S.hot, S.wide};
-        put_raw(b, sizeof(b));
-        put_raw(&S.acc, sizeof(S.acc));
-        put_raw(&S.acc32, sizeof(S.acc32));
-        put_raw(S.mult, sizeof(S.mult));
-        put_raw(S.mult32, sizeof(S.mult32));
+        static_assert(sizeof(b) + sizeof(S.acc) + sizeof(S.acc32) + sizeof(S.mult) + sizeof(S.mult32) <= 160, "room for a stage");
+        k->put(b, sizeof(b));
+        k->put(&S.acc, sizeof(S.acc));
+        k->put(&S.acc32, sizeof(S.acc32));
+        k->put(S.mult, sizeof(S.mult));
+        k->put(S.mult32, sizeof(S.mult32));
     }
-    if (const char *extra = std::getenv("SJQ_JIT_EXTRA")) k += extra;
-    return k;
 }
 
 struct Module {
@@ -239,6 +247,24 @@ struct Module {
 
 std::mutex g_mutex;
 std::unordered_map<std::string, Module> g_modules;
+
+// The modules met so far by the hash of their shape's bytes (FNV-1a over 64-bit words), so that a repeated run compares
+// one key instead of building a string; the full key decides.
+uint64_t key_hash(const ShapeKey &k)
+{
+    uint64_t h = 0xCBF29CE484222325ULL, w;
+    size_t i = 0;
+    for (; i + 8 <= k.size; i += 8) {
+        std::memcpy(&w, k.bytes + i, 8);
+        h = (h ^ w) * 0x100000001B3ULL;
+        h ^= h >> 29;
+    }
+    w = 0;
+    std::memcpy(&w, k.bytes + i, k.size - i);
+    h = (h ^ w) * 0x100000001B3ULL;
+    return h ^ (h >> 32);
+}
+std::unordered_multimap<uint64_t, std::pair<const std::string, Module> *> g_by_hash;
 std::string g_last_log;
 
 sjq_status compile(const std::string &shape, std::vector<char> *cubin, std::string *log)
@@ -300,7 +326,22 @@ sjq_status compile(const std::string &shape, std::vector<char> *cubin, std::stri
 // Find or build the module of a shape.  Called with g_mutex held.
 sjq_status module_for(const RunParams &P, int agg, bool mul, bool hash, int lb_threads, int lb_blocks, Module **out)
 {
-    const std::string key = shape_key(P, agg, mul, hash, lb_threads, lb_blocks);
+    ShapeKey shape_bytes;
+    shape_key(P, agg, mul, hash, lb_threads, lb_blocks, &shape_bytes);
+    const char *extra = std::getenv("SJQ_JIT_EXTRA");
+    const uint64_t h = key_hash(shape_bytes);
+    if (!extra) {
+        const auto range = g_by_hash.equal_range(h);
+        for (auto it = range.first; it != range.second; ++it) {
+            const std::string &k = it->second->first;
+            if (k.size() == shape_bytes.size && std::memcmp(k.data(), shape_bytes.bytes, k.size()) == 0) {
+                *out = &it->second->second;
+                return (*out)->status;
+            }
+        }
+    }
+    std::string key(reinterpret_cast<const char *>(shape_bytes.bytes), shape_bytes.size);
+    if (extra) key += extra;
     auto it = g_modules.find(key);
     if (it == g_modules.end()) {
         const std::string shape = jit_shape_header(P, agg, mul, hash, lb_threads, lb_blocks);
@@ -319,6 +360,7 @@ sjq_status module_for(const RunParams &P, int agg, bool mul, bool hash, int lb_t
             }
         }
         it = g_modules.emplace(key, M).first;
+        if (!extra) g_by_hash.emplace(h, &*it); // (elements of an unordered_map stay where they are)
     }
     *out = &it->second;
     return it->second.status;
@@ -326,8 +368,9 @@ sjq_status module_for(const RunParams &P, int agg, bool mul, bool hash, int lb_t
 
 } // namespace
 
-sjq_status jit_occupancy(const RunParams &P, int agg, bool mul, bool hash, int block, int lb_blocks, size_t smem,
-                         int *ctas_per_sm)
+// The compiled kernel of a run (a cudaKernel_t) and how many of its blocks an SM holds.
+sjq_status jit_prepare(const RunParams &P, int agg, bool mul, bool hash, int block, int lb_blocks, size_t smem,
+                       int *ctas_per_sm, const void **kernel)
 {
     std::lock_guard<std::mutex> lock(g_mutex);
     Module *M = nullptr;
@@ -355,29 +398,19 @@ sjq_status jit_occupancy(const RunParams &P, int agg, bool mul, bool hash, int b
         o = M->occupancy.emplace(okey, n).first;
     }
     *ctas_per_sm = o->second;
+    *kernel = reinterpret_cast<const void *>(M->kernel);
     return SJQ_OK;
 }
 
-sjq_status jit_launch(const RunParams &P, int agg, bool mul, bool hash, int grid, int block, int lb_blocks,
-                      size_t smem, bool behind, cudaStream_t stream)
+sjq_status jit_launch(const void *kernel, const RunParams &P, int grid, int block, size_t smem, bool behind,
+                      cudaStream_t stream)
 {
-    cudaKernel_t kernel;
-    {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        Module *M = nullptr;
-        sjq_status st = module_for(P, agg, mul, hash, block, lb_blocks, &M);
-        if (st != SJQ_OK) return st;
-        kernel = M->kernel;
-    }
     // the compiled kernel's parameter struct holds P.nstages stage descriptors (at least one), then the same
     // fields as RunParams: pack exactly that
     const size_t nst = (size_t)(P.nstages > 0 ? P.nstages : 1);
-    const size_t tail_from = offsetof(RunParams, sets), tail_bytes = sizeof(RunParams) - tail_from;
-    static_assert(offsetof(RunParams, st) == 0 && offsetof(RunParams, sets) == sizeof(DStage) * (size_t)kMaxStages,
-                  "the stage descriptors lead the parameter block and the rest follows without padding");
     alignas(16) unsigned char packed[sizeof(RunParams)];
     std::memcpy(packed, P.st, nst * sizeof(DStage));
-    std::memcpy(packed + nst * sizeof(DStage), reinterpret_cast<const unsigned char *>(&P) + tail_from, tail_bytes);
+    std::memcpy(packed + nst * sizeof(DStage), static_cast<const RunCore *>(&P), sizeof(RunCore));
     void *args[] = {packed};
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -389,7 +422,7 @@ sjq_status jit_launch(const RunParams &P, int agg, bool mul, bool hash, int grid
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), args) != cudaSuccess) {
+    if (cudaLaunchKernelExC(&cfg, kernel, args) != cudaSuccess) {
         (void)cudaGetLastError();
         return SJQ_ERR_CUDA;
     }
@@ -418,6 +451,7 @@ extern "C" int32_t sjq_jit_cache_clear(void)
             ++n;
         }
     }
+    sjq::g_by_hash.clear();
     sjq::g_modules.clear();
     return n;
 }

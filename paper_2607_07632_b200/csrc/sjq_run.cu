@@ -23,11 +23,11 @@
 
 namespace sjq {
 
-sjq_status fused_occupancy(int agg, bool mul, bool hash, int block, size_t smem, int *ctas_per_sm);
-sjq_status jit_occupancy(const RunParams &P, int agg, bool mul, bool hash, int block, int lb_blocks, size_t smem,
-                         int *ctas_per_sm);
-sjq_status jit_launch(const RunParams &P, int agg, bool mul, bool hash, int grid, int block, int lb_blocks,
-                      size_t smem, bool behind, cudaStream_t stream);
+sjq_status fused_occupancy(int agg, bool mul, bool hash, int nstages, int block, size_t smem, int *ctas_per_sm);
+sjq_status jit_prepare(const RunParams &P, int agg, bool mul, bool hash, int block, int lb_blocks, size_t smem,
+                       int *ctas_per_sm, const void **kernel);
+sjq_status jit_launch(const void *kernel, const RunParams &P, int grid, int block, size_t smem, bool behind,
+                      cudaStream_t stream);
 sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, bool behind,
                         const RunParams &P, cudaStream_t stream);
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
@@ -50,6 +50,28 @@ sjq_status merge_launch(const int64_t *keys, const int64_t *sums, const int64_t 
 
 namespace {
 
+// A list with room for everything the planner can put in it: the planning of a run allocates nothing.
+template <typename T, int N>
+struct Short {
+    T items[N];
+    int count = 0;
+
+    Short() {}
+    Short(int n, const T &v) : count(n)
+    {
+        for (int i = 0; i < n; ++i) items[i] = v;
+    }
+    void push_back(const T &v) { items[count++] = v; }
+    void resize(int n) { count = n; }
+    int size() const { return count; }
+    T &operator[](int i) { return items[i]; }
+    const T &operator[](int i) const { return items[i]; }
+    T *begin() { return items; }
+    T *end() { return items + count; }
+    const T *begin() const { return items; }
+    const T *end() const { return items + count; }
+};
+
 struct StageSpec {
     int kind;     // ST_PRED / ST_PROBE / ST_LOAD
     int index;    // predicate or join index (-1 for loads)
@@ -59,6 +81,9 @@ struct StageSpec {
     double cost;  // picoseconds per row evaluated, the column's bytes apart
     int prefilter; // 1: only the presence bitmap of a hashed join; 2: the exact probe that follows one
 };
+constexpr int kMaxFilters = SJQ_MAX_PREDS + 2 * SJQ_MAX_JOINS; // (a hashed join is two)
+typedef Short<StageSpec, kMaxFilters> Specs;
+typedef Short<int, kMaxFilters> Order;
 
 // share of the rows surviving all filters from which a compiled kernel drops the survivor queues
 constexpr double kDirectSurvival = 0.35;       // register accumulators
@@ -117,13 +142,12 @@ double column_ps(int width, double reach)
 // (Ranking by (1 - selectivity) / cost with one cost for every table below 200 KB left city x brand to chance: two
 // joins that keep one row in 25, one probing 25 KB in shared memory, the other 175 KB through the L1, which is
 // 0.67 or 3.3 ms for 600 M rows with the one or the other first.)
-std::vector<int> cheapest_order(const std::vector<StageSpec> &specs)
+Order cheapest_order(const Specs &specs)
 {
     constexpr int kExhaustive = 8;
     const int n = (int)specs.size();
-    int early[64], m = 0;
-    std::vector<int> order;
-    order.reserve(n);
+    int early[kMaxFilters], m = 0;
+    Order order;
     for (int i = 0; i < n; ++i)
         if (specs[i].prefilter != 2) early[m++] = i;
     auto cost = [&](int i, double reach, bool column_read) {
@@ -150,7 +174,7 @@ std::vector<int> cheapest_order(const std::vector<StageSpec> &specs)
         std::reverse(order.begin(), order.end());
     } else {
         double reach = 1.0;
-        std::vector<char> used(n, 0);
+        Short<char, kMaxFilters> used(n, 0);
         for (int k = 0; k < m; ++k) {
             int pick = -1;
             double least = 0.0;
@@ -176,10 +200,10 @@ std::vector<int> cheapest_order(const std::vector<StageSpec> &specs)
 // stages) with estimated selectivities and costs, and the order they are evaluated in: the caller's, or
 // the cheapest.
 sjq_status order_stages(const sjq_col *fact, const sjq_pred *preds, int npreds, const sjq_join *joins, int njoins,
-                        const sjq_run_opts &opts, std::vector<StageSpec> *specs_out, std::vector<int> *order_out)
+                        const sjq_run_opts &opts, Specs *specs_out, Order *order_out)
 {
-    std::vector<StageSpec> &specs = *specs_out;
-    std::vector<int> &order = *order_out;
+    Specs &specs = *specs_out;
+    Order &order = *order_out;
     // a measured pass fraction (parts per million) replaces the estimate where the caller supplies one
     auto hinted = [&](int i, double estimate) {
         const int32_t ppm = opts.pass_ppm[i];
@@ -216,10 +240,9 @@ sjq_status order_stages(const sjq_col *fact, const sjq_pred *preds, int npreds, 
         specs.push_back({ST_PROBE, j, joins[j].fk_col, std::min(1.0, sel), width, probe + kPsIssue, 0});
     }
     const int nfilter = (int)specs.size();
-    static_assert(SJQ_MAX_PREDS + 2 * SJQ_MAX_JOINS <= 64, "cheapest_order lists the stages in 64 places");
     if (opts.norder) {
         // the caller orders predicates and joins; a hashed join's bitmap and exact probe stay adjacent
-        std::vector<char> seen(npreds + njoins, 0);
+        Short<char, SJQ_MAX_PREDS + SJQ_MAX_JOINS> seen(npreds + njoins, 0);
         for (int i = 0; i < npreds + njoins; ++i) {
             const int o = opts.order[i];
             if (o < 0 || o >= npreds + njoins || seen[o]) return SJQ_ERR_INVALID_ARG;
@@ -389,8 +412,8 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     cudaStream_t stream = (cudaStream_t)stream_;
 
     // ------------------------------------------------------------ stage list
-    std::vector<StageSpec> specs;
-    std::vector<int> order;
+    Specs specs;
+    Order order;
     if ((st = order_stages(fact, preds, npreds, joins, njoins, opts, &specs, &order)) != SJQ_OK) return st;
     const int nfilter = (int)specs.size();
 
@@ -398,7 +421,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     // Every term adds mult * value to one accumulator; fold the expressions
     // into per-source multipliers: src_mult[source][dest].
     struct Contribution { int src, a, b, dest; int64_t mult; };
-    std::vector<Contribution> contrib;
+    Short<Contribution, SJQ_MAX_KEY_TERMS + 2> contrib;
     auto add_term = [&](const sjq_term &t, int dest, int64_t sign) {
         contrib.push_back({t.src, t.a, t.b, dest, (int64_t)((uint64_t)t.mult * (uint64_t)sign)});
     };
@@ -412,14 +435,15 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     if (agg->op == SJQ_AGG_ADD) add_term(agg->y, kAccX, 1);
 
     RunParams P;
-    std::memset(&P, 0, sizeof(P));
+    std::memset(static_cast<RunCore *>(&P), 0, sizeof(RunCore)); // (stages are cleared as they are filled)
     P.n = n;
     int ns = 0;
     int nsets = 0;
-    std::vector<int> stage_of_join(njoins, -1);
-    std::vector<int> stage_of_col(nfact, -1);
-    std::vector<int> stage_label;
+    Short<int, SJQ_MAX_JOINS> stage_of_join(njoins, -1);
+    Short<int, 64> stage_of_col(nfact, -1);
+    Short<int, kMaxStages> stage_label;
     auto fill_stage = [&](DStage &S, const StageSpec &sp) -> sjq_status {
+        std::memset(&S, 0, sizeof(S));
         S.kind = (uint8_t)sp.kind;
         S.col = fact[sp.col].data;
         S.is64 = (uint8_t)(fact[sp.col].dtype == SJQ_I64);
@@ -501,7 +525,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
 
     // ------------------------------------------------------------ dense / sparse split
     // Fraction of rows reaching each filter stage, from the estimates.
-    std::vector<double> reach(nfilter + 1, 1.0);
+    Short<double, kMaxFilters + 1> reach(nfilter + 1, 1.0);
     for (int s = 0; s < nfilter; ++s) reach[s + 1] = reach[s] * specs[order[s]].sel;
     const double survivors = (double)n * reach[nfilter];
     // Level 0 runs, on thread-owned rows, the leading filter stages that still see a fair share of
@@ -567,7 +591,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     // Sources of the accumulators.  A dense stage cannot feed an accumulator
     // (it only keeps a bit per row), so a value it would supply is gathered
     // again for the survivors by a sparse copy of the stage.
-    std::vector<int> gather_of_stage(ns, -1);
+    Short<int, kMaxStages> gather_of_stage(ns, -1);
     for (const Contribution &c : contrib) {
         int s, src;
         if (c.src == SJQ_SRC_FACT) {
@@ -615,7 +639,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
     // A filter stage on a direct table with payloads probes the table's presence bitmap (an eighth to a
     // sixty-fourth of the code array, so far more of it stays in L1/L2); the payload is gathered from the
     // codes by the sparse copy, for the survivors only.
-    std::vector<char> via_bitmap(ns, 0);
+    Short<char, kMaxStages> via_bitmap(ns, 0);
     if (!opts.no_filter_bitmap) {
         for (int s = 0; s < ndense; ++s) {
             DStage &S = P.st[s];
@@ -820,7 +844,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
         const size_t table_budget = smem_cap - fixed;
         size_t tables = 0;
         if (opts.smem_tables != 1 && !opts.unfused) {
-            std::vector<int> cand;
+            Order cand;
             for (int s = 0; s < nfilter; ++s)
                 if (is_direct_op(P.st[s].op)) cand.push_back(s);
             std::stable_sort(cand.begin(), cand.end(), [&](int a, int b) {
@@ -932,8 +956,9 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
                           : block > 512 ? 1
                           : (block <= 384 && smem_without_bulk <= ((size_t)48 << 10)) ? 3
                                                                         : 2;
-    st = jit ? jit_occupancy(P, aggp, mul, has_hash, block, lb_blocks, smem, &per_sm)
-             : fused_occupancy(aggp, mul, has_hash, block, smem, &per_sm);
+    const void *compiled = nullptr;
+    st = jit ? jit_prepare(P, aggp, mul, has_hash, block, lb_blocks, smem, &per_sm, &compiled)
+             : fused_occupancy(aggp, mul, has_hash, ns, block, smem, &per_sm);
     if (st != SJQ_OK) return st;
     if (per_sm < 1) return SJQ_ERR_UNSUPPORTED;
     if (opts.ctas_per_sm > 0) per_sm = std::min(per_sm, opts.ctas_per_sm);
@@ -979,7 +1004,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
         // stages its tables, which were complete before the clear began, and waits for the clear before it touches a
         // result (two-join query, 60 M rows: 94 -> 92 us; filter and sum, 6 M rows: 20.5 -> 18.5 us back to back).
         const bool behind = !opts.accumulate && hot_stage < 0 && !opts.event_before;
-        st = jit ? jit_launch(P, aggp, mul, has_hash, grid, block, lb_blocks, smem, behind, stream)
+        st = jit ? jit_launch(compiled, P, grid, block, smem, behind, stream)
                  : fused_launch(aggp, mul, has_hash, grid, block, smem, behind, P, stream);
         if (st != SJQ_OK) return st;
         ++launches;
@@ -1119,8 +1144,8 @@ void host_transfer_plan(const sjq_col *fact_host, int nfact, const sjq_pred *pre
         for (int t = 0; ok && t < key->nterms; ++t) ok = term_ok(key->t[t]);
     }
     ok = ok && term_ok(agg->x) && (agg->op == SJQ_AGG_COL || term_ok(agg->y));
-    std::vector<StageSpec> specs;
-    std::vector<int> order;
+    Specs specs;
+    Order order;
     // The columns are in host memory here, so predicates without a measured pass fraction are measured on
     // the spot: a few thousand evenly spaced rows read by the host.  (A guess that is far too low would send
     // a column most rows need over the bus sector by sector.)

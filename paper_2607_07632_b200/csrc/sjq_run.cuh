@@ -46,6 +46,7 @@ constexpr int kAccKey = 0, kAccX = 1, kAccY = 2;
 constexpr int kMaxStages = SJQ_JIT_nstages > 0 ? SJQ_JIT_nstages : 1;
 #else
 constexpr int kMaxStages = 72;
+constexpr int kFewStages = 12; // the interpreting kernels come for so many stages and for the most there can be
 #endif
 
 // Geometry of the fused kernel.
@@ -99,8 +100,8 @@ struct DStage {
 };
 static_assert(sizeof(DStage) % 8 == 0, "stage descriptors are copied as 64-bit words");
 
-struct RunParams {
-    DStage st[kMaxStages];
+// What a run is made of besides its stages.
+struct RunCore {
     int64_t sets[SJQ_MAX_PREDS][SJQ_MAX_IN_SET];
     int64_t n;
     int64_t key_offset;
@@ -137,14 +138,32 @@ struct RunParams {
     int32_t l0_bulk;      // compiled kernels: the first column arrives by bulk-asynchronous copies into shared memory
 };
 
+// A kernel's parameter block: its stage descriptors, then the rest.
+template <int N>
+struct RunStages {
+    DStage st[N];
+};
+template <int N>
+struct RunParamsOf : RunStages<N>, RunCore {
+};
+typedef RunParamsOf<kMaxStages> RunParams;
+static_assert(sizeof(RunParams) == sizeof(RunStages<kMaxStages>) + sizeof(RunCore), "no padding between the two");
+
 #if !defined(SJQ_JIT)
-// The sixteen ahead-of-time variants of the fused kernel (aggregation path x product aggregate x "some table is
-// open-addressing"), instantiated in one translation unit per aggregation path.
+// The ahead-of-time variants of the fused kernel (aggregation path x product aggregate x "some table is open-addressing"
+// x up to kFewStages stages or any number), instantiated in one translation unit per aggregation path and size.  A
+// launch copies its whole parameter block, 6 KB with twelve stages and 21 KB with all (a call of a small query 9.9 -> 8.1 us).
+typedef RunParamsOf<kFewStages> RunParamsFew;
+typedef void (*fused_few_fn)(const RunParamsFew);
 typedef void (*fused_fn)(const RunParams);
 fused_fn fused_variant_scalar(bool mul, bool hash);
 fused_fn fused_variant_smem(bool mul, bool hash);
 fused_fn fused_variant_global(bool mul, bool hash);
 fused_fn fused_variant_hash(bool mul, bool hash);
+fused_few_fn fused_few_scalar(bool mul, bool hash);
+fused_few_fn fused_few_smem(bool mul, bool hash);
+fused_few_fn fused_few_global(bool mul, bool hash);
+fused_few_fn fused_few_hash(bool mul, bool hash);
 #endif
 
 } // namespace sjq

@@ -28,7 +28,7 @@ def test_of_two_equally_selective_joins_the_one_in_shared_memory_goes_first(smal
     assert res.info.order[0] == names.index("small")
 
 
-@pytest.mark.parametrize("npreds", [1, 8, 9, 16])
+@pytest.mark.parametrize("npreds", [1, 8, 9, 10, 11, 12, 16])
 def test_any_number_of_filters(npreds):
     n, rng = 20_011, np.random.default_rng(npreds)
     fact = {f"c{i}": rng.integers(0, 100, n).astype(np.int32) for i in range(npreds)}
