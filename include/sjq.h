@@ -472,14 +472,14 @@ sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *preds, int np
  * Section 3.3's global table returns its groups in table order, which depends
  * on the hash function and the capacity; the paper compares results through an
  * order-free checksum (Section 2.2), this library gives the list itself an
- * order instead.  A radix sort of (key, position) pairs on the device, then
- * one gather of the three arrays.
+ * order instead.  A sample sort (up to 2^20 entries) or a radix sort of (key,
+ * position) pairs on the device; equal keys keep their order.
  *   keys/sums/counts  device arrays of `capacity` entries (8-byte aligned), of
  *                     which the first *n_groups hold the result; sorted in place
  *   n_groups          device pointer, read by the kernels (no host wait)
  *   scratch           device scratch of sjq_result_sort_scratch_bytes(capacity)
  *                     bytes, 16-byte aligned (about 40 bytes per entry)
- * capacity <= 2^31.  Enqueues 27 small kernels on `stream`; does not
+ * capacity <= 2^31.  Enqueues 4 to 17 small kernels on `stream`; does not
  * synchronise.  Errors: INVALID_ARG, ALIGN, BUFFER_SMALL, CUDA.
  */
 sjq_status sjq_result_sort_scratch_bytes(int64_t capacity, size_t *bytes);

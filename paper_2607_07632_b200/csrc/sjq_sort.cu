@@ -2,24 +2,23 @@
 //
 // The global group table of Section 3.3 hands its groups back in table order, which depends on the hash function
 // and on the capacity; two runs of the same query agree only as sets.  sjq_result_sort puts the list of
-// (key, sum, count) triples into ascending signed key order on the device: a stable least-significant-digit radix
-// sort of (key - smallest key, position) pairs, 8 bits a pass.
+// (key, sum, count) triples into ascending signed key order on the device, equal keys as they came.
 //
-// The number of groups and the range of the keys are known on the device only, so nothing waits on the host: the
-// host enqueues every pass that 64-bit keys could need, a first kernel finds smallest and largest key and whether
-// the list is in order already, and the passes that the range does not need return at once (group keys are small
-// numbers as a rule: 20 bits for a million groups, three passes; a list in order needs none).
+// The number of groups is known on the device only, so nothing waits on the host: the host enqueues the same kernels
+// whatever the list holds, each launched while its predecessor still runs and waiting for it on the device
+// (programmatic dependent launch), and a first kernel also finds out whether the list is in order already, in which
+// case the others return at once.
 //
-// What bounds it: kernel latency.  A pass over a million pairs moves 24 MB, which the L2 holds, so its two kernels
-// are short (5 to 15 us) and what they do one after the other counts.  Hence
-//   - at most kSortBlocks blocks of 1024 threads (one per SM), each owning one contiguous piece of the list: the
-//     digit counts are kSortBlocks x 256 words whatever the length, and every scatter block forms its own offsets
-//     from them (a kernel of its own that scanned 256 counts per 1024 elements with one block took 461 us a pass
-//     at a capacity of 2 million, 9/10 of the whole sort; the counts of 8 SMs' worth of loads take 2 us here);
-//   - the measures travel once: they are copied aside by the first counting kernel and gathered by the last
-//     scatter, which writes all three result arrays;
-//   - each kernel is launched while its predecessor still runs and waits for it on the device (programmatic
-//     dependent launch), so that a pass without work costs about a microsecond.
+// What bounds it: kernel latency.  A million pairs are 24 MB, which the L2 holds, so a kernel takes 3 to 15 us and it
+// is the number of kernels one after the other that counts.  Two ways, by the capacity of the list:
+//   - up to kSampleMost entries a sample sort, four kernels: splitters from a sorted sample; the bucket of every
+//     entry, counted; the entries into their buckets; every bucket sorted in shared memory (merge of eight lists of
+//     200,000 with its sort: 198 us with the radix sort, 75 with this one);
+//   - beyond, a stable least-significant-digit radix sort of (key - smallest key, position) pairs, 8 bits a pass,
+//     two kernels each; passes that the range of the keys does not need return at once.  At most kSortBlocks blocks
+//     own one contiguous piece of the list each, so that the digit counts are few and every scatter block forms its
+//     own offsets from them.
+// Both copy the measures aside once and gather them in the last kernel, which writes all three result arrays.
 #include <algorithm>
 
 #include "sjq_internal.h"
@@ -34,6 +33,12 @@ constexpr int kSortTile = kSortThreads * kSortRounds;
 constexpr int kSortBlocks = 148;                       // one per SM
 constexpr int kSortMinPiece = 2048;                    // elements a block takes before another one is put to work
 constexpr int kSortPasses = 8;
+
+constexpr int64_t kSampleMost = (int64_t)1 << 20;
+constexpr int kBuckets = 1024;      // at most; about 256 entries each in a shorter list
+constexpr int kOversample = 4;      // samples per bucket: the largest bucket is two to three times the average
+constexpr int kBucketThreads = 256;
+constexpr int kBucketRoom = 2048;   // entries of a bucket that shared memory holds
 
 struct SortRange {
     unsigned long long lo, hi; // smallest and largest key, sign bit flipped
@@ -59,6 +64,13 @@ struct SortParams {
     unsigned int *totals;          // [kSortPasses][256] elements per digit
     unsigned int *hist;            // [kSortBlocks][256] elements per block and digit of the current pass
     int32_t pass;
+    // sample sort
+    unsigned long long *split_key; // [kBuckets - 1] splitters, ascending by (key, position)
+    unsigned int *split_pos;
+    unsigned int *bucket_total;    // [kBuckets] entries per bucket
+    unsigned int *bucket_base;     // [blocks][kBuckets] places of a block's entries within their buckets
+    unsigned int *disorder;        // [blocks] a key larger than its successor was seen
+    int32_t pieces;                // blocks of the first three kernels
 };
 
 __device__ __forceinline__ unsigned long long flip(int64_t k) { return (unsigned long long)k ^ 0x8000000000000000ull; }
@@ -305,11 +317,295 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const __grid
     }
 }
 
+// ------------------------------------------------------------------ sample sort
+__device__ __forceinline__ int buckets_for(int64_t n)
+{
+    int nb = 1;
+    while (nb < kBuckets && (int64_t)nb * 256 < n) nb <<= 1;
+    return nb;
+}
+
+// Position of sample i of s in a list of n: anywhere in the i-th of s equal parts, so that no regular pattern in the
+// list meets the samples; samples ascend in position.
+__device__ __forceinline__ int64_t sample_at(int i, int s, int64_t n)
+{
+    const int64_t lo = (int64_t)i * n / s, hi = (int64_t)(i + 1) * n / s;
+    unsigned int h = (unsigned int)i * 2654435761u + 0x9E3779B9u;
+    h ^= h >> 15;
+    h *= 2246822519u;
+    h ^= h >> 13;
+    return lo + (int64_t)(h % (unsigned int)(hi - lo));
+}
+
+__device__ __forceinline__ bool list_in_order(const SortParams &S)
+{
+    int any = 0;
+    for (int b = threadIdx.x; b < S.pieces; b += blockDim.x) any |= (int)S.disorder[b];
+    return __syncthreads_or(any) == 0;
+}
+
+// Is the list in order, and the splitters: every block holds the sample and ranks its share of it, one per warp.
+__global__ void __launch_bounds__(kSortThreads) sample_split_kernel(const __grid_constant__ SortParams S)
+{
+    __shared__ unsigned long long sample[kBuckets * kOversample];
+    cudaTriggerProgrammaticLaunchCompletion();
+    const int64_t n = sort_count(S);
+    const int nb = buckets_for(n), ns = nb > 1 ? nb * kOversample : 0;
+    for (int i = threadIdx.x; i < ns; i += kSortThreads) sample[i] = flip(S.keys[sample_at(i, ns, n)]);
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < kBuckets; i += kSortThreads) S.bucket_total[i] = 0;
+    int64_t lo, hi;
+    sort_piece(n, &lo, &hi);
+    int disorder = 0;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kSortThreads)
+        if (i + 1 < n && S.keys[i + 1] < S.keys[i]) disorder = 1;
+    disorder = __syncthreads_or(disorder);
+    if (threadIdx.x == 0) S.disorder[blockIdx.x] = (unsigned int)disorder;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = blockIdx.x * kSortWarps + warp; i < ns; i += gridDim.x * kSortWarps) {
+        const unsigned long long k = sample[i];
+        unsigned int before = 0;
+        for (int j = lane; j < ns; j += 32) before += (sample[j] < k) | ((sample[j] == k) & (j < i));
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0 && before % kOversample == 0 && before > 0) {
+            S.split_key[before / kOversample - 1] = k;
+            S.split_pos[before / kOversample - 1] = (unsigned int)sample_at(i, ns, n);
+        }
+    }
+}
+
+// The bucket of every entry of this block's piece (the number of splitters not above it) and its place among the
+// block's entries of that bucket; the block's places within the buckets; the measures copied aside.
+__global__ void __launch_bounds__(kSortThreads) sample_count_kernel(const __grid_constant__ SortParams S)
+{
+    __shared__ unsigned long long split_key[kBuckets];
+    __shared__ unsigned int split_pos[kBuckets], count[kBuckets];
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    if (list_in_order(S)) return;
+    const int64_t n = sort_count(S);
+    const int nb = buckets_for(n);
+    for (int i = threadIdx.x; i < nb; i += kSortThreads) {
+        count[i] = 0;
+        if (i < nb - 1) {
+            split_key[i] = S.split_key[i];
+            split_pos[i] = S.split_pos[i];
+        }
+    }
+    __syncthreads();
+    int64_t lo, hi;
+    sort_piece(n, &lo, &hi);
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kSortThreads) {
+        const unsigned long long k = flip(S.keys[i]);
+        S.tsums[i] = S.sums[i];
+        S.tcounts[i] = S.counts[i];
+        int b = 0;
+        for (int step = nb >> 1; step > 0; step >>= 1) {
+            const unsigned long long sk = split_key[b + step - 1];
+            if (sk < k || (sk == k && split_pos[b + step - 1] <= (unsigned int)i)) b += step;
+        }
+        const unsigned int at = atomicAdd(&count[b], 1u);
+        static_assert(kSampleMost / kSortBlocks < (1 << 13) && kBuckets <= (1 << 10), "a place and a bucket fit one word");
+        S.p[0][i] = (unsigned int)b << 16 | at;
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < nb; b += kSortThreads)
+        S.bucket_base[(size_t)blockIdx.x * kBuckets + b] = count[b] ? atomicAdd(&S.bucket_total[b], count[b]) : 0u;
+}
+
+// First entry of every bucket: exclusive scan of the totals by the first kBuckets / 4 threads of a block.
+__device__ __forceinline__ void bucket_starts(const SortParams &S, int nb, unsigned int *start, unsigned int *warp_sum)
+{
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    unsigned int incl = 0;
+    if (t < kBuckets / 4) {
+        if (4 * t < nb) v = reinterpret_cast<const uint4 *>(S.bucket_total)[t]; // (totals beyond nb are zero)
+        incl = v.x + v.y + v.z + v.w;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+    }
+    __syncthreads();
+    if (t < kBuckets / 4) {
+        for (int w = 0; w < warp; ++w) incl += warp_sum[w];
+        start[4 * t + 3] = incl - v.w;
+        start[4 * t + 2] = incl - v.w - v.z;
+        start[4 * t + 1] = incl - v.w - v.z - v.y;
+        start[4 * t] = incl - v.w - v.z - v.y - v.x;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSortThreads) sample_scatter_kernel(const __grid_constant__ SortParams S)
+{
+    __shared__ unsigned int place[kBuckets], warp_sum[kBuckets / 128];
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    if (list_in_order(S)) return;
+    const int64_t n = sort_count(S);
+    const int nb = buckets_for(n);
+    int64_t lo, hi;
+    sort_piece(n, &lo, &hi);
+    if (lo >= hi) return;
+    bucket_starts(S, nb, place, warp_sum);
+    for (int b = threadIdx.x; b < nb; b += kSortThreads) place[b] += S.bucket_base[(size_t)blockIdx.x * kBuckets + b];
+    __syncthreads();
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kSortThreads) {
+        const unsigned int w = S.p[0][i], at = place[w >> 16] + (w & 0xFFFFu);
+        S.k[1][at] = flip(S.keys[i]);
+        S.p[1][at] = (unsigned int)i;
+    }
+}
+
+// Sort R * kBucketThreads values by a bitonic network; value r * kBucketThreads + thread sits in v[r].  Partners in the
+// same thread or warp meet in registers, the others in shared memory.
+template <int R>
+__device__ __forceinline__ void bitonic(unsigned long long (&v)[R], unsigned long long *buf)
+{
+    const int tid = threadIdx.x;
+    for (int k = 2; k <= R * kBucketThreads; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= kBucketThreads) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+#pragma unroll
+                    for (int o = 1; o < R; o <<= 1) {
+                        if (o * kBucketThreads != j || (r & o)) continue;
+                        const bool up = ((r * kBucketThreads) & k) == 0;
+                        const unsigned long long a = v[r], b = v[r | o], lo = a < b ? a : b, hi = a < b ? b : a;
+                        v[r] = up ? lo : hi;
+                        v[r | o] = up ? hi : lo;
+                    }
+                }
+                continue;
+            }
+            unsigned long long other[R];
+            if (j >= 32) {
+                __syncthreads(); // what was read the last time
+#pragma unroll
+                for (int r = 0; r < R; ++r) buf[r * kBucketThreads + tid] = v[r];
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < R; ++r) other[r] = buf[r * kBucketThreads + (tid ^ j)];
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) other[r] = __shfl_xor_sync(0xffffffffu, v[r], j);
+            }
+            const bool low = (tid & j) == 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const bool up = ((r * kBucketThreads + tid) & k) == 0, least = low == up;
+                v[r] = (v[r] < other[r]) == least ? v[r] : other[r];
+            }
+        }
+    }
+}
+
+// Order of a bucket's m <= R * kBucketThreads entries: order[i] = the entry that comes i-th.  The values sorted are the
+// top 53 bits of the distance from the bucket's smallest key, then the entry's number: one word instead of key and
+// position.  False when two neighbours agree in those bits.
+template <int R>
+__device__ __forceinline__ bool order_bucket(const unsigned long long *key, int m, unsigned long long kmin, int shift,
+                                             unsigned long long *buf, unsigned short *order)
+{
+    constexpr int kNumberBits = 11;
+    static_assert(kBucketRoom <= (1 << kNumberBits), "an entry's number");
+    unsigned long long v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = r * kBucketThreads + (int)threadIdx.x;
+        v[r] = e < m ? ((key[e] - kmin) >> shift) << kNumberBits | (unsigned long long)e : ~0ull;
+    }
+    bitonic<R>(v, buf);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) buf[r * kBucketThreads + threadIdx.x] = v[r];
+    __syncthreads();
+    bool same = false;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = r * kBucketThreads + (int)threadIdx.x;
+        if (e >= m) continue;
+        order[e] = (unsigned short)(v[r] & ((1u << kNumberBits) - 1u));
+        same |= e + 1 < m && (buf[e + 1] ^ v[r]) >> kNumberBits == 0;
+    }
+    return __syncthreads_or(same) == 0;
+}
+
+// Sort the buckets, a block each.  Where keys of a bucket are equal, or so far apart that the 53 bits do not tell them
+// apart, or a bucket is larger than shared memory (the sample would have to be very unlucky), its entries are ranked one
+// by one against the whole bucket.
+__global__ void __launch_bounds__(kBucketThreads) sample_bucket_kernel(const __grid_constant__ SortParams S)
+{
+    __shared__ unsigned long long key[kBucketRoom], buf[kBucketRoom];
+    __shared__ unsigned short order[kBucketRoom];
+    __shared__ unsigned int start[kBuckets], warp_sum[kBuckets / 128];
+    __shared__ unsigned long long least[kBucketThreads / 32], most[kBucketThreads / 32];
+    static_assert(kBucketThreads == kBuckets / 4, "bucket_starts takes so many threads");
+    cudaGridDependencySynchronize();
+    if (list_in_order(S)) return;
+    const int nb = buckets_for(sort_count(S));
+    bucket_starts(S, nb, start, warp_sum);
+    auto store = [&](unsigned int at, unsigned long long k, unsigned int p) {
+        S.keys[at] = (int64_t)(k ^ 0x8000000000000000ull);
+        S.sums[at] = S.tsums[p];
+        S.counts[at] = S.tcounts[p];
+    };
+    for (int b = blockIdx.x; b < nb; b += gridDim.x) {
+        const unsigned int lo = start[b], m = S.bucket_total[b];
+        bool done = m == 0;
+        if (m > 0 && m <= (unsigned int)kBucketRoom) {
+            __syncthreads(); // the bucket before has been written out
+            unsigned long long kmin = ~0ull, kmax = 0ull;
+            for (int e = threadIdx.x; e < (int)m; e += kBucketThreads) {
+                const unsigned long long k = S.k[1][lo + e];
+                key[e] = k;
+                kmin = k < kmin ? k : kmin;
+                kmax = k > kmax ? k : kmax;
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
+                kmin = x < kmin ? x : kmin;
+                kmax = y > kmax ? y : kmax;
+            }
+            if ((threadIdx.x & 31) == 0) least[threadIdx.x >> 5] = kmin, most[threadIdx.x >> 5] = kmax;
+            __syncthreads();
+            for (int w = 0; w < kBucketThreads / 32; ++w) {
+                kmin = least[w] < kmin ? least[w] : kmin;
+                kmax = most[w] > kmax ? most[w] : kmax;
+            }
+            // (all ones in the top 53 bits would meet the padding: 2^53 - 1 is the most a distance may reach, exclusive)
+            const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > 52 ? bits - 52 : 0;
+            if (m <= kBucketThreads) done = order_bucket<1>(key, (int)m, kmin, shift, buf, order);
+            else if (m <= 2 * kBucketThreads) done = order_bucket<2>(key, (int)m, kmin, shift, buf, order);
+            else if (m <= 4 * kBucketThreads) done = order_bucket<4>(key, (int)m, kmin, shift, buf, order);
+            else done = order_bucket<8>(key, (int)m, kmin, shift, buf, order);
+            if (done)
+                for (int e = threadIdx.x; e < (int)m; e += kBucketThreads) store(lo + e, key[order[e]], S.p[1][lo + order[e]]);
+        }
+        if (done) continue;
+        for (unsigned int e = threadIdx.x; e < m; e += kBucketThreads) {
+            const unsigned long long k = S.k[1][lo + e];
+            const unsigned int p = S.p[1][lo + e];
+            unsigned int before = 0;
+            for (unsigned int j = 0; j < m; ++j) {
+                const unsigned long long o = S.k[1][lo + j];
+                before += (o < k) | ((o == k) & (S.p[1][lo + j] < p));
+            }
+            store(lo + before, k, p);
+        }
+    }
+}
+
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
 struct SortLayout {
-    size_t k0, k1, p0, p1, ranges, header, totals, hist, tsums, tcounts, total;
+    size_t k0, k1, p0, p1, ranges, header, totals, hist, tsums, tcounts, split_key, split_pos, bucket_total, disorder, total;
     int nblocks;
+    bool sample;
 };
 
 SortLayout sort_layout(int64_t capacity)
@@ -325,7 +621,12 @@ SortLayout sort_layout(int64_t capacity)
     L.ranges = at, at += up256(sizeof(SortRange) * L.nblocks);
     L.header = at, at += 256;
     L.totals = at, at += (size_t)kSortPasses * 256 * 4;
-    L.hist = at, at += (size_t)256 * L.nblocks * 4;
+    L.hist = at, at += (size_t)kBuckets * L.nblocks * 4; // (the radix sort's 256 counts per block, or bucket_base)
+    L.split_key = at, at += (size_t)kBuckets * 8;
+    L.split_pos = at, at += (size_t)kBuckets * 4;
+    L.bucket_total = at, at += (size_t)kBuckets * 4;
+    L.disorder = at, at += up256((size_t)kSortBlocks * 4);
+    L.sample = capacity <= kSampleMost;
     L.tsums = at, at += up256(c * 8);
     L.tcounts = at, at += up256(c * 8);
     L.total = at;
@@ -334,14 +635,14 @@ SortLayout sort_layout(int64_t capacity)
 
 // Launch behind the previous kernel of the sort without waiting for it: every kernel but the first waits on the
 // device (cudaGridDependencySynchronize) before it touches what its predecessors wrote.
-bool launch_behind(void (*kernel)(SortParams), int grid, const SortParams &S, cudaStream_t stream)
+bool launch_behind(void (*kernel)(SortParams), int grid, int threads, const SortParams &S, cudaStream_t stream)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kSortThreads);
+    cfg.blockDim = dim3(threads);
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
@@ -389,11 +690,27 @@ extern "C" sjq_status sjq_result_sort(int64_t *keys, int64_t *sums, int64_t *cou
     S.header = reinterpret_cast<SortHeader *>(base + L.header);
     S.totals = reinterpret_cast<unsigned int *>(base + L.totals);
     S.hist = reinterpret_cast<unsigned int *>(base + L.hist);
-    sort_range_kernel<<<L.nblocks, kSortThreads, 0, stream>>>(S);
-    bool ok = cudaGetLastError() == cudaSuccess;
-    for (int pass = 0; pass < kSortPasses && ok; ++pass) {
-        S.pass = pass;
-        ok = launch_behind(sort_hist_kernel, L.nblocks, S, stream) && launch_behind(sort_scatter_kernel, L.nblocks, S, stream);
+    S.split_key = reinterpret_cast<unsigned long long *>(base + L.split_key);
+    S.split_pos = reinterpret_cast<unsigned int *>(base + L.split_pos);
+    S.bucket_total = reinterpret_cast<unsigned int *>(base + L.bucket_total);
+    S.bucket_base = S.hist;
+    S.disorder = reinterpret_cast<unsigned int *>(base + L.disorder);
+    S.pieces = L.nblocks;
+    bool ok;
+    if (L.sample) {
+        const int64_t buckets = std::min<int64_t>((capacity + 127) / 128, kBuckets);
+        sample_split_kernel<<<L.nblocks, kSortThreads, 0, stream>>>(S);
+        ok = cudaGetLastError() == cudaSuccess && launch_behind(sample_count_kernel, L.nblocks, kSortThreads, S, stream) &&
+             launch_behind(sample_scatter_kernel, L.nblocks, kSortThreads, S, stream) &&
+             launch_behind(sample_bucket_kernel, (int)buckets, kBucketThreads, S, stream);
+    } else {
+        sort_range_kernel<<<L.nblocks, kSortThreads, 0, stream>>>(S);
+        ok = cudaGetLastError() == cudaSuccess;
+        for (int pass = 0; pass < kSortPasses && ok; ++pass) {
+            S.pass = pass;
+            ok = launch_behind(sort_hist_kernel, L.nblocks, kSortThreads, S, stream) &&
+                 launch_behind(sort_scatter_kernel, L.nblocks, kSortThreads, S, stream);
+        }
     }
     if (!ok) {
         (void)cudaGetLastError();

@@ -24,22 +24,50 @@ def _check(keys, capacity):
         assert np.array_equal(got.cpu().numpy(), want[order])
 
 
-@pytest.mark.parametrize("n", [2, 31, 2047, 2048, 2049, 4095, 4096, 4097, 148 * 2048 - 1, 148 * 2048 + 1,
-                               148 * 4096 + 33, 2_000_003])
+@pytest.mark.parametrize("n", [2, 31, 255, 256, 257, 512, 513, 2047, 2048, 2049, 4095, 4096, 4097, 148 * 2048 - 1, 148 * 2048 + 1,
+                               148 * 4096 + 33, 2**20 - 7, 2**20 - 6, 2_000_003])
 def test_list_lengths_around_pieces_and_tiles(n):
     keys = np.random.default_rng(n).permutation(n).astype(np.int64) * 0x9E3779B97F4A7 - 2**40
     _check(keys, n + 7)
 
 
 @pytest.mark.parametrize("bits", [1, 8, 9, 16, 24, 33, 40, 48, 56, 63])
-def test_every_number_of_passes_with_equal_keys(bits):
+@pytest.mark.parametrize("capacity", [32_768, 2**20 + 1])  # sample sort, radix sort
+def test_every_number_of_passes_with_equal_keys(bits, capacity):
     n = 20_011
     rng = np.random.default_rng(bits)
     lo = -(2**(bits - 1)) + 12_345
     keys = rng.integers(0, 2**bits - 1, n, endpoint=True, dtype=np.int64) + np.int64(lo)
     keys[:2] = lo, lo + 2**bits - 1  # the whole range, so that the pass count is the intended one
     keys[100:5_000] = keys[7]
-    _check(keys, 32_768)
+    _check(keys, capacity)
+
+
+@pytest.mark.parametrize("capacity", [300_000, 2**20 + 5])
+def test_clustered_keys_and_a_lone_outlier(capacity):
+    rng = np.random.default_rng(4)
+    keys = np.concatenate([rng.permutation(100_000), rng.permutation(100_000) + 2**50, [-2**63, 2**63 - 1],
+                           np.full(3_000, 77), 2**62 + 2**40 * rng.integers(0, 50, 5_000)]).astype(np.int64)
+    _check(rng.permutation(keys), capacity)
+    _check(np.sort(keys)[::-1].copy(), capacity)
+
+
+def test_buckets_larger_than_shared_memory_are_ranked():
+    # the sampled positions hold small keys only: all other entries fall into one bucket
+    n = 40_000
+    keys = np.random.default_rng(1).permutation(n).astype(np.int64) + 10**6
+    nb = 1
+    while nb < 1024 and nb * 256 < n:
+        nb *= 2
+    s = 4 * nb
+    for i in range(s):
+        lo, hi = i * n // s, (i + 1) * n // s
+        h = (i * 2654435761 + 0x9E3779B9) & 0xFFFFFFFF
+        h ^= h >> 15
+        h = (h * 2246822519) & 0xFFFFFFFF
+        h ^= h >> 13
+        keys[lo + h % (hi - lo)] = i
+    _check(keys, n)
 
 
 def test_list_in_order_and_list_of_equal_keys_stay_as_they_are():
