@@ -234,8 +234,11 @@ sjq_status sjq_build_dim(const sjq_col *cols, int ncols, const sjq_pred *preds, 
  *   dims              `ndims` descriptions, as the arguments of sjq_dim_plan
  *   scratch_dev       device scratch of ndims * SJQ_PLAN_SCRATCH_BYTES bytes
  *   layouts           receives (plan) or gives (build) `ndims` layouts
- *   table_mem etc.    one entry per dimension, as the arguments of sjq_build_dim; the status words ARE cleared
+ *   table_mem etc.    one entry per dimension, as the arguments of sjq_build_dim
+ *   clear_status      non-zero: the status words are cleared first
  * sjq_dims_plan SYNCHRONISES the stream; sjq_dims_build does not.  After an error no table has been created.
+ * sjq_dims_plan_begin enqueues the scans and returns: the scan kernel writes the statistics of dimension i to
+ * host_stats[i] (eight int64 words of page-locked host memory, for sjq_dim_plan_end).
  */
 typedef struct sjq_dim_desc {
     const sjq_col *cols;
@@ -249,8 +252,11 @@ typedef struct sjq_dim_desc {
 } sjq_dim_desc;
 sjq_status sjq_dims_plan(const sjq_dim_desc *dims, int ndims, void *scratch_dev, size_t scratch_bytes, void *stream,
                          sjq_dim_layout *layouts);
+sjq_status sjq_dims_plan_begin(const sjq_dim_desc *dims, int ndims, void *scratch_dev, size_t scratch_bytes,
+                               int64_t *const *host_stats, void *stream);
 sjq_status sjq_dims_build(const sjq_dim_desc *dims, int ndims, const sjq_dim_layout *layouts, void *const *table_mem,
-                          const size_t *table_bytes, int32_t *const *status_dev, void *stream, sjq_table **tables);
+                          const size_t *table_bytes, int32_t *const *status_dev, int32_t clear_status, void *stream,
+                          sjq_table **tables);
 
 /*
  * Device bytes a table of the given shape occupies, recomputed from `kind`,

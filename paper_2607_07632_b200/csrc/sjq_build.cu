@@ -180,7 +180,7 @@ struct ScanParams {
     DimFilters filters;
     int32_t ndims;
     unsigned long long *scratch;
-    int64_t *host; // page-locked, eight words per dimension, or NULL: the statistics stay in the scratch
+    int64_t *host[kBatchDims]; // page-locked, eight words each, or NULL: the statistics stay in the scratch
 };
 
 constexpr int kExtremes = 2 + 2 * SJQ_MAX_PAYLOADS; // [min, max] of the key and of each payload
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kScanThreads, 2) plan_scan_kernel(const __grid
         __syncwarp();
         if (lane < 8) {
             scratch[i] = (unsigned long long)stat;
-            if (P.host) P.host[8 * which + i] = stat;
+            if (P.host[which]) P.host[which][i] = stat;
         }
     }
 }
@@ -735,6 +735,19 @@ sjq_status fill_rows(const sjq_dim_desc &d, DimRows *D, DimFilters *F, int *nfil
     return SJQ_OK;
 }
 
+// (argument errors come before a missing device)
+sjq_status check_dims(const sjq_dim_desc *dims, int ndims)
+{
+    for (int i = 0; i < ndims; ++i) {
+        DimRows rows;
+        DimFilters filters;
+        int nfilters = 0;
+        const sjq_status st = fill_rows(dims[i], &rows, &filters, &nfilters);
+        if (st != SJQ_OK) return st;
+    }
+    return SJQ_OK;
+}
+
 // How many of the dimensions from `first` on one launch can take.
 int batch_of(const sjq_dim_desc *dims, int ndims, int first)
 {
@@ -764,28 +777,25 @@ uint32_t share_blocks(int ntasks, int64_t room, Get task)
     return at;
 }
 
-// Enqueue the scans of a batch; the statistics of dimension i go to scratch + i * kScratchWords (and host + 8 i).
-sjq_status scan_launch(const sjq_dim_desc *dims, int ndims, unsigned long long *scratch, int64_t *host, int sm_count,
+// Enqueue the scans of a batch; the statistics of dimension i go to scratch + i * kScratchWords (and to host[i]).
+sjq_status scan_launch(const sjq_dim_desc *dims, int ndims, unsigned long long *scratch, int64_t *const *host, int sm_count,
                        cudaStream_t stream)
 {
     ScanParams P;
     int nfilters = 0;
-    bool rows = false;
     for (int i = 0; i < ndims; ++i) {
         const sjq_status st = fill_rows(dims[i], &P.dim[i], &P.filters, &nfilters);
         if (st != SJQ_OK) return st;
-        rows = rows || P.dim[i].n > 0;
+        P.host[i] = host ? host[i] : nullptr;
     }
     P.ndims = ndims;
     P.scratch = scratch;
-    P.host = host;
     if (cudaMemsetAsync(scratch, 0, (size_t)ndims * kScratchWords * 8, stream) != cudaSuccess) return SJQ_ERR_CUDA;
-    if (rows || host) { // (a dimension without rows still has its statistics written)
-        const uint32_t grid = share_blocks(ndims, 2 * sm_count, [&](int i) {
-            return std::make_pair(&P.dim[i], (P.dim[i].n + 8 * kScanThreads - 1) / (8 * kScanThreads));
-        });
-        plan_scan_kernel<<<grid, kScanThreads, 0, stream>>>(P);
-    }
+    // (a dimension without rows has a block too, which writes its statistics)
+    const uint32_t grid = share_blocks(ndims, 2 * sm_count, [&](int i) {
+        return std::make_pair(&P.dim[i], (P.dim[i].n + 8 * kScanThreads - 1) / (8 * kScanThreads));
+    });
+    plan_scan_kernel<<<grid, kScanThreads, 0, stream>>>(P);
     return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 
@@ -882,12 +892,8 @@ extern "C" sjq_status sjq_dim_plan_begin(const sjq_col *cols, int ncols, const s
     if (!aligned16(scratch_dev)) return SJQ_ERR_ALIGN;
     const sjq_dim_desc d{cols, ncols, preds, npreds, key_col, payload_cols, npayload, nullptr};
     DeviceInfo dev;
-    sjq_status st = device_info(&dev);
-    DimRows check_rows; // (argument errors come before a missing device)
-    DimFilters check_filters;
-    int nfilters = 0;
-    const sjq_status bad = fill_rows(d, &check_rows, &check_filters, &nfilters);
-    if (bad != SJQ_OK) return bad;
+    sjq_status st = check_dims(&d, 1);
+    if (st == SJQ_OK) st = device_info(&dev);
     if (st != SJQ_OK) return st;
     cudaStream_t stream = (cudaStream_t)stream_;
     st = scan_launch(&d, 1, static_cast<unsigned long long *>(scratch_dev), nullptr, dev.sm_count, stream);
@@ -913,29 +919,24 @@ extern "C" sjq_status sjq_dims_plan(const sjq_dim_desc *dims, int ndims, void *s
 {
     if (!dims || ndims <= 0 || !scratch_dev || !layouts) return SJQ_ERR_INVALID_ARG;
     if (!aligned16(scratch_dev)) return SJQ_ERR_ALIGN;
-    const int most = std::min(ndims, kBatchDims);
-    if (scratch_bytes < (size_t)most * SJQ_PLAN_SCRATCH_BYTES) return SJQ_ERR_BUFFER_SMALL;
-    for (int i = 0; i < ndims; ++i) {
-        DimRows rows;
-        DimFilters filters;
-        int nfilters = 0;
-        const sjq_status st = fill_rows(dims[i], &rows, &filters, &nfilters);
-        if (st != SJQ_OK) return st;
-    }
-    DeviceInfo dev;
-    sjq_status st = device_info(&dev);
-    if (st != SJQ_OK) return st;
-    cudaStream_t stream = (cudaStream_t)stream_;
+    if (scratch_bytes < (size_t)ndims * SJQ_PLAN_SCRATCH_BYTES) return SJQ_ERR_BUFFER_SMALL;
     int64_t *&host = g_host_stats.words;
+    DeviceInfo dev;
+    sjq_status st = check_dims(dims, ndims);
+    if (st == SJQ_OK) st = device_info(&dev);
+    if (st != SJQ_OK) return st;
     if (!host && cudaHostAlloc(reinterpret_cast<void **>(&host), kBatchDims * 8 * sizeof(int64_t),
                                cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
         (void)cudaGetLastError();
         host = nullptr;
         return SJQ_ERR_CUDA;
     }
+    int64_t *words[kBatchDims];
+    for (int i = 0; i < kBatchDims; ++i) words[i] = host + 8 * i;
+    cudaStream_t stream = (cudaStream_t)stream_;
     for (int first = 0; first < ndims;) {
         const int n = batch_of(dims, ndims, first);
-        st = scan_launch(dims + first, n, static_cast<unsigned long long *>(scratch_dev), host, dev.sm_count, stream);
+        st = scan_launch(dims + first, n, static_cast<unsigned long long *>(scratch_dev), words, dev.sm_count, stream);
         // the kernel writes the statistics into the page-locked words itself
         if (st == SJQ_OK && cudaStreamSynchronize(stream) != cudaSuccess) st = SJQ_ERR_CUDA;
         if (st != SJQ_OK) {
@@ -944,12 +945,31 @@ extern "C" sjq_status sjq_dims_plan(const sjq_dim_desc *dims, int ndims, void *s
         }
         for (int i = 0; i < n; ++i) {
             const sjq_dim_desc &d = dims[first + i];
-            st = sjq_dim_plan_end(d.cols, d.ncols, d.key_col, d.npayload, d.opts, host + 8 * i, &layouts[first + i]);
+            st = sjq_dim_plan_end(d.cols, d.ncols, d.key_col, d.npayload, d.opts, words[i], &layouts[first + i]);
             if (st != SJQ_OK) return st;
         }
         first += n;
     }
     return SJQ_OK;
+}
+
+extern "C" sjq_status sjq_dims_plan_begin(const sjq_dim_desc *dims, int ndims, void *scratch_dev, size_t scratch_bytes,
+                                          int64_t *const *host_stats, void *stream_)
+{
+    if (!dims || ndims <= 0 || !scratch_dev || !host_stats) return SJQ_ERR_INVALID_ARG;
+    if (!aligned16(scratch_dev)) return SJQ_ERR_ALIGN;
+    if (scratch_bytes < (size_t)ndims * SJQ_PLAN_SCRATCH_BYTES) return SJQ_ERR_BUFFER_SMALL;
+    DeviceInfo dev;
+    sjq_status st = check_dims(dims, ndims);
+    if (st == SJQ_OK) st = device_info(&dev);
+    for (int first = 0; first < ndims && st == SJQ_OK;) {
+        const int n = batch_of(dims, ndims, first);
+        st = scan_launch(dims + first, n, static_cast<unsigned long long *>(scratch_dev) + (size_t)first * kScratchWords,
+                         host_stats + first, dev.sm_count, (cudaStream_t)stream_);
+        first += n;
+    }
+    if (st == SJQ_ERR_CUDA) (void)cudaGetLastError();
+    return st;
 }
 
 extern "C" sjq_status sjq_dim_plan(const sjq_col *cols, int ncols, const sjq_pred *preds, int npreds, int key_col,
@@ -1213,14 +1233,14 @@ sjq_status build_launch(const sjq_dim_desc *dims, int ndims, const sjq_dim_layou
 
 extern "C" sjq_status sjq_dims_build(const sjq_dim_desc *dims, int ndims, const sjq_dim_layout *layouts,
                                      void *const *table_mem, const size_t *table_bytes, int32_t *const *status_dev,
-                                     void *stream, sjq_table **tables)
+                                     int32_t clear_status, void *stream, sjq_table **tables)
 {
     if (!dims || ndims <= 0 || !layouts || !table_mem || !table_bytes || !status_dev || !tables) return SJQ_ERR_INVALID_ARG;
     for (int i = 0; i < ndims; ++i) tables[i] = nullptr;
     for (int first = 0; first < ndims;) {
         const int n = batch_of(dims, ndims, first);
         const sjq_status st = build_launch(dims + first, n, layouts + first, table_mem + first, table_bytes + first,
-                                           status_dev + first, true, stream, tables + first);
+                                           status_dev + first, clear_status != 0, stream, tables + first);
         if (st != SJQ_OK) {
             for (int i = 0; i < ndims; ++i) {
                 delete tables[i];

@@ -204,7 +204,10 @@ def lib():
         L.sjq_dims_plan.argtypes = [ctypes.POINTER(_DimDesc), ip, vp, ctypes.c_size_t, vp, ctypes.POINTER(DimLayout)]
         L.sjq_dims_build.restype = ctypes.c_int32
         L.sjq_dims_build.argtypes = [ctypes.POINTER(_DimDesc), ip, ctypes.POINTER(DimLayout), ctypes.POINTER(vp),
-                                     ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(vp), vp, ctypes.POINTER(vp)]
+                                     ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(vp), ctypes.c_int32, vp,
+                                     ctypes.POINTER(vp)]
+        L.sjq_dims_plan_begin.restype = ctypes.c_int32
+        L.sjq_dims_plan_begin.argtypes = [ctypes.POINTER(_DimDesc), ip, vp, ctypes.c_size_t, ctypes.POINTER(vp), vp]
         L.sjq_dim_layout_bytes.restype = ctypes.c_int32
         L.sjq_dim_layout_bytes.argtypes = [ctypes.POINTER(DimLayout), ctypes.POINTER(ctypes.c_size_t)]
         L.sjq_table_info.restype = ctypes.c_int32
@@ -307,6 +310,7 @@ class Table:
 
     def __init__(self, handle: int, layout: DimLayout, mem: torch.Tensor, status: torch.Tensor):
         self.handle, self.layout, self.mem, self.status_dev = handle, layout, mem, status
+        self.scans = 1  # scan kernels enqueued for it (a batch's scan counts with its first table)
 
     def status(self) -> int:
         return int(self.status_dev.item())
@@ -367,10 +371,17 @@ def _build_tables(dims, edit_layout=None, mem_offset: int = 0) -> list:
         handles = (vp * n)()
         rc = L.sjq_dims_build(descs, n, layouts, (vp * n)(*[m.data_ptr() for m in mems]),
                               (ctypes.c_size_t * n)(*[m.numel() for m in mems]),
-                              (vp * n)(*[s.data_ptr() for s in statuses]), stream, handles)
+                              (vp * n)(*[s.data_ptr() for s in statuses]), 1, stream, handles)
         if rc != 0:
             raise SjqError(rc, "sjq_build_dim")
-    return [Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], statuses[i]) for i in range(n)]
+    return _batch_tables(Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], statuses[i]) for i in range(n))
+
+
+def _batch_tables(tables) -> list:
+    tables = list(tables)
+    for i, t in enumerate(tables):
+        t.scans = int(i % 8 == 0)  # eight dimensions to a launch
+    return tables
 
 
 class TableBuilder:
@@ -414,27 +425,47 @@ class TableBuilder:
             self.guards = [torch.cuda.Event(), torch.cuda.Event()]
             self.guard_set = [False, False]
             self.layout = DimLayout()
+            self.desc = _DimDesc(self.carr, len(self.names), self.parr, self.npreds, self.key_col, self.pay, self.npay,
+                                 ctypes.pointer(self.opts))
+            self.batch_scratch = None  # of the batches this builder is the first of
+            self.ran_on = self         # the builder on whose streams the newest scan and build were enqueued
+
+    def _move_to(self, other):
+        """Scans and builds of this builder are enqueued on the streams of `other` from now on: they follow what is
+        queued on its own, or on those of the builder it was last batched with."""
+        if self.ran_on is not other:
+            other.side.wait_stream(self.ran_on.side)
+            other.scan_side.wait_stream(self.ran_on.scan_side)
+            self.ran_on = other
+
+    def _next_stats(self) -> int:
+        j = (self.scan + 1) % len(self.stats)
+        if self.stats_used[j]:
+            self.stats_done[j].synchronize()  # the host is a whole ring ahead of the device
+        return j
+
+    def _scanned(self, j: int, stream):
+        self.stats_done[j].record(stream)
+        self.stats_used[j] = True
+        self.scan = j
 
     def begin(self):
         """Enqueue the key-range scan on the side stream.  It only reads the dimension columns, so it does
         not wait for work queued on the current stream (a previous run may still be reading the old table)."""
-        j = (self.scan + 1) % len(self.stats)
-        if self.stats_used[j]:
-            self.stats_done[j].synchronize()  # the host is a whole ring ahead of the device
+        self._move_to(self)
+        j = self._next_stats()
         rc = lib().sjq_dim_plan_begin(self.carr, len(self.names), self.parr, self.npreds, self.key_col, self.pay,
                                       self.npay, self.scratch.data_ptr(), self.stats[j].data_ptr(),
                                       self.scan_side.cuda_stream)
         if rc != 0:
             raise SjqError(rc, "sjq_dim_plan_begin")
-        self.stats_done[j].record(self.scan_side)
-        self.stats_used[j] = True
-        self.scan = j
+        self._scanned(j, self.scan_side)
 
     def after(self, stream):
         """Scans and builds enqueued from now on follow the work already queued on `stream` (e.g. copies that
         refresh the dimension columns)."""
-        self.side.wait_stream(stream)
-        self.scan_side.wait_stream(stream)
+        self.ran_on.side.wait_stream(stream)
+        self.ran_on.scan_side.wait_stream(stream)
 
     def _choose_layout(self):
         """The layout for the scan just enqueued, or (reuse_layout) for the newest one that has completed."""
@@ -459,23 +490,9 @@ class TableBuilder:
     def finish(self) -> Table:
         """Choose the layout (waiting for the scan unless reuse_layout allows an earlier one), enqueue the
         build on the side stream."""
+        self._move_to(self)
         self._choose_layout()
-        i = self.turn
-        self.turn ^= 1
-        main = torch.cuda.current_stream(self.device)
-        if self.mems[i] is None or self.mems[i].numel() < self.layout.table_bytes:
-            with torch.cuda.device(self.device):
-                self.mems[i] = torch.empty(self.layout.table_bytes, dtype=torch.uint8, device=self.device)
-            self.side.wait_stream(main)
-        # The build overwrites buffer i, which the table returned two calls ago lives in: it must follow
-        # whatever the current stream had queued by the time of the previous call (the runs on that table),
-        # not the runs on the previous table, which read the other buffer.  A table is therefore valid for
-        # work enqueued on the current stream before the next call of finish().
-        if self.guard_set[i]:
-            self.side.wait_event(self.guards[i])
-        self.guards[i ^ 1].record(main)
-        self.guard_set[i ^ 1] = True
-        mem = self.mems[i]
+        mem = self._next_memory(self.side)
         handle = ctypes.c_void_p()
         rc = lib().sjq_build_dim(self.carr, len(self.names), self.parr, self.npreds, self.key_col, self.pay,
                                  self.npay, ctypes.byref(self.layout), mem.data_ptr(), mem.numel(),
@@ -485,6 +502,58 @@ class TableBuilder:
         layout = DimLayout.from_buffer_copy(self.layout)
         return Table(handle.value, layout, mem, self.status)
 
+    def _next_memory(self, side) -> torch.Tensor:
+        """The table memory whose turn it is, for a build on the stream `side`."""
+        i = self.turn
+        self.turn ^= 1
+        main = torch.cuda.current_stream(self.device)
+        if self.mems[i] is None or self.mems[i].numel() < self.layout.table_bytes:
+            with torch.cuda.device(self.device):
+                self.mems[i] = torch.empty(self.layout.table_bytes, dtype=torch.uint8, device=self.device)
+            side.wait_stream(main)
+        # The build overwrites buffer i, which the table returned two calls ago lives in: it must follow
+        # whatever the current stream had queued by the time of the previous call (the runs on that table),
+        # not the runs on the previous table, which read the other buffer.  A table is therefore valid for
+        # work enqueued on the current stream before the next call of finish().
+        if self.guard_set[i]:
+            side.wait_event(self.guards[i])
+        self.guards[i ^ 1].record(main)
+        self.guard_set[i ^ 1] = True
+        return self.mems[i]
+
+
+def _build_batch(builders: list) -> list:
+    """begin() and finish() of several builders of one device with one launch per step: the scans on the first one's
+    scan stream, then the fills and the builds on its build stream."""
+    lead, n, vp, L = builders[0], len(builders), ctypes.c_void_p, lib()
+    for b in builders:
+        b._move_to(lead)
+    if lead.batch_scratch is None or lead.batch_scratch.numel() < n * PLAN_SCRATCH_BYTES:
+        with torch.cuda.device(lead.device):
+            lead.batch_scratch = torch.empty(n * PLAN_SCRATCH_BYTES, dtype=torch.uint8, device=lead.device)
+        lead.scan_side.wait_stream(torch.cuda.current_stream(lead.device))
+    descs = (_DimDesc * n)(*[b.desc for b in builders])
+    slots = [b._next_stats() for b in builders]
+    rc = L.sjq_dims_plan_begin(descs, n, lead.batch_scratch.data_ptr(), lead.batch_scratch.numel(),
+                               (vp * n)(*[b.stats[j].data_ptr() for b, j in zip(builders, slots)]),
+                               lead.scan_side.cuda_stream)
+    if rc != 0:
+        raise SjqError(rc, "sjq_dims_plan_begin")
+    for b, j in zip(builders, slots):
+        b._scanned(j, lead.scan_side)
+    for b in builders:
+        b._choose_layout()
+    layouts = (DimLayout * n)(*[b.layout for b in builders])
+    mems = [b._next_memory(lead.side) for b in builders]
+    handles = (vp * n)()
+    rc = L.sjq_dims_build(descs, n, layouts, (vp * n)(*[m.data_ptr() for m in mems]),
+                          (ctypes.c_size_t * n)(*[m.numel() for m in mems]),
+                          (vp * n)(*[b.status.data_ptr() for b in builders]), 0, lead.side.cuda_stream, handles)
+    if rc != 0:
+        raise SjqError(rc, "sjq_dims_build")
+    return _batch_tables(Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], builders[i].status)
+                         for i in range(n))
+
 
 def workload_builders(w, dims: dict, reuse_layout: bool = False) -> dict:
     return {d.name: TableBuilder(dims[d.name], d.key, d.preds, d.payloads,
@@ -493,12 +562,19 @@ def workload_builders(w, dims: dict, reuse_layout: bool = False) -> dict:
 
 
 def build_tables(builders: dict) -> dict:
-    """Plan all dimensions (one wait each, scans overlapping on side streams), build them concurrently,
-    and make the current stream wait for the builds."""
-    for b in builders.values():
+    """Plan all dimensions and build their tables on side streams, one scan and one build for all of them, and make
+    the current stream wait for the builds."""
+    if not builders:
+        return {}
+    each = list(builders.values())
+    if all(b.device == each[0].device for b in each) and len(set(map(id, each))) == len(each):
+        tables = dict(zip(builders, _build_batch(each)))
+        torch.cuda.current_stream(each[0].device).wait_stream(each[0].side)
+        return tables
+    for b in each:
         b.begin()
     tables = {name: b.finish() for name, b in builders.items()}
-    for b in builders.values():
+    for b in each:
         torch.cuda.current_stream(b.device).wait_stream(b.side)
     return tables
 
@@ -863,12 +939,12 @@ def jit_log() -> str:
 
 
 def build_launches(table: "Table") -> int:
-    """Kernels enqueued by sjq_dim_plan + sjq_build_dim for this table: the plan's two (counter
-    initialisation, and the scan unless the dimension is empty) and what the build reports."""
+    """Kernels enqueued to plan and build this table: the scan and what the build reports (those of a batch count
+    with its first table)."""
     L = lib()
     L.sjq_table_kernel_launches.restype = ctypes.c_int32
     L.sjq_table_kernel_launches.argtypes = [ctypes.c_void_p]
-    return 1 + (1 if table.layout.dim_rows > 0 else 0) + int(L.sjq_table_kernel_launches(table.handle))
+    return table.scans + int(L.sjq_table_kernel_launches(table.handle))
 
 
 def release() -> int:

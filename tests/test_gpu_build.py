@@ -110,3 +110,40 @@ def test_empty_dimension_in_a_batch():
     full = {"k": np.arange(9, dtype=np.int32), "p": np.arange(9, dtype=np.int32)}
     tables = sjq.sjq._build_tables([(to_dev(d), "k", (), ("p",), sjq.sjq._BuildOpts()) for d in (empty, full, empty)])
     assert [t.layout.entries for t in tables] == [0, 9, 0] and all(t.status() == 0 for t in tables)
+
+
+@pytest.mark.parametrize("reuse", [False, True])
+def test_builders_alone_and_in_changing_batches(reuse):
+    """The same builders in batches of different make-up, alone, and with their columns refreshed on another stream."""
+    rng = np.random.default_rng(9)
+    n, rows = 20_011, {"a": 4_000, "b": 700, "c": 33_000}
+    host = {d: {"k": rng.permutation(r).astype(np.int32), "p": rng.integers(0, 9, r).astype(np.int32),
+                "f": rng.integers(0, 9, r).astype(np.int32)} for d, r in rows.items()}
+    fact = {d: rng.integers(0, r, n).astype(np.int32) for d, r in rows.items()}
+    w = adhoc("batches", fact, [(d, host[d], "k", [Pred("f", "GE", 2)], ["p"]) for d in rows], [(d, d) for d in rows], [],
+              KeyExpr((Term("PAYLOAD", 0, 0),)), AggExpr("ADD", Term("PAYLOAD", 1, 0), Term("PAYLOAD", 2, 0)), "DENSE",
+              num_groups=9)
+    dev = {d: to_dev(c) for d, c in host.items()}
+    builders = sjq.workload_builders(w, dev, reuse_layout=reuse)
+    refresh = torch.cuda.Stream()
+    for turn in range(6):
+        for d in rows:  # other payloads in the same range
+            host[d]["p"] = rng.permutation(host[d]["p"])
+        torch.cuda.synchronize()
+        with torch.cuda.stream(refresh):
+            for d in rows:
+                dev[d]["p"].copy_(torch.from_numpy(host[d]["p"]).pin_memory(), non_blocking=True)
+        for b in builders.values():
+            b.after(refresh)
+        if turn % 3 == 0:
+            tables = sjq.build_tables(builders)
+        elif turn % 3 == 1:
+            tables = sjq.build_tables({d: builders[d] for d in ("c", "a")})
+            builders["b"].begin()
+            tables["b"] = builders["b"].finish()
+            torch.cuda.current_stream().wait_stream(builders["b"].side)
+        else:
+            tables = {**sjq.build_tables({"b": builders["b"]}), **sjq.build_tables({d: builders[d] for d in ("a", "c")})}
+        res, exp, _ = run_both(w, fact, host, tables=tables)
+        assert res.status() == 0 and all(t.status() == 0 for t in tables.values())
+        compare(w, res, exp)
