@@ -353,28 +353,35 @@ def _build_tables(dims, edit_layout=None, mem_offset: int = 0) -> list:
             keep.append((carr, parr, values, pay, opts))
             descs[i] = _DimDesc(carr, len(names), parr, len(preds), names.index(key), pay, len(payloads),
                                 ctypes.pointer(opts))
-        L, stream = lib(), _stream_ptr(device)
+        # everything that does not depend on the layouts comes before the plan, whose wait leaves the GPU idle until
+        # the builds are enqueued; the tables share one allocation
+        L, stream, vp = lib(), _raw_stream(device.index), ctypes.c_void_p
         scratch = torch.empty(n * PLAN_SCRATCH_BYTES, dtype=torch.uint8, device=device)
-        layouts = (DimLayout * n)()
+        status = torch.empty(n, dtype=torch.int32, device=device)  # cleared by the build
+        layouts, handles = (DimLayout * n)(), (vp * n)()
+        base = status.data_ptr()
+        status_ptrs = (vp * n)(*[base + 4 * i for i in range(n)])
+        ptrs, sizes, at = (vp * n)(), (ctypes.c_size_t * n)(), [0] * (n + 1)
         rc = L.sjq_dims_plan(descs, n, scratch.data_ptr(), scratch.numel(), stream, layouts)
         if rc != 0:
             raise SjqError(rc, "sjq_dim_plan")
-        planned = [x.table_bytes for x in layouts]
+        for i in range(n):
+            sizes[i] = layouts[i].table_bytes
         if edit_layout is not None:
-            for x in layouts:
-                edit_layout(x)
-        mems = [torch.empty(max(p, x.table_bytes) + mem_offset, dtype=torch.uint8, device=device)[mem_offset:]
-                for p, x in zip(planned, layouts)]
-        status = torch.empty(n, dtype=torch.int32, device=device)  # cleared by the build
-        statuses = [status[i:i + 1] for i in range(n)]
-        vp = ctypes.c_void_p
-        handles = (vp * n)()
-        rc = L.sjq_dims_build(descs, n, layouts, (vp * n)(*[m.data_ptr() for m in mems]),
-                              (ctypes.c_size_t * n)(*[m.numel() for m in mems]),
-                              (vp * n)(*[s.data_ptr() for s in statuses]), 1, stream, handles)
+            for i in range(n):
+                edit_layout(layouts[i])
+                sizes[i] = max(sizes[i], layouts[i].table_bytes)
+        for i in range(n):
+            at[i + 1] = at[i] + (sizes[i] + mem_offset + 255) // 256 * 256
+        mem = torch.empty(at[n], dtype=torch.uint8, device=device)
+        base = mem.data_ptr() + mem_offset
+        for i in range(n):
+            ptrs[i] = base + at[i]
+        rc = L.sjq_dims_build(descs, n, layouts, ptrs, sizes, status_ptrs, 1, stream, handles)
         if rc != 0:
             raise SjqError(rc, "sjq_build_dim")
-    return _batch_tables(Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], statuses[i]) for i in range(n))
+    return _batch_tables(Table(handles[i], DimLayout.from_buffer_copy(layouts[i]),
+                               mem[at[i] + mem_offset:at[i] + mem_offset + sizes[i]], status[i:i + 1]) for i in range(n))
 
 
 def _batch_tables(tables) -> list:
@@ -705,7 +712,10 @@ def _term(t, names) -> _Term:
     return _Term(1, int(t.a), t.b, t.mult)
 
 
-def alloc_result(mode: str, num_groups: int, capacity: int, want_count: bool, device) -> Result:
+def alloc_result(mode: str, num_groups: int, capacity: int, want_count: bool, device, cleared: bool = True) -> Result:
+    """Buffers for a result.  cleared: with the status and the number of groups at zero (a run clears them itself unless
+    it accumulates)."""
+    new = torch.zeros if cleared else torch.empty
     spec = _ResultSpec(MODES[mode], num_groups, capacity)
     n = 1 if mode == "SCALAR" else num_groups if mode == "DENSE" else capacity
     keys = n_groups = ws = joined = None
@@ -720,13 +730,13 @@ def alloc_result(mode: str, num_groups: int, capacity: int, want_count: bool, de
         counts = torch.empty(n, dtype=torch.int64, device=device)
     if mode == "HASHED":
         keys = torch.empty(n, dtype=torch.int64, device=device)
-        n_groups = torch.zeros(1, dtype=torch.int64, device=device)
+        n_groups = new(1, dtype=torch.int64, device=device)
         nbytes = ctypes.c_size_t(0)
         rc = lib().sjq_run_workspace_bytes(ctypes.byref(spec), ctypes.byref(nbytes))
         if rc != 0:
             raise SjqError(rc, "sjq_run_workspace_bytes")
         ws = torch.empty(nbytes.value, dtype=torch.uint8, device=device)
-    status = torch.zeros(1, dtype=torch.int32, device=device)
+    status = new(1, dtype=torch.int32, device=device)
     return Result(mode, sums, counts, keys, n_groups, status, ws, joined=joined)
 
 
@@ -786,7 +796,9 @@ def run(fact: dict, preds=(), joins=(), key=None, agg=None, mode: str = "SCALAR"
     if index != torch.cuda.current_device():
         with torch.cuda.device(device):
             return run(fact, preds, joins, key, agg, mode, num_groups, capacity, opts, result)
-    res = result if result is not None else alloc_result(mode, num_groups, capacity, agg.want_count, device)
+    res = result
+    if res is None:
+        res = alloc_result(mode, num_groups, capacity, agg.want_count, device, cleared=bool(opts and opts.accumulate))
     # (one hot-key scratch per device, reused by every run: runs on one stream are ordered)
     rc = marshal().run(fact, preds, joins, key, agg, MODES[mode], num_groups, capacity, opts, res,
                        _raw_stream(index), lambda: _hot_scratch(device))
