@@ -185,7 +185,7 @@ std::string jit_shape_header(const RunParams &P, int agg, bool mul, bool hash, i
           << "; S.in_smem = " << (int)S.in_smem << "; S.kind = " << (int)S.kind << "; S.simple = " << (int)S.simple
           << "; S.acc = " << (int)S.acc << "; S.acc32 = " << S.acc32 << "; S.code_bits = " << (int)S.code_bits
           << "; S.issue_after = " << (int)S.issue_after << "; S.full = " << (int)S.full << "; S.hot = " << (int)S.hot
-          << "; S.wide = " << (int)S.wide << ";\n";
+          << "; S.wide = " << (int)S.wide << "; S.col32 = " << S.col32 << ";\n";
         for (int i = 0; i < 9; ++i) {
             // INT64_MIN cannot be written as a literal
             if (S.mult[i] == INT64_MIN) o << "        S.mult[" << i << "] = (-9223372036854775807LL - 1);";
@@ -226,7 +226,7 @@ void shape_key(const RunParams &P, int agg, bool mul, bool hash, int lb_threads,
     for (int s = 0; s < P.nstages; ++s) {
         const DStage &S = P.st[s];
         const uint8_t b[] = {S.op, S.is64, S.neg, S.never, S.nset, S.set_idx, S.in_smem, S.kind, S.simple, S.code_bits,
-                             (uint8_t)S.issue_after, S.full, S.hot, S.wide};
+                             (uint8_t)S.issue_after, S.full, S.hot, S.wide, (uint8_t)S.col32};
         static_assert(sizeof(b) + sizeof(S.acc) + sizeof(S.acc32) + sizeof(S.mult) + sizeof(S.mult32) <= 160, "room for a stage");
         k->put(b, sizeof(b));
         k->put(&S.acc, sizeof(S.acc));

@@ -447,6 +447,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
         S.kind = (uint8_t)sp.kind;
         S.col = fact[sp.col].data;
         S.is64 = (uint8_t)(fact[sp.col].dtype == SJQ_I64);
+        S.col32 = S.is64 && (reinterpret_cast<uintptr_t>(S.col) & 31u) == 0;
         S.op = OP_LOAD;
         if (sp.kind == ST_PRED) {
             DPred d;

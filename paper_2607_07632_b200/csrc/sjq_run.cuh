@@ -96,7 +96,7 @@ struct DStage {
     uint8_t wide;   // open-addressing probe: the bucket array starts on a 32-byte boundary, so a bucket is one 256-bit load
     const void *hot_tab; // hot-key table in global memory (kHotSlots + 1 entries), copied to shared memory per block
     uint32_t hot_off;    // byte offset of that copy in dynamic shared memory
-    uint32_t hot_pad;
+    uint32_t col32;      // the column starts on a 32-byte boundary: four 64-bit values are one load
 };
 static_assert(sizeof(DStage) % 8 == 0, "stage descriptors are copied as 64-bit words");
 

@@ -43,7 +43,7 @@ __device__ __forceinline__ void filter_group(const RunParams &P, const DStage &S
     T v[4];
     const T *c = static_cast<const T *>(S.col) + r;
     if (valid == 0xFu) {
-        Vec4<T>::load(c, v);
+        Vec4<T>::load(c, v, false);
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) v[k] = ((valid >> k) & 1u) ? c[k] : (T)0;

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 import torch
 
-from datagen.workloads import AggExpr, Pred, Term
+from datagen.workloads import AggExpr, KeyExpr, Pred, Term
 
 pytestmark = pytest.mark.gpu
 
@@ -60,3 +60,24 @@ def test_launch_shapes_by_rows_and_survivors(n, below):
         assert res.status() == 0
         compare(w, res, exp)
         assert (res.info.reserved_levels == 0) == (n <= 2**19)
+
+
+@pytest.mark.parametrize("shift", [0, 2])
+def test_64_bit_columns_on_16_and_32_byte_boundaries(shift):
+    """Four 64-bit values are one 256-bit load where the column starts on a 32-byte boundary, else two loads."""
+    n, rng = 600_007, np.random.default_rng(8)
+    keys = rng.permutation(5_000).astype(np.int64) * 2**33
+    dim = {"k": keys, "p": rng.integers(0, 99, 5_000).astype(np.int32)}
+    fact = {"fk": rng.choice(np.concatenate([keys, keys + 1]), n), "m": rng.integers(-2**62, 2**62, n)}
+    w = adhoc("wide", fact, [("d", dim, "k", [], ["p"], True)], [("fk", "d")], [], KeyExpr((Term("PAYLOAD", 0, 0),)),
+              AggExpr("COL", Term("FACT", "m")), "DENSE", num_groups=99)
+    dev = {}
+    for c, v in fact.items():
+        room = torch.empty(n + shift, dtype=torch.int64, device="cuda")
+        dev[c] = room[shift:].copy_(torch.from_numpy(v))
+        assert dev[c].data_ptr() % 32 == 8 * shift % 32
+    tables = None
+    for opts in (sjq.RunOpts(), sjq.RunOpts(specialise=True), sjq.RunOpts(compaction=1), sjq.RunOpts(specialise=True, compaction=1)):
+        res, exp, tables = run_both(w, fact, {"d": dim}, opts=opts, dev_fact=dev, tables=tables)
+        assert res.status() == 0
+        compare(w, res, exp)
