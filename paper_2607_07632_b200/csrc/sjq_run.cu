@@ -142,7 +142,9 @@ double column_ps(int width, double reach)
 // (Ranking by (1 - selectivity) / cost with one cost for every table below 200 KB left city x brand to chance: two
 // joins that keep one row in 25, one probing 25 KB in shared memory, the other 175 KB through the L1, which is
 // 0.67 or 3.3 ms for 600 M rows with the one or the other first.)
-Order cheapest_order(const Specs &specs)
+// `column(spec, reach)`: what reading a stage's column for the rows that reach it costs.
+template <typename Column>
+Order cheapest_order(const Specs &specs, Column column)
 {
     constexpr int kExhaustive = 8;
     const int n = (int)specs.size();
@@ -151,7 +153,7 @@ Order cheapest_order(const Specs &specs)
     for (int i = 0; i < n; ++i)
         if (specs[i].prefilter != 2) early[m++] = i;
     auto cost = [&](int i, double reach, bool column_read) {
-        return (column_read ? 0.0 : column_ps(specs[i].width, reach)) + reach * specs[i].cost;
+        return (column_read ? 0.0 : column(specs[i], reach)) + reach * specs[i].cost;
     };
     if (m <= kExhaustive) {
         struct Best { double ps, reach; int last; } best[1 << kExhaustive];
@@ -254,7 +256,7 @@ sjq_status order_stages(const sjq_col *fact, const sjq_pred *preds, int npreds, 
             }
         }
     } else {
-        order = cheapest_order(specs);
+        order = cheapest_order(specs, [](const StageSpec &sp, double reach) { return column_ps(sp.width, reach); });
     }
 
     return SJQ_OK;
@@ -1115,11 +1117,24 @@ namespace {
 
 enum { HOST_COPY = 0, HOST_IN_PLACE = 1, HOST_SKIP = 2 };
 
+// What a column costs on the bus, in picoseconds per row of the table: copied whole at 53 GB/s, or, where at most
+// kInPlaceReach of the rows reach it, the 32-byte sectors that hold one of them, read by the kernel at about half that
+// (28 MB in 0.95 ms beside the copies).
+constexpr double kInPlaceReach = 0.05;
+double bus_ps(int width, double reach)
+{
+    const double copy = 18.9 * width;
+    if (reach > kInPlaceReach) return copy;
+    double dead = 1.0 - reach;
+    for (int rows = 32 / width; rows > 1; rows >>= 1) dead *= dead;
+    return std::min(copy, 1.9 * copy * (1.0 - dead));
+}
+
 // How each host-resident column reaches the kernel.  A column most rows still need is copied chunk by
 // chunk; one that only a few per cent of the rows reach (lazy loading: it is read for survivors only) is
 // read by the kernel straight from the page-locked host buffer, 32 bytes per touched sector, which moves
 // far fewer bytes over the bus than the whole column (measured on the four-join workload, 600 M rows:
-// revenue and supplycost 16 ms instead of 87 ms of copies; break-even near 5 % of the rows); a column the
+// revenue and supplycost 16 ms instead of 87 ms of copies; break-even beyond 5 % of the rows); a column the
 // query never references is not transferred at all.  `need`: share of the rows each column is first read
 // for (< 0: never).  Invalid queries get "copy everything" and are rejected later by sjq_run.
 void host_transfer_plan(const sjq_col *fact_host, int nfact, const sjq_pred *preds, int npreds,
@@ -1174,6 +1189,28 @@ void host_transfer_plan(const sjq_col *fact_host, int nfact, const sjq_pred *pre
         measured.pass_ppm[p] = ppm_of(pass, samples);
     }
     if (!ok || order_stages(fact_host, preds, npreds, joins, njoins, measured, &specs, &order) != SJQ_OK) return;
+    std::vector<const char *> mapped(nfact, nullptr); // device address of a page-locked column
+    for (int c = 0; c < nfact; ++c) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, fact_host[c].data) == cudaSuccess && attr.type == cudaMemoryTypeHost &&
+            attr.devicePointer && aligned16(attr.devicePointer))
+            mapped[c] = static_cast<const char *>(attr.devicePointer);
+        else
+            (void)cudaGetLastError(); // pageable memory: copied
+    }
+    const bool in_place_allowed = !opts.eager_loads && !opts.host_copy_all;
+    // The bus is what a run from host memory waits for, so the filters are ordered by what their columns cost there: a
+    // column is copied whole, or read in place where few rows reach it.  Four joins, 16 M rows: with the order of a
+    // device-resident run three columns are copied (4,017 us), with this one two (3,373 us); 3 M rows 822 and 711, 700
+    // thousand 244 and 218.  Below a million rows the saving is no more than that and the order stays the device's.
+    bool by_bus = in_place_allowed && !opts.norder && n >= (int64_t)1 << 20;
+    for (const StageSpec &sp : specs) by_bus = by_bus && sp.prefilter == 0 && mapped[sp.col];
+    if (by_bus) {
+        order = cheapest_order(specs, [](const StageSpec &sp, double reach) { return bus_ps(sp.width, reach); });
+        opts.norder = order.size();
+        for (int i = 0; i < order.size(); ++i)
+            opts.order[i] = specs[order[i]].kind == ST_PRED ? specs[order[i]].index : npreds + specs[order[i]].index;
+    }
     std::vector<double> &need = *need_out;
     need.assign(nfact, -1.0);
     double reach = 1.0;
@@ -1191,15 +1228,9 @@ void host_transfer_plan(const sjq_col *fact_host, int nfact, const sjq_pred *pre
     for (int c = 0; c < nfact; ++c) {
         if (need[c] < 0) {
             how[c] = HOST_SKIP;
-        } else if (need[c] <= 0.04 && !opts.eager_loads && !opts.host_copy_all) {
-            cudaPointerAttributes attr;
-            if (cudaPointerGetAttributes(&attr, fact_host[c].data) == cudaSuccess && attr.type == cudaMemoryTypeHost &&
-                attr.devicePointer && aligned16(attr.devicePointer)) {
-                how[c] = HOST_IN_PLACE;
-                direct_base[c] = static_cast<const char *>(attr.devicePointer);
-            } else {
-                (void)cudaGetLastError(); // pageable memory: copy it
-            }
+        } else if (need[c] <= kInPlaceReach && in_place_allowed && mapped[c]) {
+            how[c] = HOST_IN_PLACE;
+            direct_base[c] = mapped[c];
         }
     }
 }

@@ -81,3 +81,28 @@ def test_64_bit_columns_on_16_and_32_byte_boundaries(shift):
         res, exp, tables = run_both(w, fact, {"d": dim}, opts=opts, dev_fact=dev, tables=tables)
         assert res.status() == 0
         compare(w, res, exp)
+
+
+@pytest.mark.parametrize("n", [2**20 - 1, 2**20, 1_300_001])
+def test_host_resident_filters_are_ordered_by_the_bus(n):
+    """From 2^20 rows on the order copies as few columns as it can: of three filters that keep a fifth, a fifth and a
+    third, the first two are copied and the last is read in place; below it is the order of a device-resident run."""
+    rng = np.random.default_rng(n)
+    dims, fact, host = [], {}, {}
+    for nm, rows, of in (("wide", 400_000, 5), ("other", 400_000, 5), ("small", 3_000, 3)):
+        host[nm] = {"k": rng.permutation(rows).astype(np.int32), "a": (np.arange(rows) % of).astype(np.int32)}
+        dims.append((nm, host[nm], "k", [Pred("a", "EQ", 1)], []))
+        fact[nm] = rng.integers(0, rows, n).astype(np.int32)
+    fact["m"] = rng.integers(-2**31, 2**31 - 1, n).astype(np.int32)
+    w = adhoc("bus", fact, dims, [(d[0], d[0]) for d in dims], [], None, AggExpr("COL", Term("FACT", "m")), "SCALAR")
+    _, exp, tables = run_both(w, fact, host)
+    pinned = {c: torch.from_numpy(v).pin_memory() for c, v in fact.items()}
+    how = {c: h for c, (h, _) in sjq.host_transfer_plan(pinned, (), [(d[0], tables[d[0]]) for d in dims], None, w.agg).items()}
+    assert how["small"] == ("in place" if n >= 2**20 else "copy") and how["m"] == "in place"
+    for chunk in (2**18, 2**21):
+        staging = torch.empty(sjq.staging_bytes(pinned, chunk), dtype=torch.uint8, device="cuda")
+        for opts in (sjq.RunOpts(), sjq.RunOpts(specialise=True), sjq.RunOpts(host_copy_all=True), sjq.RunOpts(order=(2, 0, 1))):
+            res, out = sjq.run_workload_host(w, pinned, tables, staging, chunk, opts)
+            torch.cuda.synchronize()
+            assert int(out.status[0]) == 0
+            compare(w, res, exp)
