@@ -351,10 +351,12 @@ extern "C" sjq_status sjq_pred_sample(const sjq_col *fact, int nfact, const sjq_
     return sjq_pred_sample_end(h, npreds, pass_ppm);
 }
 
-extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *preds, int npreds,
+// sjq_run.  `callers_order`: the order of the filters, if the options give one, is the caller's own and not one that
+// this library chose for a run from host memory.
+static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *preds, int npreds,
                               const sjq_join *joins, int njoins, const sjq_key_expr *key, const sjq_agg_expr *agg,
                               const sjq_result_spec *spec, const sjq_result *out, const sjq_run_opts *opts_,
-                              void *stream_, sjq_run_info *info)
+                              bool callers_order, void *stream_, sjq_run_info *info)
 {
     // ------------------------------------------------------------ validation
     if (!fact || nfact <= 0 || nfact > 64 || npreds < 0 || npreds > SJQ_MAX_PREDS || (npreds && !preds) ||
@@ -565,8 +567,9 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
             // joins, the third filter reached by 6 % of the rows, 1286 us with a queue for it and 1223 without, but
             // 1295 without one for the second, reached by 20 %; filter and sum, 4 %: 1280 and 1109; two joins, 4 %:
             // 783 and 735).  The interpreting kernel loads its columns one after the other and is better off with
-            // queues (four joins, 60 M rows: 175 us against 290 without any).
-            const double queue_reach = opts.specialise ? 0.12 : 0.002;
+            // queues (four joins, 60 M rows: 175 us against 290 without any), and an order that the caller lays down
+            // is carried out with a level for every filter.
+            const double queue_reach = opts.specialise && !(opts.norder && callers_order) ? 0.12 : 0.002;
             while (nd0 + nfq < nfilter && nfq < kMaxQueues - 1 && specs[order[nd0 + nfq]].sel < 0.9 &&
                    reach[nd0 + nfq] > queue_reach && specs[order[nd0 + nfq]].prefilter != 2)
                 ++nfq;
@@ -1043,6 +1046,14 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
 }
 
 
+extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *preds, int npreds,
+                              const sjq_join *joins, int njoins, const sjq_key_expr *key, const sjq_agg_expr *agg,
+                              const sjq_result_spec *spec, const sjq_result *out, const sjq_run_opts *opts,
+                              void *stream, sjq_run_info *info)
+{
+    return run_planned(fact, nfact, preds, npreds, joins, njoins, key, agg, spec, out, opts, true, stream, info);
+}
+
 // ---------------------------------------------------------------------------
 // Merge of hashed results (the exchange step of a row-sharded run).
 extern "C" sjq_status sjq_merge_groups(const int64_t *keys, const int64_t *sums, const int64_t *counts, int64_t n,
@@ -1321,8 +1332,8 @@ extern "C" sjq_status sjq_run_host(const sjq_col *fact_host, int nfact, const sj
         if (k > 0 && cudaStreamWaitEvent(hp->s[b], hp->done[b ^ 1], 0) != cudaSuccess) return SJQ_ERR_CUDA;
         opts.accumulate = (k > 0 || (opts_ && opts_->accumulate)) ? 1 : 0;
         opts.hot_keys = 2; // a chunk's foreign keys may still be in host memory: no sampling pass over them
-        sjq_status st = sjq_run(dev_cols.data(), nfact, preds, npreds, joins, njoins, key, agg, spec, out, &opts,
-                                hp->s[b], nullptr);
+        sjq_status st = run_planned(dev_cols.data(), nfact, preds, npreds, joins, njoins, key, agg, spec, out, &opts,
+                                    opts_ && opts_->norder != 0, hp->s[b], nullptr);
         if (st != SJQ_OK) return st;
         if (cudaEventRecord(hp->done[b], hp->s[b]) != cudaSuccess) return SJQ_ERR_CUDA;
     }
