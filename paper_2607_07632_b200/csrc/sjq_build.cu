@@ -47,16 +47,18 @@ struct DimFilters {
 };
 
 // Four consecutive values of a column as T (a 32-bit column may be read as 64-bit values, not the other way round).
+// Evict first: the columns pass once and should not push the table that is being built out of the L2 (skewed keys asked
+// once, 128 MB of columns beside an 84 MB table: 289 -> 279 us in all).
 template <typename T>
 __device__ __forceinline__ void load4(const void *col, bool is64, int64_t r, int rows, T *v)
 {
     if (rows == 4) {
         if (sizeof(T) == 8 && is64) {
-            const longlong2 a = __ldg(static_cast<const longlong2 *>(col) + r / 2);
-            const longlong2 b = __ldg(static_cast<const longlong2 *>(col) + r / 2 + 1);
+            const longlong2 a = __ldcs(static_cast<const longlong2 *>(col) + r / 2);
+            const longlong2 b = __ldcs(static_cast<const longlong2 *>(col) + r / 2 + 1);
             v[0] = (T)a.x, v[1] = (T)a.y, v[2] = (T)b.x, v[3] = (T)b.y;
         } else {
-            const int4 a = __ldg(static_cast<const int4 *>(col) + r / 4);
+            const int4 a = __ldcs(static_cast<const int4 *>(col) + r / 4);
             v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
         }
         return;
