@@ -36,6 +36,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Compile the translation units that changed (all of them with force) in parallel, then link."""
     extra = os.environ.get("SJQ_NVCC_EXTRA", "").split()  # e.g. -D switches for kernel experiments
     headers = _headers()
+    if not force and not extra and not _stale(LIB, sources() + headers):  # whatever became of the objects
+        _build_marshal(False)
+        return LIB
     todo = [s for s in sources() if force or extra or _stale(_object(s), [s] + headers)]
     if not todo and not _stale(LIB, [_object(s) for s in sources()]):
         _build_marshal(force)
