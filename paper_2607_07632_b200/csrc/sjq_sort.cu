@@ -13,7 +13,7 @@
 // is the number of kernels one after the other that counts.  Two ways, by the capacity of the list:
 //   - up to kSampleMost entries a sample sort, four kernels: splitters from a sorted sample; the bucket of every
 //     entry, counted; the entries into their buckets; every bucket sorted in shared memory (merge of eight lists of
-//     200,000 with its sort: 198 us with the radix sort, 75 with this one);
+//     200,000 with its sort: 200 us with the radix sort, 106 with this one);
 //   - beyond, a stable least-significant-digit radix sort of (key - smallest key, position) pairs, 8 bits a pass,
 //     two kernels each; passes that the range of the keys does not need return at once.  At most kSortBlocks blocks
 //     own one contiguous piece of the list each, so that the digit counts are few and every scatter block forms its
@@ -39,6 +39,9 @@ constexpr int kBuckets = 1024;      // at most; about 256 entries each in a shor
 constexpr int kOversample = 4;      // samples per bucket: the largest bucket is two to three times the average
 constexpr int kBucketThreads = 256;
 constexpr int kBucketRoom = 2048;   // entries of a bucket that shared memory holds
+constexpr int kBinBits = 11;        // bins of a bucket, as many as it may have entries
+constexpr int kBins = 1 << kBinBits;
+constexpr int kBinMost = 64;        // entries of a bin that are compared with one another
 
 struct SortRange {
     unsigned long long lo, hi; // smallest and largest key, sign bit flipped
@@ -460,6 +463,23 @@ __global__ void __launch_bounds__(kSortThreads) sample_scatter_kernel(const __gr
     }
 }
 
+// Smallest and largest key of a block's bucket.
+__device__ __forceinline__ void block_range(unsigned long long &kmin, unsigned long long &kmax, unsigned long long *least,
+                                            unsigned long long *most)
+{
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
+        kmin = x < kmin ? x : kmin;
+        kmax = y > kmax ? y : kmax;
+    }
+    if ((threadIdx.x & 31) == 0) least[threadIdx.x >> 5] = kmin, most[threadIdx.x >> 5] = kmax;
+    __syncthreads();
+    for (int w = 0; w < kBucketThreads / 32; ++w) {
+        kmin = least[w] < kmin ? least[w] : kmin;
+        kmax = most[w] > kmax ? most[w] : kmax;
+    }
+}
+
 // Sort R * kBucketThreads values by a bitonic network; value r * kBucketThreads + thread sits in v[r].  Partners in the
 // same thread or warp meet in registers, the others in shared memory.
 template <int R>
@@ -535,16 +555,112 @@ __device__ __forceinline__ bool order_bucket(const unsigned long long *key, int 
     return __syncthreads_or(same) == 0;
 }
 
-// Sort the buckets, a block each.  Where keys of a bucket are equal, or so far apart that the 53 bits do not tell them
-// apart, or a bucket is larger than shared memory (the sample would have to be very unlucky), its entries are ranked one
-// by one against the whole bucket.
-__global__ void __launch_bounds__(kBucketThreads) sample_bucket_kernel(const __grid_constant__ SortParams S)
+// A bucket's m entries by one more distribution: bins of equal width over the bucket's range, as many as shared memory
+// holds entries, so that most bins take one or none; an entry's place is its bin's start plus the smaller entries of its
+// bin.  Half a dozen barriers where the network has one pair per step (lists of 400,000 entries: merge and sort 127 us
+// with the network, 106 with the bins; three waves of the network's blocks took 43 of them).  Registers are kept to four
+// blocks per SM: with five, measures spill and it takes 112.  R > 0: m <= R * kBucketThreads, and a thread's
+// entries stay in registers, keys and measures requested before the first wait; R = 0: any m <= kBucketRoom, keys read
+// again (from the L1) in each pass.  False, with nothing written, when a bin takes more than kBinMost entries (keys
+// bunched within the bucket).
+template <int R>
+__device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo, int m, unsigned long long *key,
+                                           unsigned int *bin, unsigned int *pos, unsigned short *number,
+                                           unsigned long long *least, unsigned long long *most, unsigned int *warp_sum)
 {
-    __shared__ unsigned long long key[kBucketRoom], buf[kBucketRoom];
+    constexpr int kPerThread = kBins / kBucketThreads, kKept = R > 0 ? R : 1;
+    static_assert(kPerThread % 4 == 0, "whole 128-bit words");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned long long k[kKept], kmin = ~0ull, kmax = 0ull;
+    unsigned int p[kKept];
+    int64_t sum[kKept], count[kKept];
+    if (R > 0) {
+#pragma unroll
+        for (int r = 0; r < kKept; ++r) {
+            const int e = r * kBucketThreads + tid;
+            if (e < m) k[r] = S.k[1][lo + e], p[r] = S.p[1][lo + e];
+        }
+#pragma unroll
+        for (int r = 0; r < kKept; ++r)
+            if (r * kBucketThreads + tid < m) sum[r] = S.tsums[p[r]], count[r] = S.tcounts[p[r]];
+    }
+    auto entries = [&](auto &&f) { // f(slot, entry, its key) for every entry of this thread
+        if (R > 0) {
+#pragma unroll
+            for (int r = 0; r < kKept; ++r)
+                if (r * kBucketThreads + tid < m) f(r, r * kBucketThreads + tid, k[r]);
+        } else {
+#pragma unroll 1
+            for (int e = tid; e < m; e += kBucketThreads) f(0, e, S.k[1][lo + e]);
+        }
+    };
+    uint4 *words = reinterpret_cast<uint4 *>(bin) + tid * (kPerThread / 4);
+#pragma unroll
+    for (int q = 0; q < kPerThread / 4; ++q) words[q] = make_uint4(0u, 0u, 0u, 0u);
+    entries([&](int, int, unsigned long long x) {
+        kmin = x < kmin ? x : kmin;
+        kmax = x > kmax ? x : kmax;
+    });
+    block_range(kmin, kmax, least, most);
+    const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > kBinBits ? bits - kBinBits : 0;
+    entries([&](int, int e, unsigned long long x) {
+        number[e] = (unsigned short)atomicAdd(&bin[(x - kmin) >> shift], 1u);
+    });
+    __syncthreads();
+    unsigned int mine = 0, largest = 0;
+#pragma unroll
+    for (int q = 0; q < kPerThread / 4; ++q) {
+        const uint4 w = words[q];
+        mine += w.x + w.y + w.z + w.w;
+        largest = max(max(max(largest, w.x), max(w.y, w.z)), w.w);
+    }
+    unsigned int first = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int u = __shfl_up_sync(0xffffffffu, first, o);
+        if (lane >= o) first += u;
+    }
+    if (lane == 31) warp_sum[warp] = first;
+    if (__syncthreads_or(largest > (unsigned int)kBinMost)) return false;
+    first -= mine;
+    for (int w = 0; w < warp; ++w) first += warp_sum[w];
+#pragma unroll
+    for (int q = 0; q < kPerThread / 4; ++q) {
+        const uint4 w = words[q];
+        words[q] = make_uint4(first, first + w.x, first + w.x + w.y, first + w.x + w.y + w.z);
+        first += w.x + w.y + w.z + w.w;
+    }
+    __syncthreads();
+    entries([&](int r, int e, unsigned long long x) {
+        const unsigned int i = bin[(x - kmin) >> shift] + number[e];
+        key[i] = x;
+        pos[i] = R > 0 ? p[r] : S.p[1][lo + e];
+    });
+    __syncthreads();
+    entries([&](int r, int e, unsigned long long x) {
+        const unsigned int d = (unsigned int)((x - kmin) >> shift), i0 = bin[d];
+        const unsigned int i1 = d + 1 < (unsigned int)kBins ? bin[d + 1] : (unsigned int)m;
+        const unsigned int from = R > 0 ? p[r] : pos[i0 + number[e]];
+        unsigned int place = lo + i0;
+        for (unsigned int i = i0; i < i1; ++i) place += (key[i] < x) | ((key[i] == x) & (pos[i] < from));
+        S.keys[place] = (int64_t)(x ^ 0x8000000000000000ull);
+        S.sums[place] = R > 0 ? sum[r] : S.tsums[from];
+        S.counts[place] = R > 0 ? count[r] : S.tcounts[from];
+    });
+    return true;
+}
+
+// Sort the buckets, a block each: by bins, or by the network where the keys are bunched.  Where bunched keys are equal,
+// or so far apart that the 53 bits do not tell them apart, or a bucket is larger than shared memory (the sample would
+// have to be very unlucky), its entries are ranked one by one against the whole bucket.
+__global__ void __launch_bounds__(kBucketThreads, 4) sample_bucket_kernel(const __grid_constant__ SortParams S)
+{
+    __shared__ __align__(16) unsigned long long key[kBucketRoom], buf[kBucketRoom];
     __shared__ unsigned short order[kBucketRoom];
-    __shared__ unsigned int start[kBuckets], warp_sum[kBuckets / 128];
+    __shared__ unsigned int start[kBuckets], warp_sum[kBucketThreads / 32];
     __shared__ unsigned long long least[kBucketThreads / 32], most[kBucketThreads / 32];
     static_assert(kBucketThreads == kBuckets / 4, "bucket_starts takes so many threads");
+    static_assert(8 * (size_t)kBucketRoom >= 4 * (size_t)(kBins + kBucketRoom),
+                  "bins and positions fit beside the keys");
     cudaGridDependencySynchronize();
     if (list_in_order(S)) return;
     const int nb = buckets_for(sort_count(S));
@@ -556,9 +672,17 @@ __global__ void __launch_bounds__(kBucketThreads) sample_bucket_kernel(const __g
     };
     for (int b = blockIdx.x; b < nb; b += gridDim.x) {
         const unsigned int lo = start[b], m = S.bucket_total[b];
-        bool done = m == 0;
-        if (m > 0 && m <= (unsigned int)kBucketRoom) {
-            __syncthreads(); // the bucket before has been written out
+        if (m == 0) continue;
+        bool done = false;
+        unsigned int *const bin = reinterpret_cast<unsigned int *>(buf), *const pos = bin + kBins;
+        __syncthreads(); // the bucket before has been written out
+        if (m <= kBucketThreads) done = bin_bucket<1>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
+        else if (m <= 2 * kBucketThreads) done = bin_bucket<2>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
+        else if (m <= (unsigned int)kBucketRoom)
+            done = bin_bucket<0>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
+        if (done) continue;
+        if (m <= (unsigned int)kBucketRoom) {
+            __syncthreads(); // the bins have been read
             unsigned long long kmin = ~0ull, kmax = 0ull;
             for (int e = threadIdx.x; e < (int)m; e += kBucketThreads) {
                 const unsigned long long k = S.k[1][lo + e];
@@ -566,17 +690,7 @@ __global__ void __launch_bounds__(kBucketThreads) sample_bucket_kernel(const __g
                 kmin = k < kmin ? k : kmin;
                 kmax = k > kmax ? k : kmax;
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
-                kmin = x < kmin ? x : kmin;
-                kmax = y > kmax ? y : kmax;
-            }
-            if ((threadIdx.x & 31) == 0) least[threadIdx.x >> 5] = kmin, most[threadIdx.x >> 5] = kmax;
-            __syncthreads();
-            for (int w = 0; w < kBucketThreads / 32; ++w) {
-                kmin = least[w] < kmin ? least[w] : kmin;
-                kmax = most[w] > kmax ? most[w] : kmax;
-            }
+            block_range(kmin, kmax, least, most);
             // (all ones in the top 53 bits would meet the padding: 2^53 - 1 is the most a distance may reach, exclusive)
             const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > 52 ? bits - 52 : 0;
             if (m <= kBucketThreads) done = order_bucket<1>(key, (int)m, kmin, shift, buf, order);

@@ -76,3 +76,26 @@ def test_list_in_order_and_list_of_equal_keys_stay_as_they_are():
     swapped = np.arange(60_000, dtype=np.int64)
     swapped[[2047, 2048]] = swapped[[2048, 2047]]  # out of order only across a piece's edge
     _check(swapped, 60_000)
+
+
+@pytest.mark.parametrize("n", [200, 264, 265, 500, 520, 528, 529, 1500, 2112, 2113])
+@pytest.mark.parametrize("bunch", [1, 64, 65, 66])
+def test_one_bucket_of_spread_and_of_bunched_keys(n, bunch):
+    # the sampled positions hold the smallest keys, so nearly all others share the last bucket: 256, 257, 512, 513 and
+    # 2048, 2049 entries among the sizes; `bunch` neighbours lie in one bin of the bucket's range
+    rng = np.random.default_rng(n + bunch)
+    nb = 1
+    while nb < 1024 and nb * 256 < n:
+        nb *= 2
+    keys = (rng.permutation(n).astype(np.int64) + 10**6) << 40
+    bunched = rng.choice(n, bunch, replace=False)
+    keys[bunched] = (np.int64(2**62)) + rng.permutation(bunch)
+    keys[bunched[: bunch // 8]] = 2**62 + 3  # equal ones keep their order
+    for i in range(4 * nb if nb > 1 else 0):
+        lo, hi = i * n // (4 * nb), (i + 1) * n // (4 * nb)
+        h = (i * 2654435761 + 0x9E3779B9) & 0xFFFFFFFF
+        h ^= h >> 15
+        h = (h * 2246822519) & 0xFFFFFFFF
+        h ^= h >> 13
+        keys[lo + h % (hi - lo)] = i
+    _check(keys, n + 1)
