@@ -53,7 +53,7 @@ def test_capacity_is_a_limit_in_both_forms():
             assert res.status() == 19
 
 
-@pytest.mark.parametrize("n", [1, 31, 33, 100_003])
+@pytest.mark.parametrize("n", [1, 31, 33, 100_003, 303_103, 303_105, 1_000_003])
 def test_merge_adds_zero_and_wrapping_entries(n):
     rng = np.random.default_rng(n)
     keys = rng.integers(-5, max(6, n // 3), n)
