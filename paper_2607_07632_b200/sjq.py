@@ -539,6 +539,8 @@ def _build_batch(builders: list) -> list:
         with torch.cuda.device(lead.device):
             lead.batch_scratch = torch.empty(n * PLAN_SCRATCH_BYTES, dtype=torch.uint8, device=lead.device)
         lead.scan_side.wait_stream(torch.cuda.current_stream(lead.device))
+        # scans of earlier batches may still be adding to it when a larger batch replaces it (or the builder goes)
+        lead.batch_scratch.record_stream(lead.scan_side)
     descs = (_DimDesc * n)(*[b.desc for b in builders])
     slots = [b._next_stats() for b in builders]
     rc = L.sjq_dims_plan_begin(descs, n, lead.batch_scratch.data_ptr(), lead.batch_scratch.numel(),

@@ -147,3 +147,26 @@ def test_builders_alone_and_in_changing_batches(reuse):
         res, exp, _ = run_both(w, fact, host, tables=tables)
         assert res.status() == 0 and all(t.status() == 0 for t in tables.values())
         compare(w, res, exp)
+
+
+def test_scratch_of_a_batch_that_grows_is_not_handed_out_while_a_scan_uses_it():
+    """With reuse_layout nothing waits for a scan: when a larger batch replaces its lead's scratch, the allocator may not
+    give the old block to somebody else before the scans queued on it have run."""
+    rng = np.random.default_rng(12)
+    dims = {d: to_dev({"k": rng.permutation(n).astype(np.int32), "p": rng.integers(0, 9, n).astype(np.int32)})
+            for d, n in (("a", 4_000), ("b", 700), ("c", 900))}
+    b = {d: sjq.TableBuilder(c, "k", (), ("p",), reuse_layout=True) for d, c in dims.items()}
+    for d in b:
+        sjq.build_tables({d: b[d]})
+    torch.cuda.synchronize()
+    lead, small = b["a"], b["a"].batch_scratch.data_ptr()
+    with torch.cuda.stream(lead.scan_side):
+        torch.cuda._sleep(400_000_000)  # the scan queued next stays pending for a fifth of a second
+    sjq.build_tables({"a": b["a"]})
+    tables = sjq.build_tables(b)
+    assert lead.batch_scratch.data_ptr() != small
+    taken = [torch.empty(sjq.sjq.PLAN_SCRATCH_BYTES, dtype=torch.uint8, device="cuda") for _ in range(64)]
+    assert not lead.stats_done[lead.scan].query()  # ... and is pending still
+    assert small not in [t.data_ptr() for t in taken]
+    torch.cuda.synchronize()
+    assert all(t.status() == 0 for t in tables.values())
