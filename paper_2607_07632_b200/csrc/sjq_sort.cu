@@ -34,11 +34,17 @@ constexpr int kSortBlocks = 148;                       // one per SM
 constexpr int kSortMinPiece = 2048;                    // elements a block takes before another one is put to work
 constexpr int kSortPasses = 8;
 
-constexpr int64_t kSampleMost = (int64_t)1 << 20;
 constexpr int kBuckets = 1024;      // at most; about 256 entries each in a shorter list
-constexpr int kOversample = 4;      // samples per bucket: the largest bucket is two to three times the average
+constexpr int kOversample = 4;      // samples per bucket
 constexpr int kBucketThreads = 256;
 constexpr int kBucketRoom = 2048;   // entries of a bucket that shared memory holds
+// The longest list: a bucket larger than the room is ranked entry by entry (a list of a million had forty of them and
+// took 2.3 ms; the radix sort takes 0.25), so it must be rare.  Bucket sizes depend on the ranks of the sampled entries
+// alone, not on how the keys are spread, and a bucket of four samples exceeds x times the average with the tail of a
+// gamma distribution of order four: where the average is a fifth of the room, one list in 300 has such a bucket; at half
+// the room, every list.  Six samples a bucket would do at a quarter of the room, but ranking them costs every list beyond
+// 131,072 entries 12 us (merge of eight lists of 200,000 with its sort 108 -> 120).
+constexpr int64_t kSampleMost = (int64_t)kBuckets * (kBucketRoom / 5);
 constexpr int kBinBits = 11;        // bins of a bucket, as many as it may have entries
 constexpr int kBins = 1 << kBinBits;
 constexpr int kBinMost = 64;        // entries of a bin that are compared with one another
@@ -321,7 +327,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const __grid
 }
 
 // ------------------------------------------------------------------ sample sort
-__device__ __forceinline__ int buckets_for(int64_t n)
+__host__ __device__ __forceinline__ int buckets_for(int64_t n)
 {
     int nb = 1;
     while (nb < kBuckets && (int64_t)nb * 256 < n) nb <<= 1;
@@ -330,7 +336,7 @@ __device__ __forceinline__ int buckets_for(int64_t n)
 
 // Position of sample i of s in a list of n: anywhere in the i-th of s equal parts, so that no regular pattern in the
 // list meets the samples; samples ascend in position.
-__device__ __forceinline__ int64_t sample_at(int i, int s, int64_t n)
+__host__ __device__ __forceinline__ int64_t sample_at(int i, int s, int64_t n)
 {
     const int64_t lo = (int64_t)i * n / s, hi = (int64_t)(i + 1) * n / s;
     unsigned int h = (unsigned int)i * 2654435761u + 0x9E3779B9u;
@@ -650,8 +656,8 @@ __device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo,
 }
 
 // Sort the buckets, a block each: by bins, or by the network where the keys are bunched.  Where bunched keys are equal,
-// or so far apart that the 53 bits do not tell them apart, or a bucket is larger than shared memory (the sample would
-// have to be very unlucky), its entries are ranked one by one against the whole bucket.
+// or so far apart that the 53 bits do not tell them apart, or a bucket is larger than shared memory (an unlucky sample,
+// see kSampleMost), its entries are ranked one by one against the whole bucket.
 __global__ void __launch_bounds__(kBucketThreads, 4) sample_bucket_kernel(const __grid_constant__ SortParams S)
 {
     __shared__ __align__(16) unsigned long long key[kBucketRoom], buf[kBucketRoom];
@@ -831,4 +837,17 @@ extern "C" sjq_status sjq_result_sort(int64_t *keys, int64_t *sums, int64_t *cou
         return SJQ_ERR_CUDA;
     }
     return SJQ_OK;
+}
+
+// The sampler as the kernels use it, for tests on the host (not part of the interface): the positions sampled in a list
+// of n entries (`positions` NULL: none are written); returns their number.
+extern "C" int32_t sjq_result_sort_samples(int64_t n, int64_t *positions, int32_t *per_bucket, int32_t *room,
+                                           int64_t *most)
+{
+    const int nb = buckets_for(n), ns = nb > 1 ? nb * kOversample : 0;
+    for (int i = 0; positions && i < ns; ++i) positions[i] = sample_at(i, ns, n);
+    *per_bucket = kOversample;
+    *room = kBucketRoom;
+    *most = kSampleMost;
+    return ns;
 }

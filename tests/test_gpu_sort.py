@@ -1,10 +1,12 @@
-"""Canonical order of hashed results at the sizes and key ranges where the radix sort takes another path: one tile,
-one more, the most pieces, every number of digit passes, equal keys, lists in order already."""
+"""Canonical order of hashed results at the sizes and key ranges where the sample sort and the radix sort take another
+path: one tile, one more, the most pieces, every number of digit passes, equal keys, lists in order already, buckets
+beyond shared memory and bins of bunched keys."""
 import numpy as np
 import pytest
 import torch
 
 import paper_2607_07632_b200 as sjq
+from sorthelpers import bucket_sizes, samples
 
 pytestmark = pytest.mark.gpu
 
@@ -56,17 +58,9 @@ def test_buckets_larger_than_shared_memory_are_ranked():
     # the sampled positions hold small keys only: all other entries fall into one bucket
     n = 40_000
     keys = np.random.default_rng(1).permutation(n).astype(np.int64) + 10**6
-    nb = 1
-    while nb < 1024 and nb * 256 < n:
-        nb *= 2
-    s = 4 * nb
-    for i in range(s):
-        lo, hi = i * n // s, (i + 1) * n // s
-        h = (i * 2654435761 + 0x9E3779B9) & 0xFFFFFFFF
-        h ^= h >> 15
-        h = (h * 2246822519) & 0xFFFFFFFF
-        h ^= h >> 13
-        keys[lo + h % (hi - lo)] = i
+    at, _, room, _ = samples(n)
+    keys[at] = np.arange(len(at))
+    assert bucket_sizes(keys).max() > 10 * room
     _check(keys, n)
 
 
@@ -78,24 +72,25 @@ def test_list_in_order_and_list_of_equal_keys_stay_as_they_are():
     _check(swapped, 60_000)
 
 
-@pytest.mark.parametrize("n", [200, 264, 265, 500, 520, 528, 529, 1500, 2112, 2113])
+@pytest.mark.parametrize("last", [200, 256, 257, 496, 512, 513, 1500, 2048, 2049])
 @pytest.mark.parametrize("bunch", [1, 64, 65, 66])
-def test_one_bucket_of_spread_and_of_bunched_keys(n, bunch):
-    # the sampled positions hold the smallest keys, so nearly all others share the last bucket: 256, 257, 512, 513 and
-    # 2048, 2049 entries among the sizes; `bunch` neighbours lie in one bin of the bucket's range
+def test_one_bucket_of_spread_and_of_bunched_keys(last, bunch):
+    # the sampled positions hold the smallest keys, so all others share the last bucket with the samples behind the last
+    # splitter: `last` entries in all; `bunch` neighbours lie in one bin of the bucket's range
+    n = next(n for n in range(last, 2 * last) if n - len(samples(n)[0]) + (samples(n)[1] if n > 256 else 0) == last)
     rng = np.random.default_rng(n + bunch)
-    nb = 1
-    while nb < 1024 and nb * 256 < n:
-        nb *= 2
     keys = (rng.permutation(n).astype(np.int64) + 10**6) << 40
     bunched = rng.choice(n, bunch, replace=False)
     keys[bunched] = (np.int64(2**62)) + rng.permutation(bunch)
     keys[bunched[: bunch // 8]] = 2**62 + 3  # equal ones keep their order
-    for i in range(4 * nb if nb > 1 else 0):
-        lo, hi = i * n // (4 * nb), (i + 1) * n // (4 * nb)
-        h = (i * 2654435761 + 0x9E3779B9) & 0xFFFFFFFF
-        h ^= h >> 15
-        h = (h * 2246822519) & 0xFFFFFFFF
-        h ^= h >> 13
-        keys[lo + h % (hi - lo)] = i
+    at, _, _, _ = samples(n)
+    keys[at] = np.arange(len(at))
+    assert bucket_sizes(keys)[-1] == last
     _check(keys, n + 1)
+
+
+@pytest.mark.parametrize("beyond", [-7, -6, 200_000, 600_000])
+def test_unordered_lists_on_both_sides_of_the_longest_sample_sort(beyond):
+    n = samples(1000)[3] + beyond
+    keys = np.random.default_rng(n).permutation(n).astype(np.int64) * 0x9E3779B97F4A7 - 2**40
+    _check(keys, n + 7)
