@@ -351,12 +351,21 @@ extern "C" sjq_status sjq_pred_sample(const sjq_col *fact, int nfact, const sjq_
     return sjq_pred_sample_end(h, npreds, pass_ppm);
 }
 
-// sjq_run.  `callers_order`: the order of the filters, if the options give one, is the caller's own and not one that
-// this library chose for a run from host memory.
+namespace {
+
+// What a run is part of: by default of nothing, its columns are in device memory and its options are the caller's.
+struct RunContext {
+    bool callers_order = true; // the order of the filters, if the options give one, is the caller's own and not one that
+                               // this library chose for a run from host memory
+    bool in_place = false;     // some columns are read in place from host memory
+};
+
+} // namespace
+
 static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *preds, int npreds,
                               const sjq_join *joins, int njoins, const sjq_key_expr *key, const sjq_agg_expr *agg,
                               const sjq_result_spec *spec, const sjq_result *out, const sjq_run_opts *opts_,
-                              bool callers_order, void *stream_, sjq_run_info *info)
+                              const RunContext &context, void *stream_, sjq_run_info *info)
 {
     // ------------------------------------------------------------ validation
     if (!fact || nfact <= 0 || nfact > 64 || npreds < 0 || npreds > SJQ_MAX_PREDS || (npreds && !preds) ||
@@ -552,8 +561,9 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     // Few rows: the kernel's time is a chain of memory latencies, one per queue level, and without queues it is one in
     // all (compiled, 400 thousand rows: city x city 12.5 -> 8.7 us, city x brand 14.6 -> 12.6, the others alike;
     // interpreted: four joins 16.6 -> 12.5, two joins 14.5 -> 10.5, filter and sum 12.5 -> 10.4; at 800 thousand rows
-    // some gain and some lose).
-    const bool few_rows = n <= (int64_t)1 << 19 && opts.compaction == 0;
+    // some gain and some lose).  Not where a column is read in place from host memory: a kernel without queues requests
+    // columns before it knows which rows need them, four rows at a time, and would bring most of it over the bus.
+    const bool few_rows = n <= (int64_t)1 << 19 && opts.compaction == 0 && !context.in_place;
     const bool direct = few_rows || opts.eager_loads || opts.compaction == 1 || nfilter == 0 || opts.unfused || mostly_survive;
     if (!direct) {
         nd0 = 1;
@@ -569,7 +579,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
             // 783 and 735).  The interpreting kernel loads its columns one after the other and is better off with
             // queues (four joins, 60 M rows: 175 us against 290 without any), and an order that the caller lays down
             // is carried out with a level for every filter.
-            const double queue_reach = opts.specialise && !(opts.norder && callers_order) ? 0.12 : 0.002;
+            const double queue_reach = opts.specialise && !(opts.norder && context.callers_order) ? 0.12 : 0.002;
             while (nd0 + nfq < nfilter && nfq < kMaxQueues - 1 && specs[order[nd0 + nfq]].sel < 0.9 &&
                    reach[nd0 + nfq] > queue_reach && specs[order[nd0 + nfq]].prefilter != 2)
                 ++nfq;
@@ -1051,7 +1061,7 @@ extern "C" sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *pr
                               const sjq_result_spec *spec, const sjq_result *out, const sjq_run_opts *opts,
                               void *stream, sjq_run_info *info)
 {
-    return run_planned(fact, nfact, preds, npreds, joins, njoins, key, agg, spec, out, opts, true, stream, info);
+    return run_planned(fact, nfact, preds, npreds, joins, njoins, key, agg, spec, out, opts, RunContext{}, stream, info);
 }
 
 // ---------------------------------------------------------------------------
@@ -1301,6 +1311,9 @@ extern "C" sjq_status sjq_run_host(const sjq_col *fact_host, int nfact, const sj
     std::vector<const char *> direct_base;
     std::vector<double> need_share;
     host_transfer_plan(fact_host, nfact, preds, npreds, joins, njoins, key, agg, &opts, &how, &direct_base, &need_share);
+    RunContext context;
+    context.callers_order = opts_ && opts_->norder != 0;
+    for (int c = 0; c < nfact; ++c) context.in_place |= how[c] == HOST_IN_PLACE;
 
     // internal streams start after whatever is already queued on the caller's stream
     if (cudaEventRecord(hp->start, stream) != cudaSuccess) return SJQ_ERR_CUDA;
@@ -1333,7 +1346,7 @@ extern "C" sjq_status sjq_run_host(const sjq_col *fact_host, int nfact, const sj
         opts.accumulate = (k > 0 || (opts_ && opts_->accumulate)) ? 1 : 0;
         opts.hot_keys = 2; // a chunk's foreign keys may still be in host memory: no sampling pass over them
         sjq_status st = run_planned(dev_cols.data(), nfact, preds, npreds, joins, njoins, key, agg, spec, out, &opts,
-                                    opts_ && opts_->norder != 0, hp->s[b], nullptr);
+                                    context, hp->s[b], nullptr);
         if (st != SJQ_OK) return st;
         if (cudaEventRecord(hp->done[b], hp->s[b]) != cudaSuccess) return SJQ_ERR_CUDA;
     }

@@ -1,4 +1,6 @@
 """The evaluation order the planner chooses, and parity where its search changes form."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -9,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 sjq = pytest.importorskip("paper_2607_07632_b200") if torch.cuda.is_available() else None
 
-from gpuhelpers import compare, run_both  # noqa: E402
+from gpuhelpers import compare, oracle_result, run_both  # noqa: E402
 from qhelpers import adhoc  # noqa: E402
 
 
@@ -106,3 +108,39 @@ def test_host_resident_filters_are_ordered_by_the_bus(n):
             torch.cuda.synchronize()
             assert int(out.status[0]) == 0
             compare(w, res, exp)
+
+
+def _modules():
+    """Compiled modules loaded since the last call; all are unloaded (nothing is running)."""
+    torch.cuda.synchronize()
+    lib = sjq.sjq.lib()
+    lib.sjq_jit_cache_clear.restype = ctypes.c_int32
+    return lib.sjq_jit_cache_clear()
+
+
+def _sparse_query(n):
+    """Of a thousand rows one passes both filters: q is read for a twentieth of the rows, m for one in a thousand."""
+    rng = np.random.default_rng(n)
+    fact = {c: rng.integers(0, 1000, n).astype(np.int32) for c in ("p", "q", "m")}
+    return fact, adhoc("sparse", fact, [], [], [Pred("p", "LT", 50), Pred("q", "LT", 20)], None,
+                       AggExpr("COL", Term("FACT", "m")), "SCALAR")
+
+
+@pytest.mark.parametrize("n", [100_003, 2**19])
+def test_few_rows_with_columns_in_place_are_queued_like_many(n):
+    """A kernel without queues would fetch columns in host memory for rows that need none of them: with such a column a
+    small table runs through the kernel that a large one does, with copies alone through one without queues."""
+    for copy_all, modules in ((False, 1), (True, 2)):
+        _modules()
+        for rows in (700_001, n):
+            fact, w = _sparse_query(rows)
+            pinned = {c: torch.from_numpy(v).pin_memory() for c, v in fact.items()}
+            opts = sjq.RunOpts(specialise=True, pass_ppm=(50_000, 20_000), host_copy_all=copy_all)
+            how = sjq.host_transfer_plan(pinned, w.preds, (), None, w.agg, opts)
+            assert how["m"][0] == ("copy" if copy_all else "in place")
+            staging = torch.empty(sjq.staging_bytes(pinned, 700_004), dtype=torch.uint8, device="cuda")
+            res, out = sjq.run_workload_host(w, pinned, {}, staging, 700_004, opts)
+            torch.cuda.synchronize()
+            assert int(out.status[0]) == 0
+            compare(w, res, oracle_result(w, fact, {})[1])
+        assert _modules() == modules
