@@ -358,6 +358,8 @@ struct RunContext {
     bool callers_order = true; // the order of the filters, if the options give one, is the caller's own and not one that
                                // this library chose for a run from host memory
     bool in_place = false;     // some columns are read in place from host memory
+    int64_t rows = -1;         // rows to plan for where they are not the call's own: a last chunk is planned as the others,
+                               // so that a compiled kernel is not compiled again for it
 };
 
 } // namespace
@@ -541,7 +543,8 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     // Fraction of rows reaching each filter stage, from the estimates.
     Short<double, kMaxFilters + 1> reach(nfilter + 1, 1.0);
     for (int s = 0; s < nfilter; ++s) reach[s + 1] = reach[s] * specs[order[s]].sel;
-    const double survivors = (double)n * reach[nfilter];
+    const int64_t plan_rows = context.rows >= 0 ? context.rows : n;
+    const double survivors = (double)plan_rows * reach[nfilter];
     // Level 0 runs, on thread-owned rows, the leading filter stages that still see a fair share of
     // the rows (a dense stage costs about the same per table row whatever survives, a queue-fed
     // level costs per surviving row, several times more: measured break-even between 20 % and 30 %).
@@ -563,7 +566,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     // interpreted: four joins 16.6 -> 12.5, two joins 14.5 -> 10.5, filter and sum 12.5 -> 10.4; at 800 thousand rows
     // some gain and some lose).  Not where a column is read in place from host memory: a kernel without queues requests
     // columns before it knows which rows need them, four rows at a time, and would bring most of it over the bus.
-    const bool few_rows = n <= (int64_t)1 << 19 && opts.compaction == 0 && !context.in_place;
+    const bool few_rows = plan_rows <= (int64_t)1 << 19 && opts.compaction == 0 && !context.in_place;
     const bool direct = few_rows || opts.eager_loads || opts.compaction == 1 || nfilter == 0 || opts.unfused || mostly_survive;
     if (!direct) {
         nd0 = 1;
@@ -767,7 +770,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         // rows, 2 to 4096 groups, skewed and uniform: from 0.35 rows per cell on it is never slower and soon several
         // times faster, since the global cells serialise (0.34: 18.3 against 18.3 us; 1.1: 20.6 against 12.3; 5: 240
         // against 144; 100: 3,600 against 51); at 0.1 to 0.2 the two are within 5 %, below that up to 9 us slower.
-        const double blocks = std::min((double)approx_grid, std::max(1.0, (double)n / (SJQ_LB_THREADS * 4 * P.slots)));
+        const double blocks = std::min((double)approx_grid, std::max(1.0, (double)plan_rows / (SJQ_LB_THREADS * 4 * P.slots)));
         const bool contended = survivors >= 0.35 * blocks * (double)table_groups;
         if (opts.unfused) {
             aggp = AGG_GLOBAL;
@@ -874,7 +877,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
                 if (opts.smem_tables == 0 && tb > kStageBytes) continue;
                 if (opts.smem_tables >= 1024 && tb > (size_t)opts.smem_tables) continue; // experiment: size limit in bytes
                 // worth it only if a block probes the table more often than it costs to copy
-                const double probes_per_cta = (double)n * reach[s] / approx_grid;
+                const double probes_per_cta = (double)plan_rows * reach[s] / approx_grid;
                 if (probes_per_cta * 4.0 < (double)tb) continue;
                 S.in_smem = 1;
                 S.smem_off = (uint32_t)(stage_bytes + tables);
@@ -904,7 +907,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     bool single_block = false, two_wide_queue_blocks = false;
     if (opts.specialise && !opts.block_threads && !opts.ctas_per_sm && P.nq && !opts.unfused) {
         const size_t copies = tables + hot_bytes + group_bytes, as384 = stage_bytes + copies + queue_bytes(block);
-        const int64_t tiles_per_block = n / ((int64_t)1024 * 4 * P.slots) / dev.sm_count;
+        const int64_t tiles_per_block = plan_rows / ((int64_t)1024 * 4 * P.slots) / dev.sm_count;
         size_t other = 0;
         if ((copies >= ((size_t)16 << 10) || as384 > ((size_t)80 << 10)) && tiles_per_block >= 16 && stage_tables(1024, &other)) {
             block = 1024;
@@ -1314,6 +1317,7 @@ extern "C" sjq_status sjq_run_host(const sjq_col *fact_host, int nfact, const sj
     RunContext context;
     context.callers_order = opts_ && opts_->norder != 0;
     for (int c = 0; c < nfact; ++c) context.in_place |= how[c] == HOST_IN_PLACE;
+    context.rows = std::min(n, chunk_rows);
 
     // internal streams start after whatever is already queued on the caller's stream
     if (cudaEventRecord(hp->start, stream) != cudaSuccess) return SJQ_ERR_CUDA;

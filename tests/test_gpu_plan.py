@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 sjq = pytest.importorskip("paper_2607_07632_b200") if torch.cuda.is_available() else None
 
-from gpuhelpers import compare, oracle_result, run_both  # noqa: E402
+from gpuhelpers import compare, oracle_result, run_both, to_dev  # noqa: E402
 from qhelpers import adhoc  # noqa: E402
 
 
@@ -144,3 +144,26 @@ def test_few_rows_with_columns_in_place_are_queued_like_many(n):
             assert int(out.status[0]) == 0
             compare(w, res, oracle_result(w, fact, {})[1])
         assert _modules() == modules
+
+
+@pytest.mark.parametrize("tail", [4, 50_003, 2**19])
+def test_a_short_last_chunk_runs_through_the_kernel_of_the_others(tail):
+    """One module for a whole run from host memory: groups, a staged table and columns copied or read in place."""
+    chunk = 2**20
+    rng = np.random.default_rng(tail)
+    dim = {"k": np.arange(3_000, dtype=np.int32), "a": rng.integers(0, 100, 3_000).astype(np.int32)}
+    fact, w = _sparse_query(2 * chunk + tail)
+    fact["fk"] = rng.integers(0, 3_000, len(fact["p"])).astype(np.int32)
+    w = adhoc("tail", fact, [("d", dim, "k", [], ["a"])], [("fk", "d")], w.preds, KeyExpr((Term("PAYLOAD", 0, 0),)),
+              AggExpr("COL", Term("FACT", "m")), "DENSE", num_groups=100)
+    tables = sjq.build_workload_tables(w, {"d": to_dev(dim)})
+    pinned = {c: torch.from_numpy(v).pin_memory() for c, v in fact.items()}
+    staging = torch.empty(sjq.staging_bytes(pinned, chunk), dtype=torch.uint8, device="cuda")
+    exp = oracle_result(w, fact, {"d": dim})[1]
+    for opts in (sjq.RunOpts(specialise=True), sjq.RunOpts(specialise=True, host_copy_all=True)):
+        _modules()
+        res, out = sjq.run_workload_host(w, pinned, tables, staging, chunk, opts)
+        torch.cuda.synchronize()
+        assert int(out.status[0]) == 0
+        compare(w, res, exp)
+        assert _modules() == 1
