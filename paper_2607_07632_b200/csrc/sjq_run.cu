@@ -566,7 +566,9 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     // interpreted: four joins 16.6 -> 12.5, two joins 14.5 -> 10.5, filter and sum 12.5 -> 10.4; at 800 thousand rows
     // some gain and some lose).  Not where a column is read in place from host memory: a kernel without queues requests
     // columns before it knows which rows need them, four rows at a time, and would bring most of it over the bus.
-    const bool few_rows = plan_rows <= (int64_t)1 << 19 && opts.compaction == 0 && !context.in_place;
+    // Nor where the caller sets an option that only a kernel with queues can carry out.
+    const bool asks_for_queues = opts.rows_per_lane || opts.dense_slots || opts.l0_bulk == 1 || opts.l0_bulk == 3;
+    const bool few_rows = plan_rows <= (int64_t)1 << 19 && opts.compaction == 0 && !context.in_place && !asks_for_queues;
     const bool direct = few_rows || opts.eager_loads || opts.compaction == 1 || nfilter == 0 || opts.unfused || mostly_survive;
     if (!direct) {
         nd0 = 1;
@@ -580,8 +582,8 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
             // joins, the third filter reached by 6 % of the rows, 1286 us with a queue for it and 1223 without, but
             // 1295 without one for the second, reached by 20 %; filter and sum, 4 %: 1280 and 1109; two joins, 4 %:
             // 783 and 735).  The interpreting kernel loads its columns one after the other and is better off with
-            // queues (four joins, 60 M rows: 175 us against 290 without any), and an order that the caller lays down
-            // is carried out with a level for every filter.
+            // queues (four joins, 60 M rows: 175 us against 290 without any), and beyond the few rows above an order
+            // that the caller lays down is carried out with a level for every filter.
             const double queue_reach = opts.specialise && !(opts.norder && context.callers_order) ? 0.12 : 0.002;
             while (nd0 + nfq < nfilter && nfq < kMaxQueues - 1 && specs[order[nd0 + nfq]].sel < 0.9 &&
                    reach[nd0 + nfq] > queue_reach && specs[order[nd0 + nfq]].prefilter != 2)

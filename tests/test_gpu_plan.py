@@ -167,3 +167,19 @@ def test_a_short_last_chunk_runs_through_the_kernel_of_the_others(tail):
         assert int(out.status[0]) == 0
         compare(w, res, exp)
         assert _modules() == 1
+
+
+@pytest.mark.parametrize("n", [20_011, 2**19])
+def test_options_for_queues_hold_for_few_rows_too(n):
+    """A kernel without queues has no batches of survivors, no level 0 and no staged first column."""
+    fact, w = _sparse_query(n)
+    for kw, status in ((dict(rows_per_lane=4), 0), (dict(rows_per_lane=8, specialise=True), 0),
+                       (dict(dense_slots=4, specialise=True), 0), (dict(l0_bulk=1, specialise=True), 0),
+                       (dict(l0_bulk=3, specialise=True, block_threads=128, ctas_per_sm=1), 22)):
+        res, exp, _ = run_both(w, fact, {}, opts=sjq.RunOpts(**kw))
+        assert res.info.reserved_levels > 0
+        assert res.status() == status
+        compare(w, res, exp)
+    res, exp, _ = run_both(w, fact, {}, opts=sjq.RunOpts(dense_slots=2, rows_per_lane=4, l0_bulk=2, compaction=1))
+    assert res.info.reserved_levels == 0
+    compare(w, res, exp)
