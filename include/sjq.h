@@ -274,8 +274,8 @@ sjq_status sjq_dim_layout_bytes(const sjq_dim_layout *layout, size_t *bytes);
  * whether the probed structure stays in L1 / L2 (Section 3.3: the packed map is sized to stay cache-resident). */
 sjq_status sjq_table_info(const sjq_table *table, sjq_dim_layout *layout);
 
-/* Kernels sjq_build_dim enqueued for this table: one that prepares the memory and the build unless the dimension is
- * empty.  (sjq_dims_build counts those of a batch with its first table.) */
+/* Kernels sjq_build_dim enqueued for this table: one that prepares the memory and the build, the latter unless the
+ * dimension is empty (and its layout promises no keys).  (sjq_dims_build counts those of a batch with its first table.) */
 int32_t sjq_table_kernel_launches(const sjq_table *table);
 
 /* Frees the host handle only (the device memory belongs to the caller). */

@@ -1195,8 +1195,10 @@ sjq_status build_launch(const sjq_dim_desc *dims, int ndims, const sjq_dim_layou
         BuildTask &task = to.task[to.ntasks];
         st = describe_build(dims[i], layouts[i], table_mem[i], table_bytes[i], status_dev[i], &task, &B.filters,
                             &nfilters, &I, tables[i]);
+        if (st != SJQ_OK) break;
         if (clear_status) I.clear_status[i] = status_dev[i];
-        if (task.rows.n > 0) ++to.ntasks;
+        // (a layout that promises every key of its range is checked against a dimension without rows too)
+        if (task.rows.n > 0 || task.expect_full >= 0) ++to.ntasks;
     }
     DeviceInfo dev;
     if (st == SJQ_OK) st = device_info(&dev);

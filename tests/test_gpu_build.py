@@ -112,6 +112,22 @@ def test_empty_dimension_in_a_batch():
     assert [t.layout.entries for t in tables] == [0, 9, 0] and all(t.status() == 0 for t in tables)
 
 
+@pytest.mark.parametrize("bits,kind", [(2, 9), (4, 8)])
+@pytest.mark.parametrize("rows", [0, 1, 5])
+def test_a_layout_that_promises_every_key_is_checked_against_any_number_of_rows(bits, kind, rows):
+    """Probes of such a table trust the range test alone: keys that are missing would be hits."""
+    def promise(L):
+        L.kind, L.code_bits, L.npayload = kind, bits, 1
+        L.entries, L.kmin, L.kmax, L.slots, L.filter_bits = 6, 0, 5, 6, 128
+        L.pay_min[0], L.pay_max[0], L.pay_bits[0] = 0, 2, 2
+        L.table_bytes = sjq.layout_bytes(L)
+
+    cols = {"k": np.arange(rows, dtype=np.int32), "p": np.ones(rows, np.int32)}
+    assert sjq.build_dim(to_dev(cols), "k", (), ("p",), edit_layout=promise).status() == 21
+    cols = {"k": np.arange(6, dtype=np.int32), "p": np.ones(6, np.int32)}
+    assert sjq.build_dim(to_dev(cols), "k", (), ("p",), edit_layout=promise).status() == 0
+
+
 @pytest.mark.parametrize("reuse", [False, True])
 def test_builders_alone_and_in_changing_batches(reuse):
     """The same builders in batches of different make-up, alone, and with their columns refreshed on another stream."""
