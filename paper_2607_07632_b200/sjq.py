@@ -310,7 +310,6 @@ class Table:
 
     def __init__(self, handle: int, layout: DimLayout, mem: torch.Tensor, status: torch.Tensor):
         self.handle, self.layout, self.mem, self.status_dev = handle, layout, mem, status
-        self.scans = 1  # scan kernels enqueued for it (a batch's scan counts with its first table)
 
     def status(self) -> int:
         return int(self.status_dev.item())
@@ -380,15 +379,8 @@ def _build_tables(dims, edit_layout=None, mem_offset: int = 0) -> list:
         rc = L.sjq_dims_build(descs, n, layouts, ptrs, sizes, status_ptrs, 1, stream, handles)
         if rc != 0:
             raise SjqError(rc, "sjq_build_dim")
-    return _batch_tables(Table(handles[i], DimLayout.from_buffer_copy(layouts[i]),
-                               mem[at[i] + mem_offset:at[i] + mem_offset + sizes[i]], status[i:i + 1]) for i in range(n))
-
-
-def _batch_tables(tables) -> list:
-    tables = list(tables)
-    for i, t in enumerate(tables):
-        t.scans = int(i % 8 == 0)  # eight dimensions to a launch
-    return tables
+    return [Table(handles[i], DimLayout.from_buffer_copy(layouts[i]),
+                  mem[at[i] + mem_offset:at[i] + mem_offset + sizes[i]], status[i:i + 1]) for i in range(n)]
 
 
 class TableBuilder:
@@ -560,8 +552,7 @@ def _build_batch(builders: list) -> list:
                           (vp * n)(*[b.status.data_ptr() for b in builders]), 0, lead.side.cuda_stream, handles)
     if rc != 0:
         raise SjqError(rc, "sjq_dims_build")
-    return _batch_tables(Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], builders[i].status)
-                         for i in range(n))
+    return [Table(handles[i], DimLayout.from_buffer_copy(layouts[i]), mems[i], builders[i].status) for i in range(n)]
 
 
 def workload_builders(w, dims: dict, reuse_layout: bool = False) -> dict:
@@ -953,12 +944,14 @@ def jit_log() -> str:
 
 
 def build_launches(table: "Table") -> int:
-    """Kernels enqueued to plan and build this table: the scan and what the build reports (those of a batch count
-    with its first table)."""
+    """Kernels enqueued to plan and build this table: what the build reports and the scan.  Those of a batch count with
+    its first table: the library splits the scans of several dimensions into the launches that it splits their builds
+    into, and reports none for the other tables."""
     L = lib()
     L.sjq_table_kernel_launches.restype = ctypes.c_int32
     L.sjq_table_kernel_launches.argtypes = [ctypes.c_void_p]
-    return table.scans + int(L.sjq_table_kernel_launches(table.handle))
+    builds = int(L.sjq_table_kernel_launches(table.handle))
+    return builds + (builds > 0)
 
 
 def release() -> int:

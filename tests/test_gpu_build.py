@@ -105,6 +105,22 @@ def test_more_dimensions_and_filters_than_one_launch_takes():
             assert (list(a) == list(b)) if hasattr(a, "__len__") else a == b
 
 
+def test_launches_of_a_batch_split_by_its_filters_are_all_counted():
+    """At most eight dimensions and sixteen filters a launch: 1 + ... + 5, 6 + 7 and 8 filters are three scans and three
+    fills; the first tables' builds are one launch for direct tables, one for open addressing."""
+    dims = []
+    for j in range(8):
+        cols = {"k": torch.arange(100, dtype=torch.int32, device="cuda")}
+        dims.append((cols, "k", [Pred("k", "GE", 1)] * (j + 1), (),
+                     sjq.sjq._BuildOpts(sjq.sjq.FORCE_HASH if j in (1, 7) else 0)))
+    tables = sjq.sjq._build_tables(dims)
+    assert [sjq.build_launches(t) for t in tables] == [4, 0, 0, 0, 0, 3, 0, 3]
+    assert sjq.build_launches(sjq.build_dim(dims[0][0], "k")) == 3
+    builder = sjq.TableBuilder(dims[0][0], "k")
+    assert sjq.build_launches(sjq.build_tables({"d": builder})["d"]) == 3
+    torch.cuda.synchronize()
+
+
 def test_empty_dimension_in_a_batch():
     empty = {"k": np.zeros(0, np.int32), "p": np.zeros(0, np.int32)}
     full = {"k": np.arange(9, dtype=np.int32), "p": np.arange(9, dtype=np.int32)}
