@@ -608,8 +608,9 @@ const char *sjq_version(void);
 /*
  * Give back what the library holds on behalf of the calling thread and the
  * process: the two internal streams and three events sjq_run_host creates per
- * device and thread on first use, the modules compiled at run time, and the
- * remembered occupancy answers.  Nothing the library enqueued may still be
+ * device and thread on first use, the page-locked words (512 bytes a piece, at
+ * most eight kept) that waiting plans read statistics back through, the
+ * modules compiled at run time, and the remembered occupancy answers.  Nothing the library enqueued may still be
  * running.  Later calls create what they need again.  Returns the number of
  * objects released.  (Host-side bookkeeping only; the paper has no counterpart.)
  */

@@ -7,6 +7,7 @@
 // to an open-addressing table populated with atomicCAS.  Section 4.3.1: the
 // key range is verified at run time and the packed or unpacked form chosen.
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <utility>
@@ -801,11 +802,45 @@ sjq_status scan_launch(const sjq_dim_desc *dims, int ndims, unsigned long long *
     return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 
-// Page-locked memory of this thread for the statistics that a waiting plan reads back.
+// Page-locked words for the statistics that a waiting plan reads back: a plan has a piece for as long as it waits, and
+// the process keeps up to kKeptStats of them, so that threads that come and go leave none behind.
+constexpr int kKeptStats = 8;
+constexpr size_t kStatsBytes = kBatchDims * 8 * sizeof(int64_t);
+std::mutex g_stats_mutex;
+int64_t *g_stats[kKeptStats];
+int g_nstats = 0;
+
 struct HostStats {
     int64_t *words = nullptr;
+
+    HostStats()
+    {
+        {
+            std::lock_guard<std::mutex> lock(g_stats_mutex);
+            if (g_nstats > 0) words = g_stats[--g_nstats];
+        }
+        if (!words && cudaHostAlloc(reinterpret_cast<void **>(&words), kStatsBytes,
+                                    cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            (void)cudaGetLastError();
+            words = nullptr;
+        }
+    }
+    HostStats(const HostStats &) = delete;
+    HostStats &operator=(const HostStats &) = delete;
+    ~HostStats()
+    {
+        if (!words) return;
+        {
+            std::lock_guard<std::mutex> lock(g_stats_mutex);
+            if (g_nstats < kKeptStats) {
+                g_stats[g_nstats++] = words;
+                return;
+            }
+        }
+        if (cudaFreeHost(words) != cudaSuccess) (void)cudaGetLastError();
+    }
+    void abandon() { words = nullptr; } // after a failed wait: a kernel may still write there
 };
-thread_local HostStats g_host_stats;
 
 } // namespace
 
@@ -909,10 +944,11 @@ extern "C" sjq_status sjq_dim_plan_begin(const sjq_col *cols, int ncols, const s
 namespace sjq {
 int host_stats_release()
 {
-    if (!g_host_stats.words) return 0;
-    if (cudaFreeHost(g_host_stats.words) != cudaSuccess) (void)cudaGetLastError();
-    g_host_stats.words = nullptr;
-    return 1;
+    std::lock_guard<std::mutex> lock(g_stats_mutex);
+    const int n = g_nstats;
+    while (g_nstats > 0)
+        if (cudaFreeHost(g_stats[--g_nstats]) != cudaSuccess) (void)cudaGetLastError();
+    return n;
 }
 } // namespace sjq
 
@@ -922,25 +958,23 @@ extern "C" sjq_status sjq_dims_plan(const sjq_dim_desc *dims, int ndims, void *s
     if (!dims || ndims <= 0 || !scratch_dev || !layouts) return SJQ_ERR_INVALID_ARG;
     if (!aligned16(scratch_dev)) return SJQ_ERR_ALIGN;
     if (scratch_bytes < (size_t)ndims * SJQ_PLAN_SCRATCH_BYTES) return SJQ_ERR_BUFFER_SMALL;
-    int64_t *&host = g_host_stats.words;
     DeviceInfo dev;
     sjq_status st = check_dims(dims, ndims);
     if (st == SJQ_OK) st = device_info(&dev);
     if (st != SJQ_OK) return st;
-    if (!host && cudaHostAlloc(reinterpret_cast<void **>(&host), kBatchDims * 8 * sizeof(int64_t),
-                               cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-        (void)cudaGetLastError();
-        host = nullptr;
-        return SJQ_ERR_CUDA;
-    }
+    HostStats host;
+    if (!host.words) return SJQ_ERR_CUDA;
     int64_t *words[kBatchDims];
-    for (int i = 0; i < kBatchDims; ++i) words[i] = host + 8 * i;
+    for (int i = 0; i < kBatchDims; ++i) words[i] = host.words + 8 * i;
     cudaStream_t stream = (cudaStream_t)stream_;
     for (int first = 0; first < ndims;) {
         const int n = batch_of(dims, ndims, first);
         st = scan_launch(dims + first, n, static_cast<unsigned long long *>(scratch_dev), words, dev.sm_count, stream);
         // the kernel writes the statistics into the page-locked words itself
-        if (st == SJQ_OK && cudaStreamSynchronize(stream) != cudaSuccess) st = SJQ_ERR_CUDA;
+        if (st == SJQ_OK && cudaStreamSynchronize(stream) != cudaSuccess) {
+            host.abandon();
+            st = SJQ_ERR_CUDA;
+        }
         if (st != SJQ_OK) {
             (void)cudaGetLastError();
             return st;

@@ -2,6 +2,8 @@
 warp's 128, a block's 1024; neighbouring, descending, scattered and widely spaced keys; repeated keys inside a thread,
 a warp, a block and across blocks; tables without a presence bitmap; batches of more dimensions and filters than one
 launch takes."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -119,6 +121,33 @@ def test_launches_of_a_batch_split_by_its_filters_are_all_counted():
     builder = sjq.TableBuilder(dims[0][0], "k")
     assert sjq.build_launches(sjq.build_tables({"d": builder})["d"]) == 3
     torch.cuda.synchronize()
+
+
+def test_threads_that_plan_leave_at_most_eight_pieces_of_page_locked_memory_behind():
+    """sjq_release counts what it frees: the pieces that finished plans left, whatever thread they ran on."""
+    cols, found = to_dev({"k": np.arange(5_000, dtype=np.int32)}), []
+
+    def plan():
+        table = sjq.build_dim(cols, "k")
+        found.append((table.layout.entries, table.status()))
+
+    def in_threads(n):
+        threads = [threading.Thread(target=plan) for _ in range(n)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+
+    torch.cuda.synchronize()
+    sjq.release()
+    for _ in range(3):
+        in_threads(1)  # one after the other: the same piece
+    assert sjq.release() == 1
+    in_threads(16)
+    assert 1 <= sjq.release() <= 8
+    assert sjq.release() == 0
+    plan()
+    assert found == [(5_000, 0)] * 20
 
 
 def test_empty_dimension_in_a_batch():
