@@ -196,7 +196,8 @@ bool read_term(PyObject *t, const Columns &C, sjq_term *out)
     return get_int(t, N.b, &out->b);
 }
 
-bool read_ints(PyObject *o, PyObject *name, int32_t *out, int most, int32_t *count)
+// `convert`: each entry goes through int() first, as RunOpts.to_c does with measured fractions (they may be floats).
+bool read_ints(PyObject *o, PyObject *name, int32_t *out, int most, int32_t *count, bool convert)
 {
     Ref seq(PyObject_GetAttr(o, name));
     if (!seq) return false;
@@ -209,7 +210,9 @@ bool read_ints(PyObject *o, PyObject *name, int32_t *out, int most, int32_t *cou
     }
     for (Py_ssize_t i = 0; i < n; ++i) {
         int64_t v = 0;
-        if (!as_int(PySequence_Fast_GET_ITEM(fast.p, i), &v)) return false;
+        PyObject *entry = PySequence_Fast_GET_ITEM(fast.p, i);
+        Ref whole(convert ? PyNumber_Long(entry) : Py_NewRef(entry));
+        if (!whole || !as_int(whole.p, &v)) return false;
         out[i] = (int32_t)v;
     }
     if (count) *count = (int32_t)n;
@@ -226,8 +229,8 @@ bool read_opts(PyObject *p, sjq_run_opts *o)
         !get_flag(p, N.host_copy_all, &o->host_copy_all) || !get_int(p, N.dense_slots, &o->dense_slots) ||
         !get_flag(p, N.group_hash_always, &o->group_hash_always) || !get_int(p, N.warp_agg, &o->warp_agg) ||
         !get_int(p, N.hot_keys, &o->hot_keys) || !get_int(p, N.l0_bulk, &o->l0_bulk) ||
-        !read_ints(p, N.order, o->order, SJQ_MAX_PREDS + SJQ_MAX_JOINS, &o->norder) ||
-        !read_ints(p, N.pass_ppm, o->pass_ppm, SJQ_MAX_PREDS + SJQ_MAX_JOINS, nullptr))
+        !read_ints(p, N.order, o->order, SJQ_MAX_PREDS + SJQ_MAX_JOINS, &o->norder, false) ||
+        !read_ints(p, N.pass_ppm, o->pass_ppm, SJQ_MAX_PREDS + SJQ_MAX_JOINS, nullptr, true))
         return false;
     int64_t bytes = 0;
     if (!get_pointer(p, N.hot_scratch, &o->hot_scratch, &bytes)) return false;

@@ -86,3 +86,13 @@ def test_names_and_counts_that_do_not_fit_raise():
         call(preds=[Pred("a", "EQ", "x")])
     with pytest.raises(ValueError):
         sjq.run({"a": torch.zeros(8, dtype=torch.int32)}, agg=AggExpr("COL", Term("FACT", "a")))
+
+
+def test_measured_fractions_may_be_floats():
+    """As through ctypes: int() is applied to them, and to nothing else."""
+    few = [Pred("a", "LT", 3)]
+    assert call(preds=few, opts=B.RunOpts(pass_ppm=(2.5e5, True), rows_per_lane=8)) == INVALID_ARG  # read, then refused
+    assert call(preds=few, opts=B.RunOpts(pass_ppm=torch.tensor([250_000.7]), rows_per_lane=8)) == INVALID_ARG
+    for bad in (B.RunOpts(order=(0.0,)), B.RunOpts(block_threads=128.0), B.RunOpts(pass_ppm=(None,))):
+        with pytest.raises(TypeError):
+            call(preds=few, opts=bad)
