@@ -259,9 +259,11 @@ PyObject *py_run(PyObject *, PyObject *const *args, Py_ssize_t nargs)
         return nullptr;
     }
     PyObject *fact = args[0], *joins = args[2], *key = args[3], *agg = args[4], *opts = args[8], *result = args[9];
-    if (!PyDict_Check(fact)) {
-        PyErr_SetString(PyExc_TypeError, "the fact columns come as a dict");
-        return nullptr;
+    Ref columns(nullptr); // of another mapping than a dict
+    if (!PyDict_CheckExact(fact)) {
+        columns.p = PyDict_New();
+        if (!columns || PyDict_Update(columns.p, fact) != 0) return nullptr;
+        fact = columns.p;
     }
     Columns C;
     Predicates P;

@@ -1,6 +1,9 @@
 """The extension module that fills the argument structures of sjq_run: what it accepts, what it rejects and with which
 exception.  Columns are stand-ins with a tensor's interface, so that no device is needed: a well-formed call passes all
 checks of the library that come before the device."""
+from collections import OrderedDict, UserDict
+from types import MappingProxyType
+
 import pytest
 import torch
 
@@ -96,3 +99,13 @@ def test_measured_fractions_may_be_floats():
     for bad in (B.RunOpts(order=(0.0,)), B.RunOpts(block_threads=128.0), B.RunOpts(pass_ppm=(None,))):
         with pytest.raises(TypeError):
             call(preds=few, opts=bad)
+
+
+@pytest.mark.parametrize("kind", [OrderedDict, UserDict, MappingProxyType])
+def test_columns_come_in_any_mapping(kind):
+    refused = B.RunOpts(rows_per_lane=8)  # by the library, after everything has been read
+    assert call(kind({"a": FakeColumn()}), preds=[Pred("a", "EQ", 1)], opts=refused) == INVALID_ARG
+    with pytest.raises(ValueError, match="contiguous 1-D"):
+        call(kind({"a": FakeColumn(dim=2)}))
+    with pytest.raises((TypeError, AttributeError)):
+        call([FakeColumn()])
