@@ -963,11 +963,15 @@ def release() -> int:
 
 def build_workload_tables(w, dims: dict) -> dict:
     """dims: dimension name -> dict of CUDA column tensors (a workload description's dims)."""
-    if not w.dims:
-        return {}
-    tables = _build_tables([(dims[d.name], d.key, d.preds, d.payloads, _BuildOpts(FORCE_HASH if d.force_hash else 0))
-                            for d in w.dims])
-    return {d.name: t for d, t in zip(w.dims, tables)}
+    by_device = {}  # one batch for each device that holds dimensions
+    for d in w.dims:
+        by_device.setdefault(next(iter(dims[d.name].values())).device, []).append(d)
+    tables = {}
+    for specs in by_device.values():
+        built = _build_tables([(dims[d.name], d.key, d.preds, d.payloads, _BuildOpts(FORCE_HASH if d.force_hash else 0))
+                               for d in specs])
+        tables.update((d.name, t) for d, t in zip(specs, built))
+    return {d.name: tables[d.name] for d in w.dims}
 
 
 def run_workload(w, fact: dict, tables: dict, opts: Optional[RunOpts] = None,

@@ -189,3 +189,24 @@ def test_sampled_counters_become_parts_per_million(libsjq):
     assert b.lib().sjq_pred_sample_end(counts, 4, out) == 0
     assert list(out) == [1, 99, 1_000_000, 500_000]  # none seen -> 1 ppm, never "unknown"
     assert b.lib().sjq_pred_sample_end(None, 4, out) == 1
+
+
+def test_dimensions_of_several_devices_are_built_on_their_own(monkeypatch):
+    """A batch runs on one device and one stream: the tables of a workload are batched by where their columns are."""
+    from types import SimpleNamespace
+
+    import paper_2607_07632_b200.sjq as b
+
+    batches = []
+
+    def build(batch):
+        batches.append([cols["k"].name for cols, *_ in batch])
+        return [f"table of {cols['k'].name}" for cols, *_ in batch]
+
+    monkeypatch.setattr(b, "_build_tables", build)
+    where = {"a": "cuda:0", "b": "cuda:1", "c": "cuda:0", "d": "cuda:1"}
+    dims = {n: {"k": SimpleNamespace(name=n, device=dev)} for n, dev in where.items()}
+    w = SimpleNamespace(dims=[SimpleNamespace(name=n, key="k", preds=(), payloads=(), force_hash=False) for n in where])
+    assert list(b.build_workload_tables(w, dims).items()) == [(n, f"table of {n}") for n in where]
+    assert batches == [["a", "c"], ["b", "d"]]
+    assert b.build_workload_tables(SimpleNamespace(dims=()), {}) == {}
