@@ -11,7 +11,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libsjq.so")
 OBJ = os.path.join(HERE, "csrc", "obj")  # one object per translation unit, so that an edit recompiles only its own
-MARSHAL = os.path.join(HERE, "_marshal.so")  # CPython extension: the binding's argument marshalling, linked to LIB
+# CPython extension: the binding's argument marshalling, linked to LIB.  The name carries the interpreter's tag: another
+# version of Python does not load it and builds its own.
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]
 
 
@@ -60,6 +62,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def _build_marshal(force: bool) -> None:
     src = os.path.join(HERE, "csrc", "sjq_py.cpp")
+    untagged = os.path.join(HERE, "_marshal.so")  # as it was named before: any version of Python would load it
+    if os.path.exists(untagged):
+        os.remove(untagged)
     if force or _stale(MARSHAL, [src, os.path.join(ROOT, "include", "sjq.h")]):
         subprocess.check_call(["g++", "-O2", "-std=c++17", "-Wall", "-fPIC", "-shared", "-fvisibility=hidden",
                                "-I" + os.path.join(ROOT, "include"), "-I" + sysconfig.get_paths()["include"], src, LIB,

@@ -1,6 +1,8 @@
 """The extension module that fills the argument structures of sjq_run: what it accepts, what it rejects and with which
 exception.  Columns are stand-ins with a tensor's interface, so that no device is needed: a well-formed call passes all
 checks of the library that come before the device."""
+import os
+import sysconfig
 from collections import OrderedDict, UserDict
 from types import MappingProxyType
 
@@ -109,3 +111,11 @@ def test_columns_come_in_any_mapping(kind):
         call(kind({"a": FakeColumn(dim=2)}))
     with pytest.raises((TypeError, AttributeError)):
         call([FakeColumn()])
+
+
+def test_the_module_is_the_one_built_for_this_interpreter():
+    from paper_2607_07632_b200 import build
+
+    assert build.MARSHAL.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and "cpython" in os.path.basename(build.MARSHAL)
+    assert os.path.samefile(B.marshal().__file__, build.MARSHAL)
+    assert not os.path.exists(os.path.join(os.path.dirname(build.MARSHAL), "_marshal.so"))
