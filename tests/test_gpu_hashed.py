@@ -38,6 +38,20 @@ def test_lists_of_every_length(n, groups, below):
             compare(w, res, exp)
 
 
+@pytest.mark.parametrize("groups", [1, 2, 1024, 1025, 4096, 4097, 20_000])
+@pytest.mark.parametrize("below", [1000, 10])
+def test_an_indexed_table_is_listed_in_key_order_by_one_kernel_where_it_is_small(groups, below):
+    """2 M - 1 cells: up to four blocks of 2048 count the groups before their own themselves."""
+    fact, w = _query(60_001, groups, below, groups + 8, groups)
+    for opts in (sjq.RunOpts(), sjq.RunOpts(specialise=True)):
+        res, exp, _ = run_both(w, fact, {}, opts=opts)
+        assert res.status() == 0 and res.info.kernel_launches == (3 if groups <= 4096 else 4)
+        n = int(res.n_groups.item())
+        assert np.array_equal(res.keys[:n].cpu().numpy(), exp["keys"])  # as listed, not sorted
+        assert np.array_equal(res.sums[:n].cpu().numpy(), exp["sums"])
+        compare(w, res, exp)
+
+
 def test_large_indexed_table_has_several_tiles_per_block():
     fact, w = _query(200_003, 150_000, 1000, 3_000_000, 5_000_000)  # ten million cells, 2048 to a tile
     res, exp, _ = run_both(w, fact, {}, opts=sjq.RunOpts(specialise=True))
