@@ -84,6 +84,7 @@ __device__ __forceinline__ unsigned int used_cells(const CompactParams &C, int64
 
 __global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const CompactParams C)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory"); // the pass
     asm volatile("griddepcontrol.launch_dependents;"); // the listing may start and wait for the counts on the device
     const int64_t lo = (int64_t)blockIdx.x * C.tiles_per_block * kCompactTile;
     int64_t hi = lo + C.tiles_per_block * kCompactTile;
@@ -106,11 +107,11 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(const CompactP
     __shared__ unsigned int part[kCompactThreads / 32];
     __shared__ long long draw;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    asm volatile("griddepcontrol.wait;" ::: "memory"); // the pass, and the counts where a kernel forms them
     long long place = 0;
     if (C.ordered) {
         unsigned int before = 0;
         if (C.block_counts) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int b = threadIdx.x; b < (int)blockIdx.x; b += kCompactThreads) before += C.block_counts[b];
         } else {
             before = used_cells(C, 0, (int64_t)blockIdx.x * C.tiles_per_block * kCompactTile);
@@ -401,11 +402,12 @@ sjq_status merge_launch(const int64_t *keys, const int64_t *sums, const int64_t 
 }
 
 // gslots: regular slots of the hash table (a side slot follows), or the cells of an indexed table.  `block_counts`
-// (device, one word per 2048 cells): an indexed table is listed in key order; NULL: in no order.
+// (device, one word per 2048 cells): an indexed table is listed in key order; NULL: in no order.  `beside`: directly
+// behind the fused kernel, which lets its successor start while it runs, so many blocks at most may wait beside it.
 sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gslots, bool indexed,
                           int64_t dense_base, unsigned int *block_counts, int64_t *keys, int64_t *sums,
                           int64_t *counts, int64_t capacity, int64_t *n_groups, int32_t *status, int sm_count,
-                          cudaStream_t stream, int *launches)
+                          int beside, cudaStream_t stream, int *launches)
 {
     const int64_t ncells = indexed ? gslots : gslots + 1;
     const int64_t tiles = (ncells + kCompactTile - 1) / kCompactTile;
@@ -414,20 +416,20 @@ sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gs
     const bool counted = block_counts && blocks > kCompactAlone;
     CompactParams C{gkeys, reinterpret_cast<const longlong2 *>(cells), dense_base, indexed ? 1 : 0, ncells, per,
                     block_counts ? 1 : 0, counted ? block_counts : nullptr, keys, sums, counts, capacity, n_groups, status};
-    if (counted) {
-        compact_count_kernel<<<blocks, kCompactThreads, 0, stream>>>(C);
-        ++*launches;
-        if (cudaGetLastError() != cudaSuccess) return SJQ_ERR_CUDA;
-    }
     cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization; // behind the counts, for which it waits on the device
-    attr.val.programmaticStreamSerializationAllowed = counted ? 1 : 0;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = blocks <= beside ? 1 : 0;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(kCompactThreads);
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
+    if (counted) {
+        if (cudaLaunchKernelEx(&cfg, compact_count_kernel, C) != cudaSuccess) return SJQ_ERR_CUDA;
+        ++*launches;
+        attr.val.programmaticStreamSerializationAllowed = 1; // the listing behind the counts
+    }
     ++*launches;
     return cudaLaunchKernelEx(&cfg, compact_kernel, C) == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }

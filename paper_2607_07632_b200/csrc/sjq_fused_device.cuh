@@ -1123,6 +1123,8 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
     __syncthreads();
     // launched behind the kernel that clears the results: nothing above touches them, everything below may
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (the listing of a hashed result is launched while this kernel runs and waits for its end on the device)
+    if (AGG != AGG_SCALAR) asm volatile("griddepcontrol.launch_dependents;");
 
     int64_t lsum = 0, lcnt = 0;
 

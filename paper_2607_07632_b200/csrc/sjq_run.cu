@@ -35,7 +35,7 @@ sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *
 sjq_status compact_launch(const int64_t *gkeys, const int64_t *cells, int64_t gslots, bool indexed,
                           int64_t dense_base, unsigned int *block_counts, int64_t *keys, int64_t *sums,
                           int64_t *counts, int64_t capacity, int64_t *n_groups, int32_t *status, int sm_count,
-                          cudaStream_t stream, int *launches);
+                          int beside, cudaStream_t stream, int *launches);
 
 int host_stats_release();
 size_t unfused_scratch_bytes(int64_t n, int gathering_joins);
@@ -1034,10 +1034,15 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         return SJQ_ERR_CUDA;
     if (spec->mode == SJQ_HASHED) {
         // (an indexed table has no use for the key array: it holds the block counts of the ordered list)
+        // Launched behind the pass, the listing takes 1 to 3 us less (a list of 20,000 groups, 1 % left: 20 M rows 36.4 ->
+        // 33.5 us, 2 M 18.5 -> 15.3).  Its blocks wait in the SMs meanwhile: one per SM leaves room for other streams'
+        // kernels beside a long pass.
+        const bool follows = n > 0 && !opts.unfused && !opts.event_after;
+        const int beside = !follows ? 0 : n <= (int64_t)1 << 20 ? INT32_MAX : dev.sm_count;
         st = compact_launch(gkeys, cells, direct_groups ? table_groups : (int64_t)gslots, direct_groups, P.post_offset,
                             direct_groups && !opts.unfused ? reinterpret_cast<unsigned int *>(gkeys) : nullptr,
                             out->keys, out->sums, out->counts, spec->capacity, out->n_groups, out->status,
-                            dev.sm_count, stream, &launches);
+                            dev.sm_count, beside, stream, &launches);
         if (st != SJQ_OK) return st;
     }
     if (info) {
@@ -1102,7 +1107,7 @@ extern "C" sjq_status sjq_merge_groups(const int64_t *keys, const int64_t *sums,
         return st;
     int launches = 0;
     return compact_launch(gkeys, cells, (int64_t)gslots, false, 0, nullptr, out->keys, out->sums, out->counts, capacity,
-                          out->n_groups, out->status, dev.sm_count, stream, &launches);
+                          out->n_groups, out->status, dev.sm_count, 0, stream, &launches);
 }
 
 // ---------------------------------------------------------------------------
