@@ -12,11 +12,13 @@ group-by over 600 M fact rows (14.4 GB of referenced fact columns, far larger
 than the 126 MB L2, so no L2 flush is needed between steps); every rank holds
 its own 600 M-row shard of the row space and a replica of the dimensions
 (weak scaling; `--scaling strong` cuts one 1.2 B-row table over the ranks
-instead).  Rank 0 prints ONE JSON line.  At N = 1 the line also carries
-`points`: every other configuration (config 1, 2, 5, the 20 points of the
-selectivity x cardinality sweep, the two high-cardinality shapes), each run
-ten times or more with its own roofline figures, clock record and a bit-exact
-comparison with the oracle-written expected values under tests/golden/.
+instead).  Rank 0 prints ONE JSON line on standard output, short enough for a
+reader that keeps the last 3,000 characters.  At N = 1 every other
+configuration (config 1, 2, 5, the 20 points of the selectivity x cardinality
+sweep, the two high-cardinality shapes) is run ten times or more as well and
+printed as a JSON line of its own on standard error, with its own roofline
+figures, clock record and a bit-exact comparison with the oracle-written
+expected values under tests/golden/; the line on standard output counts them.
 """
 from __future__ import annotations
 
@@ -57,6 +59,28 @@ def profiled_traffic(w, info, kernel, rows):
     if not same:
         return None, f"the plan that ran differs from the one captured in {p['summary']}"
     return p["dram_bytes_per_row"] * rows, p["summary"]
+
+
+def rounded(v, digits=7):
+    """A line's values with floats cut to `digits` significant digits."""
+    if isinstance(v, float):
+        return float(f"{v:.{digits}g}")
+    if isinstance(v, dict):
+        return {k: rounded(x, digits) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [rounded(x, digits) for x in v]
+    return v
+
+
+def print_line(line, points=None, ablation=None):
+    """One JSON line per point and per ablation row on standard error, then the line itself on standard output."""
+    for kind, rows in (("point", points), ("ablation", ablation)):
+        for row in rows or ():
+            print(json.dumps({kind: rounded(row)}), file=sys.stderr, flush=True)
+    if points is not None:
+        bad = [p["workload"] for p in points if p.get("parity") is not True]
+        line["points"] = {"run": len(points), "parity": len(points) - len(bad), "without_parity": bad[:3]}
+    print(json.dumps(rounded(line)), flush=True)
 
 
 def measured_hbm_peak():
@@ -614,8 +638,7 @@ def main():
                 "traffic": traffic, "traffic_source": traffic_note,
                 "algorithmic_bytes_per_row": alg_bpr, "kernel_ms": fused_ms,
                 "bytes_per_row_64B_model": algorithmic_bytes_per_row(w, list(info.order[: info.nstages]), pass_frac, 64),
-                "note": "achieved and frac use the 32-byte-sector model; DRAM delivers 64-byte pieces (ncu traffic), "
-                        "for which the same model gives bytes_per_row_64B_model",
+                "note": "achieved, frac: 32-byte-sector model",
                 "pass_fractions": {str(k): round(v, 6) for k, v in pass_frac.items()},
                 "effective_gbs_kernel": n * ref_bytes / (fused_ms / 1000.0) / 1e9}
 
@@ -672,13 +695,11 @@ def main():
             e2e = {"value": total_rows / dt, "unit": UNIT, "h2d_bytes_per_step": int(copied + in_place + dim_bytes),
                    "h2d_copied_bytes": int(copied), "h2d_dimension_bytes": int(dim_bytes),
                    "h2d_in_place_bytes_estimate": int(in_place),
-                   "h2d_in_place_note": "sector-model estimate from the planner's shares, not a counter",
                    "columns": {k: how for k, (how, _) in plan.items()},
                    "d2h_bytes_per_step": cells * 8 * (2 if w.agg.want_count else 1) + 4, "ms_per_step": dt * 1000.0,
                    "steps": args.e2e_steps, "chunk_rows": chunk, "matches_device_run": same,
-                   "api": "sjq_run_host (pinned host columns: chunked double-buffered copies of the columns most rows need, "
-                          "in-place reads of the sparse ones, result copied back); dimension columns copied from pinned "
-                          "host memory every step before the table builds"}
+                   # (the dimension columns are copied from pinned memory every step, before the table builds)
+                   "api": "sjq_run_host: pinned columns in chunks, sparse ones read in place, result copied back"}
             del host_fact, staging, host_dims
         except Exception as ex:  # e.g. not enough page-locked memory on the box
             e2e = {"value": None, "unit": UNIT, "error": repr(ex)[:200]}
@@ -712,21 +733,17 @@ def main():
                 "vs_baseline": None, "dtype": "int64", "data": "synthetic",
                 "config": {"workload": w.name, "rows_per_gpu": n, "rows_total": total_rows,
                            "referenced_bytes_per_row": ref_bytes,
-                           "step": "key-range scan + build of every dimension table (on side streams; the table shape comes from the newest scan that has reached the host and is checked on the device by the build, so the host never waits), then the fused pass"
-                                   + exchange,
+                           # (scans and builds on side streams; a table's shape comes from the newest scan that has
+                           # reached the host and is checked on the device by the build: the host never waits)
+                           "step": "scan + build of every dimension table, then the fused pass" + exchange,
                            "l2": "inputs (%.1f GB) exceed the 126 MB L2; no flush needed" % (n * ref_bytes / 1e9),
                            "parallelism": f"row-sharded x{world}, dimensions replicated", "plan": info.describe(),
-                           "fused_kernel": "interpreted descriptor" if args.interpret else
-                                           "compiled for the query's shape at run time during warm-up (NVRTC), cached"},
+                           "fused_kernel": "interpreted" if args.interpret else "compiled for the query during warm-up"},
                 "effective_gbs": eff_gbs, "pct_of_8tbs": 100.0 * eff_gbs / world / CONTRACT_HBM_GBS,
                 "pct_of_measured_copy_peak": 100.0 * eff_gbs / world / peak, "parity": parity,
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
                 "clocks": sampler.summary()}
-        if points is not None:
-            line["points"] = points
-        if ablation is not None:
-            line["ablation"] = ablation
-        print(json.dumps(line), flush=True)
+        print_line(line, points, ablation)
     if world > 1:
         dist.destroy_process_group()
     return 0
