@@ -217,8 +217,9 @@ sjq_status sjq_dim_plan_end(const sjq_col *cols, int ncols, int key_col, int npa
  * the open-addressing table has no free slot left).  Enqueues
  * a fill and the build kernel; does not synchronise.
  * Direct tables are written by race-free direct stores indexed by key
- * (Section 3.3), and the presence bits beside them tell a repeated key; hash tables by atomicCAS on the key word with a bounded
- * linear probe.  Keys must be unique among the passing rows: a repeated key
+ * (Section 3.3), and the presence bits beside them tell a repeated key; hash
+ * tables by atomicCAS on the key word with a bounded linear probe.  Keys must
+ * be unique among the passing rows: a repeated key
  * sets SJQ_ERR_DUP_KEY in *status_dev.  Zero passing rows is valid (every
  * probe then misses).  *status_dev is NOT cleared by this call.
  */
@@ -275,7 +276,8 @@ sjq_status sjq_dim_layout_bytes(const sjq_dim_layout *layout, size_t *bytes);
 sjq_status sjq_table_info(const sjq_table *table, sjq_dim_layout *layout);
 
 /* Kernels sjq_build_dim enqueued for this table: one that prepares the memory and the build, the latter unless the
- * dimension is empty (and its layout promises no keys).  (sjq_dims_build counts those of a batch with its first table.) */
+ * dimension is empty (and its layout promises no keys).  (sjq_dims_build counts those of a batch with its first
+ * table.) */
 int32_t sjq_table_kernel_launches(const sjq_table *table);
 
 /* Frees the host handle only (the device memory belongs to the caller). */
@@ -338,7 +340,9 @@ typedef struct sjq_run_opts {
     int32_t specialise; /* 1 = compile the fused kernel for this query's shape at run time (NVRTC) and cache the
                            module for later runs of the same shape; 0 = interpret the descriptor (default).  Key
                            ranges, thresholds, table sizes and pointers stay run-time values, so a compiled module
-                           is reused when only they change.  Same results either way. */
+                           is reused when only they change.  (The number of rows chooses between up to three kernels
+                           of a query: up to 2^19 rows, up to about 20 M, beyond; each is compiled at its first run.)
+                           Same results either way. */
     int32_t rows_per_lane; /* rows a lane handles per batch at the queue-fed levels: 0 = library chooses, 4, or 8
                               (8 only with specialise: the ahead-of-time kernels are built for 4) */
     int32_t no_filter_bitmap; /* 1 = filter stages probe a direct table's code array even when the table has a

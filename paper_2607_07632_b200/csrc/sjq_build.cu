@@ -23,9 +23,9 @@ constexpr int kMaxDimCols = 32;
 // A launch works on up to kBatchDims dimensions (and their filters, together at most kBatchPreds): the scans, the
 // fills and the builds of a query's tables are one launch each.  A block belongs to one dimension; its threads take
 // four consecutive rows at two places at a time (one where 64-bit values fill the registers), so that every column is
-// read with 128-bit loads and six of them are in flight per thread before the first is used.  What bounds these kernels: latency for the small dimensions (2,556
-// to 200,000 rows), instructions as much as the columns' bytes for those of millions; so the code for 32-bit keys and
-// payloads keeps to 32-bit arithmetic.
+// read with 128-bit loads and six of them are in flight per thread before the first is used.  What bounds these
+// kernels: latency for the small dimensions (2,556 to 200,000 rows), instructions as much as the columns' bytes for
+// those of millions; so the code for 32-bit keys and payloads keeps to 32-bit arithmetic.
 constexpr int kBatchDims = 8;
 constexpr int kBatchPreds = 16;
 constexpr int kFillThreads = 256;

@@ -25,9 +25,10 @@ constexpr unsigned int kClearSmall = 148; // blocks, of 256 threads
 // (every array starts on a 16-byte boundary; the odd last word is thread 0's)
 __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
 {
-    // The fused kernel may start and wait for this one on the device: at once where this one leaves most of the chip idle,
-    // else when its stores are out, since blocks that start beside it are spread unevenly over the SMs (sums and counts of
-    // 400,000 groups, 2 M rows: 34.3 us when started at once, 30.5 so, 32.5 one kernel after the other).
+    // The fused kernel may start and wait for this one on the device: at once where this one leaves most of the chip
+    // idle, else when its stores are out, since blocks that start beside it are spread unevenly over the SMs (sums
+    // and counts of 400,000 groups, 2 M rows: 34.3 us when started at once, 30.5 so, 32.5 one kernel after the
+    // other).
     const bool small = gridDim.x <= kClearSmall;
     if (small) asm volatile("griddepcontrol.launch_dependents;");
     const int64_t stride = (int64_t)blockDim.x * gridDim.x;
@@ -68,9 +69,9 @@ struct CompactParams {
 constexpr int kCompactThreads = 256;
 constexpr int kCompactRounds = 8; // cells per thread and tile, all loaded before the first is used
 constexpr int kCompactTile = kCompactThreads * kCompactRounds;
-// Up to so many blocks each count the groups before their own themselves: a kernel for the counts costs a query over few
-// rows 1 to 6 us (2 M rows, 1 % left, a list of 4000 groups: 15.4 us unordered, 20.0 with that kernel), the last of four
-// blocks reads 96 KB more.
+// Up to so many blocks each count the groups before their own themselves: a kernel for the counts costs a query over
+// few rows 1 to 6 us (2 M rows, 1 % left, a list of 4000 groups: 15.4 us unordered, 20.0 with that kernel), the last
+// of four blocks reads 96 KB more.
 constexpr int kCompactAlone = 4;
 
 // Cells of an indexed table that hold a group, [lo, hi), those of this thread.
@@ -157,7 +158,8 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(const CompactP
             total += part[w];
         }
         if (!C.ordered) {
-            if (threadIdx.x == 0) draw = (long long)atomicAdd(reinterpret_cast<unsigned long long *>(C.n_groups), (unsigned long long)total);
+            if (threadIdx.x == 0)
+                draw = (long long)atomicAdd(reinterpret_cast<unsigned long long *>(C.n_groups), (unsigned long long)total);
             __syncthreads();
             place = draw;
         }
@@ -257,11 +259,14 @@ __global__ void __launch_bounds__(256) sample_kernel(const __grid_constant__ Sam
 
 const void *pick_kernel(int agg, bool mul, bool hash, bool few)
 {
+    const auto of = [few](fused_few_fn little, fused_fn any) {
+        return few ? reinterpret_cast<const void *>(little) : reinterpret_cast<const void *>(any);
+    };
     switch (agg) {
-    case AGG_SCALAR: return few ? reinterpret_cast<const void *>(fused_few_scalar(mul, hash)) : reinterpret_cast<const void *>(fused_variant_scalar(mul, hash));
-    case AGG_SMEM: return few ? reinterpret_cast<const void *>(fused_few_smem(mul, hash)) : reinterpret_cast<const void *>(fused_variant_smem(mul, hash));
-    case AGG_GLOBAL: return few ? reinterpret_cast<const void *>(fused_few_global(mul, hash)) : reinterpret_cast<const void *>(fused_variant_global(mul, hash));
-    default: return few ? reinterpret_cast<const void *>(fused_few_hash(mul, hash)) : reinterpret_cast<const void *>(fused_variant_hash(mul, hash));
+    case AGG_SCALAR: return of(fused_few_scalar(mul, hash), fused_variant_scalar(mul, hash));
+    case AGG_SMEM: return of(fused_few_smem(mul, hash), fused_variant_smem(mul, hash));
+    case AGG_GLOBAL: return of(fused_few_global(mul, hash), fused_variant_global(mul, hash));
+    default: return of(fused_few_hash(mul, hash), fused_variant_hash(mul, hash));
     }
 }
 

@@ -91,8 +91,9 @@ struct Vec4<int64_t> {
     static __device__ __forceinline__ void load(const int64_t *p, int64_t *v, bool aligned)
     {
         // One 256-bit load: two 128-bit loads of neighbouring lanes would each touch every sector of the 1024 bytes,
-        // and the L1 passes one sector per cycle (the skewed 64-bit-key workload, bound by it, 300 M rows: 1689 ->
-        // 1596 us; asked once, 10 M rows: 295 -> 285).
+        // and the L1 passes one sector per cycle (the skewed 64-bit-key workload, bound by it, 300 M rows, both loads
+        // in turn three times: 1800 -> 1690, 1832 -> 1717 and 1781 -> 1680 us; asked once of the interpreting kernel,
+        // 10 M rows: 274 and 273).
 #if SJQ_HAVE_LOAD256
         if (aligned) {
             asm volatile("ld.global.nc.L1::no_allocate.v4.b64 {%0, %1, %2, %3}, [%4];"
@@ -1385,8 +1386,9 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
         const unsigned int *ss = reinterpret_cast<const unsigned int *>(smem + P.smem_groups);
         const uint64_t ng = (uint64_t)P.num_groups;
         if (SJQ_PV(cell_shift)) {
-            // sums and counts alternate: neighbouring lanes take neighbouring words, so that a warp's adds meet 8 sectors
-            // and not 16 (2 M rows into a list: 1 % left, 60 groups 18.5 -> 14.4 us; half left, a thousand 22.6 -> 19.9)
+            // sums and counts alternate: neighbouring lanes take neighbouring words, so that a warp's adds meet 8
+            // sectors and not 16 (2 M rows into a list: 1 % left, 60 groups 18.5 -> 14.4 us; half left, a thousand
+            // 22.6 -> 19.9)
             for (int64_t i = tid; i < 2 * P.num_groups; i += blockDim.x) {
                 const unsigned long long v = smem_cell((i & 1) ? ss + 2 * ng : ss, ng, (uint64_t)(i >> 1));
                 if (v != 0ull) atomicAdd(reinterpret_cast<unsigned long long *>(P.sums) + i, v);

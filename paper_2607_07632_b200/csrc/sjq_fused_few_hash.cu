@@ -1,5 +1,5 @@
-// Ahead-of-time instantiations of the fused kernel for one aggregation path (AGG_HASH) and up to kFewStages stages; one translation unit per
-// path and size of the parameter block so that they compile in parallel.
+// Ahead-of-time instantiations of the fused kernel for one aggregation path (AGG_HASH) and up to kFewStages stages;
+// one translation unit per path and size of the parameter block so that they compile in parallel.
 #include "sjq_fused_device.cuh"
 
 namespace sjq {

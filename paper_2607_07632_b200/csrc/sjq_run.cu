@@ -355,11 +355,14 @@ namespace {
 
 // What a run is part of: by default of nothing, its columns are in device memory and its options are the caller's.
 struct RunContext {
-    bool callers_order = true; // the order of the filters, if the options give one, is the caller's own and not one that
-                               // this library chose for a run from host memory
-    bool in_place = false;     // some columns are read in place from host memory
-    int64_t rows = -1;         // rows to plan for where they are not the call's own: a last chunk is planned as the others,
-                               // so that a compiled kernel is not compiled again for it
+    // the order of the filters, if the options give one, is the caller's own and not one that this library chose for a
+    // run from host memory
+    bool callers_order = true;
+    // some columns are read in place from host memory
+    bool in_place = false;
+    // rows to plan for where they are not the call's own: a last chunk is planned as the others, so that a compiled
+    // kernel is not compiled again for it
+    int64_t rows = -1;
 };
 
 } // namespace
@@ -856,7 +859,10 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         hot_stage = -1; // no room beside the group table and the queues
         hot_bytes = 0;
     }
-    auto queue_bytes = [&](int threads) { return P.nq ? (size_t)(threads / 32) * (size_t)(queue0_cap_for(P.slots) + (P.nq - 1) * queue_cap_for(P.rows)) * 4 : (size_t)0; };
+    auto queue_bytes = [&](int threads) -> size_t {
+        const size_t per_warp = (size_t)(queue0_cap_for(P.slots) + (P.nq - 1) * queue_cap_for(P.rows)) * 4;
+        return P.nq ? (size_t)(threads / 32) * per_warp : 0;
+    };
     // Direct tables (and presence bitmaps) worth a copy in shared memory, most probes per staged byte first.
     auto stage_tables = [&](int threads, size_t *tables_out) -> bool {
         for (int s2 = 0; s2 < ns; ++s2) P.st[s2].in_smem = 0, P.st[s2].smem_off = 0;
@@ -1021,9 +1027,9 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
                             dev.sm_count, stream, &launches);
         if (st != SJQ_OK) return st;
     } else if (n > 0) {
-        // Directly behind the clear the kernel is launched while that one still runs (programmatic dependent launch): it
-        // stages its tables, which were complete before the clear began, and waits for the clear before it touches a
-        // result (two-join query, 60 M rows: 94 -> 92 us; filter and sum, 6 M rows: 20.5 -> 18.5 us back to back).
+        // Directly behind the clear the kernel is launched while that one still runs (programmatic dependent launch):
+        // it stages its tables, which were complete before the clear began, and waits for the clear before it touches
+        // a result (two-join query, 60 M rows: 94 -> 92 us; filter and sum, 6 M rows: 20.5 -> 18.5 us back to back).
         const bool behind = !opts.accumulate && hot_stage < 0 && !opts.event_before;
         st = jit ? jit_launch(compiled, P, grid, block, smem, behind, stream)
                  : fused_launch(aggp, mul, has_hash, grid, block, smem, behind, P, stream);
@@ -1034,9 +1040,9 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         return SJQ_ERR_CUDA;
     if (spec->mode == SJQ_HASHED) {
         // (an indexed table has no use for the key array: it holds the block counts of the ordered list)
-        // Launched behind the pass, the listing takes 1 to 3 us less (a list of 20,000 groups, 1 % left: 20 M rows 36.4 ->
-        // 33.5 us, 2 M 18.5 -> 15.3).  Its blocks wait in the SMs meanwhile: one per SM leaves room for other streams'
-        // kernels beside a long pass.
+        // Launched behind the pass, the listing takes 1 to 3 us less (a list of 20,000 groups, 1 % left: 20 M rows
+        // 36.4 -> 33.5 us, 2 M 18.5 -> 15.3).  Its blocks wait in the SMs meanwhile: one per SM leaves room for other
+        // streams' kernels beside a long pass.
         const bool follows = n > 0 && !opts.unfused && !opts.event_after;
         const int beside = !follows ? 0 : n <= (int64_t)1 << 20 ? INT32_MAX : dev.sm_count;
         st = compact_launch(gkeys, cells, direct_groups ? table_groups : (int64_t)gslots, direct_groups, P.post_offset,

@@ -150,9 +150,10 @@ typedef RunParamsOf<kMaxStages> RunParams;
 static_assert(sizeof(RunParams) == sizeof(RunStages<kMaxStages>) + sizeof(RunCore), "no padding between the two");
 
 #if !defined(SJQ_JIT)
-// The ahead-of-time variants of the fused kernel (aggregation path x product aggregate x "some table is open-addressing"
-// x up to kFewStages stages or any number), instantiated in one translation unit per aggregation path and size.  A
-// launch copies its whole parameter block, 6 KB with twelve stages and 21 KB with all (a call of a small query 9.9 -> 8.1 us).
+// The ahead-of-time variants of the fused kernel (aggregation path x product aggregate x "some table is
+// open-addressing" x up to kFewStages stages or any number), instantiated in one translation unit per aggregation
+// path and size.  A launch copies its whole parameter block, 6 KB with twelve stages and 21 KB with all (a call of a
+// small query 9.9 -> 8.1 us).
 typedef RunParamsOf<kFewStages> RunParamsFew;
 typedef void (*fused_few_fn)(const RunParamsFew);
 typedef void (*fused_fn)(const RunParams);

@@ -41,9 +41,9 @@ constexpr int kBucketRoom = 2048;   // entries of a bucket that shared memory ho
 // The longest list: a bucket larger than the room is ranked entry by entry (a list of a million had forty of them and
 // took 2.3 ms; the radix sort takes 0.25), so it must be rare.  Bucket sizes depend on the ranks of the sampled entries
 // alone, not on how the keys are spread, and a bucket of four samples exceeds x times the average with the tail of a
-// gamma distribution of order four: where the average is a fifth of the room, one list in 300 has such a bucket; at half
-// the room, every list.  Six samples a bucket would do at a quarter of the room, but ranking them costs every list beyond
-// 131,072 entries 12 us (merge of eight lists of 200,000 with its sort 108 -> 120).
+// gamma distribution of order four: where the average is a fifth of the room, one list in 300 has such a bucket; at
+// half the room, every list.  Six samples a bucket would do at a quarter of the room, but ranking them costs every
+// list beyond 131,072 entries 12 us (merge of eight lists of 200,000 with its sort 108 -> 120).
 constexpr int64_t kSampleMost = (int64_t)kBuckets * (kBucketRoom / 5);
 constexpr int kBinBits = 11;        // bins of a bucket, as many as it may have entries
 constexpr int kBins = 1 << kBinBits;
@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const __grid
         __syncthreads();
         if (threadIdx.x < 256) {
             for (int w = 0; w < warp; ++w) incl += scan[w];
-            offset[threadIdx.x] = incl - total + part[0][threadIdx.x] + part[1][threadIdx.x] + part[2][threadIdx.x] + part[3][threadIdx.x];
+            const int t = threadIdx.x;
+            offset[t] = incl - total + part[0][t] + part[1][t] + part[2][t] + part[3][t];
         }
     }
     const unsigned long long *const kin = S.k[S.pass & 1];
@@ -562,13 +563,13 @@ __device__ __forceinline__ bool order_bucket(const unsigned long long *key, int 
 }
 
 // A bucket's m entries by one more distribution: bins of equal width over the bucket's range, as many as shared memory
-// holds entries, so that most bins take one or none; an entry's place is its bin's start plus the smaller entries of its
-// bin.  Half a dozen barriers where the network has one pair per step (lists of 400,000 entries: merge and sort 127 us
-// with the network, 106 with the bins; three waves of the network's blocks took 43 of them).  Registers are kept to four
-// blocks per SM: with five, measures spill and it takes 112.  R > 0: m <= R * kBucketThreads, and a thread's
-// entries stay in registers, keys and measures requested before the first wait; R = 0: any m <= kBucketRoom, keys read
-// again (from the L1) in each pass.  False, with nothing written, when a bin takes more than kBinMost entries (keys
-// bunched within the bucket).
+// holds entries, so that most bins take one or none; an entry's place is its bin's start plus the smaller entries of
+// its bin.  Half a dozen barriers where the network has one pair per step (lists of 400,000 entries: merge and sort
+// 127 us with the network, 106 with the bins; three waves of the network's blocks took 43 of them).  Registers are
+// kept to four blocks per SM: with five, measures spill and it takes 112.  R > 0: m <= R * kBucketThreads, and a
+// thread's entries stay in registers, keys and measures requested before the first wait; R = 0: any m <= kBucketRoom,
+// keys read again (from the L1) in each pass.  False, with nothing written, when a bin takes more than kBinMost
+// entries (keys bunched within the bucket).
 template <int R>
 __device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo, int m, unsigned long long *key,
                                            unsigned int *bin, unsigned int *pos, unsigned short *number,
@@ -697,7 +698,8 @@ __global__ void __launch_bounds__(kBucketThreads, 4) sample_bucket_kernel(const 
                 kmax = k > kmax ? k : kmax;
             }
             block_range(kmin, kmax, least, most);
-            // (all ones in the top 53 bits would meet the padding: 2^53 - 1 is the most a distance may reach, exclusive)
+            // (all ones in the top 53 bits would meet the padding: 2^53 - 1 is the most a distance may reach,
+            // exclusive)
             const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > 52 ? bits - 52 : 0;
             if (m <= kBucketThreads) done = order_bucket<1>(key, (int)m, kmin, shift, buf, order);
             else if (m <= 2 * kBucketThreads) done = order_bucket<2>(key, (int)m, kmin, shift, buf, order);

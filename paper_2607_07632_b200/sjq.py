@@ -408,8 +408,8 @@ class TableBuilder:
             self.pay = (ctypes.c_int * max(1, len(payloads)))(*[self.names.index(p) for p in payloads])
             self.opts = _BuildOpts(force_kind, hash_load_pct, max_direct_bytes, min_code_bits, 0)
             self.scratch = torch.empty(PLAN_SCRATCH_BYTES, dtype=torch.uint8, device=self.device)
-            # statistics of the last few scans (page-locked, written by an asynchronous copy), each with the
-            # event that says its copy has landed
+            # statistics of the last few scans (page-locked, written by an asynchronous copy, or by the scan itself
+            # where it is a batch's), each with the event that says they have landed
             self.stats = [torch.zeros(8, dtype=torch.int64, pin_memory=True) for _ in range(4)]
             self.stats_done = [torch.cuda.Event() for _ in self.stats]
             self.stats_used = [False] * len(self.stats)
