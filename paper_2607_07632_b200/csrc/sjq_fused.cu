@@ -18,19 +18,13 @@ struct ClearParams {
     int64_t gslots; // entries of gkeys to set to the empty marker
     int64_t *n_groups;
     int32_t *status;
+    int32_t at_once; // the kernel behind this one may start at once (it waits on the device), else when the stores are out
 };
-
-constexpr unsigned int kClearSmall = 148; // blocks, of 256 threads
 
 // (every array starts on a 16-byte boundary; the odd last word is thread 0's)
 __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
 {
-    // The fused kernel may start and wait for this one on the device: at once where this one leaves most of the chip
-    // idle, else when its stores are out, since blocks that start beside it are spread unevenly over the SMs (sums
-    // and counts of 400,000 groups, 2 M rows: 34.3 us when started at once, 30.5 so, 32.5 one kernel after the
-    // other).
-    const bool small = gridDim.x <= kClearSmall;
-    if (small) asm volatile("griddepcontrol.launch_dependents;");
+    if (C.at_once) asm volatile("griddepcontrol.launch_dependents;");
     const int64_t stride = (int64_t)blockDim.x * gridDim.x;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const longlong2 zero = make_longlong2(0, 0), empty = make_longlong2(kEmptyKey64, kEmptyKey64);
@@ -48,7 +42,7 @@ __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
         if (C.status) *C.status = 0;
         if (C.n_groups) *C.n_groups = 0;
     }
-    if (!small) asm volatile("griddepcontrol.launch_dependents;");
+    if (!C.at_once) asm volatile("griddepcontrol.launch_dependents;");
 }
 
 struct CompactParams {
@@ -353,14 +347,15 @@ sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_
     return SJQ_OK;
 }
 
+// `at_once`: the kernel behind starts beside a clear of so many blocks (of 256 threads) at most.
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
-                        int64_t *n_groups, int32_t *status, int sm_count, cudaStream_t stream)
+                        int64_t *n_groups, int32_t *status, int at_once, int sm_count, cudaStream_t stream)
 {
-    ClearParams C{sums, counts, cells, gkeys, gslots, n_groups, status};
     const int64_t work = (cells > gslots ? cells : gslots) / 2;
     int64_t blocks = (work + 255) / 256;
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     if (blocks < 1) blocks = 1;
+    const ClearParams C{sums, counts, cells, gkeys, gslots, n_groups, status, blocks <= at_once ? 1 : 0};
     clear_kernel<<<(int)blocks, 256, 0, stream>>>(C);
     return cudaGetLastError() == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
