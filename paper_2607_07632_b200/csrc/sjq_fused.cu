@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const Co
 // Group table -> list of (key, sum, count).  A block owns consecutive tiles of cells; a warp takes 256 consecutive
 // cells of a tile.  The place of a block's groups is the number of groups before it (an indexed table: the list comes
 // out in ascending key order), or is drawn from the common counter, once per tile.
-__global__ void __launch_bounds__(kCompactThreads) compact_kernel(const CompactParams C)
+// (Four blocks per SM at 64 registers: merge of eight lists of 200,000 with its sort 106.5 us, 107.9 with 80 registers.)
+__global__ void __launch_bounds__(kCompactThreads, 4) compact_kernel(const CompactParams C)
 {
     __shared__ unsigned int part[kCompactThreads / 32];
     __shared__ long long draw;
