@@ -482,7 +482,7 @@ sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *preds, int np
  * Section 3.3's global table returns its groups in table order, which depends
  * on the hash function and the capacity; the paper compares results through an
  * order-free checksum (Section 2.2), this library gives the list itself an
- * order instead.  A sample sort (up to 418,816 entries) or a radix sort of (key,
+ * order instead.  A sample sort (up to 2^20 entries) or a radix sort of (key,
  * position) pairs on the device; equal keys keep their order.
  *   keys/sums/counts  device arrays of `capacity` entries (8-byte aligned), of
  *                     which the first *n_groups hold the result; sorted in place

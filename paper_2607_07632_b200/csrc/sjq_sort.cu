@@ -11,7 +11,7 @@
 //
 // What bounds it: kernel latency.  A million pairs are 24 MB, which the L2 holds, so a kernel takes 3 to 15 us and it
 // is the number of kernels one after the other that counts.  Two ways, by the capacity of the list:
-//   - up to kSampleMost entries a sample sort, four kernels: splitters from a sorted sample; the bucket of every
+//   - up to kSampleMost entries a sample sort, four or five kernels: splitters from a sorted sample; the bucket of every
 //     entry, counted; the entries into their buckets; every bucket sorted in shared memory (merge of eight lists of
 //     200,000 with its sort: 200 us with the radix sort, 106 with this one);
 //   - beyond, a stable least-significant-digit radix sort of (key - smallest key, position) pairs, 8 bits a pass,
@@ -34,20 +34,31 @@ constexpr int kSortBlocks = 148;                       // one per SM
 constexpr int kSortMinPiece = 2048;                    // elements a block takes before another one is put to work
 constexpr int kSortPasses = 8;
 
+constexpr int64_t kSampleMost = (int64_t)1 << 20;
 constexpr int kBuckets = 1024;      // at most; about 256 entries each in a shorter list
 constexpr int kOversample = 4;      // samples per bucket
-constexpr int kBucketThreads = 256;
-constexpr int kBucketRoom = 2048;   // entries of a bucket that shared memory holds
-// The longest list: a bucket larger than the room is ranked entry by entry (a list of a million had forty of them and
-// took 2.3 ms; the radix sort takes 0.25), so it must be rare.  Bucket sizes depend on the ranks of the sampled entries
-// alone, not on how the keys are spread, and a bucket of four samples exceeds x times the average with the tail of a
-// gamma distribution of order four: where the average is a fifth of the room, one list in 300 has such a bucket; at
-// half the room, every list.  Six samples a bucket would do at a quarter of the room, but ranking them costs every
-// list beyond 131,072 entries 12 us (merge of eight lists of 200,000 with its sort 108 -> 120).
-constexpr int64_t kSampleMost = (int64_t)kBuckets * (kBucketRoom / 5);
-constexpr int kBinBits = 11;        // bins of a bucket, as many as it may have entries
-constexpr int kBins = 1 << kBinBits;
 constexpr int kBinMost = 64;        // entries of a bin that are compared with one another
+
+// The blocks that sort the buckets, by the length of the list, which only the device knows: where the capacity is
+// large both kernels are launched and one of them returns at once.  A bucket larger than the room in shared memory is
+// ranked entry by entry, so it must be rare.  Bucket sizes depend on the ranks of the sampled entries alone, not on
+// how the keys are spread, and a bucket of four samples exceeds x times the average with the tail of a gamma
+// distribution of order four.  Little: four blocks of 256 threads per SM; at its longest the average bucket is a
+// fifth of the room and one list in 300 has a larger one.  Large: one block of 1024 per SM; the average is at most an
+// eighth, one list in 10^7.  (A million unordered entries: 2,300 us with the little blocks, which had forty such
+// buckets in every list, 131 with the large ones, 253 with the radix sort; 430,000 entries 65 and 88.  Six samples a
+// bucket instead of four: ranking them costs every list beyond 131,072 entries 12 us.)
+template <int THREADS, int PER_SM, int ROOM_BITS, int BIN_BITS>
+struct BucketBlocks {
+    static constexpr int kThreads = THREADS, kPerSm = PER_SM;
+    static constexpr bool kLarge = PER_SM == 1;
+    static constexpr int kRoomBits = ROOM_BITS, kRoom = 1 << ROOM_BITS; // entries of a bucket that shared memory holds
+    static constexpr int kBinBits = BIN_BITS, kBins = 1 << BIN_BITS;    // bins of a bucket
+    static constexpr size_t kShared = (size_t)kRoom * (8 + 8 + 2);      // keys, a second array of words, numbers
+};
+typedef BucketBlocks<256, 4, 11, 11> LittleBlocks;
+typedef BucketBlocks<1024, 1, 13, 12> LargeBlocks;
+constexpr int64_t kLittleMost = (int64_t)kBuckets * (LittleBlocks::kRoom / 5);
 
 struct SortRange {
     unsigned long long lo, hi; // smallest and largest key, sign bit flipped
@@ -471,6 +482,7 @@ __global__ void __launch_bounds__(kSortThreads) sample_scatter_kernel(const __gr
 }
 
 // Smallest and largest key of a block's bucket.
+template <class B>
 __device__ __forceinline__ void block_range(unsigned long long &kmin, unsigned long long &kmax, unsigned long long *least,
                                             unsigned long long *most)
 {
@@ -481,27 +493,27 @@ __device__ __forceinline__ void block_range(unsigned long long &kmin, unsigned l
     }
     if ((threadIdx.x & 31) == 0) least[threadIdx.x >> 5] = kmin, most[threadIdx.x >> 5] = kmax;
     __syncthreads();
-    for (int w = 0; w < kBucketThreads / 32; ++w) {
+    for (int w = 0; w < B::kThreads / 32; ++w) {
         kmin = least[w] < kmin ? least[w] : kmin;
         kmax = most[w] > kmax ? most[w] : kmax;
     }
 }
 
-// Sort R * kBucketThreads values by a bitonic network; value r * kBucketThreads + thread sits in v[r].  Partners in the
+// Sort R * B::kThreads values by a bitonic network; value r * B::kThreads + thread sits in v[r].  Partners in the
 // same thread or warp meet in registers, the others in shared memory.
-template <int R>
+template <class B, int R>
 __device__ __forceinline__ void bitonic(unsigned long long (&v)[R], unsigned long long *buf)
 {
     const int tid = threadIdx.x;
-    for (int k = 2; k <= R * kBucketThreads; k <<= 1) {
+    for (int k = 2; k <= R * B::kThreads; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= kBucketThreads) {
+            if (j >= B::kThreads) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
 #pragma unroll
                     for (int o = 1; o < R; o <<= 1) {
-                        if (o * kBucketThreads != j || (r & o)) continue;
-                        const bool up = ((r * kBucketThreads) & k) == 0;
+                        if (o * B::kThreads != j || (r & o)) continue;
+                        const bool up = ((r * B::kThreads) & k) == 0;
                         const unsigned long long a = v[r], b = v[r | o], lo = a < b ? a : b, hi = a < b ? b : a;
                         v[r] = up ? lo : hi;
                         v[r | o] = up ? hi : lo;
@@ -513,10 +525,10 @@ __device__ __forceinline__ void bitonic(unsigned long long (&v)[R], unsigned lon
             if (j >= 32) {
                 __syncthreads(); // what was read the last time
 #pragma unroll
-                for (int r = 0; r < R; ++r) buf[r * kBucketThreads + tid] = v[r];
+                for (int r = 0; r < R; ++r) buf[r * B::kThreads + tid] = v[r];
                 __syncthreads();
 #pragma unroll
-                for (int r = 0; r < R; ++r) other[r] = buf[r * kBucketThreads + (tid ^ j)];
+                for (int r = 0; r < R; ++r) other[r] = buf[r * B::kThreads + (tid ^ j)];
             } else {
 #pragma unroll
                 for (int r = 0; r < R; ++r) other[r] = __shfl_xor_sync(0xffffffffu, v[r], j);
@@ -524,37 +536,36 @@ __device__ __forceinline__ void bitonic(unsigned long long (&v)[R], unsigned lon
             const bool low = (tid & j) == 0;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const bool up = ((r * kBucketThreads + tid) & k) == 0, least = low == up;
+                const bool up = ((r * B::kThreads + tid) & k) == 0, least = low == up;
                 v[r] = (v[r] < other[r]) == least ? v[r] : other[r];
             }
         }
     }
 }
 
-// Order of a bucket's m <= R * kBucketThreads entries: order[i] = the entry that comes i-th.  The values sorted are the
-// top 53 bits of the distance from the bucket's smallest key, then the entry's number: one word instead of key and
+// Order of a bucket's m <= R * B::kThreads entries: order[i] = the entry that comes i-th.  The values sorted are the
+// top bits of the distance from the bucket's smallest key, then the entry's number: one word instead of key and
 // position.  False when two neighbours agree in those bits.
-template <int R>
+template <class B, int R>
 __device__ __forceinline__ bool order_bucket(const unsigned long long *key, int m, unsigned long long kmin, int shift,
                                              unsigned long long *buf, unsigned short *order)
 {
-    constexpr int kNumberBits = 11;
-    static_assert(kBucketRoom <= (1 << kNumberBits), "an entry's number");
+    constexpr int kNumberBits = B::kRoomBits;
     unsigned long long v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int e = r * kBucketThreads + (int)threadIdx.x;
+        const int e = r * B::kThreads + (int)threadIdx.x;
         v[r] = e < m ? ((key[e] - kmin) >> shift) << kNumberBits | (unsigned long long)e : ~0ull;
     }
-    bitonic<R>(v, buf);
+    bitonic<B, R>(v, buf);
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < R; ++r) buf[r * kBucketThreads + threadIdx.x] = v[r];
+    for (int r = 0; r < R; ++r) buf[r * B::kThreads + threadIdx.x] = v[r];
     __syncthreads();
     bool same = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int e = r * kBucketThreads + (int)threadIdx.x;
+        const int e = r * B::kThreads + (int)threadIdx.x;
         if (e >= m) continue;
         order[e] = (unsigned short)(v[r] & ((1u << kNumberBits) - 1u));
         same |= e + 1 < m && (buf[e + 1] ^ v[r]) >> kNumberBits == 0;
@@ -566,16 +577,16 @@ __device__ __forceinline__ bool order_bucket(const unsigned long long *key, int 
 // holds entries, so that most bins take one or none; an entry's place is its bin's start plus the smaller entries of
 // its bin.  Half a dozen barriers where the network has one pair per step (lists of 400,000 entries: merge and sort
 // 127 us with the network, 106 with the bins; three waves of the network's blocks took 43 of them).  Registers are
-// kept to four blocks per SM: with five, measures spill and it takes 112.  R > 0: m <= R * kBucketThreads, and a
-// thread's entries stay in registers, keys and measures requested before the first wait; R = 0: any m <= kBucketRoom,
+// kept to four blocks per SM: with five, measures spill and it takes 112.  R > 0: m <= R * B::kThreads, and a
+// thread's entries stay in registers, keys and measures requested before the first wait; R = 0: any m <= B::kRoom,
 // keys read again (from the L1) in each pass.  False, with nothing written, when a bin takes more than kBinMost
 // entries (keys bunched within the bucket).
-template <int R>
+template <class B, int R>
 __device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo, int m, unsigned long long *key,
                                            unsigned int *bin, unsigned int *pos, unsigned short *number,
                                            unsigned long long *least, unsigned long long *most, unsigned int *warp_sum)
 {
-    constexpr int kPerThread = kBins / kBucketThreads, kKept = R > 0 ? R : 1;
+    constexpr int kBins = B::kBins, kPerThread = kBins / B::kThreads, kKept = R > 0 ? R : 1;
     static_assert(kPerThread % 4 == 0, "whole 128-bit words");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned long long k[kKept], kmin = ~0ull, kmax = 0ull;
@@ -584,21 +595,21 @@ __device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo,
     if (R > 0) {
 #pragma unroll
         for (int r = 0; r < kKept; ++r) {
-            const int e = r * kBucketThreads + tid;
+            const int e = r * B::kThreads + tid;
             if (e < m) k[r] = S.k[1][lo + e], p[r] = S.p[1][lo + e];
         }
 #pragma unroll
         for (int r = 0; r < kKept; ++r)
-            if (r * kBucketThreads + tid < m) sum[r] = S.tsums[p[r]], count[r] = S.tcounts[p[r]];
+            if (r * B::kThreads + tid < m) sum[r] = S.tsums[p[r]], count[r] = S.tcounts[p[r]];
     }
     auto entries = [&](auto &&f) { // f(slot, entry, its key) for every entry of this thread
         if (R > 0) {
 #pragma unroll
             for (int r = 0; r < kKept; ++r)
-                if (r * kBucketThreads + tid < m) f(r, r * kBucketThreads + tid, k[r]);
+                if (r * B::kThreads + tid < m) f(r, r * B::kThreads + tid, k[r]);
         } else {
 #pragma unroll 1
-            for (int e = tid; e < m; e += kBucketThreads) f(0, e, S.k[1][lo + e]);
+            for (int e = tid; e < m; e += B::kThreads) f(0, e, S.k[1][lo + e]);
         }
     };
     uint4 *words = reinterpret_cast<uint4 *>(bin) + tid * (kPerThread / 4);
@@ -608,8 +619,8 @@ __device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo,
         kmin = x < kmin ? x : kmin;
         kmax = x > kmax ? x : kmax;
     });
-    block_range(kmin, kmax, least, most);
-    const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > kBinBits ? bits - kBinBits : 0;
+    block_range<B>(kmin, kmax, least, most);
+    const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > B::kBinBits ? bits - B::kBinBits : 0;
     entries([&](int, int e, unsigned long long x) {
         number[e] = (unsigned short)atomicAdd(&bin[(x - kmin) >> shift], 1u);
     });
@@ -657,20 +668,23 @@ __device__ __forceinline__ bool bin_bucket(const SortParams &S, unsigned int lo,
 }
 
 // Sort the buckets, a block each: by bins, or by the network where the keys are bunched.  Where bunched keys are equal,
-// or so far apart that the 53 bits do not tell them apart, or a bucket is larger than shared memory (an unlucky sample,
-// see kSampleMost), its entries are ranked one by one against the whole bucket.
-__global__ void __launch_bounds__(kBucketThreads, 4) sample_bucket_kernel(const __grid_constant__ SortParams S)
+// or so far apart that the top bits do not tell them apart, or a bucket is larger than shared memory (an unlucky
+// sample), its entries are ranked one by one against the whole bucket.
+template <class B>
+__global__ void __launch_bounds__(B::kThreads, B::kPerSm) sample_bucket_kernel(const __grid_constant__ SortParams S)
 {
-    __shared__ __align__(16) unsigned long long key[kBucketRoom], buf[kBucketRoom];
-    __shared__ unsigned short order[kBucketRoom];
-    __shared__ unsigned int start[kBuckets], warp_sum[kBucketThreads / 32];
-    __shared__ unsigned long long least[kBucketThreads / 32], most[kBucketThreads / 32];
-    static_assert(kBucketThreads == kBuckets / 4, "bucket_starts takes so many threads");
-    static_assert(8 * (size_t)kBucketRoom >= 4 * (size_t)(kBins + kBucketRoom),
-                  "bins and positions fit beside the keys");
+    extern __shared__ __align__(16) unsigned long long key[]; // B::kShared bytes
+    unsigned long long *const buf = key + B::kRoom;
+    unsigned short *const order = reinterpret_cast<unsigned short *>(buf + B::kRoom);
+    __shared__ unsigned int start[kBuckets], warp_sum[B::kThreads / 32];
+    __shared__ unsigned long long least[B::kThreads / 32], most[B::kThreads / 32];
+    static_assert(B::kThreads >= kBuckets / 4, "bucket_starts takes so many threads");
+    static_assert(8 * (size_t)B::kRoom >= 4 * (size_t)(B::kBins + B::kRoom), "bins and positions fit beside the keys");
     cudaGridDependencySynchronize();
-    if (list_in_order(S)) return;
-    const int nb = buckets_for(sort_count(S));
+    const int64_t n = sort_count(S);
+    const bool ordered = list_in_order(S);
+    if (ordered || B::kLarge != (n > kLittleMost)) return;
+    const int nb = buckets_for(n);
     bucket_starts(S, nb, start, warp_sum);
     auto store = [&](unsigned int at, unsigned long long k, unsigned int p) {
         S.keys[at] = (int64_t)(k ^ 0x8000000000000000ull);
@@ -681,35 +695,35 @@ __global__ void __launch_bounds__(kBucketThreads, 4) sample_bucket_kernel(const 
         const unsigned int lo = start[b], m = S.bucket_total[b];
         if (m == 0) continue;
         bool done = false;
-        unsigned int *const bin = reinterpret_cast<unsigned int *>(buf), *const pos = bin + kBins;
+        unsigned int *const bin = reinterpret_cast<unsigned int *>(buf), *const pos = bin + B::kBins;
         __syncthreads(); // the bucket before has been written out
-        if (m <= kBucketThreads) done = bin_bucket<1>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
-        else if (m <= 2 * kBucketThreads) done = bin_bucket<2>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
-        else if (m <= (unsigned int)kBucketRoom)
-            done = bin_bucket<0>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
+        if (m <= B::kThreads) done = bin_bucket<B, 1>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
+        else if (m <= 2 * B::kThreads) done = bin_bucket<B, 2>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
+        else if (m <= (unsigned int)B::kRoom)
+            done = bin_bucket<B, 0>(S, lo, (int)m, key, bin, pos, order, least, most, warp_sum);
         if (done) continue;
-        if (m <= (unsigned int)kBucketRoom) {
+        if (m <= (unsigned int)B::kRoom) {
             __syncthreads(); // the bins have been read
             unsigned long long kmin = ~0ull, kmax = 0ull;
-            for (int e = threadIdx.x; e < (int)m; e += kBucketThreads) {
+            for (int e = threadIdx.x; e < (int)m; e += B::kThreads) {
                 const unsigned long long k = S.k[1][lo + e];
                 key[e] = k;
                 kmin = k < kmin ? k : kmin;
                 kmax = k > kmax ? k : kmax;
             }
-            block_range(kmin, kmax, least, most);
-            // (all ones in the top 53 bits would meet the padding: 2^53 - 1 is the most a distance may reach,
-            // exclusive)
-            const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > 52 ? bits - 52 : 0;
-            if (m <= kBucketThreads) done = order_bucket<1>(key, (int)m, kmin, shift, buf, order);
-            else if (m <= 2 * kBucketThreads) done = order_bucket<2>(key, (int)m, kmin, shift, buf, order);
-            else if (m <= 4 * kBucketThreads) done = order_bucket<4>(key, (int)m, kmin, shift, buf, order);
-            else done = order_bucket<8>(key, (int)m, kmin, shift, buf, order);
+            block_range<B>(kmin, kmax, least, most);
+            // (a distance of all ones would meet the padding: one bit less than the entry's number leaves)
+            constexpr int kDistance = 63 - B::kRoomBits;
+            const int bits = 64 - __clzll((long long)(kmax - kmin)), shift = bits > kDistance ? bits - kDistance : 0;
+            if (m <= B::kThreads) done = order_bucket<B, 1>(key, (int)m, kmin, shift, buf, order);
+            else if (m <= 2 * B::kThreads) done = order_bucket<B, 2>(key, (int)m, kmin, shift, buf, order);
+            else if (m <= 4 * B::kThreads) done = order_bucket<B, 4>(key, (int)m, kmin, shift, buf, order);
+            else done = order_bucket<B, 8>(key, (int)m, kmin, shift, buf, order);
             if (done)
-                for (int e = threadIdx.x; e < (int)m; e += kBucketThreads) store(lo + e, key[order[e]], S.p[1][lo + order[e]]);
+                for (int e = threadIdx.x; e < (int)m; e += B::kThreads) store(lo + e, key[order[e]], S.p[1][lo + order[e]]);
         }
         if (done) continue;
-        for (unsigned int e = threadIdx.x; e < m; e += kBucketThreads) {
+        for (unsigned int e = threadIdx.x; e < m; e += B::kThreads) {
             const unsigned long long k = S.k[1][lo + e];
             const unsigned int p = S.p[1][lo + e];
             unsigned int before = 0;
@@ -757,7 +771,8 @@ SortLayout sort_layout(int64_t capacity)
 
 // Launch behind the previous kernel of the sort without waiting for it: every kernel but the first waits on the
 // device (cudaGridDependencySynchronize) before it touches what its predecessors wrote.
-bool launch_behind(void (*kernel)(SortParams), int grid, int threads, const SortParams &S, cudaStream_t stream)
+bool launch_behind(void (*kernel)(SortParams), int grid, int threads, const SortParams &S, cudaStream_t stream,
+                   size_t shared = 0)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -765,10 +780,23 @@ bool launch_behind(void (*kernel)(SortParams), int grid, int threads, const Sort
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = shared;
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, S) == cudaSuccess;
+}
+
+template <class B>
+bool launch_buckets(int64_t most, const SortParams &S, cudaStream_t stream)
+{
+    void (*const kernel)(SortParams) = sample_bucket_kernel<B>;
+    if (B::kShared > ((size_t)40 << 10) &&
+        cudaFuncSetAttribute(reinterpret_cast<const void *>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)B::kShared) != cudaSuccess)
+        return false;
+    const int64_t buckets = std::min<int64_t>((S.capacity + 127) / 128, most);
+    return launch_behind(kernel, (int)buckets, B::kThreads, S, stream, B::kShared);
 }
 
 } // namespace
@@ -820,11 +848,11 @@ extern "C" sjq_status sjq_result_sort(int64_t *keys, int64_t *sums, int64_t *cou
     S.pieces = L.nblocks;
     bool ok;
     if (L.sample) {
-        const int64_t buckets = std::min<int64_t>((capacity + 127) / 128, kBuckets);
         sample_split_kernel<<<L.nblocks, kSortThreads, 0, stream>>>(S);
         ok = cudaGetLastError() == cudaSuccess && launch_behind(sample_count_kernel, L.nblocks, kSortThreads, S, stream) &&
              launch_behind(sample_scatter_kernel, L.nblocks, kSortThreads, S, stream) &&
-             launch_behind(sample_bucket_kernel, (int)buckets, kBucketThreads, S, stream);
+             launch_buckets<LittleBlocks>(kBuckets, S, stream) &&
+             (capacity <= kLittleMost || launch_buckets<LargeBlocks>(kSortBlocks, S, stream));
     } else {
         sort_range_kernel<<<L.nblocks, kSortThreads, 0, stream>>>(S);
         ok = cudaGetLastError() == cudaSuccess;
@@ -842,14 +870,16 @@ extern "C" sjq_status sjq_result_sort(int64_t *keys, int64_t *sums, int64_t *cou
 }
 
 // The sampler as the kernels use it, for tests on the host (not part of the interface): the positions sampled in a list
-// of n entries (`positions` NULL: none are written); returns their number.
+// of n entries (`positions` NULL: none are written); returns their number.  `room`: entries of a bucket that shared
+// memory holds; `little`, `most`: the longest lists of the two forms of the sample sort.
 extern "C" int32_t sjq_result_sort_samples(int64_t n, int64_t *positions, int32_t *per_bucket, int32_t *room,
-                                           int64_t *most)
+                                           int64_t *little, int64_t *most)
 {
     const int nb = buckets_for(n), ns = nb > 1 ? nb * kOversample : 0;
     for (int i = 0; positions && i < ns; ++i) positions[i] = sample_at(i, ns, n);
     *per_bucket = kOversample;
-    *room = kBucketRoom;
+    *room = n <= kLittleMost ? LittleBlocks::kRoom : LargeBlocks::kRoom;
+    *little = kLittleMost;
     *most = kSampleMost;
     return ns;
 }

@@ -7,21 +7,22 @@ import paper_2607_07632_b200.sjq as b
 
 
 def samples(n):
-    """(sampled positions, samples per bucket, entries of a bucket that shared memory holds, longest list sorted so)."""
+    """Of a list of n entries: sampled positions; samples per bucket; entries of a bucket that shared memory holds; the
+    longest lists of the two forms of the sample sort."""
     f = b.lib().sjq_result_sort_samples
     f.argtypes = [ctypes.c_int64, ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32),
-                  ctypes.POINTER(ctypes.c_int64)]
-    per, room, most = ctypes.c_int32(0), ctypes.c_int32(0), ctypes.c_int64(0)
-    count = f(n, None, ctypes.byref(per), ctypes.byref(room), ctypes.byref(most))
-    at = np.zeros(count, np.int64)
-    assert f(n, at.ctypes.data, ctypes.byref(per), ctypes.byref(room), ctypes.byref(most)) == count
-    return at, per.value, room.value, most.value
+                  ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
+    per, room, little, most = ctypes.c_int32(0), ctypes.c_int32(0), ctypes.c_int64(0), ctypes.c_int64(0)
+    refs = [ctypes.byref(v) for v in (per, room, little, most)]
+    at = np.zeros(f(n, None, *refs), np.int64)
+    assert f(n, at.ctypes.data, *refs) == len(at)
+    return at, per.value, room.value, little.value, most.value
 
 
 def bucket_sizes(keys):
     """Entries per bucket: splitters are every per-th of the sorted sample, by key and then by position."""
     n = len(keys)
-    at, per, _, _ = samples(n)
+    at, per = samples(n)[:2]
     if not len(at):
         return np.array([n])
     order = np.argsort(keys, kind="stable")

@@ -34,7 +34,7 @@ def test_list_lengths_around_pieces_and_tiles(n):
 
 
 @pytest.mark.parametrize("bits", [1, 8, 9, 16, 24, 33, 40, 48, 56, 63])
-@pytest.mark.parametrize("capacity", [32_768, 2**20 + 1])  # sample sort, radix sort
+@pytest.mark.parametrize("capacity", [32_768, 2**20, 2**20 + 1])  # sample sort in one and in either kernel; radix sort
 def test_every_number_of_passes_with_equal_keys(bits, capacity):
     n = 20_011
     rng = np.random.default_rng(bits)
@@ -45,7 +45,7 @@ def test_every_number_of_passes_with_equal_keys(bits, capacity):
     _check(keys, capacity)
 
 
-@pytest.mark.parametrize("capacity", [300_000, 2**20 + 5])
+@pytest.mark.parametrize("capacity", [300_000, 700_000, 2**20 + 5])
 def test_clustered_keys_and_a_lone_outlier(capacity):
     rng = np.random.default_rng(4)
     keys = np.concatenate([rng.permutation(100_000), rng.permutation(100_000) + 2**50, [-2**63, 2**63 - 1],
@@ -58,9 +58,9 @@ def test_buckets_larger_than_shared_memory_are_ranked():
     # the sampled positions hold small keys only: all other entries fall into one bucket
     n = 40_000
     keys = np.random.default_rng(1).permutation(n).astype(np.int64) + 10**6
-    at, _, room, _ = samples(n)
+    at = samples(n)[0]
     keys[at] = np.arange(len(at))
-    assert bucket_sizes(keys).max() > 10 * room
+    assert bucket_sizes(keys).max() > 10 * samples(n)[2]
     _check(keys, n)
 
 
@@ -83,14 +83,45 @@ def test_one_bucket_of_spread_and_of_bunched_keys(last, bunch):
     bunched = rng.choice(n, bunch, replace=False)
     keys[bunched] = (np.int64(2**62)) + rng.permutation(bunch)
     keys[bunched[: bunch // 8]] = 2**62 + 3  # equal ones keep their order
-    at, _, _, _ = samples(n)
+    at = samples(n)[0]
     keys[at] = np.arange(len(at))
     assert bucket_sizes(keys)[-1] == last
     _check(keys, n + 1)
 
 
-@pytest.mark.parametrize("beyond", [-7, -6, 200_000, 600_000])
-def test_unordered_lists_on_both_sides_of_the_longest_sample_sort(beyond):
-    n = samples(1000)[3] + beyond
+@pytest.mark.parametrize("last", [200, 1024, 1025, 2048, 2049, 4096, 4097, 8192, 8193])
+@pytest.mark.parametrize("bunch", [1, 64, 65, 66, 180])
+def test_one_bucket_of_a_long_list(last, bunch):
+    # 430,000 entries, whose buckets the larger blocks sort: samples at equal distances, `last` entries beyond the last
+    # splitter, `bunch` of them neighbours, all others below it
+    n, rng = 430_000, np.random.default_rng(last + bunch)
+    at, per = samples(n)[:2]
+    assert n > samples(n)[3]
+    top, inside = (len(at) - per) << 40, last - per
+    rest = rng.permutation(np.setdiff1d(np.arange(n), at))
+    keys = np.empty(n, np.int64)
+    keys[at] = np.arange(len(at)) << 40
+    keys[rest[inside:]] = rng.integers(0, top, n - len(at) - inside)
+    keys[rest[:inside]] = top + 1 + rng.permutation(inside) * (2**42 // inside)
+    keys[rest[:bunch]] = top + 2**41 + rng.permutation(bunch)
+    keys[rest[: bunch // 8]] = top + 2**41 + 3  # equal ones keep their order
+    assert bucket_sizes(keys)[-1] == last
+    _check(keys, n + 1)
+
+
+@pytest.mark.parametrize("form", [3, 4])
+@pytest.mark.parametrize("beyond", [-7, -6, 200_000])
+def test_unordered_lists_on_both_sides_of_the_longest_of_either_form(form, beyond):
+    n = samples(1000)[form] + beyond
     keys = np.random.default_rng(n).permutation(n).astype(np.int64) * 0x9E3779B97F4A7 - 2**40
     _check(keys, n + 7)
+
+
+@pytest.mark.parametrize("n", [1, 2, 300, 5_000, 418_816, 418_817])
+def test_lists_shorter_than_their_capacity(n):
+    rng = np.random.default_rng(n)
+    for capacity in (500_000, 2**20):
+        _check(rng.permutation(n).astype(np.int64) * 0x9E3779B97F4A7 - 2**40, capacity)
+        _check(np.arange(n, dtype=np.int64), capacity)
+        _check(rng.integers(0, 9, n), capacity)
+        _check((np.arange(n) // 200 * 2**33 + rng.integers(0, 100, n))[rng.permutation(n)], capacity)  # bunched
