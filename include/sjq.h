@@ -400,8 +400,12 @@ typedef struct sjq_run_opts {
                         SJQ_ERR_ASYNC_WAIT in *out->status and the kernel goes on with loads.  3 = as 1, but the
                         copies are never issued: every wait runs out (well under a second each), which is how the
                         tests reach that path without faulting anything; the result is still exact. */
+    void *sync; /* device scratch of SJQ_SYNC_BYTES bytes (8-byte aligned, of any content) that goes with `out`: used by
+                   this run and by nothing else until the run is over.  With it a run over few rows clears a scalar or
+                   dense result in its pass, which saves the clear kernel; NULL = a kernel of its own clears the result */
 } sjq_run_opts;
 
+#define SJQ_SYNC_BYTES 64
 #define SJQ_HOT_SCRATCH_BYTES ((size_t)3 * 1048576 + 65536)
 
 /* What the planner decided for a run (for reports and tests). */
@@ -469,8 +473,8 @@ sjq_status sjq_run_workspace_bytes(const sjq_result_spec *spec, size_t *bytes);
  *   agg          value summed per group
  *   out          result buffers; cleared by this call unless opts->accumulate
  *   info         optional: receives the plan that was used
- * Enqueues a clear kernel, the fused kernel and (HASHED) a compaction kernel
- * on `stream`; does not synchronise.  Host-detected errors are returned;
+ * Enqueues a clear kernel (unless opts->sync lets the pass clear the result), the
+ * fused kernel and (HASHED) a compaction kernel on `stream`; does not synchronise.  Host-detected errors are returned;
  * device-detected errors (GROUP_RANGE, GROUP_OVERFLOW) go to *out->status.
  */
 sjq_status sjq_run(const sjq_col *fact, int nfact, const sjq_pred *preds, int npreds, const sjq_join *joins,

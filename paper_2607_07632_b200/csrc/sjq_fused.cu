@@ -252,16 +252,16 @@ __global__ void __launch_bounds__(256) sample_kernel(const __grid_constant__ Sam
         atomicAdd(&S.counts[threadIdx.x], (unsigned long long)block_counts[threadIdx.x]);
 }
 
-const void *pick_kernel(int agg, bool mul, bool hash, bool few)
+const void *pick_kernel(int agg, bool mul, int form, bool few)
 {
     const auto of = [few](fused_few_fn little, fused_fn any) {
         return few ? reinterpret_cast<const void *>(little) : reinterpret_cast<const void *>(any);
     };
     switch (agg) {
-    case AGG_SCALAR: return of(fused_few_scalar(mul, hash), fused_variant_scalar(mul, hash));
-    case AGG_SMEM: return of(fused_few_smem(mul, hash), fused_variant_smem(mul, hash));
-    case AGG_GLOBAL: return of(fused_few_global(mul, hash), fused_variant_global(mul, hash));
-    default: return of(fused_few_hash(mul, hash), fused_variant_hash(mul, hash));
+    case AGG_SCALAR: return of(fused_few_scalar(mul, form), fused_variant_scalar(mul, form));
+    case AGG_SMEM: return of(fused_few_smem(mul, form), fused_variant_smem(mul, form));
+    case AGG_GLOBAL: return of(fused_few_global(mul, form), fused_variant_global(mul, form));
+    default: return of(fused_few_hash(mul, form), fused_variant_hash(mul, form));
     }
 }
 
@@ -285,7 +285,7 @@ int fused_cache_clear()
     return n;
 }
 
-sjq_status fused_occupancy(int agg, bool mul, bool hash, int nstages, int block, size_t smem, int *ctas_per_sm)
+sjq_status fused_occupancy(int agg, bool mul, int form, int nstages, int block, size_t smem, int *ctas_per_sm)
 {
     const bool few = nstages <= kFewStages;
     std::mutex &mutex = g_occ_mutex;
@@ -293,11 +293,11 @@ sjq_status fused_occupancy(int agg, bool mul, bool hash, int nstages, int block,
     std::unordered_map<uint32_t, int> &opted = g_opted;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SJQ_ERR_CUDA;
-    const uint32_t variant = (uint32_t)(agg * 8 + (mul ? 4 : 0) + (hash ? 2 : 0) + (few ? 1 : 0));
-    const uint32_t fkey = (uint32_t)dev * 64u + variant;
+    const uint32_t variant = (uint32_t)(agg * 32 + form * 4 + (mul ? 2 : 0) + (few ? 1 : 0));
+    const uint32_t fkey = (uint32_t)dev * 128u + variant;
     const uint64_t okey = ((uint64_t)fkey << 40) | ((uint64_t)block << 24) | (uint64_t)(smem & 0xFFFFFF);
     std::lock_guard<std::mutex> lock(mutex);
-    const void *fn = pick_kernel(agg, mul, hash, few);
+    const void *fn = pick_kernel(agg, mul, form, few);
     auto o = opted.find(fkey);
     if (o == opted.end() || o->second < (int)smem) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
@@ -319,7 +319,7 @@ sjq_status fused_occupancy(int agg, bool mul, bool hash, int nstages, int block,
     return SJQ_OK;
 }
 
-sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, bool behind,
+sjq_status fused_launch(int agg, bool mul, int form, int grid, int block, size_t smem, bool behind,
                         const RunParams &P, cudaStream_t stream)
 {
     cudaLaunchAttribute attr{};
@@ -341,7 +341,7 @@ sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_
     } else {
         args[0] = const_cast<RunParams *>(&P);
     }
-    if (cudaLaunchKernelExC(&cfg, pick_kernel(agg, mul, hash, P.nstages <= kFewStages), args) != cudaSuccess) {
+    if (cudaLaunchKernelExC(&cfg, pick_kernel(agg, mul, form, P.nstages <= kFewStages), args) != cudaSuccess) {
         (void)cudaGetLastError();
         return SJQ_ERR_CUDA;
     }

@@ -171,9 +171,9 @@ __device__ __forceinline__ uint32_t body_pred_set(const RunArg &P, const DStage 
     return m & pass;
 }
 
-template <typename T, int OP, bool SMEM, int NR, bool WANT>
+template <typename T, int OP, bool SMEM, int NR, bool WANT, typename C>
 __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned char *smem, const T (&v)[NR],
-                                                uint32_t m, uint64_t (&code)[NR])
+                                                uint32_t m, C (&code)[NR])
 {
     const unsigned char *base = SMEM ? smem + S.smem_off : static_cast<const unsigned char *>(S.tab);
     // A key outside the table's range is a miss, never an out-of-range access: its index is clamped to the
@@ -230,10 +230,12 @@ __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned 
         }
         return m & hit;
     } else {
-        uint64_t c[NR];
+        // (codes stay in the caller's word: a compiled kernel, whose words have 64 bits, takes 86.3 us with 32-bit ones
+        // here and 84.4 without, two joins, 60 M rows)
+        C c[NR];
 #pragma unroll
         for (int i = 0; i < NR; ++i) {
-            c[i] = ~0ULL;
+            c[i] = (C)~0ULL;
             if ((m >> i) & 1u) {
                 if (OP == OP_DIRECT_U8) {
                     const uint8_t *p = base + idx[i];
@@ -250,8 +252,8 @@ __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned 
                 }
             }
         }
-        const uint64_t miss = OP == OP_DIRECT_U8 ? 0xFFull : OP == OP_DIRECT_U16 ? 0xFFFFull
-                              : OP == OP_DIRECT_U32 ? 0xFFFFFFFFull : ~0ULL;
+        const C miss = OP == OP_DIRECT_U8 ? (C)0xFFull : OP == OP_DIRECT_U16 ? (C)0xFFFFull
+                       : OP == OP_DIRECT_U32 ? (C)0xFFFFFFFFull : (C)~0ULL;
 #pragma unroll
         for (int i = 0; i < NR; ++i) {
             hit |= (uint32_t)(c[i] != miss) << i;
@@ -411,10 +413,13 @@ __device__ __forceinline__ uint32_t body_hashbits(const DStage &S, const unsigne
     return hit | known;
 }
 
-template <typename T, int NR, bool WANT, bool HASH>
+// C: the word codes are held in; with 32 bits there are neither 64-bit codes nor open-addressing tables.
+template <typename T, int NR, bool WANT, bool HASH, typename C>
 __device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, const unsigned char *smem,
-                                              const T (&v)[NR], uint32_t m, uint64_t (&code)[NR])
+                                              const T (&v)[NR], uint32_t m, C (&code)[NR])
 {
+    constexpr bool kWide = sizeof(C) == 8;
+    static_assert(kWide || !HASH, "open-addressing tables have 64-bit codes");
     switch (S.op * 2 + S.in_smem) {
     case OP_PRED_RANGE * 2: return body_pred_range<T, NR>(S, v, m);
     case OP_PRED_SET * 2: return body_pred_set<T, NR>(P, S, v, m);
@@ -426,8 +431,8 @@ __device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, 
     case OP_DIRECT_U16 * 2 + 1: return body_direct<T, OP_DIRECT_U16, true, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U32 * 2: return body_direct<T, OP_DIRECT_U32, false, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U32 * 2 + 1: return body_direct<T, OP_DIRECT_U32, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U64 * 2: return body_direct<T, OP_DIRECT_U64, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U64 * 2 + 1: return body_direct<T, OP_DIRECT_U64, true, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U64 * 2: return !kWide ? m : body_direct<T, OP_DIRECT_U64, false, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U64 * 2 + 1: return !kWide ? m : body_direct<T, OP_DIRECT_U64, true, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U4 * 2: return body_direct<T, OP_DIRECT_U4, false, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U4 * 2 + 1: return body_direct<T, OP_DIRECT_U4, true, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U2 * 2: return body_direct<T, OP_DIRECT_U2, false, NR, WANT>(S, smem, v, m, code);
@@ -435,7 +440,7 @@ __device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, 
     case OP_HASHBITS * 2: return HASH ? body_hashbits<T, NR>(S, smem, v, m) : 0u; // comes with an exact probe stage
     case OP_HASH32 * 2:
     case OP_HASH64 * 2:
-        if (HASH) {
+        if constexpr (HASH) {
             if (S.code_bits == 0) return body_hash<T, 0, NR, WANT>(S, smem, v, m, code);
             if (S.code_bits == 32) return body_hash<T, 4, NR, WANT>(S, smem, v, m, code);
             return body_hash<T, 8, NR, WANT>(S, smem, v, m, code);
@@ -466,12 +471,12 @@ __device__ __forceinline__ void add_scaled32(int64_t (&dst)[NR], int32_t mult, c
         if ((m >> k) & 1u) dst[k] += (int64_t)mult * val[k]; // one widening multiply-add
 }
 
-template <bool MUL, typename T, int NR>
-__device__ __forceinline__ void accumulate(const DStage &S, const T (&v)[NR], const uint64_t (&code)[NR], uint32_t m,
+template <bool MUL, typename T, int NR, typename C>
+__device__ __forceinline__ void accumulate(const DStage &S, const T (&v)[NR], const C (&code)[NR], uint32_t m,
                                            int64_t (&key)[NR], int64_t (&X)[NR], int64_t (&Y)[NR])
 {
     const uint32_t acc = S.acc;
-    if (S.acc32 && sizeof(T) == 4) {
+    if (sizeof(C) == 4 || (S.acc32 && sizeof(T) == 4)) {
         if (acc & 0x7u) {
             int32_t r[NR];
 #pragma unroll
@@ -592,15 +597,26 @@ __device__ __forceinline__ uint64_t smem_cell(const unsigned int *words, uint64_
     return ((uint64_t)words[ng + g] << 32) | words[g];
 }
 
+// A row's group key is out of range.  Where a block's sums are its own (registers, a shared group table) the fused kernel
+// notes it in shared memory and tells it at the end, when the status word is known to be clear.
+__shared__ uint32_t range_seen;
+template <bool LATER>
+__device__ __forceinline__ void note_range(const RunArg &P)
+{
+    if (LATER) range_seen = 1u;
+    else set_status(P.status, SJQ_ERR_GROUP_RANGE);
+}
+
 // The terminal on a batch: group keys of all rows first (their divisions overlap), then the
 // aggregation; every test on the query shape is uniform and outside the row loops.
-// PAIRS: every lane of the warp arrives here (with or without rows), so lanes may work on each other's rows.
-template <int AGG, bool MUL, int NR, bool PAIRS = true>
+// FUSED: called by the fused kernel, where every lane of the warp arrives here (with or without rows), so that lanes may
+// work on each other's rows.
+template <int AGG, bool MUL, int NR, bool FUSED = true>
 __device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, const int64_t (&key)[NR],
                                          const int64_t (&X)[NR], const int64_t (&Y)[NR], uint32_t m, int64_t &lsum,
                                          int64_t &lcnt)
 {
-    const bool pairs = PAIRS && (AGG == AGG_GLOBAL || AGG == AGG_HASH) && SJQ_PV(pairs) != 0;
+    const bool pairs = FUSED && (AGG == AGG_GLOBAL || AGG == AGG_HASH) && SJQ_PV(pairs) != 0;
     if (pairs ? !__any_sync(0xffffffffu, m != 0u) : m == 0u) return;
     int64_t val[NR];
 #pragma unroll
@@ -634,7 +650,7 @@ __device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, c
 #pragma unroll
             for (int k = 0; k < NR; ++k)
                 if (((m >> k) & 1u) && g[k] != 0) {
-                    set_status(P.status, SJQ_ERR_GROUP_RANGE);
+                    note_range<FUSED>(P);
                     m &= ~(1u << k);
                 }
         }
@@ -662,7 +678,7 @@ __device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, c
 #pragma unroll
     for (int k = 0; k < NR; ++k)
         if (((m >> k) & 1u) && (uint64_t)g[k] >= ng) {
-            set_status(P.status, SJQ_ERR_GROUP_RANGE);
+            note_range<FUSED && AGG == AGG_SMEM>(P);
             m &= ~(1u << k);
         }
     const bool want_count = SJQ_PV(want_count) != 0;
@@ -762,16 +778,28 @@ __device__ __forceinline__ void load_rows(const DStage &S, int64_t base, const u
     }
 }
 
+// NARROW kernels: every fact column and every code of the query has 32 bits.
+template <bool NARROW>
+struct CodeWord {
+    typedef uint64_t type;
+};
+template <>
+struct CodeWord<true> {
+    typedef uint32_t type;
+};
+
 // One pure filter stage on a batch: returns the mask of rows that pass.
-template <bool HASH, int NR>
+template <bool HASH, bool NARROW, int NR>
 __device__ __forceinline__ uint32_t filter_rows(const RunArg &P, const DStage &S, const unsigned char *smem,
                                                 int64_t base, const uint32_t (&off)[NR], uint32_t valid)
 {
-    uint64_t unused[NR];
-    if (S.is64) {
-        int64_t v[NR];
-        load_rows<int64_t, false, NR>(S, base, off, valid, valid, v);
-        return run_stage<int64_t, NR, false, HASH>(P, S, smem, v, valid, unused);
+    typename CodeWord<NARROW>::type unused[NR];
+    if constexpr (!NARROW) {
+        if (S.is64) {
+            int64_t v[NR];
+            load_rows<int64_t, false, NR>(S, base, off, valid, valid, v);
+            return run_stage<int64_t, NR, false, HASH>(P, S, smem, v, valid, unused);
+        }
     }
     int32_t v[NR];
     load_rows<int32_t, false, NR>(S, base, off, valid, valid, v);
@@ -781,7 +809,7 @@ __device__ __forceinline__ uint32_t filter_rows(const RunArg &P, const DStage &S
 // Stages [first, nstages) with accumulators, then the terminal.  The column of
 // the next stage is requested before the current stage's probe is resolved, so
 // a stage costs one memory latency, not two.
-template <int AGG, bool MUL, bool CONTIG, bool HASH, int NR>
+template <int AGG, bool MUL, bool CONTIG, bool HASH, bool NARROW, int NR>
 __device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, unsigned char *smem, int first,
                                            int64_t base, const uint32_t (&off)[NR], uint32_t valid, int64_t &lsum,
                                            int64_t &lcnt)
@@ -810,7 +838,7 @@ __device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, un
             } else {
                 load_rows<int32_t, CONTIG, NR>(S, base, off, valid, need, v);
             }
-            have_next = (s + 1 < SJQ_PV(nstages)) && !SJQ_STAGE(s + 1).is64;
+            have_next = (s + 1 < SJQ_PV(nstages)) && (NARROW || !SJQ_STAGE(s + 1).is64);
             if (have_next) load_rows<int32_t, CONTIG, NR>(SJQ_STAGE(s + 1), base, off, valid, need, vnext);
             const int32_t mult = S.mult32[simple - 1];
             if (simple == 2) add_scaled32<NR>(X, mult, v, m);
@@ -818,28 +846,30 @@ __device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, un
             else if (MUL) add_scaled32<NR>(Y, mult, v, m);
             continue;
         }
-        uint64_t code[NR];
+        typename CodeWord<NARROW>::type code[NR];
 #pragma unroll
         for (int k = 0; k < NR; ++k) code[k] = 0;
-        if (S.is64) {
-            int64_t v[NR];
-            load_rows<int64_t, CONTIG, NR>(S, base, off, valid, need, v);
-            have_next = false;
-            m = run_stage<int64_t, NR, true, HASH>(P, S, smem, v, m, code);
-            if (S.acc) accumulate<MUL, int64_t, NR>(S, v, code, m, key, X, Y);
-        } else {
-            int32_t v[NR];
-            if (have_next) {
-#pragma unroll
-                for (int k = 0; k < NR; ++k) v[k] = vnext[k];
-            } else {
-                load_rows<int32_t, CONTIG, NR>(S, base, off, valid, need, v);
+        if constexpr (!NARROW) {
+            if (S.is64) {
+                int64_t v[NR];
+                load_rows<int64_t, CONTIG, NR>(S, base, off, valid, need, v);
+                have_next = false;
+                m = run_stage<int64_t, NR, true, HASH>(P, S, smem, v, m, code);
+                if (S.acc) accumulate<MUL, int64_t, NR>(S, v, code, m, key, X, Y);
+                continue;
             }
-            have_next = (s + 1 < SJQ_PV(nstages)) && !SJQ_STAGE(s + 1).is64;
-            if (have_next) load_rows<int32_t, CONTIG, NR>(SJQ_STAGE(s + 1), base, off, valid, need, vnext);
-            m = run_stage<int32_t, NR, true, HASH>(P, S, smem, v, m, code);
-            if (S.acc) accumulate<MUL, int32_t, NR>(S, v, code, m, key, X, Y);
         }
+        int32_t v[NR];
+        if (have_next) {
+#pragma unroll
+            for (int k = 0; k < NR; ++k) v[k] = vnext[k];
+        } else {
+            load_rows<int32_t, CONTIG, NR>(S, base, off, valid, need, v);
+        }
+        have_next = (s + 1 < SJQ_PV(nstages)) && (NARROW || !SJQ_STAGE(s + 1).is64);
+        if (have_next) load_rows<int32_t, CONTIG, NR>(SJQ_STAGE(s + 1), base, off, valid, need, vnext);
+        m = run_stage<int32_t, NR, true, HASH>(P, S, smem, v, m, code);
+        if (S.acc) accumulate<MUL, int32_t, NR>(S, v, code, m, key, X, Y);
     }
     terminal<AGG, MUL, NR>(P, smem, key, X, Y, m, lsum, lcnt);
 }
@@ -917,7 +947,7 @@ __device__ __forceinline__ void final_rows_scheduled(const RunArg &P, unsigned c
 // alive.  FULL: the whole tile lies inside the table (no bounds masks).
 // `staged` != nullptr: the tile's values of this column were copied into shared memory by a bulk-asynchronous
 // copy (in table order); the thread reads its four values of each slice from there.
-template <typename T, bool FULL, bool HASH>
+template <typename T, bool FULL, bool HASH, bool NARROW>
 __device__ __forceinline__ uint32_t dense_stage(const RunArg &P, const DStage &S, const unsigned char *smem,
                                                 int64_t row0, int32_t slot_stride, uint32_t valid, uint32_t alive,
                                                 const unsigned char *staged = nullptr)
@@ -949,11 +979,11 @@ __device__ __forceinline__ uint32_t dense_stage(const RunArg &P, const DStage &S
             }
         }
     }
-    uint64_t unused[kDenseRows];
+    typename CodeWord<NARROW>::type unused[kDenseRows];
     return run_stage<T, kDenseRows, false, HASH>(P, S, smem, v, alive, unused);
 }
 
-template <bool FULL, bool HASH>
+template <bool FULL, bool HASH, bool NARROW>
 __device__ __forceinline__ uint32_t level0(const RunArg &P, const DStage *st, const unsigned char *smem,
                                            int64_t row0, int32_t slot_stride, uint32_t valid,
                                            const unsigned char *staged = nullptr)
@@ -964,8 +994,13 @@ __device__ __forceinline__ uint32_t level0(const RunArg &P, const DStage *st, co
         if (!alive) break;
         const DStage &S = SJQ_STAGE(s);
         const unsigned char *from = s == 0 ? staged : nullptr; // only the first column is staged
-        alive = S.is64 ? dense_stage<int64_t, FULL, HASH>(P, S, smem, row0, slot_stride, valid, alive, from)
-                       : dense_stage<int32_t, FULL, HASH>(P, S, smem, row0, slot_stride, valid, alive, from);
+        if constexpr (!NARROW) {
+            if (S.is64) {
+                alive = dense_stage<int64_t, FULL, HASH, NARROW>(P, S, smem, row0, slot_stride, valid, alive, from);
+                continue;
+            }
+        }
+        alive = dense_stage<int32_t, FULL, HASH, NARROW>(P, S, smem, row0, slot_stride, valid, alive, from);
     }
     return alive;
 }
@@ -1049,9 +1084,60 @@ __device__ __forceinline__ uint32_t queue_base(int l)
     return l == 0 ? 0u : (uint32_t)(kQueue0Cap + (l - 1) * kQueueCap);
 }
 
+// ------------------------------------------------------------------ results cleared by the pass itself
+// A clear kernel in front of the pass costs a small query a fifth of its time: a launch on the host and a kernel boundary
+// on the device.  With words to meet at (P.sync) the first few blocks of the pass clear the results while the others
+// begin; a block looks at their flags before it first touches a result, at its end where its sums are its own
+// (registers, a shared group table), else before its first row.  A flag is up when it holds the number of this very
+// call, so that the words may hold anything before the first one; the last block to finish takes all flags down, so that
+// a captured call can be replayed.  The blocks that clear wait for nobody before their flags are up and are the first
+// of the grid, so the others never wait for a block that waits for them; every wait is bounded all the same.
+// (100 thousand rows, filter and sum, interpreted, back to back: 10.2 -> 8.2 us.)
+constexpr int kClearSpins = 1 << 20;
+__device__ __forceinline__ void clear_share(const RunArg &P)
+{
+    const int64_t step = (int64_t)P.clear_blocks * blockDim.x;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = first; i < P.clear_cells / 2; i += step) {
+        reinterpret_cast<longlong2 *>(P.sums)[i] = make_longlong2(0, 0);
+        if (P.clear_counts) reinterpret_cast<longlong2 *>(P.clear_counts)[i] = make_longlong2(0, 0);
+    }
+    if (first == 0) {
+        if (P.clear_cells & 1) {
+            P.sums[P.clear_cells - 1] = 0;
+            if (P.clear_counts) P.clear_counts[P.clear_cells - 1] = 0;
+        }
+        *P.status = 0;
+        P.sync[0] = 0;
+    }
+}
+// (thread 0, behind a barrier of the block)
+__device__ __forceinline__ void clear_told(const RunArg &P)
+{
+    __threadfence();
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(P.sync + 1 + blockIdx.x), "l"(P.epoch) : "memory");
+}
+// (thread 0, before a barrier of the block)
+__device__ __forceinline__ void clear_wait(const RunArg &P)
+{
+    for (int b = 0; b < P.clear_blocks; ++b) {
+        uint64_t seen = 0;
+        for (int spin = 0; spin < kClearSpins && seen != P.epoch; ++spin)
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(P.sync + 1 + b) : "memory");
+        if (seen != P.epoch) set_status(P.status, SJQ_ERR_ASYNC_WAIT);
+    }
+}
+// (thread 0, behind the block's last use of the results and a barrier)
+__device__ __forceinline__ void clear_over(const RunArg &P)
+{
+    __threadfence();
+    if (atomicAdd(reinterpret_cast<unsigned long long *>(P.sync), 1ull) != (unsigned long long)gridDim.x - 1ull) return;
+    for (int b = 0; b <= P.clear_blocks; ++b) P.sync[b] = 0;
+}
+
 // The scalar terminal's tail (Section 3.2: one atomic per block instead of one per matching row): warp
 // shuffle reduce, block reduce through shared memory, one global atomic per block.
-__device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsum, int64_t lcnt)
+__device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsum, int64_t lcnt, bool self_clear = false)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
@@ -1072,6 +1158,7 @@ __device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsu
             lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
             lcnt += __shfl_xor_sync(0xffffffffu, lcnt, o);
         }
+        if (lane == 0 && self_clear) clear_wait(P);
         if (lane == 0 && lcnt != 0) {
             atomicAdd(reinterpret_cast<unsigned long long *>(P.sums), (unsigned long long)lsum);
             if (P.counts) atomicAdd(reinterpret_cast<unsigned long long *>(P.counts), (unsigned long long)lcnt);
@@ -1080,12 +1167,18 @@ __device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsu
 }
 
 // `given`: the stage descriptors of the parameter block.
-template <int AGG, bool MUL, bool HASH>
+// DIRECT: no queues, every stage runs on thread-owned rows.
+template <int AGG, bool MUL, bool HASH, bool DIRECT, bool NARROW>
 __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given, unsigned char *smem)
 {
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int warp = tid >> 5;
+
+    // (only in kernels for few rows: the registers that it takes cost a pass over many rows up to 30 %, and the clear kernel
+    // costs that one next to nothing, since the pass starts behind it)
+    const bool self_clear = DIRECT && SJQ_PV(may_clear) && P.sync;
+    if (self_clear && (int)blockIdx.x < P.clear_blocks) clear_share(P);
 
     // Stage descriptors and small direct tables -> shared memory (once per block).
     DStage *st = reinterpret_cast<DStage *>(smem + P.smem_stages);
@@ -1121,7 +1214,16 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
         const int64_t cells = P.num_groups * (SJQ_PV(want_count) ? 2 : 1);
         for (int64_t i = tid; i < cells; i += blockDim.x) ss[i] = 0ull;
     }
+    constexpr bool kOwnSums = AGG == AGG_SCALAR || AGG == AGG_SMEM; // a block touches the results at its end only
+    if (kOwnSums && tid == 0) range_seen = 0u;
     __syncthreads();
+    if (self_clear) {
+        if (tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P);
+        if (!kOwnSums) {
+            if (tid == 0) clear_wait(P);
+            __syncthreads();
+        }
+    }
     // launched behind the kernel that clears the results: nothing above touches them, everything below may
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // (the listing of a hashed result is launched while this kernel runs and waits for its end on the device)
@@ -1129,7 +1231,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
 
     int64_t lsum = 0, lcnt = 0;
 
-    if (SJQ_PV(nq) == 0) {
+    if constexpr (DIRECT) {
         // No queue: every stage runs on the thread's own four consecutive rows.
         const int64_t tile_rows = (int64_t)blockDim.x * kDirectRows;
         const int64_t ntiles = (P.n + tile_rows - 1) / tile_rows;
@@ -1143,7 +1245,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
 #if defined(SJQ_JIT)
             final_rows_scheduled<AGG, MUL, HASH, true, kDirectRows>(P, smem, 0, base, off, valid, lsum, lcnt);
 #else
-            final_rows<AGG, MUL, true, HASH, kDirectRows>(P, st, smem, 0, base, off, valid, lsum, lcnt);
+            final_rows<AGG, MUL, true, HASH, NARROW, kDirectRows>(P, st, smem, 0, base, off, valid, lsum, lcnt);
 #endif
         }
     } else {
@@ -1237,7 +1339,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
                                 if (lane == 0) set_status(P.status, SJQ_ERR_ASYNC_WAIT);
                             }
                         }
-                        alive = level0<true, HASH>(P, st, smem, row0, slot_stride, kDenseRows >= 32 ? 0xFFFFFFFFu : ((1u << kDenseRows) - 1u), staged);
+                        alive = level0<true, HASH, NARROW>(P, st, smem, row0, slot_stride, kDenseRows >= 32 ? 0xFFFFFFFFu : ((1u << kDenseRows) - 1u), staged);
                         if (kBulk && staged != nullptr) {
                             __syncwarp(); // every lane of this warp has its values
                             if (lane == 0) {
@@ -1263,7 +1365,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
                             const uint32_t nv = rem >= 4 ? 0xFu : (rem > 0 ? ((1u << (int)rem) - 1u) : 0u);
                             valid |= nv << (4 * k);
                         }
-                        alive = level0<false, HASH>(P, st, smem, row0, slot_stride, valid);
+                        alive = level0<false, HASH, NARROW>(P, st, smem, row0, slot_stride, valid);
                     }
                     if (!__any_sync(0xffffffffu, alive != 0)) { // a very selective first stage: nothing to push
                         tile += gridDim.x;
@@ -1334,18 +1436,18 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
 #if defined(SJQ_JIT)
                 final_rows_scheduled<AGG, MUL, HASH, false, kRows>(P, smem, SJQ_JIT_nd0 + SJQ_JIT_nq - 1, qbase, off, valid, lsum, lcnt);
 #else
-                final_rows<AGG, MUL, false, HASH, kRows>(P, st, smem, SJQ_PV(nd0) + nq - 1, qbase, off, valid, lsum, lcnt);
+                final_rows<AGG, MUL, false, HASH, NARROW, kRows>(P, st, smem, SJQ_PV(nd0) + nq - 1, qbase, off, valid, lsum, lcnt);
 #endif
             } else {
 #if defined(SJQ_JIT)
                 // one copy of the filter level per queue-fed filter stage of this query
                 uint32_t m;
                 if (SJQ_JIT_nq <= 2 || l == 0)
-                    m = filter_rows<HASH, kRows>(P, SJQ_STAGE(SJQ_JIT_nd0), smem, qbase, off, valid);
+                    m = filter_rows<HASH, NARROW, kRows>(P, SJQ_STAGE(SJQ_JIT_nd0), smem, qbase, off, valid);
                 else
-                    m = filter_rows<HASH, kRows>(P, SJQ_STAGE(SJQ_JIT_nd0 + 1), smem, qbase, off, valid);
+                    m = filter_rows<HASH, NARROW, kRows>(P, SJQ_STAGE(SJQ_JIT_nd0 + 1), smem, qbase, off, valid);
 #else
-                const uint32_t m = filter_rows<HASH, kRows>(P, st[P.nd0 + l], smem, qbase, off, valid);
+                const uint32_t m = filter_rows<HASH, NARROW, kRows>(P, st[P.nd0 + l], smem, qbase, off, valid);
 #endif
                 const uint32_t mine = (uint32_t)__popc(m);
                 uint32_t incl = mine;
@@ -1379,9 +1481,10 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
     }
 
     if (AGG == AGG_SCALAR) {
-        scalar_block_reduce(P, lsum, lcnt);
+        scalar_block_reduce(P, lsum, lcnt, self_clear);
     } else if (AGG == AGG_SMEM) {
         // one global atomic per touched group per block
+        if (self_clear && tid == 0) clear_wait(P);
         __syncthreads();
         const unsigned int *ss = reinterpret_cast<const unsigned int *>(smem + P.smem_groups);
         const uint64_t ng = (uint64_t)P.num_groups;
@@ -1402,23 +1505,26 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
             }
         }
     }
+    if (kOwnSums && tid == 0 && range_seen) set_status(P.status, SJQ_ERR_GROUP_RANGE);
+    if (self_clear) {
+        if (AGG != AGG_SCALAR) __syncthreads(); // (a scalar result is added by thread 0)
+        if (tid == 0) clear_over(P);
+    }
 }
 
-
 #if !defined(SJQ_JIT)
-template <typename Params, int AGG, bool MUL, bool HASH>
+template <typename Params, int AGG, bool MUL, int FORM>
 __global__ void __launch_bounds__(SJQ_LB_THREADS, SJQ_LB_BLOCKS) fused_kernel(const __grid_constant__ Params P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    fused_body<AGG, MUL, HASH>(P, P.st, smem);
+    fused_body<AGG, MUL, (FORM & kFormHash) != 0, (FORM & kFormDirect) != 0, (FORM & kFormNarrow) != 0>(P, P.st, smem);
 }
 
-// The kernel of one aggregation path for a parameter block.
-template <typename Params, int AGG>
-auto fused_variant(bool mul, bool hash) -> void (*)(const Params)
+// The kernel of one aggregation path and form for a parameter block.
+template <typename Params, int AGG, int FORM>
+auto fused_of(bool mul) -> void (*)(const Params)
 {
-    if (mul) return hash ? fused_kernel<Params, AGG, true, true> : fused_kernel<Params, AGG, true, false>;
-    return hash ? fused_kernel<Params, AGG, false, true> : fused_kernel<Params, AGG, false, false>;
+    return mul ? fused_kernel<Params, AGG, true, FORM> : fused_kernel<Params, AGG, false, FORM>;
 }
 #endif
 
@@ -1431,7 +1537,7 @@ extern "C" __global__ void __launch_bounds__(SJQ_LB_THREADS, SJQ_LB_BLOCKS)
     sjq_jit_kernel(const __grid_constant__ sjq::RunParams P)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    sjq::fused_body<SJQ_JIT_AGG, (SJQ_JIT_MUL != 0), (SJQ_JIT_HASH != 0)>(P, P.st, smem);
+    sjq::fused_body<SJQ_JIT_AGG, (SJQ_JIT_MUL != 0), (SJQ_JIT_HASH != 0), (SJQ_JIT_nq == 0), false>(P, P.st, smem);
 }
 #endif
 #endif

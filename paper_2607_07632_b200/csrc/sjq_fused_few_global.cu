@@ -4,6 +4,16 @@
 
 namespace sjq {
 
-fused_few_fn fused_few_global(bool mul, bool hash) { return fused_variant<RunParamsFew, AGG_GLOBAL>(mul, hash); }
+fused_few_fn fused_few_global(bool mul, int form)
+{
+    switch (form) {
+    case 0: return fused_of<RunParamsFew, AGG_GLOBAL, 0>(mul);
+    case kFormHash: return fused_of<RunParamsFew, AGG_GLOBAL, kFormHash>(mul);
+    case kFormDirect: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect>(mul);
+    case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect | kFormHash>(mul);
+    case kFormNarrow: return fused_of<RunParamsFew, AGG_GLOBAL, kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect | kFormNarrow>(mul);
+    }
+}
 
 } // namespace sjq

@@ -4,6 +4,16 @@
 
 namespace sjq {
 
-fused_few_fn fused_few_hash(bool mul, bool hash) { return fused_variant<RunParamsFew, AGG_HASH>(mul, hash); }
+fused_few_fn fused_few_hash(bool mul, int form)
+{
+    switch (form) {
+    case 0: return fused_of<RunParamsFew, AGG_HASH, 0>(mul);
+    case kFormHash: return fused_of<RunParamsFew, AGG_HASH, kFormHash>(mul);
+    case kFormDirect: return fused_of<RunParamsFew, AGG_HASH, kFormDirect>(mul);
+    case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_HASH, kFormDirect | kFormHash>(mul);
+    case kFormNarrow: return fused_of<RunParamsFew, AGG_HASH, kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_HASH, kFormDirect | kFormNarrow>(mul);
+    }
+}
 
 } // namespace sjq

@@ -4,6 +4,16 @@
 
 namespace sjq {
 
-fused_few_fn fused_few_scalar(bool mul, bool hash) { return fused_variant<RunParamsFew, AGG_SCALAR>(mul, hash); }
+fused_few_fn fused_few_scalar(bool mul, int form)
+{
+    switch (form) {
+    case 0: return fused_of<RunParamsFew, AGG_SCALAR, 0>(mul);
+    case kFormHash: return fused_of<RunParamsFew, AGG_SCALAR, kFormHash>(mul);
+    case kFormDirect: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect>(mul);
+    case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect | kFormHash>(mul);
+    case kFormNarrow: return fused_of<RunParamsFew, AGG_SCALAR, kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect | kFormNarrow>(mul);
+    }
+}
 
 } // namespace sjq

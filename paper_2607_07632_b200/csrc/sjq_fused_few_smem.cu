@@ -4,6 +4,16 @@
 
 namespace sjq {
 
-fused_few_fn fused_few_smem(bool mul, bool hash) { return fused_variant<RunParamsFew, AGG_SMEM>(mul, hash); }
+fused_few_fn fused_few_smem(bool mul, int form)
+{
+    switch (form) {
+    case 0: return fused_of<RunParamsFew, AGG_SMEM, 0>(mul);
+    case kFormHash: return fused_of<RunParamsFew, AGG_SMEM, kFormHash>(mul);
+    case kFormDirect: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect>(mul);
+    case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect | kFormHash>(mul);
+    case kFormNarrow: return fused_of<RunParamsFew, AGG_SMEM, kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect | kFormNarrow>(mul);
+    }
+}
 
 } // namespace sjq

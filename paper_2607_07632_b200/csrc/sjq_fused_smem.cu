@@ -1,9 +1,17 @@
-// Ahead-of-time instantiations of the fused kernel for one aggregation path (AGG_SMEM); one translation unit per
-// path and size of the parameter block so that they compile in parallel.
+// Ahead-of-time instantiations of the fused kernel for one aggregation path (AGG_SMEM) and any number of stages;
+// one translation unit per path and size of the parameter block so that they compile in parallel.
 #include "sjq_fused_device.cuh"
 
 namespace sjq {
 
-fused_fn fused_variant_smem(bool mul, bool hash) { return fused_variant<RunParams, AGG_SMEM>(mul, hash); }
+fused_fn fused_variant_smem(bool mul, int form)
+{
+    switch (form) {
+    case 0: return fused_of<RunParams, AGG_SMEM, 0>(mul);
+    case kFormHash: return fused_of<RunParams, AGG_SMEM, kFormHash>(mul);
+    case kFormDirect: return fused_of<RunParams, AGG_SMEM, kFormDirect>(mul);
+    default: return fused_of<RunParams, AGG_SMEM, kFormDirect | kFormHash>(mul);
+    }
+}
 
 } // namespace sjq

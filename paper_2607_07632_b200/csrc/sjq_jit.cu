@@ -172,6 +172,7 @@ std::string jit_shape_header(const RunParams &P, int agg, bool mul, bool hash, i
       << "\n#define SJQ_JIT_has_key " << P.has_key << "\n#define SJQ_JIT_mod32 " << P.mod32
       << "\n#define SJQ_JIT_warp_agg " << P.warp_agg << "\n#define SJQ_JIT_l0_bulk " << P.l0_bulk << "\n#define SJQ_JIT_count32 " << P.count32 << "\n#define SJQ_JIT_sparse_push " << P.sparse_push
       << "\n#define SJQ_JIT_cell_shift " << P.cell_shift << "\n#define SJQ_JIT_pairs " << P.pairs
+      << "\n#define SJQ_JIT_may_clear " << P.may_clear
       << "\n";
     put(o, "modulo", P.modulo);
     o << "#define SJQ_JIT_modmask " << P.modmask << "ULL\n";
@@ -218,7 +219,7 @@ void shape_key(const RunParams &P, int agg, bool mul, bool hash, int lb_threads,
 {
     const int32_t head[] = {agg, mul ? 1 : 0, hash ? 1 : 0, lb_threads, lb_blocks, P.nstages, P.nd0, P.nq,
                             P.rows, P.want_count, P.eager, P.has_key, P.mod32, (int32_t)P.qfold, P.slots, P.warp_agg,
-                            P.l0_bulk, P.count32, P.sparse_push, P.cell_shift, P.pairs};
+                            P.l0_bulk, P.count32, P.sparse_push, P.cell_shift, P.pairs, P.may_clear};
     static_assert(sizeof(head) + 16 <= 128, "room for the head");
     k->put(head, sizeof(head));
     k->put(&P.modulo, sizeof(P.modulo));

@@ -17,7 +17,7 @@ namespace {
 #define SJQ_NAMES(X)                                                                                                   \
     X(data_ptr) X(dtype) X(is_cuda) X(is_contiguous) X(dim) X(numel) X(col) X(op) X(lo) X(hi) X(values) X(handle)       \
     X(terms) X(offset) X(modulo) X(src) X(a) X(b) X(mult) X(x) X(y) X(want_count) X(sums) X(counts) X(keys)             \
-    X(n_groups) X(status_dev) X(workspace) X(info) X(block_threads) X(ctas_per_sm) X(eager_loads) X(agg_path)           \
+    X(n_groups) X(status_dev) X(workspace) X(sync) X(info) X(block_threads) X(ctas_per_sm) X(eager_loads) X(agg_path)           \
     X(smem_tables) X(compaction) X(accumulate) X(order) X(events) X(cuda_event) X(specialise) X(rows_per_lane)          \
     X(no_filter_bitmap) X(host_copy_all) X(dense_slots) X(group_hash_always) X(warp_agg) X(unfused_scratch)             \
     X(pass_ppm) X(hot_keys) X(hot_scratch) X(l0_bulk)
@@ -334,6 +334,7 @@ PyObject *py_run(PyObject *, PyObject *const *args, Py_ssize_t nargs)
         !get_pointer(result, N.status_dev, &R.status) || !get_pointer(result, N.workspace, &R.workspace, &workspace_bytes))
         return nullptr;
     R.workspace_bytes = (size_t)workspace_bytes;
+    if (!get_pointer(result, N.sync, &o.sync)) return nullptr;
 
     Ref scratch(nullptr); // held until the call has enqueued its work
     if (hashed && !o.hot_scratch && o.hot_keys != 2) {

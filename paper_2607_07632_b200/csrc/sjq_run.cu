@@ -10,6 +10,8 @@
 // thread choice of Section 4.3.1 ("asymmetric batching") is the fixed four
 // rows per 128-bit load here; occupancy supplies the memory-level parallelism.
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <cstring>
 #include <vector>
 
@@ -23,12 +25,12 @@
 
 namespace sjq {
 
-sjq_status fused_occupancy(int agg, bool mul, bool hash, int nstages, int block, size_t smem, int *ctas_per_sm);
+sjq_status fused_occupancy(int agg, bool mul, int form, int nstages, int block, size_t smem, int *ctas_per_sm);
 sjq_status jit_prepare(const RunParams &P, int agg, bool mul, bool hash, int block, int lb_blocks, size_t smem,
                        int *ctas_per_sm, const void **kernel);
 sjq_status jit_launch(const void *kernel, const RunParams &P, int grid, int block, size_t smem, bool behind,
                       cudaStream_t stream);
-sjq_status fused_launch(int agg, bool mul, bool hash, int grid, int block, size_t smem, bool behind,
+sjq_status fused_launch(int agg, bool mul, int form, int grid, int block, size_t smem, bool behind,
                         const RunParams &P, cudaStream_t stream);
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
                         int64_t *n_groups, int32_t *status, int at_once, int sm_count, cudaStream_t stream);
@@ -353,6 +355,16 @@ extern "C" sjq_status sjq_pred_sample(const sjq_col *fact, int nfact, const sjq_
 
 namespace {
 
+// Groups of a dense result that a pass over few rows may clear itself: seven blocks of 384 threads take four steps.
+constexpr int64_t kClearByPass = 1 << 14;
+
+// A number that no other call has: the flags of a pass that clears its results hold it.
+uint64_t next_epoch()
+{
+    static std::atomic<uint64_t> last{(uint64_t)std::chrono::steady_clock::now().time_since_epoch().count() << 20};
+    return ++last | 1ull << 63;
+}
+
 // What a run is part of: by default of nothing, its columns are in device memory and its options are the caller's.
 struct RunContext {
     // the order of the filters, if the options give one, is the caller's own and not one that this library chose for a
@@ -423,6 +435,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     if (opts.norder && opts.norder != npreds + njoins) return SJQ_ERR_INVALID_ARG;
     if (opts.hot_keys < 0 || opts.hot_keys > 2) return SJQ_ERR_INVALID_ARG;
     if (opts.hot_scratch && !aligned16(opts.hot_scratch)) return SJQ_ERR_ALIGN;
+    if (reinterpret_cast<uintptr_t>(opts.sync) & 7u) return SJQ_ERR_ALIGN;
 
     DeviceInfo dev;
     sjq_status st = device_info(&dev);
@@ -967,9 +980,19 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         }
     }
 
+    P.may_clear = few_rows && !opts.unfused && spec->mode != SJQ_HASHED && P.num_groups <= kClearByPass;
+    const bool self_clear = P.may_clear && opts.sync && !opts.accumulate && n > 0;
+
+    // ------------------------------------------------------------ form of the ahead-of-time kernel
     bool has_hash = false; // kernels without the hash probe are leaner; pick by what the stages need
-    for (int s2 = 0; s2 < ns; ++s2)
-        has_hash |= P.st[s2].op == OP_HASH32 || P.st[s2].op == OP_HASH64 || P.st[s2].op == OP_HASHBITS;
+    bool narrow = ns <= kFewStages;
+    for (int s2 = 0; s2 < ns; ++s2) {
+        const DStage &S = P.st[s2];
+        has_hash |= S.op == OP_HASH32 || S.op == OP_HASH64 || S.op == OP_HASHBITS;
+        narrow = narrow && !S.is64 && S.op != OP_DIRECT_U64 && (S.acc32 || !S.acc);
+    }
+    narrow = narrow && !has_hash;
+    const int form = (has_hash ? kFormHash : 0) | (P.nq == 0 ? kFormDirect : 0) | (narrow ? kFormNarrow : 0);
 
     // ------------------------------------------------------------ launch shape
     int per_sm = 0;
@@ -985,7 +1008,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
                                                                         : 2;
     const void *compiled = nullptr;
     st = jit ? jit_prepare(P, aggp, mul, has_hash, block, lb_blocks, smem, &per_sm, &compiled)
-             : fused_occupancy(aggp, mul, has_hash, ns, block, smem, &per_sm);
+             : fused_occupancy(aggp, mul, form, ns, block, smem, &per_sm);
     if (st != SJQ_OK) return st;
     if (per_sm < 1) return SJQ_ERR_UNSUPPORTED;
     if (opts.ctas_per_sm > 0) per_sm = std::min(per_sm, opts.ctas_per_sm);
@@ -996,7 +1019,13 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
 
     // ------------------------------------------------------------ launches
     int launches = 0;
-    if (!opts.accumulate) {
+    if (self_clear) {
+        P.sync = static_cast<uint64_t *>(opts.sync);
+        P.epoch = next_epoch();
+        P.clear_counts = out->counts;
+        P.clear_cells = spec->mode == SJQ_SCALAR ? 1 : spec->num_groups;
+        P.clear_blocks = (int32_t)std::min<int64_t>(std::min(grid, kClearBlocks), 1 + P.clear_cells / (2 * block));
+    } else if (!opts.accumulate) {
         const int64_t words = spec->mode == SJQ_SCALAR ? 1
                               : spec->mode == SJQ_DENSE ? spec->num_groups
                               : direct_groups           ? 2 * table_groups
@@ -1035,9 +1064,9 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         // Directly behind the clear the kernel is launched while that one still runs (programmatic dependent launch):
         // it stages its tables, which were complete before the clear began, and waits for the clear before it touches
         // a result (two-join query, 60 M rows: 94 -> 92 us; filter and sum, 6 M rows: 20.5 -> 18.5 us back to back).
-        const bool behind = !opts.accumulate && hot_stage < 0 && !opts.event_before;
+        const bool behind = !opts.accumulate && !self_clear && hot_stage < 0 && !opts.event_before;
         st = jit ? jit_launch(compiled, P, grid, block, smem, behind, stream)
-                 : fused_launch(aggp, mul, has_hash, grid, block, smem, behind, P, stream);
+                 : fused_launch(aggp, mul, form, grid, block, smem, behind, P, stream);
         if (st != SJQ_OK) return st;
         ++launches;
     }

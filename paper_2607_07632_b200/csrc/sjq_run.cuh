@@ -136,7 +136,19 @@ struct RunCore {
     int32_t cell_shift;   // log2 of the distance between two groups' sums: 1 when sums and counts alternate, else 0
     int32_t pairs;        // ... and two lanes share a row's two adds
     int32_t l0_bulk;      // compiled kernels: the first column arrives by bulk-asynchronous copies into shared memory
+    // Results that the pass clears itself.
+    int32_t may_clear;     // a kernel for few rows: it does so where sync is given
+    int32_t clear_blocks;  // blocks that share the work: 1 .. kClearBlocks
+    uint64_t *sync;
+    uint64_t epoch;        // of this call alone, never 0
+    int64_t *clear_counts; // counts to zero, also where they are not asked for; may be NULL
+    int64_t clear_cells;   // words of sums and of clear_counts
 };
+
+// Words through which the blocks of a pass tell one another that the results are clear: the blocks that are done with
+// the whole pass, then the flags of the blocks that clear.  All are zero between two passes (the last block leaves
+// them so), whatever they held before the first.
+constexpr int kClearBlocks = SJQ_SYNC_BYTES / 8 - 1;
 
 // A kernel's parameter block: its stage descriptors, then the rest.
 template <int N>
@@ -150,21 +162,25 @@ typedef RunParamsOf<kMaxStages> RunParams;
 static_assert(sizeof(RunParams) == sizeof(RunStages<kMaxStages>) + sizeof(RunCore), "no padding between the two");
 
 #if !defined(SJQ_JIT)
-// The ahead-of-time variants of the fused kernel (aggregation path x product aggregate x "some table is
-// open-addressing" x up to kFewStages stages or any number), instantiated in one translation unit per aggregation
-// path and size.  A launch copies its whole parameter block, 6 KB with twelve stages and 21 KB with all (a call of a
-// small query 9.9 -> 8.1 us).
+// The ahead-of-time kernels: aggregation path x product aggregate x form x up to kFewStages stages or any number,
+// instantiated in one translation unit per aggregation path and size.  A launch copies its whole parameter block, 6 KB
+// with twelve stages and 21 KB with all (a call of a small query 9.9 -> 8.1 us).
+// Forms: kFormHash, some table is open-addressing; kFormDirect, no queues; kFormNarrow (few stages, no open-addressing
+// table), every fact column and every code has 32 bits and accumulators take 32-bit contributions.  A form holds only the
+// bodies that its queries use: fewer registers and fewer instructions to fetch (four joins asked once, 60 M rows, the
+// whole call 262 -> 252 us).
+constexpr int kFormHash = 1, kFormDirect = 2, kFormNarrow = 4;
 typedef RunParamsOf<kFewStages> RunParamsFew;
 typedef void (*fused_few_fn)(const RunParamsFew);
 typedef void (*fused_fn)(const RunParams);
-fused_fn fused_variant_scalar(bool mul, bool hash);
-fused_fn fused_variant_smem(bool mul, bool hash);
-fused_fn fused_variant_global(bool mul, bool hash);
-fused_fn fused_variant_hash(bool mul, bool hash);
-fused_few_fn fused_few_scalar(bool mul, bool hash);
-fused_few_fn fused_few_smem(bool mul, bool hash);
-fused_few_fn fused_few_global(bool mul, bool hash);
-fused_few_fn fused_few_hash(bool mul, bool hash);
+fused_fn fused_variant_scalar(bool mul, int form);
+fused_fn fused_variant_smem(bool mul, int form);
+fused_fn fused_variant_global(bool mul, int form);
+fused_fn fused_variant_hash(bool mul, int form);
+fused_few_fn fused_few_scalar(bool mul, int form);
+fused_few_fn fused_few_smem(bool mul, int form);
+fused_few_fn fused_few_global(bool mul, int form);
+fused_few_fn fused_few_hash(bool mul, int form);
 #endif
 
 } // namespace sjq

@@ -104,7 +104,8 @@ class _RunOpts(ctypes.Structure):
                 ("group_hash_always", ctypes.c_int32), ("warp_agg", ctypes.c_int32), ("unfused", ctypes.c_int32),
                 ("unfused_scratch", ctypes.c_void_p), ("unfused_scratch_bytes", ctypes.c_size_t),
                 ("pass_ppm", ctypes.c_int32 * (MAX_PREDS + MAX_JOINS)), ("hot_keys", ctypes.c_int32),
-                ("hot_scratch", ctypes.c_void_p), ("hot_scratch_bytes", ctypes.c_size_t), ("l0_bulk", ctypes.c_int32)]
+                ("hot_scratch", ctypes.c_void_p), ("hot_scratch_bytes", ctypes.c_size_t), ("l0_bulk", ctypes.c_int32),
+                ("sync", ctypes.c_void_p)]
 
 
 class RunInfo(ctypes.Structure):
@@ -656,6 +657,7 @@ class Result:
     info: RunInfo = field(default_factory=RunInfo)
     joined: Optional[torch.Tensor] = None  # SCALAR / DENSE: sums, counts and one spare cell as views of one int64
     #                                        buffer, so that a multi-GPU merge is a single all-reduce
+    sync: Optional[torch.Tensor] = None  # SYNC_BYTES of scratch with which a pass over few rows clears its result itself
 
     def status(self) -> int:
         return int(self.status_dev.item())
@@ -730,7 +732,8 @@ def alloc_result(mode: str, num_groups: int, capacity: int, want_count: bool, de
             raise SjqError(rc, "sjq_run_workspace_bytes")
         ws = torch.empty(nbytes.value, dtype=torch.uint8, device=device)
     status = new(1, dtype=torch.int32, device=device)
-    return Result(mode, sums, counts, keys, n_groups, status, ws, joined=joined)
+    sync = torch.empty(SYNC_BYTES // 8, dtype=torch.int64, device=device)
+    return Result(mode, sums, counts, keys, n_groups, status, ws, joined=joined, sync=sync)
 
 
 def merge_groups(keys: torch.Tensor, sums: torch.Tensor, counts: torch.Tensor, capacity: int,
@@ -801,6 +804,7 @@ def run(fact: dict, preds=(), joins=(), key=None, agg=None, mode: str = "SCALAR"
 
 
 STATIC_MAX_GROUPS = 65536
+SYNC_BYTES = 64  # SJQ_SYNC_BYTES
 HOT_SCRATCH_BYTES = 3 * 1048576 + 65536  # SJQ_HOT_SCRATCH_BYTES
 _hot_scratch_by_device: dict = {}
 
@@ -912,6 +916,7 @@ def run_host(fact: dict, staging: torch.Tensor, chunk_rows: int, preds=(), joins
                               torch.zeros(1, dtype=torch.int32, **pin))
         cres = _result_struct(res)
         copts = (opts or RunOpts()).to_c()
+        copts.sync = res.sync.data_ptr() if res.sync is not None else None
         rc = lib().sjq_run_host(carr, len(names), parr, len(preds), jarr, len(joins),
                                 ctypes.byref(kexpr) if kexpr is not None else None, ctypes.byref(aexpr),
                                 ctypes.byref(spec), ctypes.byref(cres), ctypes.byref(copts), staging.data_ptr(),
