@@ -597,13 +597,13 @@ __device__ __forceinline__ uint64_t smem_cell(const unsigned int *words, uint64_
     return ((uint64_t)words[ng + g] << 32) | words[g];
 }
 
-// A row's group key is out of range.  Where a block's sums are its own (registers, a shared group table) the fused kernel
-// notes it in shared memory and tells it at the end, when the status word is known to be clear.
+// A row's group key is out of range.  A pass that clears its results itself notes it in shared memory and tells it at the
+// end, when the status word is known to be clear.
 __shared__ uint32_t range_seen;
-template <bool LATER>
+template <bool FUSED>
 __device__ __forceinline__ void note_range(const RunArg &P)
 {
-    if (LATER) range_seen = 1u;
+    if (FUSED && SJQ_PV(may_clear)) range_seen = 1u;
     else set_status(P.status, SJQ_ERR_GROUP_RANGE);
 }
 
@@ -678,7 +678,7 @@ __device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, c
 #pragma unroll
     for (int k = 0; k < NR; ++k)
         if (((m >> k) & 1u) && (uint64_t)g[k] >= ng) {
-            note_range<FUSED && AGG == AGG_SMEM>(P);
+            note_range<FUSED>(P);
             m &= ~(1u << k);
         }
     const bool want_count = SJQ_PV(want_count) != 0;
@@ -1087,8 +1087,9 @@ __device__ __forceinline__ uint32_t queue_base(int l)
 // ------------------------------------------------------------------ results cleared by the pass itself
 // A clear kernel in front of the pass costs a small query a fifth of its time: a launch on the host and a kernel boundary
 // on the device.  With words to meet at (P.sync) the first few blocks of the pass clear the results while the others
-// begin; a block looks at their flags before it first touches a result, at its end where its sums are its own
-// (registers, a shared group table), else before its first row.  A flag is up when it holds the number of this very
+// begin; a block's sums are its own (registers, a shared group table), and it looks at the flags at its end, before it
+// adds them to the results (a pass that adds its rows one by one to a global table would have to look before its first row:
+// 300 thousand rows, skewed keys, 4096 groups 23.4 us with the clear kernel and 26.9 so).  A flag is up when it holds the number of this very
 // call, so that the words may hold anything before the first one; the last block to finish takes all flags down, so that
 // a captured call can be replayed.  The blocks that clear wait for nobody before their flags are up and are the first
 // of the grid, so the others never wait for a block that waits for them; every wait is bounded all the same.
@@ -1177,7 +1178,8 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
 
     // (only in kernels for few rows: the registers that it takes cost a pass over many rows up to 30 %, and the clear kernel
     // costs that one next to nothing, since the pass starts behind it)
-    const bool self_clear = DIRECT && SJQ_PV(may_clear) && P.sync;
+    const bool may_clear = (AGG == AGG_SCALAR || AGG == AGG_SMEM) && DIRECT && SJQ_PV(may_clear);
+    const bool self_clear = may_clear && P.sync;
     if (self_clear && (int)blockIdx.x < P.clear_blocks) clear_share(P);
 
     // Stage descriptors and small direct tables -> shared memory (once per block).
@@ -1214,16 +1216,9 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
         const int64_t cells = P.num_groups * (SJQ_PV(want_count) ? 2 : 1);
         for (int64_t i = tid; i < cells; i += blockDim.x) ss[i] = 0ull;
     }
-    constexpr bool kOwnSums = AGG == AGG_SCALAR || AGG == AGG_SMEM; // a block touches the results at its end only
-    if (kOwnSums && tid == 0) range_seen = 0u;
+    if (may_clear && tid == 0) range_seen = 0u;
     __syncthreads();
-    if (self_clear) {
-        if (tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P);
-        if (!kOwnSums) {
-            if (tid == 0) clear_wait(P);
-            __syncthreads();
-        }
-    }
+    if (self_clear && tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P);
     // launched behind the kernel that clears the results: nothing above touches them, everything below may
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // (the listing of a hashed result is launched while this kernel runs and waits for its end on the device)
@@ -1505,7 +1500,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
             }
         }
     }
-    if (kOwnSums && tid == 0 && range_seen) set_status(P.status, SJQ_ERR_GROUP_RANGE);
+    if (may_clear && tid == 0 && range_seen) set_status(P.status, SJQ_ERR_GROUP_RANGE);
     if (self_clear) {
         if (AGG != AGG_SCALAR) __syncthreads(); // (a scalar result is added by thread 0)
         if (tid == 0) clear_over(P);

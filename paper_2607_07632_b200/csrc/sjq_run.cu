@@ -355,9 +355,6 @@ extern "C" sjq_status sjq_pred_sample(const sjq_col *fact, int nfact, const sjq_
 
 namespace {
 
-// Groups of a dense result that a pass over few rows may clear itself: seven blocks of 384 threads take four steps.
-constexpr int64_t kClearByPass = 1 << 14;
-
 // A number that no other call has: the flags of a pass that clears its results hold it.
 uint64_t next_epoch()
 {
@@ -980,7 +977,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         }
     }
 
-    P.may_clear = few_rows && !opts.unfused && spec->mode != SJQ_HASHED && P.num_groups <= kClearByPass;
+    P.may_clear = few_rows && !opts.unfused && spec->mode != SJQ_HASHED && (aggp == AGG_SCALAR || aggp == AGG_SMEM);
     const bool self_clear = P.may_clear && opts.sync && !opts.accumulate && n > 0;
 
     // ------------------------------------------------------------ form of the ahead-of-time kernel

@@ -137,7 +137,7 @@ struct RunCore {
     int32_t pairs;        // ... and two lanes share a row's two adds
     int32_t l0_bulk;      // compiled kernels: the first column arrives by bulk-asynchronous copies into shared memory
     // Results that the pass clears itself.
-    int32_t may_clear;     // a kernel for few rows: it does so where sync is given
+    int32_t may_clear;     // a kernel for few rows whose blocks keep sums of their own: it does so where sync is given
     int32_t clear_blocks;  // blocks that share the work: 1 .. kClearBlocks
     uint64_t *sync;
     uint64_t epoch;        // of this call alone, never 0

@@ -27,17 +27,17 @@ def _query(fact, groups):
 
 
 @pytest.mark.parametrize("n", [1, 1537, 2**19, 2**19 + 1])
-@pytest.mark.parametrize("groups", [0, 1, 2, 767, 769, 5_377, 16_384, 16_385])
+@pytest.mark.parametrize("groups", [0, 1, 2, 767, 769, 4_096, 4_097])
 @pytest.mark.parametrize("compiled", [False, True])
 def test_small_results_are_cleared_by_their_pass(n, groups, compiled):
     """Buffers and words full of what earlier runs left: one launch clears and fills them, again and again, and leaves the
     words at zero; without the words, or beyond the limits, a kernel before the pass does."""
-    opts = sjq.RunOpts(specialise=compiled)
+    opts = sjq.RunOpts(specialise=compiled, agg_path=1 if 1 < groups <= 4_096 else 0)  # the largest shared table
     fact = _grouped(n, max(1, groups), n + groups)
     w = _query(fact, groups)
     res, exp, _ = run_both(w, fact, {}, opts)
     dev = to_dev(fact)
-    by_pass = n <= 2**19 and groups <= 16_384
+    by_pass = n <= 2**19 and groups <= 4_096
     for words in (torch.full((8,), -1, dtype=torch.int64, device="cuda"), torch.zeros(8, dtype=torch.int64, device="cuda"), None):
         res.sync = words
         for _ in range(3):
@@ -49,13 +49,14 @@ def test_small_results_are_cleared_by_their_pass(n, groups, compiled):
         if by_pass and words is not None:
             assert words[0] == 0 and ((words == 0) | (words == -1)).all()  # (as many flags as blocks that clear)
     res.sync = torch.full((8,), 5, dtype=torch.int64, device="cuda")  # a run that accumulates clears nothing
-    sjq.run_workload(w, dev, {}, sjq.RunOpts(specialise=compiled, accumulate=True), result=res)
+    opts.accumulate = True
+    sjq.run_workload(w, dev, {}, opts, result=res)
     torch.cuda.synchronize()
     assert (res.sync == 5).all()
     compare(w, res, {k: (2 * v if k in ("sum", "count", "sums", "counts") else v) for k, v in exp.items()})
 
 
-@pytest.mark.parametrize("groups,limit", [(500, 499), (500, 1), (9_000, 8_999)])  # shared table, registers, global table
+@pytest.mark.parametrize("groups,limit", [(100, 99), (500, 1)])  # shared table, registers
 def test_a_key_out_of_range_is_told_by_a_pass_that_clears(groups, limit):
     fact = _grouped(40_001, groups, 3)
     fact["g"][:groups] = np.arange(groups)
@@ -70,7 +71,7 @@ def test_a_key_out_of_range_is_told_by_a_pass_that_clears(groups, limit):
     compare(w, res, oracle_result(w, fact, {})[1])
 
 
-@pytest.mark.parametrize("groups", [0, 500, 9_000])
+@pytest.mark.parametrize("groups", [0, 20])
 @pytest.mark.parametrize("compiled", [False, True])
 def test_a_captured_pass_that_clears_replays_on_new_data(groups, compiled):
     n, opts = 100_003, sjq.RunOpts(specialise=compiled)
