@@ -1180,7 +1180,11 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
     // costs that one next to nothing, since the pass starts behind it)
     const bool may_clear = (AGG == AGG_SCALAR || AGG == AGG_SMEM) && DIRECT && SJQ_PV(may_clear);
     const bool self_clear = may_clear && P.sync;
-    if (self_clear && (int)blockIdx.x < P.clear_blocks) clear_share(P);
+    if (self_clear) {
+        // launched while the kernel before it still runs (four joins, 400 thousand rows, interpreted: 12.4 -> 10.5 us)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if ((int)blockIdx.x < P.clear_blocks) clear_share(P);
+    }
 
     // Stage descriptors and small direct tables -> shared memory (once per block).
     DStage *st = reinterpret_cast<DStage *>(smem + P.smem_stages);
@@ -1221,8 +1225,9 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
     if (self_clear && tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P);
     // launched behind the kernel that clears the results: nothing above touches them, everything below may
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // (the listing of a hashed result is launched while this kernel runs and waits for its end on the device)
-    if (AGG != AGG_SCALAR) asm volatile("griddepcontrol.launch_dependents;");
+    // (the listing of a hashed result, or the clear of the next pass, is launched while this kernel runs and waits for its
+    // end on the device)
+    asm volatile("griddepcontrol.launch_dependents;");
 
     int64_t lsum = 0, lcnt = 0;
 

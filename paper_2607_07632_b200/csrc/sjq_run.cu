@@ -1061,7 +1061,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         // Directly behind the clear the kernel is launched while that one still runs (programmatic dependent launch):
         // it stages its tables, which were complete before the clear began, and waits for the clear before it touches
         // a result (two-join query, 60 M rows: 94 -> 92 us; filter and sum, 6 M rows: 20.5 -> 18.5 us back to back).
-        const bool behind = !opts.accumulate && !self_clear && hot_stage < 0 && !opts.event_before;
+        const bool behind = !opts.accumulate && hot_stage < 0 && !opts.event_before;
         st = jit ? jit_launch(compiled, P, grid, block, smem, behind, stream)
                  : fused_launch(aggp, mul, form, grid, block, smem, behind, P, stream);
         if (st != SJQ_OK) return st;
