@@ -282,9 +282,9 @@ __device__ __forceinline__ uint32_t hot_lookup(const DStage &S, const unsigned c
 // codes are not wanted), compares every key in it, and stops at a match or at the first bucket with a
 // free slot.  A hit finds its code in the words already loaded: one sector per probe step.  The rows of a
 // chunk advance in lock step so that their loads overlap; bounded by the bucket count.
-template <typename T, int CB, int NR, bool WANT>
+template <typename T, int CB, int NR, bool WANT, typename C>
 __device__ __forceinline__ uint32_t body_hash(const DStage &S, const unsigned char *smem, const T (&v)[NR], uint32_t m,
-                                              uint64_t (&code)[NR])
+                                              C (&code)[NR])
 {
     constexpr int KB = (int)sizeof(T);
     constexpr int K = bucket_keys(KB, CB);
@@ -350,7 +350,7 @@ __device__ __forceinline__ uint32_t body_hash(const DStage &S, const unsigned ch
             for (int i = 0; i < CH; ++i) {
                 if ((pending >> i) & 1u) {
                     bool found = false, has_free = false;
-                    uint64_t c = 0;
+                    C c = 0;
 #pragma unroll
                     for (int j = 0; j < K; ++j) {
                         T kj;
@@ -359,7 +359,7 @@ __device__ __forceinline__ uint32_t body_hash(const DStage &S, const unsigned ch
                         if (kj == v[base + i]) {
                             found = true;
                             if (WANT && CB == 4) c = u[i][CODE_WORD + j];
-                            if (WANT && CB == 8) c = ((uint64_t)u[i][CODE_WORD + 2 * j + 1] << 32) | u[i][CODE_WORD + 2 * j];
+                            if (WANT && CB == 8) c = (C)(((uint64_t)u[i][CODE_WORD + 2 * j + 1] << 32) | u[i][CODE_WORD + 2 * j]);
                         }
                         has_free |= kj == empty;
                     }
@@ -413,13 +413,18 @@ __device__ __forceinline__ uint32_t body_hashbits(const DStage &S, const unsigne
     return hit | known;
 }
 
-// C: the word codes are held in; with 32 bits there are neither 64-bit codes nor open-addressing tables.
+// C: the word codes are held in.  With 32 bits there are no 64-bit codes; the tables of 32-bit keys are direct, those of
+// 64-bit keys (HASH) open-addressing, and nothing else filters on a 64-bit column.
 template <typename T, int NR, bool WANT, bool HASH, typename C>
 __device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, const unsigned char *smem,
                                               const T (&v)[NR], uint32_t m, C (&code)[NR])
 {
     constexpr bool kWide = sizeof(C) == 8;
-    static_assert(kWide || !HASH, "open-addressing tables have 64-bit codes");
+    if constexpr (!kWide && sizeof(T) == 8) {
+        if (S.op == OP_HASHBITS) return body_hashbits<T, NR>(S, smem, v, m);
+        if (S.op != OP_HASH64) return m; // OP_LOAD
+        return S.code_bits == 0 ? body_hash<T, 0, NR, WANT>(S, smem, v, m, code) : body_hash<T, 4, NR, WANT>(S, smem, v, m, code);
+    }
     switch (S.op * 2 + S.in_smem) {
     case OP_PRED_RANGE * 2: return body_pred_range<T, NR>(S, v, m);
     case OP_PRED_SET * 2: return body_pred_set<T, NR>(P, S, v, m);
@@ -437,10 +442,10 @@ __device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, 
     case OP_DIRECT_U4 * 2 + 1: return body_direct<T, OP_DIRECT_U4, true, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U2 * 2: return body_direct<T, OP_DIRECT_U2, false, NR, WANT>(S, smem, v, m, code);
     case OP_DIRECT_U2 * 2 + 1: return body_direct<T, OP_DIRECT_U2, true, NR, WANT>(S, smem, v, m, code);
-    case OP_HASHBITS * 2: return HASH ? body_hashbits<T, NR>(S, smem, v, m) : 0u; // comes with an exact probe stage
+    case OP_HASHBITS * 2: return HASH && kWide ? body_hashbits<T, NR>(S, smem, v, m) : 0u; // comes with an exact probe stage
     case OP_HASH32 * 2:
     case OP_HASH64 * 2:
-        if constexpr (HASH) {
+        if constexpr (HASH && kWide) {
             if (S.code_bits == 0) return body_hash<T, 0, NR, WANT>(S, smem, v, m, code);
             if (S.code_bits == 32) return body_hash<T, 4, NR, WANT>(S, smem, v, m, code);
             return body_hash<T, 8, NR, WANT>(S, smem, v, m, code);
@@ -778,7 +783,7 @@ __device__ __forceinline__ void load_rows(const DStage &S, int64_t base, const u
     }
 }
 
-// NARROW kernels: every fact column and every code of the query has 32 bits.
+// NARROW kernels: every code of the query has 32 bits, and every fact column but the keys of open-addressing tables.
 template <bool NARROW>
 struct CodeWord {
     typedef uint64_t type;
@@ -794,7 +799,7 @@ __device__ __forceinline__ uint32_t filter_rows(const RunArg &P, const DStage &S
                                                 int64_t base, const uint32_t (&off)[NR], uint32_t valid)
 {
     typename CodeWord<NARROW>::type unused[NR];
-    if constexpr (!NARROW) {
+    if constexpr (!NARROW || HASH) {
         if (S.is64) {
             int64_t v[NR];
             load_rows<int64_t, false, NR>(S, base, off, valid, valid, v);
@@ -838,7 +843,7 @@ __device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, un
             } else {
                 load_rows<int32_t, CONTIG, NR>(S, base, off, valid, need, v);
             }
-            have_next = (s + 1 < SJQ_PV(nstages)) && (NARROW || !SJQ_STAGE(s + 1).is64);
+            have_next = (s + 1 < SJQ_PV(nstages)) && ((NARROW && !HASH) || !SJQ_STAGE(s + 1).is64);
             if (have_next) load_rows<int32_t, CONTIG, NR>(SJQ_STAGE(s + 1), base, off, valid, need, vnext);
             const int32_t mult = S.mult32[simple - 1];
             if (simple == 2) add_scaled32<NR>(X, mult, v, m);
@@ -849,7 +854,7 @@ __device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, un
         typename CodeWord<NARROW>::type code[NR];
 #pragma unroll
         for (int k = 0; k < NR; ++k) code[k] = 0;
-        if constexpr (!NARROW) {
+        if constexpr (!NARROW || HASH) {
             if (S.is64) {
                 int64_t v[NR];
                 load_rows<int64_t, CONTIG, NR>(S, base, off, valid, need, v);
@@ -866,7 +871,7 @@ __device__ __forceinline__ void final_rows(const RunArg &P, const DStage *st, un
         } else {
             load_rows<int32_t, CONTIG, NR>(S, base, off, valid, need, v);
         }
-        have_next = (s + 1 < SJQ_PV(nstages)) && (NARROW || !SJQ_STAGE(s + 1).is64);
+        have_next = (s + 1 < SJQ_PV(nstages)) && ((NARROW && !HASH) || !SJQ_STAGE(s + 1).is64);
         if (have_next) load_rows<int32_t, CONTIG, NR>(SJQ_STAGE(s + 1), base, off, valid, need, vnext);
         m = run_stage<int32_t, NR, true, HASH>(P, S, smem, v, m, code);
         if (S.acc) accumulate<MUL, int32_t, NR>(S, v, code, m, key, X, Y);
@@ -994,7 +999,7 @@ __device__ __forceinline__ uint32_t level0(const RunArg &P, const DStage *st, co
         if (!alive) break;
         const DStage &S = SJQ_STAGE(s);
         const unsigned char *from = s == 0 ? staged : nullptr; // only the first column is staged
-        if constexpr (!NARROW) {
+        if constexpr (!NARROW || HASH) {
             if (S.is64) {
                 alive = dense_stage<int64_t, FULL, HASH, NARROW>(P, S, smem, row0, slot_stride, valid, alive, from);
                 continue;

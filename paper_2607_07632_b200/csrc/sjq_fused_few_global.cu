@@ -12,7 +12,9 @@ fused_few_fn fused_few_global(bool mul, int form)
     case kFormDirect: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect>(mul);
     case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect | kFormHash>(mul);
     case kFormNarrow: return fused_of<RunParamsFew, AGG_GLOBAL, kFormNarrow>(mul);
-    default: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect | kFormNarrow>(mul);
+    case kFormDirect | kFormNarrow: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect | kFormNarrow>(mul);
+    case kFormHash | kFormNarrow: return fused_of<RunParamsFew, AGG_GLOBAL, kFormHash | kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_GLOBAL, kFormDirect | kFormHash | kFormNarrow>(mul);
     }
 }
 

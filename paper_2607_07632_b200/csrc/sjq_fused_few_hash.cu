@@ -12,7 +12,9 @@ fused_few_fn fused_few_hash(bool mul, int form)
     case kFormDirect: return fused_of<RunParamsFew, AGG_HASH, kFormDirect>(mul);
     case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_HASH, kFormDirect | kFormHash>(mul);
     case kFormNarrow: return fused_of<RunParamsFew, AGG_HASH, kFormNarrow>(mul);
-    default: return fused_of<RunParamsFew, AGG_HASH, kFormDirect | kFormNarrow>(mul);
+    case kFormDirect | kFormNarrow: return fused_of<RunParamsFew, AGG_HASH, kFormDirect | kFormNarrow>(mul);
+    case kFormHash | kFormNarrow: return fused_of<RunParamsFew, AGG_HASH, kFormHash | kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_HASH, kFormDirect | kFormHash | kFormNarrow>(mul);
     }
 }
 

@@ -12,7 +12,9 @@ fused_few_fn fused_few_scalar(bool mul, int form)
     case kFormDirect: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect>(mul);
     case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect | kFormHash>(mul);
     case kFormNarrow: return fused_of<RunParamsFew, AGG_SCALAR, kFormNarrow>(mul);
-    default: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect | kFormNarrow>(mul);
+    case kFormDirect | kFormNarrow: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect | kFormNarrow>(mul);
+    case kFormHash | kFormNarrow: return fused_of<RunParamsFew, AGG_SCALAR, kFormHash | kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_SCALAR, kFormDirect | kFormHash | kFormNarrow>(mul);
     }
 }
 

@@ -12,7 +12,9 @@ fused_few_fn fused_few_smem(bool mul, int form)
     case kFormDirect: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect>(mul);
     case kFormDirect | kFormHash: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect | kFormHash>(mul);
     case kFormNarrow: return fused_of<RunParamsFew, AGG_SMEM, kFormNarrow>(mul);
-    default: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect | kFormNarrow>(mul);
+    case kFormDirect | kFormNarrow: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect | kFormNarrow>(mul);
+    case kFormHash | kFormNarrow: return fused_of<RunParamsFew, AGG_SMEM, kFormHash | kFormNarrow>(mul);
+    default: return fused_of<RunParamsFew, AGG_SMEM, kFormDirect | kFormHash | kFormNarrow>(mul);
     }
 }
 

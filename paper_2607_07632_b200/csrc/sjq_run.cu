@@ -689,7 +689,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     // 32-bit fast path of the accumulators: int32 column, multipliers and payload ranges within int32
     for (int s2 = 0; s2 < ns; ++s2) {
         DStage &S = P.st[s2];
-        bool ok = !S.is64;
+        bool ok = !S.is64 || (S.acc & 0x7u) == 0; // (a payload's contribution does not depend on the key's width)
         for (int i = 0; i < 9; ++i) {
             ok = ok && S.mult[i] >= INT32_MIN && S.mult[i] <= INT32_MAX;
             S.mult32[i] = (int32_t)S.mult[i];
@@ -986,9 +986,11 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     for (int s2 = 0; s2 < ns; ++s2) {
         const DStage &S = P.st[s2];
         has_hash |= S.op == OP_HASH32 || S.op == OP_HASH64 || S.op == OP_HASHBITS;
-        narrow = narrow && !S.is64 && S.op != OP_DIRECT_U64 && (S.acc32 || !S.acc);
+        const bool hashed_key = S.is64 && (S.acc & 0x7u) == 0 &&
+                                (S.op == OP_LOAD || S.op == OP_HASHBITS || (S.op == OP_HASH64 && S.code_bits <= 32));
+        const bool plain = !S.is64 && S.op != OP_DIRECT_U64 && S.op != OP_HASH32 && S.op != OP_HASHBITS;
+        narrow = narrow && (plain || hashed_key) && (S.acc32 || !S.acc);
     }
-    narrow = narrow && !has_hash;
     const int form = (has_hash ? kFormHash : 0) | (P.nq == 0 ? kFormDirect : 0) | (narrow ? kFormNarrow : 0);
 
     // ------------------------------------------------------------ launch shape

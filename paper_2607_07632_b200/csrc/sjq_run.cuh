@@ -165,10 +165,10 @@ static_assert(sizeof(RunParams) == sizeof(RunStages<kMaxStages>) + sizeof(RunCor
 // The ahead-of-time kernels: aggregation path x product aggregate x form x up to kFewStages stages or any number,
 // instantiated in one translation unit per aggregation path and size.  A launch copies its whole parameter block, 6 KB
 // with twelve stages and 21 KB with all (a call of a small query 9.9 -> 8.1 us).
-// Forms: kFormHash, some table is open-addressing; kFormDirect, no queues; kFormNarrow (few stages, no open-addressing
-// table), every fact column and every code has 32 bits and accumulators take 32-bit contributions.  A form holds only the
-// bodies that its queries use: fewer registers and fewer instructions to fetch (four joins asked once, 60 M rows, the
-// whole call 262 -> 252 us).
+// Forms: kFormHash, some table is open-addressing; kFormDirect, no queues; kFormNarrow (few stages), every code has 32
+// bits, every fact column too except the keys of open-addressing tables, and accumulators take 32-bit contributions.  A
+// form holds only the bodies that its queries use: fewer registers and fewer instructions to fetch (four joins asked
+// once, 60 M rows, the whole call 262 -> 252 us; skewed 64-bit keys into an open-addressing table, 20 M rows 215 -> 174).
 constexpr int kFormHash = 1, kFormDirect = 2, kFormNarrow = 4;
 typedef RunParamsOf<kFewStages> RunParamsFew;
 typedef void (*fused_few_fn)(const RunParamsFew);
