@@ -553,42 +553,57 @@ __global__ void __launch_bounds__(kBuildThreads, 4) direct_build_kernel(const __
 // Open addressing.  A key claims the first free slot on its probe path (bucket after bucket from its home bucket, the
 // slots of a bucket in order) with atomicCAS on the key word, one CAS a step and no look before it (at the default load
 // 1.3 steps place a key), then its code goes beside it.  Bounded by the number of buckets; a key met on the way is a
-// duplicate.  The passing rows of a warp are gathered in shared memory and placed 32 at a time, so that every lane of
-// the chain of CASes, whose latency bounds the kernel, has a key.  2 M keys of 8 M rows of 16 bytes into 80 MB: 100 us,
-// 135 with each lane placing its own rows, 125 one row per thread; the CASes alone, random, take 45, the rows 20.
+// duplicate.  The latency of the CASes bounds the kernel, so a warp gathers its passing rows in shared memory and every
+// lane whose key has found its place takes the next one from there: a step costs the warp one latency, nearly all lanes
+// have a key in it, and a lane still walking when the queue is empty goes on with the keys of the warp's next rows.
+// 2 M keys of 8 M rows of 16 bytes into 80 MB, planned, built and probed by 10 M rows: 277 us with a warp placing 32 keys
+// at a time and waiting for the last of them, 264 so.  (The CASes alone, random, take 45, the rows 20.)
 constexpr int kHashThreads = 256;
-constexpr int kHashQueue = 31 + 128; // what is left of a batch and a warp's next rows
+constexpr int kHashQueue = 128; // a warp's next rows: the queue is empty before they come
+
+// A key on its way to its place.
+template <typename W, typename C>
+struct HashWalk {
+    W key;
+    C code;
+    uint32_t bucket, tried; // tried: buckets seen full
+    int slot;
+    bool on;
+};
 
 template <typename W, typename C>
-__device__ __forceinline__ void hash_place(const BuildTask &B, W key, C code)
+__device__ __forceinline__ void hash_start(const BuildTask &B, HashWalk<W, C> &H)
 {
-    const W empty = sizeof(W) == 8 ? (W)kEmptyKey64 : (W)(uint32_t)kEmptyKey32;
-    const uint64_t hashed = sizeof(W) == 8 ? (uint64_t)key : (uint64_t)(int64_t)(int32_t)key;
+    const uint64_t hashed = sizeof(W) == 8 ? (uint64_t)H.key : (uint64_t)(int64_t)(int32_t)H.key;
     if (B.filter) {
         const uint32_t fb = filter_hash(hashed) & B.fmask;
         atomicOr(B.filter + (fb >> 5), 1u << (fb & 31));
     }
-    uint32_t b = home_bucket(hashed, B.buckets), it = 0;
-    int j = 0;
-    for (;;) {
-        char *const bucket = static_cast<char *>(B.slots) + (size_t)b * kBucketBytes;
-        const W old = atomicCAS(reinterpret_cast<W *>(bucket) + j, empty, key);
-        if (old == empty) {
-            if (B.code_bits == 32) reinterpret_cast<uint32_t *>(bucket + B.code_off)[j] = (uint32_t)code;
-            else if (B.code_bits == 64) reinterpret_cast<uint64_t *>(bucket + B.code_off)[j] = code;
-            return;
-        }
-        if (old == key) {
-            set_status(B.status, SJQ_ERR_DUP_KEY);
-            return;
-        }
-        if (++j == B.bucket_k) {
-            j = 0;
-            b = b + 1 == B.buckets ? 0 : b + 1;
-            if (++it == B.buckets) {
-                set_status(B.status, SJQ_ERR_TABLE_FULL);
-                return;
-            }
+    H.bucket = home_bucket(hashed, B.buckets);
+    H.tried = 0;
+    H.slot = 0;
+    H.on = true;
+}
+
+template <typename W, typename C>
+__device__ __forceinline__ void hash_step(const BuildTask &B, HashWalk<W, C> &H)
+{
+    const W empty = sizeof(W) == 8 ? (W)kEmptyKey64 : (W)(uint32_t)kEmptyKey32;
+    char *const at = static_cast<char *>(B.slots) + (size_t)H.bucket * kBucketBytes;
+    const W old = atomicCAS(reinterpret_cast<W *>(at) + H.slot, empty, H.key);
+    if (old == empty) {
+        if (B.code_bits == 32) reinterpret_cast<uint32_t *>(at + B.code_off)[H.slot] = (uint32_t)H.code;
+        else if (B.code_bits == 64) reinterpret_cast<uint64_t *>(at + B.code_off)[H.slot] = H.code;
+        H.on = false;
+    } else if (old == H.key) {
+        set_status(B.status, SJQ_ERR_DUP_KEY);
+        H.on = false;
+    } else if (++H.slot == B.bucket_k) {
+        H.slot = 0;
+        H.bucket = H.bucket + 1 == B.buckets ? 0 : H.bucket + 1;
+        if (++H.tried == B.buckets) {
+            set_status(B.status, SJQ_ERR_TABLE_FULL);
+            H.on = false;
         }
     }
 }
@@ -600,13 +615,16 @@ __device__ __forceinline__ void hash_rows(const BuildTask &B, const DimFilters &
     static_assert(Set::kQuads == 1, "the queue takes 128 rows at a time");
     const W empty = sizeof(W) == 8 ? (W)kEmptyKey64 : (W)(uint32_t)kEmptyKey32;
     const int lane = threadIdx.x & 31;
+    const unsigned int below = (1u << lane) - 1u;
     W *const qkey = static_cast<W *>(queue);
-    C *const qcode = reinterpret_cast<C *>(qkey + kHashQueue + 1);
-    int waiting = 0;
+    C *const qcode = reinterpret_cast<C *>(qkey + kHashQueue);
+    HashWalk<W, C> H;
+    H.on = false;
     for (int64_t r = 4 * ((int64_t)(blockIdx.x - B.rows.block0) * kHashThreads + threadIdx.x);
          r - 4 * lane < B.rows.n; r += 4 * (int64_t)B.rows.blocks * kHashThreads) { // whole warps stay together
         Set R;
         read_rows(B.rows, F, r, 0, R);
+        int waiting = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             bool on = (R.m >> k) & 1u;
@@ -621,35 +639,49 @@ __device__ __forceinline__ void hash_rows(const BuildTask &B, const DimFilters &
             }
             const unsigned int lanes = __ballot_sync(0xffffffffu, on);
             if (on) {
-                const int at = waiting + __popc(lanes & ((1u << lane) - 1u));
+                const int at = waiting + __popc(lanes & below);
                 qkey[at] = (W)R.key[k];
                 qcode[at] = code;
             }
             waiting += __popc(lanes);
         }
         __syncwarp();
-        while (waiting >= 32) {
-            waiting -= 32;
-            hash_place<W>(B, qkey[waiting + lane], qcode[waiting + lane]);
-            __syncwarp();
+        while (waiting > 0) {
+            const unsigned int idle = __ballot_sync(0xffffffffu, !H.on);
+            const int mine = waiting - 1 - __popc(idle & below);
+            if (!H.on && mine >= 0) {
+                H.key = qkey[mine];
+                H.code = qcode[mine];
+                hash_start(B, H);
+            }
+            waiting -= __popc(idle);
+            if (H.on) hash_step(B, H);
         }
+        __syncwarp(); // the queue has been read
     }
-    if (lane < waiting) hash_place<W>(B, qkey[lane], qcode[lane]);
+    while (H.on) hash_step(B, H);
 }
 
 template <typename K>
 using UsualQuad = RowSet<K, int32_t, 1, 1>;
 
-__global__ void __launch_bounds__(kHashThreads, 5) hash_build_kernel(const __grid_constant__ BuildParams P)
+// USUAL: every dimension of the launch has at most one payload, of 32 bits (the other forms need more registers).
+template <bool USUAL>
+constexpr int kHashPerSm = USUAL ? 5 : 4;
+template <bool USUAL>
+__global__ void __launch_bounds__(kHashThreads, kHashPerSm<USUAL>) hash_build_kernel(const __grid_constant__ BuildParams P)
 {
-    __shared__ __align__(16) unsigned char queues[kHashThreads / 32][(kHashQueue + 1) * 16];
+    __shared__ __align__(16) unsigned char queues[kHashThreads / 32][kHashQueue * 16];
     const BuildTask &B = P.task[task_of_block(P.task, P.ntasks)];
     void *const queue = queues[threadIdx.x >> 5];
     cudaGridDependencySynchronize(); // the tables' memory is prepared by the kernel before this one
-    if (B.usual && !B.rows.key64) hash_rows<UsualQuad<int32_t>, uint32_t>(B, P.filters, queue);
-    else if (B.usual) hash_rows<UsualQuad<int64_t>, uint32_t>(B, P.filters, queue);
-    else if (!B.rows.key64) hash_rows<Wide<int32_t>, uint64_t>(B, P.filters, queue);
-    else hash_rows<Wide<int64_t>, uint64_t>(B, P.filters, queue);
+    if constexpr (USUAL) {
+        if (!B.rows.key64) hash_rows<UsualQuad<int32_t>, uint32_t>(B, P.filters, queue);
+        else hash_rows<UsualQuad<int64_t>, uint32_t>(B, P.filters, queue);
+    } else {
+        if (!B.rows.key64) hash_rows<Wide<int32_t>, uint64_t>(B, P.filters, queue);
+        else hash_rows<Wide<int64_t>, uint64_t>(B, P.filters, queue);
+    }
 }
 
 int bits_for(uint64_t range)
@@ -1249,7 +1281,10 @@ sjq_status build_launch(const sjq_dim_desc *dims, int ndims, const sjq_dim_layou
         }
         if (ok && H.ntasks) {
             H.filters = B.filters;
-            ok = launch_behind(hash_build_kernel, H, kHashThreads, 5, dev.sm_count, stream);
+            bool usual = true;
+            for (int i = 0; i < H.ntasks; ++i) usual = usual && H.task[i].usual;
+            ok = usual ? launch_behind(hash_build_kernel<true>, H, kHashThreads, kHashPerSm<true>, dev.sm_count, stream)
+                       : launch_behind(hash_build_kernel<false>, H, kHashThreads, kHashPerSm<false>, dev.sm_count, stream);
             ++launches;
         }
         tables[0]->launches = launches;
