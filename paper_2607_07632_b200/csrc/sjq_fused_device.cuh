@@ -603,12 +603,23 @@ __device__ __forceinline__ uint64_t smem_cell(const unsigned int *words, uint64_
 }
 
 // A row's group key is out of range.  A pass that clears its results itself notes it in shared memory and tells it at the
-// end, when the status word is known to be clear.
+// end, when the status word is known to be clear.  So do all ahead-of-time kernels whose blocks keep sums of their own (a
+// store is shorter than an atomic: four joins asked once, 60 M rows, 254 us and 262), while a compiled kernel over many
+// rows is better off telling it at once (a list of 500 groups, 3 M rows, 11.6 us and 12.3).
 __shared__ uint32_t range_seen;
-template <bool FUSED>
+template <int AGG>
+__device__ __forceinline__ constexpr bool range_noted()
+{
+#if defined(SJQ_JIT)
+    return (AGG == AGG_SCALAR || AGG == AGG_SMEM) && SJQ_JIT_may_clear != 0;
+#else
+    return AGG == AGG_SCALAR || AGG == AGG_SMEM;
+#endif
+}
+template <bool NOTED>
 __device__ __forceinline__ void note_range(const RunArg &P)
 {
-    if (FUSED && SJQ_PV(may_clear)) range_seen = 1u;
+    if (NOTED) range_seen = 1u;
     else set_status(P.status, SJQ_ERR_GROUP_RANGE);
 }
 
@@ -655,7 +666,7 @@ __device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, c
 #pragma unroll
             for (int k = 0; k < NR; ++k)
                 if (((m >> k) & 1u) && g[k] != 0) {
-                    note_range<FUSED>(P);
+                    note_range<FUSED && range_noted<AGG>()>(P);
                     m &= ~(1u << k);
                 }
         }
@@ -683,7 +694,7 @@ __device__ __forceinline__ void terminal(const RunArg &P, unsigned char *smem, c
 #pragma unroll
     for (int k = 0; k < NR; ++k)
         if (((m >> k) & 1u) && (uint64_t)g[k] >= ng) {
-            note_range<FUSED>(P);
+            note_range<FUSED && range_noted<AGG>()>(P);
             m &= ~(1u << k);
         }
     const bool want_count = SJQ_PV(want_count) != 0;
@@ -1183,8 +1194,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
 
     // (only in kernels for few rows: the registers that it takes cost a pass over many rows up to 30 %, and the clear kernel
     // costs that one next to nothing, since the pass starts behind it)
-    const bool may_clear = (AGG == AGG_SCALAR || AGG == AGG_SMEM) && DIRECT && SJQ_PV(may_clear);
-    const bool self_clear = may_clear && P.sync;
+    const bool self_clear = (AGG == AGG_SCALAR || AGG == AGG_SMEM) && DIRECT && SJQ_PV(may_clear) && P.sync;
     if (self_clear) {
         // launched while the kernel before it still runs (four joins, 400 thousand rows, interpreted: 12.4 -> 10.5 us)
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1225,7 +1235,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
         const int64_t cells = P.num_groups * (SJQ_PV(want_count) ? 2 : 1);
         for (int64_t i = tid; i < cells; i += blockDim.x) ss[i] = 0ull;
     }
-    if (may_clear && tid == 0) range_seen = 0u;
+    if (range_noted<AGG>() && tid == 0) range_seen = 0u;
     __syncthreads();
     if (self_clear && tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P);
     // launched behind the kernel that clears the results: nothing above touches them, everything below may
@@ -1510,7 +1520,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
             }
         }
     }
-    if (may_clear && tid == 0 && range_seen) set_status(P.status, SJQ_ERR_GROUP_RANGE);
+    if (range_noted<AGG>() && tid == 0 && range_seen) set_status(P.status, SJQ_ERR_GROUP_RANGE);
     if (self_clear) {
         if (AGG != AGG_SCALAR) __syncthreads(); // (a scalar result is added by thread 0)
         if (tid == 0) clear_over(P);
