@@ -125,9 +125,6 @@ __device__ __forceinline__ int64_t ld_sparse(const int64_t *p)
     return v;
 }
 
-// One word of a direct-mapped table.
-__device__ __forceinline__ uint32_t ld_table(const uint32_t *p) { return __ldg(p); }
-
 template <typename T>
 struct Index {
     typedef uint64_t type;
@@ -171,11 +168,26 @@ __device__ __forceinline__ uint32_t body_pred_set(const RunArg &P, const DStage 
     return m & pass;
 }
 
-template <typename T, int OP, bool SMEM, int NR, bool WANT, typename C>
+// A word of a direct-mapped table, `at` words from its start: from the copy in shared memory, from global memory, or, where
+// the copy is the first part of a larger table (kTabPart), from either.
+struct TablePlaces {
+    const unsigned char *global, *shared;
+    uint32_t held; // bytes of the copy
+};
+template <int WHERE, typename W, typename I>
+__device__ __forceinline__ W table_word(const TablePlaces &T, I at)
+{
+    if (WHERE == kTabShared || (WHERE == kTabPart && at < (I)(T.held / sizeof(W)))) return reinterpret_cast<const W *>(T.shared)[at];
+    return __ldg(reinterpret_cast<const W *>(T.global) + at);
+}
+
+template <typename T, int OP, int WHERE, int NR, bool WANT, typename C>
 __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned char *smem, const T (&v)[NR],
                                                 uint32_t m, C (&code)[NR])
 {
-    const unsigned char *base = SMEM ? smem + S.smem_off : static_cast<const unsigned char *>(S.tab);
+    // (formed once: an ahead-of-time kernel would read the descriptor at every row, four joins 256 -> 262 us)
+    const TablePlaces places{WHERE == kTabShared ? nullptr : static_cast<const unsigned char *>(S.tab),
+                         WHERE == kTabGlobal ? nullptr : smem + S.smem_off, WHERE == kTabPart ? S.tab_bytes : 0u};
     // A key outside the table's range is a miss, never an out-of-range access: its index is clamped to the
     // spare entry after the last slot, which is never set (one min instead of a range test and a mask).
     typename Index<T>::type idx[NR];
@@ -195,10 +207,7 @@ __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned 
 #pragma unroll
         for (int i = 0; i < NR; ++i) {
             w[i] = 0;
-            if ((m >> i) & 1u) {
-                const uint32_t *p = reinterpret_cast<const uint32_t *>(base) + (idx[i] >> 5);
-                w[i] = SMEM ? *p : ld_table(p);
-            }
+            if ((m >> i) & 1u) w[i] = table_word<WHERE, uint32_t>(places, idx[i] >> 5);
         }
         // rotate the wanted bit of the word straight into position i of the mask (the funnel shift takes its
         // amount modulo 32): subtract, rotate, and-or
@@ -214,10 +223,7 @@ __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned 
 #pragma unroll
         for (int i = 0; i < NR; ++i) {
             w[i] = ~0u;
-            if ((m >> i) & 1u) {
-                const uint32_t *p = reinterpret_cast<const uint32_t *>(base) + (idx[i] / PER);
-                w[i] = SMEM ? *p : ld_table(p);
-            }
+            if ((m >> i) & 1u) w[i] = table_word<WHERE, uint32_t>(places, idx[i] / PER);
         }
 #pragma unroll
         for (int i = 0; i < NR; ++i) {
@@ -237,19 +243,10 @@ __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned 
         for (int i = 0; i < NR; ++i) {
             c[i] = (C)~0ULL;
             if ((m >> i) & 1u) {
-                if (OP == OP_DIRECT_U8) {
-                    const uint8_t *p = base + idx[i];
-                    c[i] = SMEM ? *p : __ldg(p);
-                } else if (OP == OP_DIRECT_U16) {
-                    const uint16_t *p = reinterpret_cast<const uint16_t *>(base) + idx[i];
-                    c[i] = SMEM ? *p : __ldg(p);
-                } else if (OP == OP_DIRECT_U32) {
-                    const uint32_t *p = reinterpret_cast<const uint32_t *>(base) + idx[i];
-                    c[i] = SMEM ? *p : __ldg(p);
-                } else {
-                    const uint64_t *p = reinterpret_cast<const uint64_t *>(base) + idx[i];
-                    c[i] = SMEM ? *p : __ldg(p);
-                }
+                if (OP == OP_DIRECT_U8) c[i] = table_word<WHERE, uint8_t>(places, idx[i]);
+                else if (OP == OP_DIRECT_U16) c[i] = table_word<WHERE, uint16_t>(places, idx[i]);
+                else if (OP == OP_DIRECT_U32) c[i] = table_word<WHERE, uint32_t>(places, idx[i]);
+                else c[i] = (C)table_word<WHERE, uint64_t>(places, idx[i]);
             }
         }
         const C miss = OP == OP_DIRECT_U8 ? (C)0xFFull : OP == OP_DIRECT_U16 ? (C)0xFFFFull
@@ -425,23 +422,33 @@ __device__ __forceinline__ uint32_t run_stage(const RunArg &P, const DStage &S, 
         if (S.op != OP_HASH64) return m; // OP_LOAD
         return S.code_bits == 0 ? body_hash<T, 0, NR, WANT>(S, smem, v, m, code) : body_hash<T, 4, NR, WANT>(S, smem, v, m, code);
     }
+#if defined(SJQ_JIT)
+    if (S.in_smem == kTabPart) {
+        switch (S.op) {
+        case OP_DIRECT_BITMAP: return body_direct<T, OP_DIRECT_BITMAP, kTabPart, NR, WANT>(S, smem, v, m, code);
+        case OP_DIRECT_U2: return body_direct<T, OP_DIRECT_U2, kTabPart, NR, WANT>(S, smem, v, m, code);
+        case OP_DIRECT_U4: return body_direct<T, OP_DIRECT_U4, kTabPart, NR, WANT>(S, smem, v, m, code);
+        default: return body_direct<T, OP_DIRECT_U8, kTabPart, NR, WANT>(S, smem, v, m, code); // (no wider codes)
+        }
+    }
+#endif
     switch (S.op * 2 + S.in_smem) {
     case OP_PRED_RANGE * 2: return body_pred_range<T, NR>(S, v, m);
     case OP_PRED_SET * 2: return body_pred_set<T, NR>(P, S, v, m);
-    case OP_DIRECT_BITMAP * 2: return body_direct<T, OP_DIRECT_BITMAP, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_BITMAP * 2 + 1: return body_direct<T, OP_DIRECT_BITMAP, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U8 * 2: return body_direct<T, OP_DIRECT_U8, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U8 * 2 + 1: return body_direct<T, OP_DIRECT_U8, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U16 * 2: return body_direct<T, OP_DIRECT_U16, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U16 * 2 + 1: return body_direct<T, OP_DIRECT_U16, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U32 * 2: return body_direct<T, OP_DIRECT_U32, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U32 * 2 + 1: return body_direct<T, OP_DIRECT_U32, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U64 * 2: return !kWide ? m : body_direct<T, OP_DIRECT_U64, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U64 * 2 + 1: return !kWide ? m : body_direct<T, OP_DIRECT_U64, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U4 * 2: return body_direct<T, OP_DIRECT_U4, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U4 * 2 + 1: return body_direct<T, OP_DIRECT_U4, true, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U2 * 2: return body_direct<T, OP_DIRECT_U2, false, NR, WANT>(S, smem, v, m, code);
-    case OP_DIRECT_U2 * 2 + 1: return body_direct<T, OP_DIRECT_U2, true, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_BITMAP * 2: return body_direct<T, OP_DIRECT_BITMAP, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_BITMAP * 2 + 1: return body_direct<T, OP_DIRECT_BITMAP, kTabShared, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U8 * 2: return body_direct<T, OP_DIRECT_U8, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U8 * 2 + 1: return body_direct<T, OP_DIRECT_U8, kTabShared, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U16 * 2: return body_direct<T, OP_DIRECT_U16, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U16 * 2 + 1: return body_direct<T, OP_DIRECT_U16, kTabShared, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U32 * 2: return body_direct<T, OP_DIRECT_U32, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U32 * 2 + 1: return body_direct<T, OP_DIRECT_U32, kTabShared, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U64 * 2: return !kWide ? m : body_direct<T, OP_DIRECT_U64, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U64 * 2 + 1: return !kWide ? m : body_direct<T, OP_DIRECT_U64, kTabShared, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U4 * 2: return body_direct<T, OP_DIRECT_U4, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U4 * 2 + 1: return body_direct<T, OP_DIRECT_U4, kTabShared, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U2 * 2: return body_direct<T, OP_DIRECT_U2, kTabGlobal, NR, WANT>(S, smem, v, m, code);
+    case OP_DIRECT_U2 * 2 + 1: return body_direct<T, OP_DIRECT_U2, kTabShared, NR, WANT>(S, smem, v, m, code);
     case OP_HASHBITS * 2: return HASH && kWide ? body_hashbits<T, NR>(S, smem, v, m) : 0u; // comes with an exact probe stage
     case OP_HASH32 * 2:
     case OP_HASH64 * 2:

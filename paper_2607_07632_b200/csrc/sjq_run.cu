@@ -120,6 +120,10 @@ bool valid_term(const sjq_term &t, int nfact, const sjq_join *joins, int njoins)
     return false;
 }
 
+// A map staged in part (see there): from so many rows on, so much of it.
+constexpr int64_t kPartRows = (int64_t)1 << 24;
+constexpr size_t kPartBytes = (size_t)192 << 10;
+
 // What a filter stage costs, in picoseconds per fact row on the whole chip (148 SMs, 1.9 GHz, 6.5 TB/s).
 constexpr double kPsByte = 0.154;  // a byte of DRAM traffic
 constexpr double kPsIssue = 0.3;   // evaluating a row (about ten instructions)
@@ -939,6 +943,35 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
         } else if (!stage_tables(block, &tables)) {
             return SJQ_ERR_UNSUPPORTED;
         }
+    }
+    // Every row probes a map too large for the 32 KB above and adds to a global table: the pass is bound by the L2's tags
+    // and the requests of the SMs, of which a row costs two to three.  The first part of the map, or all of it, is then
+    // staged in the shared memory that such a plan has to itself, and a probe asks the L2 only beyond it (the L1 answers
+    // next to none of those probes: its lines fill sector by sector).  192 KB leave an L1 of 32 KB; with more it is too
+    // small for the columns.  The sweep's lists with every row left, 750 KB map: a million groups, 600 M rows 5619 -> 4898
+    // us (64 KB 5516, 128 KB 5416, 176 KB 5335, 192 KB with blocks of 1024 threads 5086, 768 4996, 640 5098, 200 KB 5523);
+    // 20 thousand groups, 100 M rows 1063 -> 996; a 250 KB map, 20 M rows 190 -> 175; the same groups as a dense array, 50
+    // thousand, 1435 -> 1392; a 75 KB map, 500 thousand groups 719 -> 708; no gain for 3 M rows.  With a shared group table or register sums the L1's own rate is the bound, and
+    // the second, divergent load costs what it saves (a thousand groups, 600 K and 3 M keys: 332 -> 350, 420 -> 397).
+    int part = -1;
+    if (opts.specialise && !opts.unfused && !opts.block_threads && !opts.ctas_per_sm && opts.smem_tables == 0 && P.nq == 0 &&
+        aggp == AGG_GLOBAL && hot_stage < 0 && plan_rows >= kPartRows) {
+        for (int s = 0; s < nfilter; ++s) {
+            const DStage &S = P.st[s];
+            const bool narrow_codes = S.op == OP_DIRECT_BITMAP || S.op == OP_DIRECT_U2 || S.op == OP_DIRECT_U4 || S.op == OP_DIRECT_U8;
+            if (narrow_codes && !S.in_smem && reach[s] >= 0.5 && (part < 0 || S.tab_bytes < P.st[part].tab_bytes)) part = s;
+        }
+    }
+    if (part >= 0 && stage_bytes + tables + kPartBytes <= smem_cap) {
+        DStage &S = P.st[part];
+        const size_t whole = S.tab_bytes;
+        S.in_smem = align_up(S.tab_bytes, 16) <= kPartBytes ? kTabShared : kTabPart;
+        S.smem_off = (uint32_t)(stage_bytes + tables);
+        if (S.in_smem == kTabPart) S.tab_bytes = (uint32_t)kPartBytes;
+        tables += align_up(S.tab_bytes, 16);
+        // fewer, longer chains where every row goes all the way and most of the map is beyond the copy
+        block = reach[nfilter] >= 0.9 && P.st[part].in_smem == kTabPart && whole > 3 * kPartBytes ? 512 : 768;
+        single_block = true;
     }
     P.smem_stages = 0;
     P.smem_groups = (uint32_t)(stage_bytes + tables + hot_bytes);

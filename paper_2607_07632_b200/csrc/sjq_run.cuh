@@ -28,6 +28,9 @@ enum : uint8_t {
     OP_DIRECT_U4 = 11, // sub-byte codes, eight / sixteen to a 32-bit word
     OP_DIRECT_U2 = 12
 };
+// where a direct table is probed: in global memory, in a copy in shared memory, or, where the copy is the first part of a
+// larger table, in either (compiled kernels)
+enum : uint8_t { kTabGlobal = 0, kTabShared = 1, kTabPart = 2 };
 __host__ __device__ constexpr bool is_code_op(int op)
 {
     return (op >= OP_DIRECT_U8 && op <= OP_DIRECT_U64) || op == OP_DIRECT_U4 || op == OP_DIRECT_U2;

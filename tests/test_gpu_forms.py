@@ -115,3 +115,32 @@ def test_forms_by_key_code_and_multiplier(n, key64, payloads, mult, hashed):
         res, exp, _ = run_both(w, fact, {"d": dim})
         assert res.status() == 0
         compare(w, res, exp)
+
+
+@pytest.mark.parametrize("keys", [200_000, 786_431, 786_432, 786_433, 1_600_000])  # 2-bit codes: 192 KB hold 786,432
+@pytest.mark.parametrize("payload", [3, 200])
+@pytest.mark.parametrize("hashed", [False, True])
+def test_a_map_staged_whole_and_in_part(keys, payload, hashed):
+    """2- and 8-bit codes on both sides of what is staged; keys below, on the edges of and beyond the map's range."""
+    n, rng = 2**24 + 3, np.random.default_rng(keys)
+    dim = {"k": np.arange(7, keys + 7, dtype=np.int32), "v": rng.integers(0, payload + 1, keys).astype(np.int32)}
+    fact = {"fk": rng.integers(5, keys + 9, n).astype(np.int32), "g": rng.integers(0, 2**30, n).astype(np.int32)}
+    edges = np.array([6, 7, 7 + 196_607, 7 + 196_608, 7 + 786_431, 7 + 786_432, 6 + keys, 7 + keys, -2**31, 2**31 - 1])
+    fact["fk"][:10] = edges
+    groups = 50_000
+    w = adhoc("part", fact, [("d", dim, "k", [], ["v"])], [("fk", "d")], [], KeyExpr((Term("FACT", "g"),), modulo=groups),
+              AggExpr("ADD", Term("FACT", "fk"), Term("PAYLOAD", 0, 0)), "HASHED" if hashed else "DENSE", num_groups=groups,
+              capacity=2 * groups)
+    opts = sjq.RunOpts(specialise=True)
+    tables = sjq.build_workload_tables(w, {"d": to_dev(dim)})
+    dev = to_dev(fact)
+    res = sjq.run_workload(w, dev, tables, opts)
+    assert res.status() == 0 and res.info.describe()["in_smem"][0] == (1 if keys * (2 if payload == 3 else 8) < 8 * 192 * 1024 else 2)
+    hit = (fact["fk"] >= 7) & (fact["fk"] < keys + 7)
+    at, g = fact["fk"][hit].astype(np.int64), fact["g"][hit] % groups
+    value = at + dim["v"][at - 7]
+    sums = np.bincount(g, weights=value.astype(np.float64), minlength=groups)  # below 2**53: exact
+    counts = np.bincount(g, minlength=groups)
+    k, s, c = res.hashed_sorted() if hashed else (None, res.sums, res.counts)
+    assert hashed is False or np.array_equal(k.cpu().numpy(), np.arange(groups))
+    assert np.array_equal(s.cpu().numpy(), sums.astype(np.int64)) and np.array_equal(c.cpu().numpy(), counts)
