@@ -732,7 +732,7 @@ def alloc_result(mode: str, num_groups: int, capacity: int, want_count: bool, de
             raise SjqError(rc, "sjq_run_workspace_bytes")
         ws = torch.empty(nbytes.value, dtype=torch.uint8, device=device)
     status = new(1, dtype=torch.int32, device=device)
-    sync = torch.empty(SYNC_BYTES // 8, dtype=torch.int64, device=device)
+    sync = None if mode == "HASHED" else torch.empty(SYNC_BYTES // 8, dtype=torch.int64, device=device)
     return Result(mode, sums, counts, keys, n_groups, status, ws, joined=joined, sync=sync)
 
 
