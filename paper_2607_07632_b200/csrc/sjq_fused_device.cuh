@@ -185,7 +185,7 @@ template <typename T, int OP, int WHERE, int NR, bool WANT, typename C>
 __device__ __forceinline__ uint32_t body_direct(const DStage &S, const unsigned char *smem, const T (&v)[NR],
                                                 uint32_t m, C (&code)[NR])
 {
-    // (formed once: an ahead-of-time kernel would read the descriptor at every row, four joins 256 -> 262 us)
+    // (formed once: an ahead-of-time kernel would read the descriptor at every row, four joins asked once 252 -> 262 us)
     const TablePlaces places{WHERE == kTabShared ? nullptr : static_cast<const unsigned char *>(S.tab),
                          WHERE == kTabGlobal ? nullptr : smem + S.smem_off, WHERE == kTabPart ? S.tab_bytes : 0u};
     // A key outside the table's range is a miss, never an out-of-range access: its index is clamped to the
@@ -610,9 +610,8 @@ __device__ __forceinline__ uint64_t smem_cell(const unsigned int *words, uint64_
 }
 
 // A row's group key is out of range.  A pass that clears its results itself notes it in shared memory and tells it at the
-// end, when the status word is known to be clear.  So do all ahead-of-time kernels whose blocks keep sums of their own (a
-// store is shorter than an atomic: four joins asked once, 60 M rows, 254 us and 262), while a compiled kernel over many
-// rows is better off telling it at once (a list of 500 groups, 3 M rows, 11.6 us and 12.3).
+// end, when the status word is known to be clear; so do all ahead-of-time kernels whose blocks keep sums of their own,
+// which do not know at compile time whether they will clear.
 __shared__ uint32_t range_seen;
 template <int AGG>
 __device__ __forceinline__ constexpr bool range_noted()
