@@ -17,7 +17,8 @@ namespace {
 #define SJQ_NAMES(X)                                                                                                   \
     X(data_ptr) X(dtype) X(is_cuda) X(is_contiguous) X(dim) X(numel) X(col) X(op) X(lo) X(hi) X(values) X(handle)       \
     X(terms) X(offset) X(modulo) X(src) X(a) X(b) X(mult) X(x) X(y) X(want_count) X(sums) X(counts) X(keys)             \
-    X(n_groups) X(status_dev) X(workspace) X(sync) X(info) X(block_threads) X(ctas_per_sm) X(eager_loads) X(agg_path)           \
+    X(n_groups) X(status_dev) X(workspace) X(sync) X(element_size) X(get_device) X(info) X(block_threads)               \
+    X(ctas_per_sm) X(eager_loads) X(agg_path)                                                                          \
     X(smem_tables) X(compaction) X(accumulate) X(order) X(events) X(cuda_event) X(specialise) X(rows_per_lane)          \
     X(no_filter_bitmap) X(host_copy_all) X(dense_slots) X(group_hash_always) X(warp_agg) X(unfused_scratch)             \
     X(pass_ppm) X(hot_keys) X(hot_scratch) X(l0_bulk)
@@ -250,12 +251,37 @@ bool read_opts(PyObject *p, sjq_run_opts *o)
     return true;
 }
 
-// run(fact, preds, joins, key, agg, mode, num_groups, capacity, opts, result, stream, hot_scratch) -> status
+// The scratch with which a pass clears its result: the kernel writes SJQ_SYNC_BYTES through it, so a tensor that is shorter,
+// or not on the device of the call, must not reach it.  A result without the attribute, or with None, brings none.
+bool read_sync(PyObject *result, int64_t device, void **sync, bool *small)
+{
+    *small = false;
+    Ref t(PyObject_GetAttr(result, N.sync));
+    if (!t) {
+        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return false;
+        PyErr_Clear();
+        return true;
+    }
+    int64_t cells = 0, width = 0, at = 0;
+    if (!pointer_of(t.p, sync, &cells)) return false;
+    if (t.p == Py_None) return true;
+    if (!call_int(t.p, N.element_size, &width) || !call_int(t.p, N.get_device, &at)) return false;
+    Ref contiguous(PyObject_CallMethodNoArgs(t.p, N.is_contiguous));
+    if (!contiguous) return false;
+    if (at != device || contiguous.p != Py_True) {
+        PyErr_SetString(PyExc_ValueError, "the sync words of a result must be a contiguous tensor on the device of its columns");
+        return false;
+    }
+    *small = cells * width < SJQ_SYNC_BYTES;
+    return true;
+}
+
+// run(fact, preds, joins, key, agg, mode, num_groups, capacity, opts, result, stream, hot_scratch, device) -> status
 // `hot_scratch()` supplies the scratch of the hot-key table where the options bring none and a join could use it.
 PyObject *py_run(PyObject *, PyObject *const *args, Py_ssize_t nargs)
 {
-    if (nargs != 12) {
-        PyErr_SetString(PyExc_TypeError, "run takes 12 arguments");
+    if (nargs != 12 && nargs != 13) {
+        PyErr_SetString(PyExc_TypeError, "run takes 12 or 13 arguments");
         return nullptr;
     }
     PyObject *fact = args[0], *joins = args[2], *key = args[3], *agg = args[4], *opts = args[8], *result = args[9];
@@ -334,7 +360,10 @@ PyObject *py_run(PyObject *, PyObject *const *args, Py_ssize_t nargs)
         !get_pointer(result, N.status_dev, &R.status) || !get_pointer(result, N.workspace, &R.workspace, &workspace_bytes))
         return nullptr;
     R.workspace_bytes = (size_t)workspace_bytes;
-    if (!get_pointer(result, N.sync, &o.sync)) return nullptr;
+    int64_t device = 0;
+    bool small = false;
+    if ((nargs > 12 && !as_int(args[12], &device)) || !read_sync(result, device, &o.sync, &small)) return nullptr;
+    if (small) return PyLong_FromLong(SJQ_ERR_BUFFER_SMALL);
 
     Ref scratch(nullptr); // held until the call has enqueued its work
     if (hashed && !o.hot_scratch && o.hot_keys != 2) {

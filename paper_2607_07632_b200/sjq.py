@@ -797,7 +797,7 @@ def run(fact: dict, preds=(), joins=(), key=None, agg=None, mode: str = "SCALAR"
         res = alloc_result(mode, num_groups, capacity, agg.want_count, device, cleared=bool(opts and opts.accumulate))
     # (one hot-key scratch per device, reused by every run: runs on one stream are ordered)
     rc = marshal().run(fact, preds, joins, key, agg, MODES[mode], num_groups, capacity, opts, res,
-                       _raw_stream(index), lambda: _hot_scratch(device))
+                       _raw_stream(index), lambda: _hot_scratch(device), index)
     if rc != 0:
         raise SjqError(rc, "sjq_run")
     return res
@@ -889,6 +889,19 @@ def host_transfer_plan(fact: dict, preds=(), joins=(), key=None, agg=None, opts:
     return {n: (label[how[i]], share[i]) for i, n in enumerate(names)}
 
 
+def _sync_pointer(res, device) -> Optional[int]:
+    """Address of the scratch with which a pass clears its result, if the result brings it: the kernel writes SYNC_BYTES
+    through it, so what is shorter, or not on the device of the run, is refused here."""
+    sync = getattr(res, "sync", None)
+    if sync is None:
+        return None
+    if sync.device != device or not sync.is_contiguous():
+        raise ValueError("the sync words of a result must be a contiguous tensor on the device of its columns")
+    if sync.numel() * sync.element_size() < SYNC_BYTES:
+        raise SjqError(5, "sjq_run_host")  # SJQ_ERR_BUFFER_SMALL
+    return sync.data_ptr()
+
+
 def run_host(fact: dict, staging: torch.Tensor, chunk_rows: int, preds=(), joins=(), key=None, agg=None,
              mode: str = "SCALAR", num_groups: int = 1, capacity: int = 0, opts: Optional[RunOpts] = None,
              result: Optional[Result] = None, host: Optional[HostResult] = None):
@@ -916,7 +929,7 @@ def run_host(fact: dict, staging: torch.Tensor, chunk_rows: int, preds=(), joins
                               torch.zeros(1, dtype=torch.int32, **pin))
         cres = _result_struct(res)
         copts = (opts or RunOpts()).to_c()
-        copts.sync = res.sync.data_ptr() if res.sync is not None else None
+        copts.sync = _sync_pointer(res, device)
         rc = lib().sjq_run_host(carr, len(names), parr, len(preds), jarr, len(joins),
                                 ctypes.byref(kexpr) if kexpr is not None else None, ctypes.byref(aexpr),
                                 ctypes.byref(spec), ctypes.byref(cres), ctypes.byref(copts), staging.data_ptr(),
