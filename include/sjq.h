@@ -62,8 +62,9 @@ enum {
     SJQ_ERR_GROUP_OVERFLOW = 19, /* hashed mode: more distinct groups than the capacity */
     SJQ_ERR_RESERVED_KEY = 20,   /* a dimension key equals the reserved empty marker (minimum of its type) */
     SJQ_ERR_LAYOUT_MISMATCH = 21, /* build saw a key or payload outside the planned layout */
-    SJQ_ERR_ASYNC_WAIT = 22       /* a bounded wait for a bulk-asynchronous copy ran out; the kernel went on with
-                                     plain loads, so the result is still exact, but the device needs a look */
+    SJQ_ERR_ASYNC_WAIT = 22       /* a bounded wait ran out, so the device needs a look: for a bulk-asynchronous copy, where
+                                     the kernel went on with plain loads and the result is still exact, or for the clear
+                                     of a result by its pass (sjq_run_opts.sync), where rows are missing from it */
 };
 
 enum { SJQ_I32 = 0, SJQ_I64 = 1 };
@@ -402,7 +403,11 @@ typedef struct sjq_run_opts {
                         tests reach that path without faulting anything; the result is still exact. */
     void *sync; /* device scratch of SJQ_SYNC_BYTES bytes (8-byte aligned, of any content) that goes with `out`: used by
                    this run and by nothing else until the run is over.  With it a run over few rows clears a scalar or
-                   dense result in its pass, which saves the clear kernel; NULL = a kernel of its own clears the result */
+                   dense result in its pass, which saves the clear kernel; NULL = a kernel of its own clears the result.
+                   The blocks of the pass wait for one another's clear, for half a second or so; a block whose wait runs
+                   out leaves its rows out and the run ends with SJQ_ERR_ASYNC_WAIT in *out->status. */
+    int32_t sync_late_ms; /* 0; otherwise the block that clears first sleeps so many milliseconds (at most 5000) before it
+                             does, which is how the tests reach that path without faulting anything */
 } sjq_run_opts;
 
 #define SJQ_SYNC_BYTES 64

@@ -1111,16 +1111,33 @@ __device__ __forceinline__ uint32_t queue_base(int l)
 // on the device.  With words to meet at (P.sync) the first few blocks of the pass clear the results while the others
 // begin; a block's sums are its own (registers, a shared group table), and it looks at the flags at its end, before it
 // adds them to the results (a pass that adds its rows one by one to a global table would have to look before its first row:
-// 300 thousand rows, skewed keys, 4096 groups 23.4 us with the clear kernel and 26.9 so).  A flag is up when it holds the number of this very
-// call, so that the words may hold anything before the first one; the last block to finish takes all flags down, so that
-// a captured call can be replayed.  The blocks that clear wait for nobody before their flags are up and are the first
-// of the grid, so the others never wait for a block that waits for them; every wait is bounded all the same.
+// 300 thousand rows, skewed keys, 4096 groups 23.4 us with the clear kernel and 26.9 so).  A flag is up when it holds the
+// number of this very call, so that the words may hold anything before the first one; the last block to finish takes all
+// flags down, so that a captured call can be replayed.  The blocks that clear wait for nobody before their flags are up
+// and are the first of the grid, so the others never wait for a block that waits for them.
+// Every wait is bounded all the same.  A block whose wait ran out does not add its sums, which the late clear might wipe,
+// and arrives as late; the last block to arrive, behind every clear, turns that into the status.  The word that counts the
+// arrivals names the call too, and whoever finds it without that name gives it one: arrivals are counted before block 0
+// has got there, and the last one is known, and leaves the words at rest, however late a block is.
 // (100 thousand rows, filter and sum, interpreted, back to back: 10.2 -> 8.2 us.)
 constexpr int kClearSpins = 1 << 20;
-__device__ __forceinline__ void clear_share(const RunArg &P)
+constexpr uint64_t kClearArrivals = (1ull << 20) - 1, kClearLate = 1ull << 20; // the rest of the word: the call
+constexpr int kClearCall = 21;
+__device__ __forceinline__ bool clear_of_call(const RunArg &P, uint64_t word) { return ((word ^ (P.epoch << kClearCall)) >> kClearCall) == 0; }
+__device__ __forceinline__ uint64_t clear_swap(const RunArg &P, uint64_t from, uint64_t to)
+{
+    return atomicCAS(reinterpret_cast<unsigned long long *>(P.sync), (unsigned long long)from, (unsigned long long)to);
+}
+// Returns what thread 0 of block 0 found in the word of the arrivals: looked at behind the barrier, so that the answer's way
+// back is not waited for alone.
+__device__ __forceinline__ uint64_t clear_share(const RunArg &P)
 {
     const int64_t step = (int64_t)P.clear_blocks * blockDim.x;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (P.clear_late_ms && blockIdx.x == 0)
+        for (int ms = 0; ms < P.clear_late_ms; ++ms) __nanosleep(1000000u);
+    uint64_t word = 0;
+    if (first == 0) word = clear_swap(P, 0, P.epoch << kClearCall);
     for (int64_t i = first; i < P.clear_cells / 2; i += step) {
         reinterpret_cast<longlong2 *>(P.sums)[i] = make_longlong2(0, 0);
         if (P.clear_counts) reinterpret_cast<longlong2 *>(P.clear_counts)[i] = make_longlong2(0, 0);
@@ -1131,37 +1148,56 @@ __device__ __forceinline__ void clear_share(const RunArg &P)
             if (P.clear_counts) P.clear_counts[P.clear_cells - 1] = 0;
         }
         *P.status = 0;
-        P.sync[0] = 0;
     }
+    return word;
 }
 // (thread 0, behind a barrier of the block)
-__device__ __forceinline__ void clear_told(const RunArg &P)
+__device__ __forceinline__ void clear_told(const RunArg &P, uint64_t word)
 {
+    // left by another user of the memory (only a late block can change it meanwhile, and that gives it this call's name)
+    while (word != 0 && !clear_of_call(P, word)) {
+        const uint64_t now = clear_swap(P, word, P.epoch << kClearCall);
+        word = now == word ? 0 : now;
+    }
     __threadfence();
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(P.sync + 1 + blockIdx.x), "l"(P.epoch) : "memory");
 }
-// (thread 0, before a barrier of the block)
-__device__ __forceinline__ void clear_wait(const RunArg &P)
+// (thread 0, before a barrier of the block)  Whether all flags are up.
+__device__ __forceinline__ bool clear_wait(const RunArg &P)
 {
+    int spins = kClearSpins;
     for (int b = 0; b < P.clear_blocks; ++b) {
         uint64_t seen = 0;
-        for (int spin = 0; spin < kClearSpins && seen != P.epoch; ++spin)
+        for (; spins > 0 && seen != P.epoch; --spins)
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(P.sync + 1 + b) : "memory");
-        if (seen != P.epoch) set_status(P.status, SJQ_ERR_ASYNC_WAIT);
+        if (seen != P.epoch) return false;
     }
+    return true;
 }
 // (thread 0, behind the block's last use of the results and a barrier)
-__device__ __forceinline__ void clear_over(const RunArg &P)
+__device__ __forceinline__ void clear_over(const RunArg &P, bool late)
 {
     __threadfence();
-    if (atomicAdd(reinterpret_cast<unsigned long long *>(P.sync), 1ull) != (unsigned long long)gridDim.x - 1ull) return;
+    uint64_t word;
+    if (!late) {
+        word = atomicAdd(reinterpret_cast<unsigned long long *>(P.sync), 1ull);
+    } else {
+        uint64_t found = 0, now; // (a try fails because another block has arrived: bounded by the grid)
+        while ((now = clear_swap(P, found, word = ((clear_of_call(P, found) ? found : P.epoch << kClearCall) | kClearLate) + 1)) != found) found = now;
+        --word;
+    }
+    if ((word & kClearArrivals) != gridDim.x - 1) return;
+    __threadfence();
+    if (word & kClearLate) set_status(P.status, SJQ_ERR_ASYNC_WAIT);
     for (int b = 0; b <= P.clear_blocks; ++b) P.sync[b] = 0;
 }
 
 // The scalar terminal's tail (Section 3.2: one atomic per block instead of one per matching row): warp
-// shuffle reduce, block reduce through shared memory, one global atomic per block.
-__device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsum, int64_t lcnt, bool self_clear = false)
+// shuffle reduce, block reduce through shared memory, one global atomic per block.  False (thread 0) if the block waited for
+// the clear in vain and its sums were not added.
+__device__ __forceinline__ bool scalar_block_reduce(const RunArg &P, int64_t lsum, int64_t lcnt, bool self_clear = false)
 {
+    bool cleared = true;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
         lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
@@ -1181,12 +1217,13 @@ __device__ __forceinline__ void scalar_block_reduce(const RunArg &P, int64_t lsu
             lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
             lcnt += __shfl_xor_sync(0xffffffffu, lcnt, o);
         }
-        if (lane == 0 && self_clear) clear_wait(P);
-        if (lane == 0 && lcnt != 0) {
+        if (lane == 0 && self_clear) cleared = clear_wait(P);
+        if (lane == 0 && lcnt != 0 && cleared) {
             atomicAdd(reinterpret_cast<unsigned long long *>(P.sums), (unsigned long long)lsum);
             if (P.counts) atomicAdd(reinterpret_cast<unsigned long long *>(P.counts), (unsigned long long)lcnt);
         }
     }
+    return cleared;
 }
 
 // `given`: the stage descriptors of the parameter block.
@@ -1201,10 +1238,11 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
     // (only in kernels for few rows: the registers that it takes cost a pass over many rows up to 30 %, and the clear kernel
     // costs that one next to nothing, since the pass starts behind it)
     const bool self_clear = (AGG == AGG_SCALAR || AGG == AGG_SMEM) && DIRECT && SJQ_PV(may_clear) && P.sync;
+    uint64_t arrivals = 0;
     if (self_clear) {
         // launched while the kernel before it still runs (four joins, 400 thousand rows, interpreted: 12.4 -> 10.5 us)
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if ((int)blockIdx.x < P.clear_blocks) clear_share(P);
+        if ((int)blockIdx.x < P.clear_blocks) arrivals = clear_share(P);
     }
 
     // Stage descriptors and small direct tables -> shared memory (once per block).
@@ -1243,7 +1281,7 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
     }
     if (range_noted<AGG>() && tid == 0) range_seen = 0u;
     __syncthreads();
-    if (self_clear && tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P);
+    if (self_clear && tid == 0 && (int)blockIdx.x < P.clear_blocks) clear_told(P, arrivals);
     // launched behind the kernel that clears the results: nothing above touches them, everything below may
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // (the listing of a hashed result, or the clear of the next pass, is launched while this kernel runs and waits for its
@@ -1501,15 +1539,18 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
         }
     }
 
+    bool cleared = true; // what this block found when it waited for the clear (every thread's, or thread 0's)
     if (AGG == AGG_SCALAR) {
-        scalar_block_reduce(P, lsum, lcnt, self_clear);
+        cleared = scalar_block_reduce(P, lsum, lcnt, self_clear);
     } else if (AGG == AGG_SMEM) {
         // one global atomic per touched group per block
-        if (self_clear && tid == 0) clear_wait(P);
-        __syncthreads();
+        if (self_clear) cleared = !__syncthreads_or(tid == 0 && !clear_wait(P));
+        else __syncthreads();
         const unsigned int *ss = reinterpret_cast<const unsigned int *>(smem + P.smem_groups);
         const uint64_t ng = (uint64_t)P.num_groups;
-        if (SJQ_PV(cell_shift)) {
+        if (!cleared) {
+            // (the late clear might wipe what is added now)
+        } else if (SJQ_PV(cell_shift)) {
             // sums and counts alternate: neighbouring lanes take neighbouring words, so that a warp's adds meet 8
             // sectors and not 16 (2 M rows into a list: 1 % left, 60 groups 18.5 -> 14.4 us; half left, a thousand
             // 22.6 -> 19.9)
@@ -1526,10 +1567,10 @@ __device__ __forceinline__ void fused_body(const RunArg &P, const DStage *given,
             }
         }
     }
-    if (range_noted<AGG>() && tid == 0 && range_seen) set_status(P.status, SJQ_ERR_GROUP_RANGE);
+    if (range_noted<AGG>() && tid == 0 && range_seen && cleared) set_status(P.status, SJQ_ERR_GROUP_RANGE);
     if (self_clear) {
         if (AGG != AGG_SCALAR) __syncthreads(); // (a scalar result is added by thread 0)
-        if (tid == 0) clear_over(P);
+        if (tid == 0) clear_over(P, !cleared);
     }
 }
 

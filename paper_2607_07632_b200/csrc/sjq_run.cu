@@ -1056,6 +1056,7 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     if (self_clear) {
         P.sync = static_cast<uint64_t *>(opts.sync);
         P.epoch = next_epoch();
+        P.clear_late_ms = std::min(std::max(opts.sync_late_ms, 0), 5000);
         P.clear_counts = out->counts;
         P.clear_cells = spec->mode == SJQ_SCALAR ? 1 : spec->num_groups;
         P.clear_blocks = (int32_t)std::min<int64_t>(std::min(grid, kClearBlocks), 1 + P.clear_cells / (2 * block));

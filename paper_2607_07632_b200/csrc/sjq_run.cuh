@@ -142,15 +142,16 @@ struct RunCore {
     // Results that the pass clears itself.
     int32_t may_clear;     // a kernel for few rows whose blocks keep sums of their own: it does so where sync is given
     int32_t clear_blocks;  // blocks that share the work: 1 .. kClearBlocks
+    int32_t clear_late_ms; // milliseconds that block 0 sleeps before its share: how tests make the others' waits run out
     uint64_t *sync;
     uint64_t epoch;        // of this call alone, never 0
     int64_t *clear_counts; // counts to zero, also where they are not asked for; may be NULL
     int64_t clear_cells;   // words of sums and of clear_counts
 };
 
-// Words through which the blocks of a pass tell one another that the results are clear: the blocks that are done with
-// the whole pass, then the flags of the blocks that clear.  All are zero between two passes (the last block leaves
-// them so), whatever they held before the first.
+// Words through which the blocks of a pass tell one another that the results are clear: the number of blocks that are done
+// with the whole pass beside the number of the call, then the flags of the blocks that clear.  All are zero between two
+// passes (the last block leaves them so), whatever they held before the first.
 constexpr int kClearBlocks = SJQ_SYNC_BYTES / 8 - 1;
 
 // A kernel's parameter block: its stage descriptors, then the rest.

@@ -105,7 +105,7 @@ class _RunOpts(ctypes.Structure):
                 ("unfused_scratch", ctypes.c_void_p), ("unfused_scratch_bytes", ctypes.c_size_t),
                 ("pass_ppm", ctypes.c_int32 * (MAX_PREDS + MAX_JOINS)), ("hot_keys", ctypes.c_int32),
                 ("hot_scratch", ctypes.c_void_p), ("hot_scratch_bytes", ctypes.c_size_t), ("l0_bulk", ctypes.c_int32),
-                ("sync", ctypes.c_void_p)]
+                ("sync", ctypes.c_void_p), ("sync_late_ms", ctypes.c_int32)]
 
 
 class RunInfo(ctypes.Structure):
