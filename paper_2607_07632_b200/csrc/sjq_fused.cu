@@ -353,6 +353,11 @@ sjq_status fused_launch(int agg, bool mul, int form, int grid, int block, size_t
 }
 
 // `at_once`: the kernel behind starts beside a clear of so many blocks (of 256 threads) at most.
+// Launched while the kernel before it still runs, a clear's blocks wait in the SMs: one per SM at most, which leaves other
+// streams their room beside a long pass.  (Another stream's two joins over 2 M rows, a call, while filter and sum over 300 M
+// rows and the clear of 8 M groups take turns: 206 us with eight waiting blocks per SM, 92 so, 99 to 103 with none launched
+// early.  One per SM for every clear takes longer than it saves: 8 M groups, few rows, 28.7 us as now, 26.6 with eight
+// waiting, 39.2 with one.)
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
                         int64_t *n_groups, int32_t *status, int at_once, int sm_count, cudaStream_t stream)
 {
@@ -369,7 +374,7 @@ sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *
     cfg.blockDim = dim3(256);
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = blocks <= sm_count ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, clear_kernel, C) == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 
