@@ -120,9 +120,12 @@ bool valid_term(const sjq_term &t, int nfact, const sjq_join *joins, int njoins)
     return false;
 }
 
-// A map staged in part (see there): from so many rows on, so much of it.
+// A map staged in part (see there): from so many rows on, so much of it, in so much dynamic shared memory (a carve-out of 196
+// KB less what the system and the kernel's own arrays take); and the rows from which chains are longer.
 constexpr int64_t kPartRows = (int64_t)1 << 24;
 constexpr size_t kPartBytes = (size_t)192 << 10;
+constexpr size_t kPartCarveOut = ((size_t)196 << 10) - 1024 - 640;
+constexpr int64_t kLongChainRows = (int64_t)1 << 26;
 
 // What a filter stage costs, in picoseconds per fact row on the whole chip (148 SMs, 1.9 GHz, 6.5 TB/s).
 constexpr double kPsByte = 0.154;  // a byte of DRAM traffic
@@ -944,35 +947,57 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
             return SJQ_ERR_UNSUPPORTED;
         }
     }
-    // Every row probes a map too large for the 32 KB above and adds to a global table: the pass is bound by the L2's tags
-    // and the requests of the SMs, of which a row costs two to three.  The first part of the map, or all of it, is then
-    // staged in the shared memory that such a plan has to itself, and a probe asks the L2 only beyond it (the L1 answers
-    // next to none of those probes: its lines fill sector by sector).  192 KB leave an L1 of 32 KB; with more it is too
-    // small for the columns.  The sweep's lists with every row left, 750 KB map: a million groups, 600 M rows 5619 -> 4898
-    // us (64 KB 5516, 128 KB 5416, 176 KB 5335, 192 KB with blocks of 1024 threads 5086, 768 4996, 640 5098, 200 KB 5523);
-    // 20 thousand groups, 100 M rows 1063 -> 996; a 250 KB map, 20 M rows 190 -> 175; the same groups as a dense array, 50
-    // thousand, 1435 -> 1392; a 75 KB map, 500 thousand groups 719 -> 708; no gain for 3 M rows.  With a shared group table or register sums the L1's own rate is the bound, and
-    // the second, divergent load costs what it saves (a thousand groups, 600 K and 3 M keys: 332 -> 350, 420 -> 397).
-    int part = -1;
-    if (opts.specialise && !opts.unfused && !opts.block_threads && !opts.ctas_per_sm && opts.smem_tables == 0 && P.nq == 0 &&
-        aggp == AGG_GLOBAL && hot_stage < 0 && plan_rows >= kPartRows) {
+    // Nearly every row probes a map too large for the 32 KB above and adds to a global table: the pass is bound by the
+    // L2's tags and the requests of the SMs, of which a row costs two to three.  The first part of the map, or all of it,
+    // is then staged in shared memory, and a probe asks the L2 only beyond it.  The part is what fits beside the other
+    // staged tables in a carve-out of 196 KB, which leaves the L1 60 KB: one step more and it has 28 (a first join with
+    // a map of 10 or 30 KB, then one of 750 KB, 100 M rows: 853 and 858 us without staging, 962 and 961 beyond the step,
+    // 797 and 809 so).  With a shared group table or register sums the L1's own rate is the bound and the second,
+    // divergent load costs what it saves.  No gain for 3 M rows.
+    // A million groups as a list, every row left, one block of 768 threads, without and with, 100 M rows: maps of 35 KB
+    // 703 and 681, 150 KB 705 and 688, 250 KB 772 and 680, 500 KB 956 and 895, 750 KB 880 and 841; 17 M rows: 75 KB 143
+    // and 139, 250 KB 157 and 141, 750 KB 176 and 168.  Lists take no part of a map
+    //   of up to 1.25 parts, most of which the L1 holds (200 KB 666 and 690; from 235 KB on 782 and 671), with codes of
+    //   a byte, whose divergent loads cost more, of up to 1.75 (260 KB 839 and 854, 340 KB 903 and 873);
+    //   of more than five parts, where too few probes are answered (17 M rows: 880 KB 179 and 174, 1.2 MB 172 and 181,
+    //   1.5 MB 171 and 184), unless the group table is moderate (200 thousand groups, 1.2 MB, 166 and 159);
+    //   beside a group table of more than 64 MB, whose own misses bound them (4 M groups, 750 KB, 1066 and 1076; 2 M
+    //   groups 959 and 855).
+    // Lists of few groups and dense results gain from all of these or lose little (20 thousand groups: 200 KB 931 and
+    // 928, at 17 M rows 144 and 147; 900 KB 1055 and 961; dense, 50 thousand, 1.5 MB 1482 and 1446).
+    int part = -1, probes = 0;
+    const size_t beside_part = align_up(stage_bytes + tables, 16);
+    const size_t part_bytes = beside_part < kPartCarveOut ? std::min(kPartBytes, (kPartCarveOut - beside_part) & ~(size_t)15) : 0;
+    if (mostly_survive && !opts.unfused && !opts.block_threads && !opts.ctas_per_sm && opts.smem_tables == 0 && P.nq == 0 &&
+        aggp == AGG_GLOBAL && hot_stage < 0 && plan_rows >= kPartRows && part_bytes > kStageBytes) {
         for (int s = 0; s < nfilter; ++s) {
             const DStage &S = P.st[s];
-            const bool narrow_codes = S.op == OP_DIRECT_BITMAP || S.op == OP_DIRECT_U2 || S.op == OP_DIRECT_U4 || S.op == OP_DIRECT_U8;
-            if (narrow_codes && !S.in_smem && reach[s] >= 0.5 && (part < 0 || S.tab_bytes < P.st[part].tab_bytes)) part = s;
+            const bool bytes = S.op == OP_DIRECT_U8;
+            const bool narrow_codes = bytes || S.op == OP_DIRECT_BITMAP || S.op == OP_DIRECT_U2 || S.op == OP_DIRECT_U4;
+            const bool whole = align_up(S.tab_bytes, 16) <= part_bytes;
+            const bool some = !P.pairs || table_groups <= (int64_t)1 << 17 ||
+                              (S.tab_bytes >= kPartBytes / 4 * (bytes ? 7 : 5) && table_groups <= (int64_t)1 << 22 &&
+                               (S.tab_bytes <= 5 * part_bytes || table_groups <= (int64_t)1 << 19));
+            probes += S.kind == ST_PROBE;
+            if (narrow_codes && !S.in_smem && (whole || some) && (part < 0 || S.tab_bytes < P.st[part].tab_bytes)) part = s;
         }
     }
-    if (part >= 0 && stage_bytes + tables + kPartBytes <= smem_cap) {
+    if (part >= 0) {
         DStage &S = P.st[part];
-        const size_t whole = S.tab_bytes;
-        S.in_smem = align_up(S.tab_bytes, 16) <= kPartBytes ? kTabShared : kTabPart;
-        S.smem_off = (uint32_t)(stage_bytes + tables);
-        if (S.in_smem == kTabPart) S.tab_bytes = (uint32_t)kPartBytes;
-        tables += align_up(S.tab_bytes, 16);
-        // fewer, longer chains where every row goes all the way and most of the map is beyond the copy (512 against 768
-        // threads: the million groups 4898 and 4996 us; 300 M rows of which 80 % are left 2305 and 1961; a 250 KB map, 20 M
-        // rows 192 and 181)
-        block = reach[nfilter] >= 0.9 && P.st[part].in_smem == kTabPart && whole > 3 * kPartBytes ? 512 : 768;
+        // Fewer, longer chains where every row goes all the way, half of the probes or more go beyond the copy and no
+        // other probe fills the time.  A million groups, 100 M rows, 768 and 512 threads: 2-bit codes of 350 KB 750 and
+        // 761, 400 KB 793 and 785, 500 KB 895 and 822, 625 KB 842 and 818, 750 KB 841 and 831, 900 KB 830 and 843; 4-bit
+        // codes of 500 KB 894 and 822, 700 KB 839 and 827; bitmaps of 500 KB 893 and 836, 750 KB 817 and 828; 300 M rows,
+        // 400 KB 2467 and 2268, 600 KB 2565 and 2391.  Not so with nine rows in ten left (300 M rows, 750 KB, 2234 and
+        // 2305; 19 in 20, 100 M rows, 847 and 814), fewer rows (17 M, 400 KB, 162 and 166), codes of a byte (780 KB, 816
+        // and 934) or behind a first join (750 KB, 796 and 846).
+        const bool long_chains = S.op != OP_DIRECT_U8 && S.tab_bytes > 2 * kPartBytes && S.tab_bytes <= 4 * kPartBytes &&
+                                 probes == 1 && reach[nfilter] >= 0.95 && plan_rows >= kLongChainRows;
+        block = long_chains ? 512 : 768;
+        S.in_smem = align_up(S.tab_bytes, 16) <= part_bytes ? kTabShared : kTabPart;
+        S.smem_off = (uint32_t)beside_part;
+        if (S.in_smem == kTabPart) S.tab_bytes = (uint32_t)part_bytes;
+        tables = beside_part - stage_bytes + align_up(S.tab_bytes, 16);
         single_block = true;
     }
     P.smem_stages = 0;
