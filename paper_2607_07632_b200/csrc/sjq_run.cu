@@ -957,10 +957,11 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
     // A million groups as a list, every row left, one block of 768 threads, without and with, 100 M rows: maps of 35 KB
     // 703 and 681, 150 KB 705 and 688, 250 KB 772 and 680, 500 KB 956 and 895, 750 KB 880 and 841; 17 M rows: 75 KB 143
     // and 139, 250 KB 157 and 141, 750 KB 176 and 168.  Lists take no part of a map
-    //   of up to 1.25 parts, most of which the L1 holds (200 KB 666 and 690; from 235 KB on 782 and 671), with codes of
-    //   a byte, whose divergent loads cost more, of up to 1.75 (260 KB 839 and 854, 340 KB 903 and 873);
-    //   of more than five parts, where too few probes are answered (17 M rows: 880 KB 179 and 174, 1.2 MB 172 and 181,
-    //   1.5 MB 171 and 184), unless the group table is moderate (200 thousand groups, 1.2 MB, 166 and 159);
+    //   of less than 1 1/8 parts, most of which the L1 holds (200 KB 666 and 690, 220 KB 745 and 670), with codes of a
+    //   byte, whose divergent loads cost more, of less than 1 3/4 (260 KB 839 and 854, 340 KB 903 and 873);
+    //   of more than six parts, where too few probes are answered (17 M rows: 880 KB 179 and 174, 1.1 MB 179 and 179,
+    //   1.2 MB 172 and 181, 1.5 MB 171 and 184), unless the group table is moderate (200 thousand groups, 1.2 MB, 166
+    //   and 159);
     //   beside a group table of more than 64 MB, whose own misses bound them (4 M groups, 750 KB, 1066 and 1076; 2 M
     //   groups 959 and 855).
     // Lists of few groups and dense results gain from all of these or lose little (20 thousand groups: 200 KB 931 and
@@ -976,8 +977,8 @@ static sjq_status run_planned(const sjq_col *fact, int nfact, const sjq_pred *pr
             const bool narrow_codes = bytes || S.op == OP_DIRECT_BITMAP || S.op == OP_DIRECT_U2 || S.op == OP_DIRECT_U4;
             const bool whole = align_up(S.tab_bytes, 16) <= part_bytes;
             const bool some = !P.pairs || table_groups <= (int64_t)1 << 17 ||
-                              (S.tab_bytes >= kPartBytes / 4 * (bytes ? 7 : 5) && table_groups <= (int64_t)1 << 22 &&
-                               (S.tab_bytes <= 5 * part_bytes || table_groups <= (int64_t)1 << 19));
+                              (S.tab_bytes >= kPartBytes / 8 * (bytes ? 14 : 9) && table_groups <= (int64_t)1 << 22 &&
+                               (S.tab_bytes <= 6 * part_bytes || table_groups <= (int64_t)1 << 19));
             probes += S.kind == ST_PROBE;
             if (narrow_codes && !S.in_smem && (whole || some) && (part < 0 || S.tab_bytes < P.st[part].tab_bytes)) part = s;
         }

@@ -56,12 +56,13 @@ ROWS = 2**24 + 3
     (800_000, 3, 1_000_000, True, 0),    # 200 KB: left to the L1
     (800_000, 3, 20_000, True, 2),       # (of few groups, and of a dense result, the first 192 KB)
     (800_000, 3, 200_000, False, 2),
-    (1_000_000, 3, 1_000_000, True, 2),  # 250 KB
+    (880_000, 3, 1_000_000, True, 0),    # 215 KB
+    (890_000, 3, 1_000_000, True, 2),
     (250_000, 200, 1_000_000, True, 0),  # 250 KB, codes of a byte
     (350_000, 200, 1_000_000, True, 2),
-    (3_900_000, 3, 1_000_000, True, 2),  # 950 KB
-    (4_000_000, 3, 1_000_000, True, 0),  # 980 KB: too little of it
-    (4_000_000, 3, 200_000, True, 2),
+    (4_700_000, 3, 1_000_000, True, 2),  # 1,148 KB
+    (4_750_000, 3, 1_000_000, True, 0),  # 1,160 KB: too little of it
+    (4_750_000, 3, 200_000, True, 2),
     (2_000_000, 3, 2_097_152, True, 2),  # the largest group table
     (2_000_000, 3, 2_097_153, True, 0),
 ])
