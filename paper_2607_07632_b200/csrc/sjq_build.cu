@@ -665,20 +665,24 @@ __device__ __forceinline__ void hash_rows(const BuildTask &B, const DimFilters &
 template <typename K>
 using UsualQuad = RowSet<K, int32_t, 1, 1>;
 
-// USUAL: every dimension of the launch has at most one payload, of 32 bits (the other forms need more registers).
-template <bool USUAL>
-constexpr int kHashPerSm = USUAL ? 5 : 4;
-template <bool USUAL>
-__global__ void __launch_bounds__(kHashThreads, kHashPerSm<USUAL>) hash_build_kernel(const __grid_constant__ BuildParams P)
+// FORMS: what the dimensions of the launch are, usual (at most one payload, of 32 bits), others, which need more registers,
+// or both.  A kernel that holds both keeps the usual ones at their 32-bit payloads and costs the others 1 to 3 %: tables of
+// 8 M rows, one in four kept, beside one of 1,000 of the other form, others alone and both: usual 153 and 141 us, the other
+// 163 and 166; 8 M rows of each 336 and 340.
+constexpr int kFormUsual = 1, kFormOther = 2;
+template <int FORMS>
+constexpr int kHashPerSm = FORMS == kFormUsual ? 5 : 4;
+template <int FORMS>
+__global__ void __launch_bounds__(kHashThreads, kHashPerSm<FORMS>) hash_build_kernel(const __grid_constant__ BuildParams P)
 {
     __shared__ __align__(16) unsigned char queues[kHashThreads / 32][kHashQueue * 16];
     const BuildTask &B = P.task[task_of_block(P.task, P.ntasks)];
     void *const queue = queues[threadIdx.x >> 5];
     cudaGridDependencySynchronize(); // the tables' memory is prepared by the kernel before this one
-    if constexpr (USUAL) {
+    if (FORMS == kFormUsual || (FORMS != kFormOther && B.usual)) {
         if (!B.rows.key64) hash_rows<UsualQuad<int32_t>, uint32_t>(B, P.filters, queue);
         else hash_rows<UsualQuad<int64_t>, uint32_t>(B, P.filters, queue);
-    } else {
+    } else if constexpr (FORMS != kFormUsual) {
         if (!B.rows.key64) hash_rows<Wide<int32_t>, uint64_t>(B, P.filters, queue);
         else hash_rows<Wide<int64_t>, uint64_t>(B, P.filters, queue);
     }
@@ -1240,6 +1244,12 @@ bool launch_behind(void (*kernel)(BuildParams), BuildParams &B, int threads, int
     return cudaLaunchKernelEx(&cfg, kernel, B) == cudaSuccess;
 }
 
+template <int FORMS>
+bool launch_hash_build(BuildParams &H, int sm_count, cudaStream_t stream)
+{
+    return launch_behind(hash_build_kernel<FORMS>, H, kHashThreads, kHashPerSm<FORMS>, sm_count, stream);
+}
+
 // Enqueue the fills and the builds of a batch: one launch for the direct tables, one for those with open addressing.
 sjq_status build_launch(const sjq_dim_desc *dims, int ndims, const sjq_dim_layout *layouts, void *const *table_mem,
                         const size_t *table_bytes, int32_t *const *status_dev, bool clear_status, void *stream_,
@@ -1281,10 +1291,11 @@ sjq_status build_launch(const sjq_dim_desc *dims, int ndims, const sjq_dim_layou
         }
         if (ok && H.ntasks) {
             H.filters = B.filters;
-            bool usual = true;
-            for (int i = 0; i < H.ntasks; ++i) usual = usual && H.task[i].usual;
-            ok = usual ? launch_behind(hash_build_kernel<true>, H, kHashThreads, kHashPerSm<true>, dev.sm_count, stream)
-                       : launch_behind(hash_build_kernel<false>, H, kHashThreads, kHashPerSm<false>, dev.sm_count, stream);
+            int64_t usual = 0, other = 0;
+            for (int i = 0; i < H.ntasks; ++i) (H.task[i].usual ? usual : other) += H.task[i].rows.n;
+            ok = other == 0     ? launch_hash_build<kFormUsual>(H, dev.sm_count, stream)
+                 : usual > other ? launch_hash_build<kFormUsual | kFormOther>(H, dev.sm_count, stream)
+                                 : launch_hash_build<kFormOther>(H, dev.sm_count, stream);
             ++launches;
         }
         tables[0]->launches = launches;
