@@ -25,8 +25,8 @@ struct ClearParams {
 __global__ void __launch_bounds__(256) clear_kernel(const ClearParams C)
 {
     // Launched while the kernel before it still runs: that one, and all before it, first; then the pass may start, whose
-    // reads of its tables rely on it.  (Back to back: filter and sum, 6 M rows 16.5 -> 15.3 us; two joins, 60 M rows 84.2
-    // -> 82.1.)
+    // reads of its tables rely on it.  (Filter and sum, 6 M rows, calls back to back: 18.4 -> 16.5 us; a call that nothing
+    // runs before gains nothing.)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (C.at_once) asm volatile("griddepcontrol.launch_dependents;");
     const int64_t stride = (int64_t)blockDim.x * gridDim.x;
@@ -355,9 +355,13 @@ sjq_status fused_launch(int agg, bool mul, int form, int grid, int block, size_t
 // `at_once`: the kernel behind starts beside a clear of so many blocks (of 256 threads) at most.
 // Launched while the kernel before it still runs, a clear's blocks wait in the SMs: one per SM at most, which leaves other
 // streams their room beside a long pass.  (Another stream's two joins over 2 M rows, a call, while filter and sum over 300 M
-// rows and the clear of 8 M groups take turns: 206 us with eight waiting blocks per SM, 92 so, 99 to 103 with none launched
-// early.  One per SM for every clear takes longer than it saves: 8 M groups, few rows, 28.7 us as now, 26.6 with eight
-// waiting, 39.2 with one.)
+// rows and the clear of 8 M groups take turns: 206 us with eight waiting blocks per SM, 87 to 92 so, 99 to 103 with none
+// launched early.)  The clear of a list's cells is held to that many blocks up to 32 MB (back to back, in its turn and so:
+// a hundred thousand groups, 100 thousand rows 10.0 and 9.5 us; merge of eight lists of 58 thousand 22.2 and 21.8).  A dense
+// result, which the pass adds to at once, needs all its blocks, and from half a block per SM on its clear waits for its turn
+// (2 M rows, 5 thousand groups 6.65 in its turn and 6.35 early, 30 thousand 6.75 and 6.9, 60 thousand 6.75 and 7.05; a
+// million 8.9 and, with one block per SM, 13.2; eight million, few rows, 28.7 and 39.2).
+constexpr size_t kEarlyList = (size_t)32 << 20;
 sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *gkeys, int64_t gslots,
                         int64_t *n_groups, int32_t *status, int at_once, int sm_count, cudaStream_t stream)
 {
@@ -366,6 +370,8 @@ sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     if (blocks < 1) blocks = 1;
     const ClearParams C{sums, counts, cells, gkeys, gslots, n_groups, status, blocks <= at_once ? 1 : 0};
+    const bool list = gkeys != nullptr;
+    if (list && blocks > sm_count && ((size_t)cells + (size_t)gslots) * 8 <= kEarlyList) blocks = sm_count;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -374,7 +380,7 @@ sjq_status clear_launch(int64_t *sums, int64_t *counts, int64_t cells, int64_t *
     cfg.blockDim = dim3(256);
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = blocks <= sm_count ? 1 : 0;
+    cfg.numAttrs = (list ? blocks : 2 * blocks) <= sm_count ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, clear_kernel, C) == cudaSuccess ? SJQ_OK : SJQ_ERR_CUDA;
 }
 
