@@ -417,7 +417,8 @@ typedef struct sjq_run_opts {
 typedef struct sjq_run_info {
     int32_t nstages;
     int32_t order[SJQ_MAX_PREDS + SJQ_MAX_JOINS + 8]; /* as in sjq_run_opts.order; -1 = plain column load */
-    int32_t stage_in_smem[SJQ_MAX_PREDS + SJQ_MAX_JOINS + 8];
+    int32_t stage_in_smem[SJQ_MAX_PREDS + SJQ_MAX_JOINS + 8]; /* 0 the table is probed in global memory, 1 in a copy in
+                                                                 shared memory, 2 its first part is such a copy */
     int32_t first_sparse_stage; /* stages before this one filter thread-owned rows (level 0); later stages run
                                    on compacted survivors; 0 = no queues at all */
     int32_t reserved_levels;    /* number of queue-fed levels (the last one is the final level) */

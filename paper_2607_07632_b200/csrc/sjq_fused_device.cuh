@@ -1123,7 +1123,10 @@ __device__ __forceinline__ uint32_t queue_base(int l)
 constexpr int kClearSpins = 1 << 20;
 constexpr uint64_t kClearArrivals = (1ull << 20) - 1, kClearLate = 1ull << 20; // the rest of the word: the call
 constexpr int kClearCall = 21;
-__device__ __forceinline__ bool clear_of_call(const RunArg &P, uint64_t word) { return ((word ^ (P.epoch << kClearCall)) >> kClearCall) == 0; }
+__device__ __forceinline__ bool clear_of_call(const RunArg &P, uint64_t word)
+{
+    return ((word ^ (P.epoch << kClearCall)) >> kClearCall) == 0;
+}
 __device__ __forceinline__ uint64_t clear_swap(const RunArg &P, uint64_t from, uint64_t to)
 {
     return atomicCAS(reinterpret_cast<unsigned long long *>(P.sync), (unsigned long long)from, (unsigned long long)to);
@@ -1182,9 +1185,12 @@ __device__ __forceinline__ void clear_over(const RunArg &P, bool late)
     if (!late) {
         word = atomicAdd(reinterpret_cast<unsigned long long *>(P.sync), 1ull);
     } else {
-        uint64_t found = 0, now; // (a try fails because another block has arrived: bounded by the grid)
-        while ((now = clear_swap(P, found, word = ((clear_of_call(P, found) ? found : P.epoch << kClearCall) | kClearLate) + 1)) != found) found = now;
-        --word;
+        for (uint64_t found = 0;;) { // (a try fails because another block has arrived: bounded by the grid)
+            word = (clear_of_call(P, found) ? found : P.epoch << kClearCall) | kClearLate;
+            const uint64_t now = clear_swap(P, found, word + 1);
+            if (now == found) break;
+            found = now;
+        }
     }
     if ((word & kClearArrivals) != gridDim.x - 1) return;
     __threadfence();
