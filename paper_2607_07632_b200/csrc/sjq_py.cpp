@@ -17,7 +17,7 @@ namespace {
 #define SJQ_NAMES(X)                                                                                                   \
     X(data_ptr) X(dtype) X(is_cuda) X(is_contiguous) X(dim) X(numel) X(col) X(op) X(lo) X(hi) X(values) X(handle)       \
     X(terms) X(offset) X(modulo) X(src) X(a) X(b) X(mult) X(x) X(y) X(want_count) X(sums) X(counts) X(keys)             \
-    X(n_groups) X(status_dev) X(workspace) X(sync) X(element_size) X(get_device) X(info) X(block_threads)               \
+    X(n_groups) X(status_dev) X(workspace) X(sync) X(nbytes) X(get_device) X(info) X(block_threads)                     \
     X(ctas_per_sm) X(eager_loads) X(agg_path)                                                                          \
     X(smem_tables) X(compaction) X(accumulate) X(order) X(events) X(cuda_event) X(specialise) X(rows_per_lane)          \
     X(no_filter_bitmap) X(host_copy_all) X(dense_slots) X(group_hash_always) X(warp_agg) X(unfused_scratch)             \
@@ -262,17 +262,17 @@ bool read_sync(PyObject *result, int64_t device, void **sync, bool *small)
         PyErr_Clear();
         return true;
     }
-    int64_t cells = 0, width = 0, at = 0;
-    if (!pointer_of(t.p, sync, &cells)) return false;
+    int64_t bytes = 0, at = 0;
+    if (!pointer_of(t.p, sync)) return false;
     if (t.p == Py_None) return true;
-    if (!call_int(t.p, N.element_size, &width) || !call_int(t.p, N.get_device, &at)) return false;
+    if (!get_int(t.p, N.nbytes, &bytes) || !call_int(t.p, N.get_device, &at)) return false;
     Ref contiguous(PyObject_CallMethodNoArgs(t.p, N.is_contiguous));
     if (!contiguous) return false;
     if (at != device || contiguous.p != Py_True) {
         PyErr_SetString(PyExc_ValueError, "the sync words of a result must be a contiguous tensor on the device of its columns");
         return false;
     }
-    *small = cells * width < SJQ_SYNC_BYTES;
+    *small = bytes < SJQ_SYNC_BYTES;
     return true;
 }
 

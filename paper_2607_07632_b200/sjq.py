@@ -897,7 +897,7 @@ def _sync_pointer(res, device) -> Optional[int]:
         return None
     if sync.device != device or not sync.is_contiguous():
         raise ValueError("the sync words of a result must be a contiguous tensor on the device of its columns")
-    if sync.numel() * sync.element_size() < SYNC_BYTES:
+    if sync.nbytes < SYNC_BYTES:
         raise SjqError(5, "sjq_run_host")  # SJQ_ERR_BUFFER_SMALL
     return sync.data_ptr()
 

@@ -19,8 +19,9 @@ class Words(FakeColumn):
         super().__init__(n, **kw)
         self.width, self.at, self.device = width, device, torch.device("cpu" if device < 0 else "cuda:%d" % device)
 
-    def element_size(self):
-        return self.width
+    @property
+    def nbytes(self):
+        return self.n * self.width
 
     def get_device(self):
         return self.at
